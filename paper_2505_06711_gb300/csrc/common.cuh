@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -278,6 +279,22 @@ struct GraphSlot {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
+// Device memory of a context's lists: a stream-ordered pool, so that building and
+// freeing one structure after another re-uses blocks instead of mapping and
+// unmapping memory for each of its ~45 buffers (cudaMalloc + cudaFree of a
+// 4,000-atom list: 0.8 ms of a 1.37 ms build + evaluation).  It keeps at most
+// kKeep unused bytes and gives everything back with the last of its context and
+// lists (each holds a reference).  Blocks are taken on the building context's
+// stream.  They go back on the pool's own stream after a device synchronisation (as
+// cudaFree implies one), so that no stream of the caller needs to outlive a list
+// and a block is never handed on while work of any stream may still use it.
+struct ListPool {
+    static constexpr uint64_t kKeep = 512ull << 20;
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;
+    static std::shared_ptr<ListPool> create();  // null when the device has no memory pools
+    ~ListPool();
+};
 enum GraphSlotId { GS_REBUILD = 0, GS_EVAL, GS_HOST_REBUILD, GS_HOST_EVAL, GS_COUNT };
 
 }  // namespace reann
@@ -358,9 +375,11 @@ struct reann_nlist {
     int rank_grid[3] = {1, 1, 1};
     std::vector<int64_t> rank_local, rank_ghost, rank_remote;
     std::vector<void*> allocs;
-    // stream-ordered allocation (serving builds): blocks come from mem_pool on
-    // alloc_stream and go back with cudaFreeAsync on the same stream, so neither
-    // side waits for unrelated device work; null pool: cudaMalloc / cudaFree
+    // stream-ordered allocation: blocks come from mem_pool on alloc_stream.  Serving
+    // builds return them with cudaFreeAsync on the same stream, so neither side waits
+    // for unrelated device work; other lists as described at ListPool (list_pool set).
+    // Null mem_pool: cudaMalloc / cudaFree.
+    std::shared_ptr<reann::ListPool> list_pool;
     cudaMemPool_t mem_pool = nullptr;
     cudaStream_t alloc_stream = nullptr;
 };
@@ -379,7 +398,9 @@ struct reann_ctx {
     void* d_fp8 = nullptr;         // FP8 E4M3 weight images for the tensor-core networks
     reann::TcTable tc{};
     int* d_flags = nullptr;        // reann::NFLAGS ints
-    int* h_flags = nullptr;        // pinned mirror
+    int* h_flags = nullptr;        // pinned mirror, then kHostInts ints for the build's sizes
+    static constexpr int kHostInts = reann::MAX_ELEM + 2;
+    std::shared_ptr<reann::ListPool> list_pool;  // created by the first build
     std::string err;
     int num_sms = 0;
     // a non-blocking stream the MD step graph and the replayed rebuild / evaluation graphs run on

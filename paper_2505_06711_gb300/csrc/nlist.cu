@@ -761,8 +761,18 @@ static cudaError_t counting_sort(cudaStream_t s, const int* gate, int64_t n, int
 void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes) {
     void* p = nullptr;
     bytes = std::max<size_t>(bytes, 1);
-    const cudaError_t e = nl->mem_pool ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream)
-                                       : cudaMalloc(&p, bytes);
+    auto take = [&] {
+        return nl->mem_pool ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream) : cudaMalloc(&p, bytes);
+    };
+    cudaError_t e = take();
+    if (e != cudaSuccess && nl->list_pool) {  // give the pool's unused blocks back and try again
+        (void)cudaGetLastError();
+        cudaMemPoolTrimTo(nl->mem_pool, 0);
+        e = take();
+    }
+    // after the build the block may be used on any stream
+    if (e == cudaSuccess && nl->list_pool && nl->alloc_stream == nl->list_pool->stream)
+        e = cudaStreamSynchronize(nl->alloc_stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
@@ -857,9 +867,8 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
         !w.tsum)
         return set_error(ctx, REANN_E_NOMEM, "neighbour-list allocation failed");
     {
-        const int32_t state0[4] = {1, 0, 0, 0};  // this build sorts; rebuilds count from 1
+        static const int32_t state0[4] = {1, 0, 0, 0};  // this build sorts; rebuilds count from 1
         REANN_CUDA_TRY(ctx, cudaMemcpyAsync(w.rb_state, state0, sizeof(state0), cudaMemcpyHostToDevice, s));
-        REANN_CUDA_TRY(ctx, cudaStreamSynchronize(s));  // state0 lives on this stack frame
     }
     REANN_CUDA_TRY(ctx, cudaMemcpyAsync(w.species_c, species, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
     REANN_CUDA_TRY(ctx, cudaMemsetAsync(w.counts, 0, sizeof(int32_t) * nkeys, s));  // kept zero between sorts
@@ -867,16 +876,16 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
                                         sizeof(int32_t) * std::max(scan_status_words(nkeys), scan_status_words(n)), s));
     REANN_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_flags, 0, sizeof(int) * NFLAGS, s));
     REANN_CUDA_TRY(ctx, stage_sort_and_count(s, nl, pos, ctx->d_flags, nullptr, nullptr, nullptr));
-    // sizes: element ranges of the internal order and the ghost count
-    std::vector<int32_t> es(nl->n_elem + 1);
+    // sizes: element ranges of the internal order and the ghost count, read back together
+    int32_t* es = ctx->h_flags + NFLAGS;
     const int64_t nbins = nkeys / nl->n_elem;
-    for (int e = 0; e <= nl->n_elem; ++e)
-        REANN_CUDA_TRY(ctx, cudaMemcpyAsync(&es[e], w.start + (int64_t)e * nbins, sizeof(int32_t),
+    for (int e = 0; e <= nl->n_elem; ++e)  // (pinned: the copies queue up, one synchronisation below)
+        REANN_CUDA_TRY(ctx, cudaMemcpyAsync(es + e, w.start + (int64_t)e * nbins, sizeof(int32_t),
                                             cudaMemcpyDeviceToHost, s));
-    int32_t G = 0;
-    REANN_CUDA_TRY(ctx, cudaMemcpyAsync(&G, w.goff + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    REANN_CUDA_TRY(ctx, cudaMemcpyAsync(es + MAX_ELEM + 1, w.goff + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     REANN_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(int) * NFLAGS, cudaMemcpyDeviceToHost, s));
     REANN_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    const int32_t G = es[MAX_ELEM + 1];
     if (ctx->h_flags[FLAG_SPECIES]) return set_error(ctx, REANN_E_ARG, "species index out of range");
     if (ctx->h_flags[FLAG_GEOM]) return set_error(ctx, REANN_E_GEOM, "non-finite atom position");
     for (int e = 0; e <= nl->n_elem; ++e) nl->elem_start[e] = es[e];

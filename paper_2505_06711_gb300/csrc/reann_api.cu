@@ -28,6 +28,33 @@ int set_error(reann_ctx* ctx, int code, const std::string& msg) {
 
 }  // namespace reann
 
+std::shared_ptr<reann::ListPool> reann::ListPool::create() {
+    int dev = 0, has = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&has, cudaDevAttrMemoryPoolsSupported, dev) != cudaSuccess || !has)
+        return nullptr;
+    std::shared_ptr<ListPool> p(new (std::nothrow) ListPool);
+    if (!p) return nullptr;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = kKeep;
+    if (cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaMemPoolCreate(&p->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+reann::ListPool::~ListPool() {
+    if (stream) cudaStreamSynchronize(stream);
+    if (pool) cudaMemPoolDestroy(pool);
+    if (stream) cudaStreamDestroy(stream);
+}
+
 namespace {
 
 constexpr int64_t expected_params(int n_elem, int T, bool pairs = false) {
@@ -161,7 +188,13 @@ void free_nlist(reann_nlist* nl) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         if (g.graph) cudaGraphDestroy(g.graph);
     }
+    bool idle = true;  // (as with cudaFree, nothing is given back where the device cannot be waited for)
+    if (nl->list_pool) {
+        idle = cudaDeviceSynchronize() == cudaSuccess;
+        nl->alloc_stream = nl->list_pool->stream;
+    }
     for (void* p : nl->allocs) {
+        if (!idle) break;
         if (nl->mem_pool)
             cudaFreeAsync(p, nl->alloc_stream);
         else
@@ -441,7 +474,7 @@ extern "C" int reann_ctx_create(const reann_model* model, void* cuda_stream, rea
     if (M.pairs && upload_pair_table() != cudaSuccess) return fail(REANN_E_CUDA);
     if (cudaMalloc(&ctx->d_flags, sizeof(int) * NFLAGS) != cudaSuccess) return fail(REANN_E_NOMEM);
     if (cudaMemset(ctx->d_flags, 0, sizeof(int) * NFLAGS) != cudaSuccess) return fail(REANN_E_CUDA);
-    if (cudaMallocHost(&ctx->h_flags, sizeof(int) * NFLAGS) != cudaSuccess) return fail(REANN_E_NOMEM);
+    if (cudaMallocHost(&ctx->h_flags, sizeof(int) * (NFLAGS + reann_ctx::kHostInts)) != cudaSuccess) return fail(REANN_E_NOMEM);
     *out = ctx;
     return REANN_OK;
 }
@@ -540,11 +573,20 @@ int build_list(reann_ctx* ctx, int64_t n_atoms, const double* pos, const int32_t
     nl->T = ctx->model.T;
     nl->r_c = r_c;
     nl->skin = skin;
+    if (!mem_pool && eval_buffers) {  // a caller's list (the others are freed again by their own builds)
+        if (!ctx->list_pool) ctx->list_pool = ListPool::create();
+        nl->list_pool = ctx->list_pool;
+        if (nl->list_pool) mem_pool = nl->list_pool->pool;
+    }
     nl->mem_pool = mem_pool;
     nl->alloc_stream = ctx->stream;
     int rc = make_geometry(ctx, cell, r_c + skin, &nl->geom);
     if (!rc) rc = build_nlist_device(ctx, nl, pos, species);
     if (!rc && eval_buffers) rc = alloc_eval_buffers(ctx, nl);
+    if (!rc && nl->list_pool) {  // from here on the list's memory is valid on every stream
+        if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = set_error(ctx, REANN_E_CUDA, "list build failed");
+        nl->alloc_stream = nl->list_pool->stream;
+    }
     if (rc) {
         cudaStreamSynchronize(ctx->stream);
         free_nlist(nl);

@@ -1,0 +1,101 @@
+"""Lists built and freed one after another re-use device memory of their context's pool.
+
+Results must not depend on what a block held before, a list may outlive its context and the
+stream it was built on, and lists of several threads share no block.
+"""
+
+from __future__ import annotations
+
+import threading
+
+import numpy as np
+import pytest
+
+from synth import fcc_box, make_model, water_box
+
+pytestmark = pytest.mark.gpu
+
+
+def _evaluate(pot, s):
+    import torch
+
+    sy = pot.system(s.pos, s.species, s.cell)
+    sy.evaluate(virial=True)
+    sy.check()
+    out = float(sy.energy), sy.forces.cpu().numpy().copy(), sy.virial.cpu().numpy().copy()
+    sy.close()
+    return out
+
+
+def _same(a, b):
+    return a[0] == b[0] and np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+
+
+def test_reused_memory_gives_the_same_results():
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=3)
+    boxes = [water_box(64, seed=1), fcc_box(8, seed=2), water_box(400, seed=3), fcc_box(3, seed=4)]
+    alone = []
+    for s in boxes:
+        pot = Potential(spec)
+        alone.append(_evaluate(pot, s))
+        pot.close()
+    pot = Potential(spec)
+    for order in ([0, 1, 2, 3], [3, 2, 1, 0], [2, 0, 3, 1]):
+        for k in order:
+            assert _same(_evaluate(pot, boxes[k]), alone[k]), k
+    pot.close()
+
+
+def test_list_outlives_its_context_and_stream():
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=2)
+    s = water_box(100, seed=5)
+    other = Potential(spec)
+    want = _evaluate(other, s)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        pot = Potential(spec, stream=stream)
+        sy = pot.system(s.pos, s.species, s.cell)
+    pot.close()
+    del stream
+    sy.pot = other  # evaluate the list on another context
+    sy.evaluate(virial=True)
+    sy.check()
+    assert _same((float(sy.energy), sy.forces.cpu().numpy(), sy.virial.cpu().numpy()), want)
+    sy.close()
+    other.close()
+
+
+def test_threads_build_and_free_together():
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=2)
+    boxes = [water_box(50 + 13 * k, seed=k) for k in range(4)]
+    pot = Potential(spec)
+    want = [_evaluate(pot, s) for s in boxes]
+    pot.close()
+    bad = []
+
+    def work(k):
+        import torch
+
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            mine = Potential(spec, stream=stream)
+            for _ in range(6):
+                got = _evaluate(mine, boxes[k])
+                if not _same(got, want[k]):
+                    bad.append(k)
+            mine.close()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
