@@ -487,7 +487,7 @@ def source_sha(name: str) -> str:
 
 REGION_SOURCE = {
     "density_fwd": "density.cu", "density_adj": "density.cu", "bbar": "density.cu", "mlp_fwd": "mlp_fp32.cu",
-    "mlp_bwd": "mlp_fp32.cu", "nlist_rebuild": "nlist.cu", "live_edges": "nlist.cu",
+    "mlp_bwd": "mlp_fp32.cu", "nlist_rebuild": "nlist.cu", "live_edges": "density.cu",
 }
 
 

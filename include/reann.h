@@ -326,7 +326,7 @@ int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const double* pos,
  *   reann_serve_create  reserve a pool of max_atoms owned slots, max_ghosts
  *                       ghost slots, max_structures structures and neighbour
  *                       rows of `stride` entries on ctx's device; its device
- *                       memory (about 3.5 kB per atom at T = 3 plus 8 B per row
+ *                       memory (about 3.5 kB per atom at T = 3 plus 36 B per row
  *                       entry) is the admission budget.  Synchronous.
  *   reann_serve_submit  build the structure's list with build_ctx (its own
  *                       stream, so builds overlap pool launches in flight),
@@ -419,7 +419,7 @@ int64_t reann_energy_sum_noalloc_max_atoms(void);
 
 /*
  * Per-region event profile: when enabled, every region of the evaluation
- * (neighbour rebuild, position refresh, live-edge filter, coefficient init,
+ * (neighbour rebuild, position refresh, live edges and their records, coefficient init,
  * ghost gathers, density forward, networks forward, energy sum, networks
  * backward, bbar, density adjoint, output scatter) is bracketed by CUDA events
  * on the context's stream.  Enabling or disabling resets the totals.

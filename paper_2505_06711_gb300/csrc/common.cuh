@@ -26,8 +26,8 @@ constexpr int NFEAT_P = (LMAX + 1) * NORB_P * (NORB_P + 1) / 2;
 constexpr int NB = NANG * NPHI;           // 80 per-atom density partials b_{a,m}
 // Adjoint record of an atom (the reverse pass's per-atom row): 3 lines of
 // 128 B, line v / 4 holding value v of channel m at float 4 m + v % 4, with
-// values v = 0..9 the adjoint bbar_{a = v, m}, v = 10 the coefficient c_m of
-// the layer and v = 11 zero.  Channel m's 12 values are then 3 aligned float4s,
+// values v = 0..9 the adjoint bbar_{a = v, m} (v = 4..6, the squares, doubled:
+// rec_scale), v = 10 the coefficient c_m of the layer and v = 11 zero.  Channel m's 12 values are then 3 aligned float4s,
 // one per line, so the 8 lanes of an atom read one full line per load.
 constexpr int NREC = 3 * 4 * NPHI;  // 96 floats
 __host__ __device__ constexpr int rec_at(int v, int m) { return (v >> 2) * (4 * NPHI) + 4 * m + (v & 3); }
@@ -41,7 +41,9 @@ constexpr int MLP_TILE = 64;  // rows per FP32 network tile
 #ifdef __CUDACC__
 __device__ __forceinline__ int ang_l(int a) { return a == 0 ? 0 : (a < 4 ? 1 : 2); }
 __device__ __forceinline__ float ang_w(int a) { return a >= 7 ? 2.f : 1.f; }
-__device__ __forceinline__ float ang_sign(int a) { return (a >= 1 && a <= 3) ? -1.f : 1.f; }
+// factor of bbar_a in the adjoint records: the squares' adjoints are kept doubled, so
+// that the quadratic's gradient needs no doubled coordinates
+__device__ __forceinline__ float rec_scale(int a) { return (a >= 4 && a <= 6) ? 2.f : 1.f; }
 
 // Programmatic dependent launch.  A kernel started by launch_pdl() may become
 // resident while the previous kernel on its stream is still draining; before
@@ -176,7 +178,9 @@ struct Radial {
     float alpha_hi, alpha_lo;  // alpha
     float tad_hi, tad_lo;      // 2 alpha Delta, Delta = r_c / (N_phi - 1)
     float mu_hi[NPHI], mu_lo[NPHI];      // Gaussian centres m Delta
+    float two_a_mu[NPHI];                // 2 alpha m Delta
     float kap_hi[NPHI], kap_lo[NPHI];    // exp(-alpha Delta^2 (2m+1)) for the Gaussian recurrence
+    float scale, unscale;                // 2^s, 2^-s: s = 0 unless exp(-alpha r_c^2) f_c would leave the normal range
 };
 
 // Cell geometry for the neighbour build (FP64) and ghost refresh.
@@ -327,15 +331,19 @@ struct reann_nlist {
     int32_t* g_shift = nullptr;    // g_cap, packed (n0+128) | (n1+128)<<8 | (n2+128)<<16
     int32_t* nbr = nullptr;        // N x stride ext slots
     int32_t* nbr_cnt = nullptr;    // N
-    int32_t* live = nullptr;       // N x stride, live (d < r_c) entries first
-    int32_t* live_cnt = nullptr;   // N
+    int32_t* live_cnt = nullptr;   // N live (d < r_c) entries of each row
+    // records of the live edges, edge_rows x stride (k_edges): normally one row per atom, fewer
+    // when device memory is short (the passes then rebuild them for one run of rows at a time)
+    int64_t edge_rows = 0;
+    float4* edge_xyzj = nullptr;   // r_j - r_i, j
+    float2* edge_phi = nullptr;    // first Gaussian x cutoff, recurrence factor
+    float2* edge_der = nullptr;    // 1/d, radial derivative part
     reann::Tile* tiles = nullptr;  // MLP tiles (64 rows, FP32 networks)
     std::vector<reann::Tile> tiles128_h;
     reann::Tile* tiles128 = nullptr;  // 128-row tiles of the tensor-core networks
     double* pos_ref = nullptr;     // N x 3 FP64 caller positions at build (caller order)
     // per-evaluation state (resident)
-    float4* pos_hi = nullptr;      // N + g_cap
-    float4* pos_lo = nullptr;      // N + g_cap
+    float4* pos = nullptr;         // (N + g_cap) x 2: hi, lo parts of each slot's position (one 32 B sector)
     float* coef = nullptr;         // T x (N + g_cap) x 8
     float* rho = nullptr;          // T x N x 48
     float* bck = nullptr;          // T x N x 80
@@ -430,11 +438,14 @@ int set_error(reann_ctx* ctx, int code, const std::string& msg);
 
 // Launches k with the programmatic-stream-serialization attribute; every
 // kernel of the library calls pdl_enter() first.  In a captured graph the
-// attribute becomes a programmatic edge.  The network kernels are launched
-// without it: their grids are one wave of tiles, and blocks that become
-// resident while the previous kernel drains pile up on the SMs that freed
-// first (measured: FP32 step 0.489 -> 0.502 ms with them, 0.489 -> 0.487 ms
-// for the edge and rebuild kernels alone).
+// attribute becomes a programmatic edge.  The network kernels and the two edge
+// passes are launched without it.  Blocks of the networks' one-wave grids that
+// become resident while the previous kernel drains pile up on the SMs that freed
+// first (measured: FP32 step 0.489 -> 0.502 ms with them).  Blocks of an edge pass
+// that become resident beside a network kernel keep that kernel's split of the
+// SM's 256 KB into shared memory and L1, up to 207 KB of shared memory, and leave
+// the gathers of the whole pass little L1 (1,048,576 atoms: reverse pass 1.17 -> 1.62 ms
+// with the attribute; 24,576: evaluation 0.342 -> 0.349 ms; 192: no difference).
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute at[1];
@@ -489,21 +500,24 @@ const int32_t* ghost_count_ptr(const reann_nlist* nl);
 // with c0: also the first layer's coefficients of every slot (k_init_coef's work)
 cudaError_t launch_refresh_positions(cudaStream_t s, const reann_nlist* nl, const double* pos,
                                      const float* c0 = nullptr);
-cudaError_t launch_live_edges(cudaStream_t s, const reann_nlist* nl, float rc2, int* flags);
 int export_nlist(reann_ctx* ctx, const reann_nlist* nl, int64_t cap, int32_t* i, int32_t* j, int32_t* n, int64_t* count);
 
 // density (density.cu)
 cudaError_t launch_init_coef(cudaStream_t s, const reann_nlist* nl, const float* c0);
 cudaError_t launch_gather_ghost_rows(cudaStream_t s, const reann_nlist* nl, float* base, int width);
-cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, const float* W, const float* coef,
-                               float* rho, float* bck, bool pairs = false);
+// the edge kernels cover rows [row0, row0 + rows); record row k belongs to row row0 + k
+cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                         int* flags);
+cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                               const float* W, const float* coef, float* rho, float* bck, bool pairs = false);
 cudaError_t launch_bbar(cudaStream_t s, const reann_nlist* nl, const float* W, const float* bck, const float* rhobar,
                         const float* coef, float* rec, bool pairs = false, GhostOut gh = {});
 // forces / atom_energy (caller order): the last reverse layer writes the outputs itself;
 // first: the first reverse layer writes grad (and vir) instead of accumulating
-cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radial& r, const float* rec, float* cbar,
-                               float* grad, bool want_cbar, int* flags, float* vir = nullptr,
-                               float* forces = nullptr, float* atom_energy = nullptr, bool first = false);
+cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                               const float* rec, const float* bck, float* cbar, float* grad, bool want_cbar,
+                               float* vir = nullptr, float* forces = nullptr, float* atom_energy = nullptr,
+                               bool first = false);
 cudaError_t upload_pair_table();
 cudaError_t launch_virial_sum(cudaStream_t s, const reann_nlist* nl, const float* vir, double* partial, double* out);
 cudaError_t launch_energy_sum(cudaStream_t s, const reann_nlist* nl, double* energy);

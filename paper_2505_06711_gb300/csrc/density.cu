@@ -14,17 +14,17 @@
 //   the paper's ghost-gradient exchange as a vector-Jacobian product, Sec. 2.2).
 // No atomics: every output row is written by the lanes of its own centre atom.
 //
-// Forward layout: a quad of 4 lanes per centre atom (8 atoms per warp).  Each
-// lane walks every 4th live neighbour, whose hi/lo FP32 position (32 B) and
-// coefficients (32 B) are copied into shared memory with cp.async one edge
-// ahead, and accumulates the 80 products in registers; a butterfly
-// reduce-scatter leaves 20 of the 80 b values in each lane, which then
-// contracts its 4 orbitals from shared memory.  The adjoint gathers each
-// neighbour's 384 B adjoint record (bbar and c) and uses 8 lanes per atom
-// instead (below).
+// Edge records.  The list of live (d < r_c) edges and everything about an edge
+// that is the same in all 2T edge passes of an evaluation is computed once per
+// evaluation (k_edges): r = r_j - r_i and j, the first Gaussian times the cutoff
+// and the factor of the Gaussian recurrence, 1/d and the cutoff's logarithmic
+// derivative (32 B per live edge, in the row order of the list).  The passes
+// stream the records of their atom (coalesced) and gather only what belongs to
+// the neighbour: its coefficients (forward) or its adjoint record (reverse).
+// Both passes give one warp to a centre atom: its lanes first expand 32 edges'
+// records, one edge per lane, into shared memory, then the four groups of 8
+// lanes (lane m of a group: radial channel m) take every fourth edge.
 #include <cuda_runtime.h>
-
-#include <mutex>
 
 #include "common.cuh"
 
@@ -32,29 +32,21 @@ namespace reann {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int kWarps = 4;          // warps per block
-constexpr int kFwdStages = 2;      // forward: a lane's next kFwdStages - 1 edges are in flight (3, 4 measured slower)
-constexpr int kAtomsPerWarp = 8;   // quads per warp
-constexpr int kBStride = 84;       // padded per-atom row in shared memory (16 B aligned)
+constexpr int kEdgeWarps = 8;  // warps (centre atoms) per block of the edge kernels
 
-
-struct Edge {
-    float x, y, z, d;
-    float phi[NPHI];
-};
-
-// exp(a) for |a| < 80 by Cody-Waite range reduction (W. J. Cody and W. Waite,
-// Software Manual for the Elementary Functions, 1980): a = k ln2 + r with ln2
-// split into a short high part (k ln2_hi exact) and a correction, |r| <= ln2/2,
-// then the degree-7 Taylor polynomial of exp(r) (truncation < 6e-9 relative) in
-// Horner form and an exact scaling by 2^k.  Measured on the GPU against FP64 its
-// mean relative error is ~1e-9 (unbiased), so the m-fold Gaussian recurrence
-// below does not turn a one-sided rounding habit into a shift of every phi_m.
-__device__ __forceinline__ float exp_cw(float a) {
+// exp(a + b) for |a| < 80 and a small correction b (the rounding error of a) by
+// Cody-Waite range reduction (W. J. Cody and W. Waite, Software Manual for the
+// Elementary Functions, 1980): a = k ln2 + r with ln2 split into a short high part
+// (k ln2_hi exact) and a correction, |r| <= ln2/2, then the degree-7 Taylor
+// polynomial of exp(r + b) (truncation < 6e-9 relative) in Horner form and an exact
+// scaling by 2^k.  Measured on the GPU against FP64 its mean relative error is
+// ~1e-9 (unbiased), so the m-fold Gaussian recurrence below does not turn a
+// one-sided rounding habit into a shift of every phi_m.
+__device__ __forceinline__ float exp_cw(float a, float b) {
     a = fminf(fmaxf(a, -87.f), 88.f);  // keeps 2^k a normal float
     const float k = rintf(a * 1.44269504f);
     float r = fmaf(-k, 0.693145751953125f, a);
-    r = fmaf(-k, 1.428606820309417e-06f, r);
+    r = fmaf(-k, 1.428606820309417e-06f, r) + b;
     float p = 1.f / 5040.f;
     p = fmaf(p, r, 1.f / 720.f);
     p = fmaf(p, r, 1.f / 120.f);
@@ -66,17 +58,23 @@ __device__ __forceinline__ float exp_cw(float a) {
     return p * __int_as_float(((int)k + 127) << 23);
 }
 
-// Gaussians by the equal-spacing recurrence exp(-a(d-mu_{m+1})^2) = exp(-a(d-mu_m)^2) q kappa_m,
-// q = exp(2 a Delta d): two exponentials per edge instead of eight.  The constants
-// a, 2 a Delta and kappa_m enter as float pairs (see Radial).
-__device__ __forceinline__ void gaussians(const Radial& R, float d, float gs[NPHI]) {
-    const float dd = d * d;
-    gs[0] = exp_cw(-fmaf(R.alpha_hi, dd, R.alpha_lo * dd));
-    const float q = exp_cw(fmaf(R.tad_hi, d, R.tad_lo * d));
+// exp(sign (x + x_lo) (c_hi + c_lo)) with the product's rounding error carried along
+__device__ __forceinline__ float exp_prod(float sign, float x, float x_lo, float c_hi, float c_lo) {
+    const float a = x * c_hi;
+    return exp_cw(sign * a, sign * (fmaf(x, c_hi, -a) + fmaf(x, c_lo, x_lo * c_hi)));
+}
+
+// All Gaussians from the first one by the equal-spacing recurrence
+//   exp(-a(d-mu_{m+1})^2) = exp(-a(d-mu_m)^2) q kappa_m,  q = exp(2 a Delta d),
+// kappa_m a float pair (see Radial).  The first value carries f_c and the power of
+// two R.scale, which keeps it normal near r_c for every a r_c^2 <= 80; the passes
+// multiply their sums by R.unscale.
+__device__ __forceinline__ void phi_chain(const Radial& R, float phi_first, float q, float phi[NPHI]) {
+    phi[0] = phi_first;
 #pragma unroll
     for (int m = 0; m + 1 < NPHI; ++m) {
-        const float p = gs[m] * q;
-        gs[m + 1] = fmaf(p, R.kap_hi[m], p * R.kap_lo[m]);
+        const float p = phi[m] * q;
+        phi[m + 1] = fmaf(p, R.kap_hi[m], p * R.kap_lo[m]);
     }
 }
 
@@ -85,180 +83,273 @@ __device__ __forceinline__ void gaussians(const Radial& R, float d, float gs[NPH
 // correctly rounded quotient and without the one-sided error of a rounded 1/r_c,
 // which near r_c, where the cutoff's logarithmic derivative is large, would
 // bias every atom), no rounded pi constant, and no cancellation of 1/2 + cos/2
-// near d = r_c.  dfc = -(2 pi / r_c) cos^3 sin (half angle).
-__device__ __forceinline__ void cutoff(const Radial& R, float d, float& fc, float& dfc) {
+// near d = r_c.  f_c' / f_c = -(2 pi / r_c) tan(pi x / 2), finite also where the
+// cosine rounds to zero (f_c is zero there).
+__device__ __forceinline__ void cutoff(const Radial& R, float d, float& fc, float& dlog) {
     float s, c;
     const float x = fmaf(d, R.inv_rc_hi, d * R.inv_rc_lo);
     sincospif(0.5f * x, &s, &c);
     const float c2 = c * c;
     fc = c2 * c2;
-    const float u = -6.28318530717959f * c2 * c * s;
-    dfc = fmaf(u, R.inv_rc_hi, u * R.inv_rc_lo);
-}
-
-__device__ __forceinline__ void monomials(float x, float y, float z, float A[NANG]) {
-    A[0] = 1.f;
-    A[1] = x;
-    A[2] = y;
-    A[3] = z;
-    A[4] = x * x;
-    A[5] = y * y;
-    A[6] = z * z;
-    A[7] = x * y;
-    A[8] = x * z;
-    A[9] = y * z;
+    const float u = -6.28318530717959f * s / (c == 0.f ? 1e-20f : c);
+    dlog = fmaf(u, R.inv_rc_hi, u * R.inv_rc_lo);
 }
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 
+// 32 consecutive bytes (32 B aligned) in one load: one instruction and one tag lookup for a
+// neighbour's coefficients or position
+__device__ __forceinline__ void ldg8(const void* p, float4& a, float4& b) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// K = 1, 2 or 4 consecutive floats (aligned to their size)
+template <int K>
+__device__ __forceinline__ void ldk(const float* p, float* v) {
+    if constexpr (K == 4) {
+        const float4 x = ld4(p);
+        v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+    } else if constexpr (K == 2) {
+        const float2 x = *reinterpret_cast<const float2*>(p);
+        v[0] = x.x, v[1] = x.y;
+    } else {
+        v[0] = p[0];
+    }
+}
+template <int K>
+__device__ __forceinline__ void stk(float* p, const float* v) {
+    if constexpr (K == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (K == 2)
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else
+        p[0] = v[0];
+}
+
 // Orbital pair (k, k'), k <= k', of pair feature p = 0..35 (row-major over k)
 __constant__ unsigned char c_pair_k[NORB_P * (NORB_P + 1) / 2];
 __constant__ unsigned char c_pair_k2[NORB_P * (NORB_P + 1) / 2];
 
-__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
+// -------------------------------------------------------------- edges ----
+// Live (d < r_c) entries of the list rows [row0, row0 + rows) and their records,
+// one warp per row; row row0 + k's records go to record row k.  A batch of 32
+// entries is tested, one per lane; the kept ones are queued in shared memory and
+// their records computed 32 at a time, so that the transcendental functions run
+// with full warps and the records are stored as whole lines.  (Queues that run on
+// over 2, 4 or 8 rows of a warp, to fill the last batch of a row as well, were
+// measured at 1.13 x, 1.08 x and 1.05 x the time for 24,576 to 32,000 atoms and
+// 0.91 x for 1,048,576.)
+//   xyzj = (r, j as bits); phi = (phi_0 R.scale, q) of phi_chain; der = (1/d, r1) with
+//   phi_m' / d = phi_m (r1 + 2 a mu_m / d), r1 = (f_c' / f_c) / d - 2 a
+__global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t rows, int stride, Radial R,
+                                                           const int32_t* __restrict__ nbr,
+                                                           const int32_t* __restrict__ cnt,
+                                                           const float4* __restrict__ pos, float4* __restrict__ xyzj,
+                                                           float2* __restrict__ phi, float2* __restrict__ der,
+                                                           int32_t* __restrict__ live_cnt, int* __restrict__ flags) {
+    pdl_enter();
+    __shared__ float4 queue[kEdgeWarps][64];
+    const int lane = threadIdx.x & 31;
+    const int64_t k = (int64_t)blockIdx.x * kEdgeWarps + (threadIdx.x >> 5);
+    if (k >= rows) return;
+    const int64_t i = row0 + k;
+    float4* q = queue[threadIdx.x >> 5];
+    float4 hi_i, lo_i;
+    ldg8(pos + 2 * i, hi_i, lo_i);
+    const int c = cnt[i];
+    const int32_t* row = nbr + (size_t)i * stride;
+    const size_t out = (size_t)k * stride;
+    int done = 0, tail = 0;  // records written, entries ever queued (queue index mod 64)
+    auto emit = [&]() {      // the record of queue entry done + lane
+        const float4 e = q[(done + lane) & 63];
+        const float d = sqrtf(e.x * e.x + e.y * e.y + e.z * e.z);
+        const float inv_d = 1.f / d;
+        float fc, dlog;
+        cutoff(R, d, fc, dlog);
+        // every radial function is that of the same rounded d (its rounding then acts like a
+        // displacement of 1e-7 A, to which all of them respond together)
+        const float dd = d * d;
+        const float g0 = exp_prod(-1.f, dd, fmaf(d, d, -dd), R.alpha_hi, R.alpha_lo);
+        const float qf = exp_prod(1.f, d, 0.f, R.tad_hi, R.tad_lo);
+        xyzj[out + done + lane] = e;
+        phi[out + done + lane] = make_float2(g0 * R.scale * fc, qf);
+        der[out + done + lane] = make_float2(inv_d, fmaf(dlog, inv_d, -2.f * R.alpha_hi));
+    };
+    int j_nx = lane < c ? row[lane] : 0;
+    for (int base = 0; base < c; base += 32) {
+        const int j = j_nx;
+        const bool in = base + lane < c;
+        j_nx = base + 32 + lane < c ? row[base + 32 + lane] : 0;
+        bool keep = false;
+        float x = 0.f, y = 0.f, z = 0.f;
+        if (in) {
+            float4 hj, lj;
+            ldg8(pos + 2 * (int64_t)j, hj, lj);
+            x = (hj.x - hi_i.x) + (lj.x - lo_i.x);
+            y = (hj.y - hi_i.y) + (lj.y - lo_i.y);
+            z = (hj.z - hi_i.z) + (lj.z - lo_i.z);
+            const float d2 = x * x + y * y + z * z;
+            keep = d2 < R.rc2;
+            if (!(d2 > 1e-16f)) {
+                keep = false;
+                atomicOr(&flags[FLAG_GEOM], 4);
+            }
+        }
+        const unsigned m = __ballot_sync(FULL, keep);
+        if (keep) q[(tail + __popc(m & ((1u << lane) - 1u))) & 63] = make_float4(x, y, z, __int_as_float(j));
+        tail += __popc(m);
+        __syncwarp();
+        if (tail - done >= 32) {
+            emit();
+            done += 32;
+            __syncwarp();  // the emitted entries are read before their places are queued again
+        }
+    }
+    if (lane < tail - done) emit();
+    if (lane == 0) live_cnt[i] = tail;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // ------------------------------------------------------------- forward ---
+// LPA lanes per centre atom (32 / LPA atoms per warp).  Lane q walks the edges
+// q, q + LPA, ... of its atom and accumulates the 80 products t_m A_a,
+// t_m = c_{j,m} phi_m, in registers; the record two edges ahead and the
+// coefficients one edge ahead are in flight meanwhile.  A butterfly
+// reduce-scatter over the LPA lanes leaves 80 / LPA of the sums in each lane
+// (stored as the b checkpoint), and lane q contracts its 16 / LPA orbitals.
+// Bound by the latency of the record stream and the coefficient gathers at 16
+// warps per SM (126 registers, 80 of them sums; issue slots 55 % busy).  Reading
+// records instead of recomputing the edge's geometry took a launch from 29.7 to
+// 19.9 us (24,576 atoms) and from 692 to 541 us (1,048,576 atoms).  Eight lanes per
+// edge with the sums of one channel each (48 registers, 37 warps) were slower, 39
+// against 21 us for 32,000 atoms: 5 shared-memory wavefronts per edge.
 // PAIRS = false: Eq. 1, rho_{l,k} = sum_{a in l} w_a g_{a,k}^2 over 16 orbitals.
 // PAIRS = true: the orbital-pair products rho_{l,(k,k')} = sum_{a in l} w_a g_{a,k} g_{a,k'},
 // k <= k' over 8 orbitals (108 features).
-template <bool PAIRS>
-__global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) k_density_fwd(int64_t n, int stride, Radial R,
-                                                            const int32_t* __restrict__ live,
+constexpr int kFwdWarps = 4;
+constexpr int kBStride = 84;  // padded b row of an atom in shared memory (16 B aligned)
+
+// one butterfly stage over CNT values: lanes with bit O set keep the upper half
+template <int CNT, int O>
+__device__ __forceinline__ void rs_half(float* v, int q) {
+    const bool upper = q & O;
+#pragma unroll
+    for (int k = 0; k < CNT / 2; ++k) {
+        const float send = upper ? v[k] : v[CNT / 2 + k];
+        const float keep = upper ? v[CNT / 2 + k] : v[k];
+        v[k] = keep + __shfl_xor_sync(FULL, send, O);
+    }
+}
+
+template <bool PAIRS, int LPA>
+__global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0, int64_t rows, int stride, Radial R,
                                                             const int32_t* __restrict__ live_cnt,
-                                                            const float4* __restrict__ phi_hi,
-                                                            const float4* __restrict__ plo,
+                                                            const float4* __restrict__ xyzj,
+                                                            const float2* __restrict__ phi,
                                                             const float* __restrict__ coef,
                                                             const float* __restrict__ Wt, float* __restrict__ rho,
-                                                            float* __restrict__ bck) {
+                                                            float* __restrict__ bck, bool far) {
     pdl_enter();
-    constexpr int KO = PAIRS ? NORB_P : NORB;
+    constexpr int KO = PAIRS ? NORB_P : NORB, APW = 32 / LPA;
+    static_assert(LPA == 4 || LPA == 8 || LPA == 16, "80 sums split evenly");
     __shared__ __align__(16) float sW[(LMAX + 1) * NPHI * KO];
-    // During the edge loop: kFwdStages stages of a lane's next neighbours (hi, lo
-    // position and c of j), [stage][part][thread] float4; afterwards the b rows.
-    constexpr int kStage = kFwdStages * 4 * kWarps * 32 * 4;
-    static_assert(kStage >= kWarps * kAtomsPerWarp * kBStride, "b rows must fit in the staging area");
-    __shared__ __align__(16) float sU[kStage];
-    float4* stg = reinterpret_cast<float4*>(sU);
+    __shared__ __align__(16) float sB[kFwdWarps * APW][kBStride];
     for (int i = threadIdx.x; i < (LMAX + 1) * NPHI * KO; i += blockDim.x) sW[i] = Wt[i];
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3, slot = lane >> 2;
-    const int64_t atom = ((int64_t)blockIdx.x * kWarps + warp) * kAtomsPerWarp + slot;
-    const bool valid = atom < n;
-
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & (LPA - 1), slot = lane / LPA;
+    const int64_t kr = ((int64_t)blockIdx.x * kFwdWarps + warp) * APW + slot;
+    const bool valid = kr < rows;
+    const int64_t atom = row0 + kr;
     float acc[NB];
 #pragma unroll
     for (int v = 0; v < NB; ++v) acc[v] = 0.f;
     if (valid) {
-        const float4 hi_i = phi_hi[atom], lo_i = plo[atom];
         const int cnt = live_cnt[atom];
-        const int32_t* row = live + (size_t)atom * stride;
-        constexpr int kT = kWarps * 32;
-        auto stage = [&](int st, int j) {
-            float4* d = stg + st * 4 * kT + threadIdx.x;
-            cp_async16(d, phi_hi + j);
-            cp_async16(d + kT, plo + j);
-            cp_async16(d + 2 * kT, coef + (size_t)j * NPHI);
-            cp_async16(d + 3 * kT, coef + (size_t)j * NPHI + 4);
-        };
-        // the lane's edges e = q, q + 4, ...: the copies of the next kFwdStages - 1 edges
-        // are in flight while edge e is computed, and the index after them is loaded
-        constexpr int NST = kFwdStages;
-#pragma unroll
-        for (int p = 0; p < NST - 1; ++p) {
-            if (q + 4 * p < cnt) stage(p, row[q + 4 * p]);
-            cp_async_commit();
+        const float4* ex = xyzj + (size_t)kr * stride;
+        const float2* ep = phi + (size_t)kr * stride;
+        // the row's records start on their way to L2 at once (large systems stream them from HBM)
+        if (far) {
+            for (int e = 8 * q; e < cnt; e += 8 * LPA) prefetch_l2(ex + e);
+            for (int e = 16 * q; e < cnt; e += 16 * LPA) prefetch_l2(ep + e);
         }
-        int j_nx = q + 4 * (NST - 1) < cnt ? row[q + 4 * (NST - 1)] : 0;
-        int st = 0;  // stage of edge e
-        for (int e = q; e < cnt; e += 4) {
-            const int e_st = e + 4 * (NST - 1);  // the edge copied now, into the stage edge e - 4 used
-            if (e_st < cnt) stage(st == 0 ? NST - 1 : st - 1, j_nx);
-            cp_async_commit();
-            j_nx = e_st + 4 < cnt ? row[e_st + 4] : 0;
-            cp_async_wait<NST - 1>();  // edge e's stage has landed
-            const float4* src = stg + st * 4 * kT + threadIdx.x;
-            const float4 hj = src[0], lj = src[kT], c0 = src[2 * kT], c1 = src[3 * kT];
-            st = st == NST - 1 ? 0 : st + 1;
-            const float x = (hj.x - hi_i.x) + (lj.x - lo_i.x);
-            const float y = (hj.y - hi_i.y) + (lj.y - lo_i.y);
-            const float z = (hj.z - hi_i.z) + (lj.z - lo_i.z);
-            const float d = sqrtf(x * x + y * y + z * z);
-            float gs[NPHI], fc, dfc;
-            gaussians(R, d, gs);
-            cutoff(R, d, fc, dfc);
-            const float cj[NPHI] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-            float tm[NPHI];
-#pragma unroll
-            for (int m = 0; m < NPHI; ++m) tm[m] = cj[m] * gs[m] * fc;
-            float A[NANG];
-            monomials(x, y, z, A);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 e1 = zero, c0 = zero, c1 = zero;
+        float2 p1 = make_float2(0.f, 0.f);
+        if (q < cnt) {
+            e1 = ex[q];
+            p1 = ep[q];
+            ldg8(coef + (size_t)__float_as_int(e1.w) * NPHI, c0, c1);
+        }
+        float4 e2 = zero;
+        float2 p2 = make_float2(0.f, 0.f);
+        if (q + LPA < cnt) e2 = ex[q + LPA], p2 = ep[q + LPA];
+        for (int e = q; e < cnt; e += LPA) {
+            const float x = e1.x, y = e1.y, z = e1.z;
+            float ph[NPHI];
+            phi_chain(R, p1.x, p1.y, ph);
+            const float t[NPHI] = {c0.x * ph[0], c0.y * ph[1], c0.z * ph[2], c0.w * ph[3],
+                                   c1.x * ph[4], c1.y * ph[5], c1.z * ph[6], c1.w * ph[7]};
+            e1 = e2;
+            p1 = p2;
+            if (e + LPA < cnt) ldg8(coef + (size_t)__float_as_int(e2.w) * NPHI, c0, c1);
+            if (e + 2 * LPA < cnt) e2 = ex[e + 2 * LPA], p2 = ep[e + 2 * LPA];
+            const float A[NANG] = {1.f, x, y, z, x * x, y * y, z * z, x * y, x * z, y * z};
 #pragma unroll
             for (int a = 0; a < NANG; ++a)
 #pragma unroll
-                for (int m = 0; m < NPHI; ++m) acc[a * NPHI + m] = fmaf(tm[m], A[a], acc[a * NPHI + m]);
+                for (int m = 0; m < NPHI; ++m) acc[a * NPHI + m] = fmaf(t[m], A[a], acc[a * NPHI + m]);
         }
     }
-    cp_async_wait_all();
-    __syncthreads();  // the staging area becomes the b rows
-    // butterfly reduce-scatter over the quad: lane q keeps b[20q, 20q+20)
-    float r1[NB / 2];
-    const bool hi_half = (q >> 1) & 1;
+    // reduce-scatter: lane q keeps b[80 / LPA * rev(q) ..), rev the order the halves were taken in
+    constexpr int NL = NB / LPA;
+    if constexpr (LPA == 16) rs_half<NB, 8>(acc, q);
+    if constexpr (LPA >= 8) rs_half<(LPA == 16 ? NB / 2 : NB), 4>(acc, q);
+    rs_half<NL * 4, 2>(acc, q);
+    rs_half<NL * 2, 1>(acc, q);
+    float* sb = sB[warp * APW + slot];
 #pragma unroll
-    for (int v = 0; v < NB / 2; ++v) {
-        const float send = hi_half ? acc[v] : acc[NB / 2 + v];
-        const float keep = hi_half ? acc[NB / 2 + v] : acc[v];
-        r1[v] = keep + __shfl_xor_sync(FULL, send, 2);
-    }
-    float r2[NB / 4];
-    const bool odd = q & 1;
+    for (int v = 0; v < NL; ++v) acc[v] *= R.unscale;
+    if constexpr (LPA == 16) {
 #pragma unroll
-    for (int v = 0; v < NB / 4; ++v) {
-        const float send = odd ? r1[v] : r1[NB / 4 + v];
-        const float keep = odd ? r1[NB / 4 + v] : r1[v];
-        r2[v] = keep + __shfl_xor_sync(FULL, send, 1);
-    }
-    float* sb = sU + (warp * kAtomsPerWarp + slot) * kBStride;
+        for (int v = 0; v < NL; ++v) sb[NL * q + v] = acc[v];
+    } else {
 #pragma unroll
-    for (int v = 0; v < NB / 4; v += 4) {
-        const float4 w4 = make_float4(r2[v], r2[v + 1], r2[v + 2], r2[v + 3]);
-        *reinterpret_cast<float4*>(sb + 20 * q + v) = w4;
-        if (valid) *reinterpret_cast<float4*>(bck + (size_t)atom * NB + 20 * q + v) = w4;
+        for (int v = 0; v < NL; v += 2) *reinterpret_cast<float2*>(sb + NL * q + v) = make_float2(acc[v], acc[v + 1]);
     }
     __syncwarp();
+    if (valid)
+#pragma unroll
+        for (int v = 4 * q; v < NB; v += 4 * LPA) *reinterpret_cast<float4*>(bck + (size_t)atom * NB + v) = ld4(sb + v);
     if constexpr (PAIRS) {
-        // g_{a,k} = sum_m b_{a,m} W_{l,m,k}: lane q the orbitals 2q, 2q+1 of every a,
-        // into the b row's place (after all four lanes have read it); then lane q
-        // the 27 features 27q .. 27q+26
-        float g[NANG][2];
+        // g_{a,k} = sum_m b_{a,m} W_{l,m,k} into the b row's place: lane q the orbitals k = q, q + LPA, ...
+        constexpr int KL = LPA >= NORB_P ? 1 : NORB_P / LPA;
+        float g[NANG][KL];
 #pragma unroll
         for (int a = 0; a < NANG; ++a) {
             const int l = ang_l(a);
             const float4 b0 = ld4(sb + a * NPHI), b1 = ld4(sb + a * NPHI + 4);
             const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-            g[a][0] = g[a][1] = 0.f;
 #pragma unroll
-            for (int m = 0; m < NPHI; ++m) {
-                const float2 w = *reinterpret_cast<const float2*>(sW + (l * NPHI + m) * KO + 2 * q);
-                g[a][0] = fmaf(bm[m], w.x, g[a][0]);
-                g[a][1] = fmaf(bm[m], w.y, g[a][1]);
+            for (int i = 0; i < KL; ++i) {
+                g[a][i] = 0.f;
+#pragma unroll
+                for (int m = 0; m < NPHI; ++m)
+                    g[a][i] = fmaf(bm[m], sW[(l * NPHI + m) * KO + ((q + i * LPA) & (NORB_P - 1))], g[a][i]);
             }
         }
         __syncwarp();
 #pragma unroll
         for (int a = 0; a < NANG; ++a)
-            *reinterpret_cast<float2*>(sb + a * NORB_P + 2 * q) = make_float2(g[a][0], g[a][1]);
+#pragma unroll
+            for (int i = 0; i < KL; ++i)
+                if (q + i * LPA < NORB_P) sb[a * NORB_P + q + i * LPA] = g[a][i];
         __syncwarp();
         if (!valid) return;
         constexpr int KP = NORB_P * (NORB_P + 1) / 2;
-        for (int f = 27 * q; f < 27 * q + 27; ++f) {
+        for (int f = q; f < NFEAT_P; f += LPA) {
             const int l = f / KP, p = f - l * KP;
             const int k = c_pair_k[p], k2 = c_pair_k2[p];
             const int a0 = l == 0 ? 0 : (l == 1 ? 1 : 4), a1 = l == 0 ? 1 : (l == 1 ? 4 : NANG);
@@ -269,34 +360,34 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) k_density_fwd(int64_
         return;
     }
     if (!valid) return;
-    // contraction over m and the squared multinomial sum; lane q owns orbitals 4q..4q+3
-    float racc[LMAX + 1][4];
+    // contraction over m and the squared multinomial sum; lane q owns KL consecutive orbitals
+    constexpr int KL = NORB / LPA;
+    float racc[LMAX + 1][KL];
 #pragma unroll
     for (int l = 0; l <= LMAX; ++l)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) racc[l][k] = 0.f;
+        for (int k = 0; k < KL; ++k) racc[l][k] = 0.f;
 #pragma unroll
     for (int a = 0; a < NANG; ++a) {
         const int l = ang_l(a);
         const float4 b0 = ld4(sb + a * NPHI), b1 = ld4(sb + a * NPHI + 4);
         const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-        float g[4] = {0.f, 0.f, 0.f, 0.f};
+        float g[KL];
+#pragma unroll
+        for (int k = 0; k < KL; ++k) g[k] = 0.f;
 #pragma unroll
         for (int m = 0; m < NPHI; ++m) {
-            const float4 w = ld4(sW + (l * NPHI + m) * NORB + 4 * q);
-            g[0] = fmaf(bm[m], w.x, g[0]);
-            g[1] = fmaf(bm[m], w.y, g[1]);
-            g[2] = fmaf(bm[m], w.z, g[2]);
-            g[3] = fmaf(bm[m], w.w, g[3]);
+            float w[KL];
+            ldk<KL>(sW + (l * NPHI + m) * NORB + KL * q, w);
+#pragma unroll
+            for (int k = 0; k < KL; ++k) g[k] = fmaf(bm[m], w[k], g[k]);
         }
         const float wa = ang_w(a);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) racc[l][k] = fmaf(wa * g[k], g[k], racc[l][k]);
+        for (int k = 0; k < KL; ++k) racc[l][k] = fmaf(wa * g[k], g[k], racc[l][k]);
     }
 #pragma unroll
-    for (int l = 0; l <= LMAX; ++l)
-        *reinterpret_cast<float4*>(rho + (size_t)atom * NFEAT + l * NORB + 4 * q) =
-            make_float4(racc[l][0], racc[l][1], racc[l][2], racc[l][3]);
+    for (int l = 0; l <= LMAX; ++l) stk<KL>(rho + (size_t)atom * NFEAT + l * NORB + KL * q, racc[l]);
 }
 
 // -------------------------------------------------------------- bbar -----
@@ -354,13 +445,13 @@ __global__ void __launch_bounds__(4 * kBbarAtoms) k_bbar(int64_t n, const float*
                     gb[k] = fmaf(rv, g[k2], gb[k]);
                     gb[k2] = fmaf(rv, g[k], gb[k2]);
                 }
-            const float wa = ang_w(a);
+            const float wa = rec_scale(a) * ang_w(a);
 #pragma unroll
             for (int m = 0; m < NPHI; ++m)
 #pragma unroll
                 for (int k = 0; k < NORB_P; ++k) out[m] = fmaf(wa * gb[k], sW[(l * NPHI + m) * KO + k], out[m]);
         } else {
-            bbar_term(bm, 2.f * ang_w(a), sW + l * NPHI * NORB, rhobar + (size_t)atom * NFEAT + l * NORB, out);
+            bbar_term(bm, 2.f * rec_scale(a) * ang_w(a), sW + l * NPHI * NORB, rhobar + (size_t)atom * NFEAT + l * NORB, out);
         }
         stage_rec(sRec, r, v, out);
     }
@@ -370,27 +461,26 @@ __global__ void __launch_bounds__(4 * kBbarAtoms) k_bbar(int64_t n, const float*
 
 // ---------------------------------------------------------- adjoint ------
 
-// Reverse pass (header formulas), laid out for coalesced gathers: 8
-// lanes per centre atom k (4 atoms per warp), lane m owning radial channel m.
-// Per batch of 8 live edges each lane first computes the geometry of one edge
-// (d, f_c, f_c', the 8 Gaussians) into shared memory; then every lane walks the
-// 8 edges and, for its channel m, gathers bbar_{j,a,m} (a = 0..9) and c_{j,m}
-// from j's adjoint record (3 float4 loads per lane; per load the 8 lanes read
-// one full 128 B line of the record), and accumulates its share of dE/dr_k;
-// cbar_{k,m} is lane m's own sum.  The force is reduced over the 8 lanes once
-// per atom.  Each record is gathered just before its edge is computed: without
-// records held in registers ahead of use the kernel fits 64 registers and 32
-// warps per SM (prefetching one edge ahead took 80 registers and 24 warps, and
-// was 3 % slower).
-constexpr int kAdjWarps = 2;  // small blocks: the block scheduler balances the SMs at fine grain
-constexpr int kAdjGroups = 4;  // centre atoms per warp
-// Edge record in shared memory: x y z 1/d | d fc fc' - | g_0..g_7 (16 floats).
-// Strides chosen bank-conflict free: a record every 20 floats (8 lanes' float4
-// stores hit 32 distinct banks), a group every 168 floats (the 4 groups'
-// reads of g_m land on disjoint banks).
-constexpr int kGeoStride = 20;
-constexpr int kGroupStride = 8 * kGeoStride + 8;
-
+// Reverse pass (header formulas), LPA lanes per centre atom k (32 / LPA atoms per
+// warp), lane (g, m) owning radial channel m of the edges s = g mod LPA / 8.  Per
+// batch of LPA edges each lane expands one edge's record into shared memory (the
+// next batch's record is on its way meanwhile).  Then, for its edges, lane (g, m)
+// gathers channel m of the neighbour's adjoint record (3 float4 loads; per load the
+// 8 lanes of a group read one full 128 B line) and accumulates its share of
+// dE/dr_k; cbar_{k,m} is summed over the groups.
+//   Bound by the L2 latency and the L1 wavefronts of the record gathers (384 B per
+// edge; the L1 data stage is 70 % busy while blocks are resident, issue slots 56 %).
+// 59 -> 41 us per launch (24,576 atoms), 1,408 -> 1,166 us (1,048,576 atoms), 28 -> 7 us
+// (192 atoms, where the number of edges that follow one another decides).  Records
+// gathered one edge ahead in a second register set gained nothing.
+//   With Q_k(r) = sum_a bbar_{k,a} A_a and Q_j(r) = sum_a (-1)^l bbar_{j,a} A_a (both
+// quadratics per channel) the edge's share of -dE/dr_k is, per channel,
+//   c_j (psi Q_k r + phi grad Q_k) + c_k (psi Q_j r + phi grad Q_j).
+// Summed over the edges, the term c_j phi grad Q_k needs only the moments sum_j
+// c_j phi A_a = b_{k,a} that the forward pass kept (grad Q_k is linear in r), so
+// it is added once per atom from the checkpoint b instead of once per edge.
+// Small blocks: the block scheduler balances the SMs at fine grain.
+constexpr int kAdjWarps = 4;
 // With forces set (the last reverse layer), the kernel also writes F = -dE/dr
 // and the atomic energies in caller order (perm: internal -> caller index);
 // with first set (the first reverse layer), grad and vir are written, not
@@ -405,188 +495,198 @@ struct Outputs {
 
 // WANT_VIR: also W -= (dE/dr_e) r_e^T over the atom's own edges (their
 // bbar_k c_j terms: every directed edge once) into vir (N x 9, accumulated
-// over the layers like grad).
-template <bool WANT_CBAR, bool WANT_VIR>
-__global__ void __launch_bounds__(kAdjWarps * 32) k_density_adj8(int64_t n, int stride, Radial R,
-                                                                const int32_t* __restrict__ live,
+// over the layers like grad); the part with grad Q_k again comes from b.
+template <bool WANT_CBAR, bool WANT_VIR, int LPA>
+__global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_adj(int64_t row0, int64_t rows, int stride, Radial R,
                                                                 const int32_t* __restrict__ live_cnt,
-                                                                const float4* __restrict__ phi_hi,
-                                                                const float4* __restrict__ plo,
+                                                                const float4* __restrict__ xyzj,
+                                                                const float2* __restrict__ phi,
+                                                                const float2* __restrict__ der,
                                                                 const float* __restrict__ rec,
+                                                                const float* __restrict__ bck,
                                                                 float* __restrict__ cbar, float* __restrict__ grad,
                                                                 float* __restrict__ vir, Outputs out) {
     pdl_enter();
-    __shared__ __align__(16) float sGeo[kAdjWarps][kAdjGroups * kGroupStride];
-    __shared__ __align__(16) float4 sPos[2][kAdjWarps * 32];  // a lane's next edge: hi, lo position of j
-    __shared__ __align__(16) float4 sCen[kAdjWarps * kAdjGroups][2];  // hi, lo position of the centre atom
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane & 7, grp = lane >> 3;
-    const int64_t atom = ((int64_t)blockIdx.x * kAdjWarps + warp) * kAdjGroups + grp;
-    const bool valid = atom < n;
-    // the 12 values of channel m in an atom's record: bbar_{0..9,m}, c_m, 0
-    auto load_rec = [&](int64_t r, float* v) {
+    constexpr int APW = 32 / LPA, G = LPA / 8;  // atoms per warp, groups of 8 lanes per atom
+    // per atom, for its batch of LPA edges: (r, 1/d) [LPA][4], (j, r1) [LPA][2], phi [LPA][8]; an
+    // atom's blocks are padded so that the words its groups and the other atoms of the warp read
+    // together lie in different banks
+    constexpr int PAD = LPA == 32 ? 0 : (LPA == 16 ? 16 : 8), LE = 4 * LPA + PAD, LJ = 2 * LPA + PAD, LP = 8 * LPA + PAD;
+    __shared__ __align__(16) float sE[kAdjWarps * APW][LE + LJ + LP];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane & 7, sub = lane & (LPA - 1), g = sub >> 3;
+    const int64_t kr = ((int64_t)blockIdx.x * kAdjWarps + warp) * APW + lane / LPA;
+    const bool valid = kr < rows;
+    const int64_t atom = row0 + kr;
+    float* s_e = sE[warp * APW + lane / LPA];
+    float *s_j = s_e + LE, *s_phi = s_j + LJ;
+    const float two_a_mu = R.two_a_mu[m];
+    // the 12 values of channel m in an atom's record: bbar_{0..9,m} (the squares' doubled), c_m, 0
+    auto load_rec = [&](int r, float* v) {
         const float* p = rec + (size_t)r * NREC + 4 * m;
+        if constexpr (LPA < 32) {
+            asm volatile(
+                "ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%12];\n\t"
+                "ld.global.nc.v4.f32 {%4, %5, %6, %7}, [%12 + 128];\n\t"
+                "ld.global.nc.v4.f32 {%8, %9, %10, %11}, [%12 + 256];"
+                : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                  "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11])
+                : "l"(p));
+        } else {
 #pragma unroll
-        for (int line = 0; line < 3; ++line) {
-            const float4 x = ldg4(p + line * 4 * NPHI);
-            v[4 * line] = x.x, v[4 * line + 1] = x.y, v[4 * line + 2] = x.z, v[4 * line + 3] = x.w;
+            for (int line = 0; line < 3; ++line) {
+                const float4 x = ldg4(p + line * 4 * NPHI);
+                v[4 * line] = x.x, v[4 * line + 1] = x.y, v[4 * line + 2] = x.z, v[4 * line + 3] = x.w;
+            }
         }
     };
-    float bk[12];
     int cnt = 0;
-    const int32_t* row = live;
-    float4* cen = sCen[warp * kAdjGroups + grp];
+    float bk[12];
+#pragma unroll
+    for (int v = 0; v < 12; ++v) bk[v] = 0.f;
     if (valid) {
-        load_rec(atom, bk);
         cnt = live_cnt[atom];
-        if (m < 2) cen[m] = (m == 0 ? phi_hi : plo)[atom];
-        row = live + (size_t)atom * stride;
-    } else {
-#pragma unroll
-        for (int a = 0; a < 12; ++a) bk[a] = 0.f;
+        load_rec((int)atom, bk);
     }
+    int cmax = cnt;  // longest row of the warp's atoms
+#pragma unroll
+    for (int o = LPA; o < 32; o <<= 1) cmax = max(cmax, __shfl_xor_sync(FULL, cmax, o));
     const float ck = bk[NANG];
-    int cmax = cnt;
-    cmax = max(cmax, __shfl_xor_sync(FULL, cmax, 8));
-    cmax = max(cmax, __shfl_xor_sync(FULL, cmax, 16));
-    __syncwarp();  // the centre positions are visible to the group
-    const float mu_hi = R.mu_hi[m], mu_lo = R.mu_lo[m], two_alpha = 2.f * R.alpha_hi;
-    float* geo = sGeo[warp] + grp * kGroupStride;
-    float4* my_hi = &sPos[0][threadIdx.x];
-    float4* my_lo = &sPos[1][threadIdx.x];
+    bk[4] *= 0.5f, bk[5] *= 0.5f, bk[6] *= 0.5f;
+    const float4* ex = xyzj + (size_t)kr * stride;
+    const float2* ep = phi + (size_t)kr * stride;
+    const float2* ed = der + (size_t)kr * stride;
     float gx = 0.f, gy = 0.f, gz = 0.f, cb = 0.f;
-    float w[9];
+    float w6[6];  // sum c_j psi Q_k r r^T: xx, yy, zz, xy, xz, yz
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = 0.f;
-    // Pipeline across batches of 8 edges: while batch b is computed, the
-    // positions of batch b + 1 are copied into shared memory (cp.async) and the
-    // indices of batch b + 2 are loaded.
-    int j_cur = 0;
-    if (m < cnt) {
-        j_cur = row[m];
-        cp_async16(my_hi, phi_hi + j_cur);
-        cp_async16(my_lo, plo + j_cur);
-    }
-    cp_async_commit();
-    int j_nx = 8 + m < cnt ? row[8 + m] : 0;
-    for (int e0 = 0; e0 < cmax; e0 += 8) {
-        const int ns = cnt - e0;
-        // geometry of edge e0 + m, one edge per lane, from the staged positions
-        cp_async_wait_all();
-        if (m < ns) {
-            const float4 hj = *my_hi, lj = *my_lo, hi_i = cen[0], lo_i = cen[1];
-            const float x = (hj.x - hi_i.x) + (lj.x - lo_i.x);
-            const float y = (hj.y - hi_i.y) + (lj.y - lo_i.y);
-            const float z = (hj.z - hi_i.z) + (lj.z - lo_i.z);
-            const float d = sqrtf(x * x + y * y + z * z);
-            float gs[NPHI], fc, dfc;
-            gaussians(R, d, gs);
-            cutoff(R, d, fc, dfc);
-            float* g = geo + m * kGeoStride;
-            *reinterpret_cast<float4*>(g) = make_float4(x, y, z, 1.f / d);
-            *reinterpret_cast<float4*>(g + 4) = make_float4(d, fc, dfc, __int_as_float(j_cur));
-            *reinterpret_cast<float4*>(g + 8) = make_float4(gs[0], gs[1], gs[2], gs[3]);
-            *reinterpret_cast<float4*>(g + 12) = make_float4(gs[4], gs[5], gs[6], gs[7]);
+    for (int q = 0; q < 6; ++q) w6[q] = 0.f;
+    float w9[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) w9[q] = 0.f;
+    float4 e_nx = make_float4(0.f, 0.f, 0.f, 0.f);  // the next batch's record of this lane
+    float2 p_nx = make_float2(0.f, 0.f), d_nx = p_nx;
+    if (sub < cnt) e_nx = ex[sub], p_nx = ep[sub], d_nx = ed[sub];
+    for (int e0 = 0; e0 < cmax; e0 += LPA) {
+        const int ne = min(cnt - e0, LPA);
+        if (sub < ne) {
+            float ph[NPHI];
+            phi_chain(R, p_nx.x, p_nx.y, ph);
+            *reinterpret_cast<float4*>(s_e + 4 * sub) = make_float4(e_nx.x, e_nx.y, e_nx.z, d_nx.x);
+            *reinterpret_cast<float2*>(s_j + 2 * sub) = make_float2(e_nx.w, d_nx.y);
+            // lanes 4-7 of every 8 store the halves the other way round: no bank conflicts
+            const bool sw = sub & 4;
+            float* f = s_phi + 8 * sub;
+            const int h0 = sw ? 4 : 0, h1 = 4 - h0;
+            *reinterpret_cast<float4*>(f + h0) =
+                make_float4(sw ? ph[4] : ph[0], sw ? ph[5] : ph[1], sw ? ph[6] : ph[2], sw ? ph[7] : ph[3]);
+            *reinterpret_cast<float4*>(f + h1) =
+                make_float4(sw ? ph[0] : ph[4], sw ? ph[1] : ph[5], sw ? ph[2] : ph[6], sw ? ph[3] : ph[7]);
+            if (e0 + LPA + sub < cnt) e_nx = ex[e0 + LPA + sub], p_nx = ep[e0 + LPA + sub], d_nx = ed[e0 + LPA + sub];
         }
         __syncwarp();
-        // this lane's slot has been read (its values are used above): stage the next batch
-        if (8 + m < ns) {
-            cp_async16(my_hi, phi_hi + j_nx);
-            cp_async16(my_lo, plo + j_nx);
-        }
-        cp_async_commit();
-        const int j_nx2 = 16 + m < ns ? row[e0 + 16 + m] : 0;
-        auto gather = [&](int s, float* bj) {
-            if (s < ns) load_rec(__float_as_int(geo[s * kGeoStride + 7]), bj);
-        };
-        auto edge = [&](int s, const float* bj) {
-            if (s >= ns) return;
-            const float cj = bj[NANG];
-            const float* g = geo + s * kGeoStride;
-            const float4 g0 = *reinterpret_cast<const float4*>(g);
-            const float4 g1 = *reinterpret_cast<const float4*>(g + 4);
-            const float gsm = g[8 + m];
-            const float x = g0.x, y = g0.y, z = g0.z, inv_d = g0.w;
-            const float d = g1.x, fc = g1.y, dfc = g1.z;
-            const float phi = gsm * fc;
-            const float dphi = gsm * (dfc - two_alpha * ((d - mu_hi) - mu_lo) * fc);  // d - mu_m as a float pair
-            // Gk = sum_a bbar_k grad A_a,  Gj = sum_a (-1)^l bbar_j grad A_a
-            const float x2 = 2.f * x, y2 = 2.f * y, z2 = 2.f * z;
-            const float gkx = fmaf(z, bk[8], fmaf(y, bk[7], fmaf(x2, bk[4], bk[1])));
-            const float gky = fmaf(z, bk[9], fmaf(x, bk[7], fmaf(y2, bk[5], bk[2])));
-            const float gkz = fmaf(y, bk[9], fmaf(x, bk[8], fmaf(z2, bk[6], bk[3])));
-            const float gjx = fmaf(z, bj[8], fmaf(y, bj[7], fmaf(x2, bj[4], -bj[1])));
-            const float gjy = fmaf(z, bj[9], fmaf(x, bj[7], fmaf(y2, bj[5], -bj[2])));
-            const float gjz = fmaf(y, bj[9], fmaf(x, bj[8], fmaf(z2, bj[6], -bj[3])));
-            // Sk = sum_a A_a bbar_k,  Sj = sum_a (-1)^l A_a bbar_j  (also cbar's edge term): both are
-            // quadratics P(r) = p0 + l.r + r^T M r, and P = p0 + (r . (l + grad P)) / 2
-            const float Sk = fmaf(0.5f, fmaf(z, bk[3] + gkz, fmaf(y, bk[2] + gky, x * (bk[1] + gkx))), bk[0]);
-            const float Sj = fmaf(0.5f, fmaf(z, gjz - bj[3], fmaf(y, gjy - bj[2], x * (gjx - bj[1]))), bj[0]);
-            // radial part (d phi / dd) A along r/d, angular part phi grad A
-            const float sc = fmaf(cj * dphi, Sk, ck * dphi * Sj) * inv_d;
-            const float qv = cj * phi, qt = ck * phi;
-            gx -= fmaf(sc, x, fmaf(qv, gkx, qt * gjx));
-            gy -= fmaf(sc, y, fmaf(qv, gky, qt * gjy));
-            gz -= fmaf(sc, z, fmaf(qv, gkz, qt * gjz));
-            if (WANT_CBAR) cb = fmaf(phi, Sj, cb);
-            if (WANT_VIR) {
-                // dE/dr_e of this edge: the bbar_k c_j part
-                const float sa = cj * dphi * Sk * inv_d;
-                const float t3[3] = {fmaf(sa, x, qv * gkx), fmaf(sa, y, qv * gky), fmaf(sa, z, qv * gkz)};
-                const float r3[3] = {x, y, z};
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) w[3 * a + b] = fmaf(-t3[a], r3[b], w[3 * a + b]);
-            }
-        };
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
+#pragma unroll 1
+        for (int s = g; s < ne; s += G) {
+            const float2 jr = *reinterpret_cast<const float2*>(s_j + 2 * s);
             float bj[12];
-            gather(s, bj);
-            edge(s, bj);
+            load_rec(__float_as_int(jr.x), bj);
+            const float4 e = ld4(s_e + 4 * s);
+            const float ph = s_phi[8 * s + m], ps = ph * fmaf(two_a_mu, e.w, jr.y);  // phi, phi' / d
+            const float x = e.x, y = e.y, z = e.z, cj = bj[NANG];
+            // grad Q_j; Q_j = q0 + (r . (l + grad Q_j)) / 2 for a quadratic with linear part l
+            const float gjx = fmaf(z, bj[8], fmaf(y, bj[7], fmaf(x, bj[4], -bj[1])));
+            const float gjy = fmaf(z, bj[9], fmaf(x, bj[7], fmaf(y, bj[5], -bj[2])));
+            const float gjz = fmaf(y, bj[9], fmaf(x, bj[8], fmaf(z, bj[6], -bj[3])));
+            const float Qj = fmaf(0.5f, fmaf(z, gjz - bj[3], fmaf(y, gjy - bj[2], x * (gjx - bj[1]))), bj[0]);
+            // Q_k by Horner's rule (bk's squares halved below)
+            const float Qk = fmaf(x, fmaf(z, bk[8], fmaf(y, bk[7], fmaf(x, bk[4], bk[1]))),
+                                  fmaf(y, fmaf(z, bk[9], fmaf(y, bk[5], bk[2])), fmaf(z, fmaf(z, bk[6], bk[3]), bk[0])));
+            const float sk = cj * Qk;
+            const float sc = ps * fmaf(ck, Qj, sk);
+            const float qt = ck * ph;
+            gx -= fmaf(sc, x, qt * gjx);
+            gy -= fmaf(sc, y, qt * gjy);
+            gz -= fmaf(sc, z, qt * gjz);
+            if (WANT_CBAR) cb = fmaf(ph, Qj, cb);
+            if (WANT_VIR) {
+                const float a = ps * sk, ax = a * x, ay = a * y, az = a * z;
+                w6[0] = fmaf(ax, x, w6[0]);
+                w6[1] = fmaf(ay, y, w6[1]);
+                w6[2] = fmaf(az, z, w6[2]);
+                w6[3] = fmaf(ax, y, w6[3]);
+                w6[4] = fmaf(ax, z, w6[4]);
+                w6[5] = fmaf(ay, z, w6[5]);
+            }
         }
         __syncwarp();
-        j_cur = j_nx;
-        j_nx = j_nx2;
+    }
+    gx *= R.unscale, gy *= R.unscale, gz *= R.unscale, cb *= R.unscale;
+    if (WANT_VIR)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) w6[q] *= R.unscale;
+    if (g == 0 && valid) {
+        // sum_j c_j phi grad Q_k (and, for the virial, times r) from the forward's moments b_{k,a,m}
+        const float* b = bck + (size_t)atom * NB + m;
+        const float h4 = 2.f * bk[4], h5 = 2.f * bk[5], h6 = 2.f * bk[6];
+        const float b0 = __ldg(b), b1 = __ldg(b + NPHI), b2 = __ldg(b + 2 * NPHI), b3 = __ldg(b + 3 * NPHI);
+        gx -= fmaf(bk[1], b0, fmaf(h4, b1, fmaf(bk[7], b2, bk[8] * b3)));
+        gy -= fmaf(bk[2], b0, fmaf(bk[7], b1, fmaf(h5, b2, bk[9] * b3)));
+        gz -= fmaf(bk[3], b0, fmaf(bk[8], b1, fmaf(bk[9], b2, h6 * b3)));
+        if (WANT_VIR) {
+            const float b4 = __ldg(b + 4 * NPHI), b5 = __ldg(b + 5 * NPHI), b6 = __ldg(b + 6 * NPHI);
+            const float b7 = __ldg(b + 7 * NPHI), b8 = __ldg(b + 8 * NPHI), b9 = __ldg(b + 9 * NPHI);
+            w9[0] = fmaf(bk[1], b1, fmaf(h4, b4, fmaf(bk[7], b7, bk[8] * b8)));
+            w9[1] = fmaf(bk[1], b2, fmaf(h4, b7, fmaf(bk[7], b5, bk[8] * b9)));
+            w9[2] = fmaf(bk[1], b3, fmaf(h4, b8, fmaf(bk[7], b9, bk[8] * b6)));
+            w9[3] = fmaf(bk[2], b1, fmaf(bk[7], b4, fmaf(h5, b7, bk[9] * b8)));
+            w9[4] = fmaf(bk[2], b2, fmaf(bk[7], b7, fmaf(h5, b5, bk[9] * b9)));
+            w9[5] = fmaf(bk[2], b3, fmaf(bk[7], b8, fmaf(h5, b9, bk[9] * b6)));
+            w9[6] = fmaf(bk[3], b1, fmaf(bk[8], b4, fmaf(bk[9], b7, h6 * b8)));
+            w9[7] = fmaf(bk[3], b2, fmaf(bk[8], b7, fmaf(bk[9], b5, h6 * b9)));
+            w9[8] = fmaf(bk[3], b3, fmaf(bk[8], b8, fmaf(bk[9], b9, h6 * b6)));
+        }
     }
 #pragma unroll
-    for (int o = 1; o <= 4; o <<= 1) {
+    for (int o = 1; o < LPA; o <<= 1) {
         gx += __shfl_xor_sync(FULL, gx, o);
         gy += __shfl_xor_sync(FULL, gy, o);
         gz += __shfl_xor_sync(FULL, gz, o);
     }
     if (WANT_VIR) {
+        w9[0] += w6[0], w9[4] += w6[1], w9[8] += w6[2];
+        w9[1] += w6[3], w9[3] += w6[3], w9[2] += w6[4], w9[6] += w6[4], w9[5] += w6[5], w9[7] += w6[5];
 #pragma unroll
-        for (int o = 1; o <= 4; o <<= 1)
+        for (int o = 1; o < LPA; o <<= 1)
 #pragma unroll
-            for (int q = 0; q < 9; ++q) w[q] += __shfl_xor_sync(FULL, w[q], o);
+            for (int q = 0; q < 9; ++q) w9[q] += __shfl_xor_sync(FULL, w9[q], o);
     }
-    if (!valid) return;
-    if (m == 0) {
+    if (WANT_CBAR) {
+#pragma unroll
+        for (int o = 8; o < LPA; o <<= 1) cb += __shfl_xor_sync(FULL, cb, o);
+        if (g == 0 && valid) cbar[(size_t)atom * NPHI + m] = cb;
+    }
+    if (sub == 0 && valid) {
         float* gr = grad + (size_t)atom * 3;
-        if (out.first) {  // the first reverse layer starts the sums (no memset)
-            gr[0] = gx;
-            gr[1] = gy;
-            gr[2] = gz;
-        } else {
-            gr[0] += gx;
-            gr[1] += gy;
-            gr[2] += gz;
+        if (!out.first) {  // the first reverse layer starts the sums (no memset)
+            gx += gr[0];
+            gy += gr[1];
+            gz += gr[2];
         }
         if (out.forces) {  // the last layer: F = -dE/dr and eps_i in caller order
             const int64_t c = out.perm[atom];
-            out.forces[3 * c] = -gr[0];
-            out.forces[3 * c + 1] = -gr[1];
-            out.forces[3 * c + 2] = -gr[2];
+            out.forces[3 * c] = -gx;
+            out.forces[3 * c + 1] = -gy;
+            out.forces[3 * c + 2] = -gz;
             if (out.atom_energy) out.atom_energy[c] = out.eps[atom];
+        } else {
+            gr[0] = gx;
+            gr[1] = gy;
+            gr[2] = gz;
         }
         if (WANT_VIR) {
             float* vr = vir + (size_t)atom * 9;
 #pragma unroll
-            for (int q = 0; q < 9; ++q) vr[q] = out.first ? w[q] : vr[q] + w[q];
+            for (int q = 0; q < 9; ++q) vr[q] = out.first ? -w9[q] : vr[q] - w9[q];
         }
     }
-    if (WANT_CBAR) cbar[(size_t)atom * NPHI + m] = cb;
 }
 
 // ------------------------------------------------------- small kernels ---
@@ -739,47 +839,43 @@ cudaError_t launch_gather_ghost_rows(cudaStream_t s, const reann_nlist* nl, floa
     return cudaGetLastError();
 }
 
-// Preferred shared-memory carveout (percent of the 228 KB maximum) of the edge
-// kernels; the rest of the 256 KB per SM serves as L1 for the neighbour
-// gathers.  40 % (a 100 KB configuration) holds four forward blocks and 50 %
-// (132 KB) sixteen adjoint blocks, their occupancy limits by registers (60 % and
-// 80 % were 1 % and 4 % slower for the adjoint); on the
-// 24,576-atom water box this is 2 % faster for the forward than the driver's
-// choice, and a 0 % hint (fewer resident blocks) 1.5-6 x slower.
-constexpr int kFwdCarveout = 40;
-constexpr int kAdjCarveout = 50;
-static void ensure_edge_attrs() {
-    static std::mutex mu;
-    static uint64_t done = 0;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 64 && ((done >> dev) & 1)) return;
-    const auto carve = [](const void* k, int pct) {
-        if (pct >= 0) cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-    };
-    carve((const void*)k_density_fwd<false>, kFwdCarveout);
-    carve((const void*)k_density_fwd<true>, kFwdCarveout);
-    carve((const void*)k_density_adj8<false, false>, kAdjCarveout);
-    carve((const void*)k_density_adj8<false, true>, kAdjCarveout);
-    carve((const void*)k_density_adj8<true, false>, kAdjCarveout);
-    carve((const void*)k_density_adj8<true, true>, kAdjCarveout);
-    if (dev < 64) done |= (uint64_t)1 << dev;
+cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                         int* flags) {
+    if (rows == 0) return cudaSuccess;
+    launch_pdl(k_edges, blocks_for(rows, kEdgeWarps), kEdgeWarps * 32, 0, s, row0, rows, nl->stride, r, nl->nbr,
+               nl->nbr_cnt, nl->pos, nl->edge_xyzj, nl->edge_phi, nl->edge_der, nl->live_cnt, flags);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, const float* W, const float* coef,
-                               float* rho, float* bck, bool pairs) {
-    ensure_edge_attrs();
-    const int64_t per_block = kWarps * kAtomsPerWarp;
-    const int64_t nr = rows_of(nl);
-    if (nr == 0) return cudaSuccess;
-    const unsigned nb = blocks_for(nr, per_block);
-    if (pairs)
-        launch_pdl(k_density_fwd<true>, nb, kWarps * 32, 0, s, nr, nl->stride, r, nl->live, nl->live_cnt, nl->pos_hi,
-                   nl->pos_lo, coef, W, rho, bck);
-    else
-        launch_pdl(k_density_fwd<false>, nb, kWarps * 32, 0, s, nr, nl->stride, r, nl->live, nl->live_cnt, nl->pos_hi,
-                   nl->pos_lo, coef, W, rho, bck);
+cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                               const float* W, const float* coef, float* rho, float* bck, bool pairs) {
+    if (rows == 0) return cudaSuccess;
+    // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer need
+    // less reduction work per atom (many).  us per launch with 16 / 8 / 4 lanes: 192 atoms 4.5 / 5.6 /
+    // 7.9, 4,000 5.5 / 5.8 / 7.1, 10,976 11.8 / 10.8 / 9.1, 24,576 25 / 20 / 20, 1,048,576 914 / 670 / 536.
+    const int lpa = rows <= 4096 ? 16 : (rows <= 8192 ? 8 : 4);
+    // records of more rows than this outgrow L2 between the passes: prefetch each atom's when it
+    // starts (1,048,576 atoms: 580 -> 541 us; 24,576 atoms: 19.9 -> 20.2 us, so not there)
+    const bool far = rows > (int64_t)1 << 16;
+#define REANN_FWD(P, L)                                                                                              \
+    k_density_fwd<P, L><<<blocks_for(rows, kFwdWarps * (32 / L)), kFwdWarps * 32, 0, s>>>(                             \
+        row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, coef, W, rho, bck, far)
+    if (pairs) {
+        if (lpa == 16)
+            REANN_FWD(true, 16);
+        else if (lpa == 8)
+            REANN_FWD(true, 8);
+        else
+            REANN_FWD(true, 4);
+    } else {
+        if (lpa == 16)
+            REANN_FWD(false, 16);
+        else if (lpa == 8)
+            REANN_FWD(false, 8);
+        else
+            REANN_FWD(false, 4);
+    }
+#undef REANN_FWD
     return cudaGetLastError();
 }
 
@@ -807,19 +903,27 @@ cudaError_t upload_pair_table() {
     return e;
 }
 
-cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radial& r, const float* rec, float* cbar,
-                               float* grad, bool want_cbar, int* flags, float* vir, float* forces, float* atom_energy,
-                               bool first) {
+cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
+                               const float* rec, const float* bck, float* cbar, float* grad, bool want_cbar,
+                               float* vir, float* forces, float* atom_energy, bool first) {
     const Outputs out{forces ? nl->perm : nullptr, forces ? nl->eps : nullptr, forces, atom_energy, first};
-    (void)flags;
-    ensure_edge_attrs();
-    const int64_t per_block = kAdjWarps * kAdjGroups;
-    const int64_t nr = rows_of(nl);
-    if (nr == 0) return cudaSuccess;
-    const unsigned nb = blocks_for(nr, per_block);
-#define REANN_ADJ(C, V)                                                                                              \
-    launch_pdl(k_density_adj8<C, V>, nb, kAdjWarps * 32, 0, s, nr, nl->stride, r, nl->live, nl->live_cnt,       \
-               nl->pos_hi, nl->pos_lo, rec, cbar, grad, vir, out)
+    if (rows == 0) return cudaSuccess;
+    // Lanes per atom, as in the forward pass.  us per launch with 32 / 16 / 8 lanes: 192 atoms 7.2 /
+    // 10.6 / 18.3, 4,000 8.6 / 11.1 / 16.1, 24,576 43.5 / 41.1 / 49, 32,000 53 / 47.0 / 45.6,
+    // 1,048,576 1,644 / 1,242 / 1,161.
+    const int lpa = rows <= 16384 ? 32 : (rows <= 28672 ? 16 : 8);
+#define REANN_ADJ_L(C, V, L)                                                                                       \
+    k_density_adj<C, V, L><<<blocks_for(rows, kAdjWarps * (32 / L)), kAdjWarps * 32, 0, s>>>(                          \
+        row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, nl->edge_der, rec, bck, cbar, grad, vir, out)
+#define REANN_ADJ(C, V)              \
+    do {                             \
+        if (lpa == 32)               \
+            REANN_ADJ_L(C, V, 32);   \
+        else if (lpa == 16)          \
+            REANN_ADJ_L(C, V, 16);   \
+        else                         \
+            REANN_ADJ_L(C, V, 8);    \
+    } while (0)
     if (want_cbar && vir)
         REANN_ADJ(true, true);
     else if (want_cbar)
@@ -829,6 +933,7 @@ cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radi
     else
         REANN_ADJ(false, false);
 #undef REANN_ADJ
+#undef REANN_ADJ_L
     return cudaGetLastError();
 }
 

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
         const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
         for (int m = 0; m < NPHI; ++m) o[m] = 0.f;
-        const float two_w = 2.f * ang_w(a);
+        const float two_w = 2.f * rec_scale(a) * ang_w(a);
         const float* wl = sWc + l * NORB * NPHI;
 #pragma unroll 4
         for (int k = 0; k < NORB; ++k) {

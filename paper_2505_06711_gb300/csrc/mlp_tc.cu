@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
                 const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
                 for (int m = 0; m < NPHI; ++m) o[m] = 0.f;
-                const float two_w = 2.f * ang_w(a_);
+                const float two_w = 2.f * rec_scale(a_) * ang_w(a_);
                 const float* wl = par + B_WC + l * NORB * NPHI;
                 const float* rl = rb + l * NORB;
 #pragma unroll 4

@@ -640,7 +640,7 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
 __global__ void k_refresh(int64_t n, const int32_t* __restrict__ g_count, int64_t g_cap, CellGeom g,
                           const double* __restrict__ pos, const int32_t* __restrict__ perm,
                           const int32_t* __restrict__ wrapm, const int32_t* __restrict__ owner,
-                          const int32_t* __restrict__ shift, float4* __restrict__ hi, float4* __restrict__ lo,
+                          const int32_t* __restrict__ shift, float4* __restrict__ out,
                           const int32_t* __restrict__ species, const float* __restrict__ c0,
                           float* __restrict__ coef) {
     pdl_enter();
@@ -665,64 +665,14 @@ __global__ void k_refresh(int64_t n, const int32_t* __restrict__ g_count, int64_
         h[k] = (float)x[k];
         l[k] = (float)(x[k] - (double)h[k]);
     }
-    hi[s] = make_float4(h[0], h[1], h[2], 0.f);
-    lo[s] = make_float4(l[0], l[1], l[2], 0.f);
+    out[2 * s] = make_float4(h[0], h[1], h[2], 0.f);
+    out[2 * s + 1] = make_float4(l[0], l[1], l[2], 0.f);
     if (c0) {
         const float4* src = reinterpret_cast<const float4*>(c0 + species[o] * NPHI);
         float4* dst = reinterpret_cast<float4*>(coef + (size_t)s * NPHI);
         dst[0] = src[0];
         dst[1] = src[1];
     }
-}
-
-// per evaluation: live (d < r_c) entries of every row, moved to the row's front
-__global__ void __launch_bounds__(256) k_live(int64_t n, int stride, float rc2, float band,
-                                             const int32_t* __restrict__ nbr,
-                                             const int32_t* __restrict__ cnt, const float4* __restrict__ hi,
-                                             const float4* __restrict__ lo, int32_t* __restrict__ live,
-                                             int32_t* __restrict__ live_cnt, int* __restrict__ flags) {
-    pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n) return;
-    const float4 hi_i = hi[i], lo_i = lo[i];
-    const int c = cnt[i];
-    const int32_t* row = nbr + (size_t)i * stride;
-    int32_t* out = live + (size_t)i * stride;
-    int count = 0;
-    for (int base = 0; base < c; base += 32) {
-        const int e = base + lane;
-        bool keep = false;
-        int j = 0;
-        if (e < c) {
-            j = row[e];
-            // the high parts decide unless d^2 is within `band` of rc2 (or tiny): then the hi + lo
-            // difference decides, as it always did, so the decision is the same with half the loads
-            const float4 hj = hi[j];
-            const float xh = hj.x - hi_i.x, yh = hj.y - hi_i.y, zh = hj.z - hi_i.z;
-            const float d2h = xh * xh + yh * yh + zh * zh;
-            if (d2h < rc2 - band && d2h > 0.01f) {
-                keep = true;
-            } else if (d2h > rc2 + band) {
-                keep = false;
-            } else {
-                const float4 lj = lo[j];
-                const float x = (hj.x - hi_i.x) + (lj.x - lo_i.x);
-                const float y = (hj.y - hi_i.y) + (lj.y - lo_i.y);
-                const float z = (hj.z - hi_i.z) + (lj.z - lo_i.z);
-                const float d2 = x * x + y * y + z * z;
-                keep = d2 < rc2;
-                if (!(d2 > 1e-16f)) {
-                    keep = false;
-                    atomicOr(&flags[FLAG_GEOM], 4);
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (keep) out[count + __popc(m & ((1u << lane) - 1u))] = j;
-        count += __popc(m);
-    }
-    if (lane == 0) live_cnt[i] = count;
 }
 
 // largest displacement since the build: flag when any atom moved more than half the skin
@@ -959,19 +909,8 @@ const int32_t* ghost_count_ptr(const reann_nlist* nl) { return nl->w.goff + nl->
 cudaError_t launch_refresh_positions(cudaStream_t s, const reann_nlist* nl, const double* pos, const float* c0) {
     const int64_t total = nl->n + nl->g_cap;
     launch_pdl(k_refresh, blocks_for(total, kFp64Threads), kFp64Threads, 0, s, nl->n, ghost_count_ptr(nl), nl->g_cap,
-               nl->geom, pos, nl->perm, nl->wrapm, nl->g_owner, nl->g_shift, nl->pos_hi, nl->pos_lo, nl->species, c0,
+               nl->geom, pos, nl->perm, nl->wrapm, nl->g_owner, nl->g_shift, nl->pos, nl->species, c0,
                nl->coef);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_live_edges(cudaStream_t s, const reann_nlist* nl, float rc2, int* flags) {
-    const int64_t nr = rows_of(nl);
-    if (nr == 0) return cudaSuccess;
-    // the band bounds the low parts' share of d^2 with room to spare: the search's FP32 margin
-    // (16 r_cut ulp(largest coordinate) + 1e-4 A^2) plus 0.05 A^2
-    const float band = nl->geom.margin + 0.05f;
-    launch_pdl(k_live, blocks_for(nr * 32, 256), 256, 0, s, nr, nl->stride, rc2, band, nl->nbr, nl->nbr_cnt,
-               nl->pos_hi, nl->pos_lo, nl->live, nl->live_cnt, flags);
     return cudaGetLastError();
 }
 

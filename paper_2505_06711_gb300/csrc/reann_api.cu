@@ -130,13 +130,35 @@ T* nl_alloc(reann_nlist* nl, size_t count) {
     return nlist_alloc<T>(nl, count);
 }
 
+// Edge records (32 B per row entry) of `rows` rows, or of the largest half, quarter, ... of
+// them that device memory has room for (at least 1,024 rows): an evaluation then recomputes
+// the records of one run of rows at a time in every pass instead of keeping all of them.
+bool alloc_edge_records(reann_nlist* nl, int64_t rows) {
+    for (;;) {
+        const size_t count = (size_t)rows * nl->stride, first = nl->allocs.size();
+        nl->edge_xyzj = nl_alloc<float4>(nl, count);
+        nl->edge_phi = nl->edge_xyzj ? nl_alloc<float2>(nl, count) : nullptr;
+        nl->edge_der = nl->edge_phi ? nl_alloc<float2>(nl, count) : nullptr;
+        nl->edge_rows = rows;
+        if (nl->edge_der) return true;
+        while (nl->allocs.size() > first) {
+            void* p = nl->allocs.back();
+            nl->allocs.pop_back();
+            if (nl->mem_pool)
+                cudaFreeAsync(p, nl->alloc_stream);
+            else
+                cudaFree(p);
+        }
+        if (rows <= 1024) return false;
+        rows = std::max<int64_t>(1024, (rows + 1) / 2);
+    }
+}
+
 // ranges: (element, first row, end row) of the network tiles; default the element ranges
 int alloc_eval_buffers(reann_ctx* ctx, reann_nlist* nl, const std::vector<std::array<int, 3>>* ranges = nullptr) {
     const int64_t n = nl->n, ne = nl->n + nl->g_cap, T = nl->T;
-    nl->live = nl_alloc<int32_t>(nl, (size_t)n * nl->stride);
     nl->live_cnt = nl_alloc<int32_t>(nl, n);
-    nl->pos_hi = nl_alloc<float4>(nl, ne);
-    nl->pos_lo = nl_alloc<float4>(nl, ne);
+    nl->pos = nl_alloc<float4>(nl, 2 * ne);
     nl->coef = nl_alloc<float>(nl, (size_t)T * ne * NPHI);
     nl->n_feat = ctx->model.n_feat();
     nl->rho = nl_alloc<float>(nl, (size_t)T * n * nl->n_feat);
@@ -168,12 +190,13 @@ int alloc_eval_buffers(reann_ctx* ctx, reann_nlist* nl, const std::vector<std::a
     if (!nl->tiles128_h.empty())
         REANN_CUDA_TRY(ctx, cudaMemcpyAsync(nl->tiles128, nl->tiles128_h.data(), sizeof(Tile) * nl->tiles128_h.size(),
                                             cudaMemcpyHostToDevice, ctx->stream));
-    if (!nl->live || !nl->live_cnt || !nl->pos_hi || !nl->pos_lo || !nl->coef || !nl->rho || !nl->bck || !nl->eps ||
+    if (!nl->live_cnt || !nl->pos || !nl->coef || !nl->rho || !nl->bck || !nl->eps ||
         !nl->rhobar || !nl->dsave || !nl->bbar || !nl->cbar || !nl->grad || !nl->partial || !nl->tiles)
         return set_error(ctx, REANN_E_NOMEM, "evaluation buffers: out of device memory");
     if (!nl->tiles_h.empty())
         REANN_CUDA_TRY(ctx, cudaMemcpyAsync(nl->tiles, nl->tiles_h.data(), sizeof(Tile) * nl->tiles_h.size(),
                                             cudaMemcpyHostToDevice, ctx->stream));
+    if (!alloc_edge_records(nl, n)) return set_error(ctx, REANN_E_NOMEM, "edge records: out of device memory");
     // unused ghost capacity keeps finite values; no live edges before the first evaluation
     REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->bbar, 0, sizeof(float) * ne * NREC, ctx->stream));
     REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->live_cnt, 0, sizeof(int32_t) * n, ctx->stream));
@@ -360,7 +383,12 @@ extern "C" int reann_ctx_create(const reann_model* model, void* cuda_stream, rea
     for (int m = 0; m < NPHI; ++m) {
         split(m * delta, R.mu_hi[m], R.mu_lo[m]);
         split(std::exp(-M.alpha * delta * delta * (2 * m + 1)), R.kap_hi[m], R.kap_lo[m]);
+        R.two_a_mu[m] = (float)(2.0 * M.alpha * m * delta);
     }
+    // exp(-40) f_c is normal down to f_c = 1e-20; wider Gaussian ranges are scaled up to that (2^58 at most)
+    const int sh = (int)std::ceil(std::max(0.0, M.alpha * M.r_c * M.r_c - 40.0) / std::log(2.0));
+    R.scale = (float)std::ldexp(1.0, sh);
+    R.unscale = (float)std::ldexp(1.0, -sh);
     // device image of the parameters: c0, W, then per (t, e) W1 b1 W2 b2 W3 b3 W1t W2t W3t
     std::vector<float> img;
     const float* p = M.params.data();
@@ -920,10 +948,26 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
         ProfScope p(ctx, PR_INIT);
         REANN_CUDA_TRY(ctx, launch_init_coef(s, nl, ctx->d_c0));
     }
-    {
+    // live edges and their records: once for all passes, or, when the records of only a part of
+    // the rows fit, before each pass for one run of rows at a time
+    const int64_t nr = rows_of(nl);
+    const bool keep_edges = nr <= nl->edge_rows;
+    auto edges = [&](int64_t row0, int64_t rows) -> int {
         ProfScope p(ctx, PR_LIVE);
-        REANN_CUDA_TRY(ctx, launch_live_edges(s, nl, ctx->radial.rc2, ctx->d_flags));
-    }
+        REANN_CUDA_TRY(ctx, launch_edges(s, nl, ctx->radial, row0, rows, ctx->d_flags));
+        return REANN_OK;
+    };
+    auto edge_pass = [&](auto&& pass) -> int {  // pass(row0, rows) over all rows
+        for (int64_t r0 = 0; r0 < nr; r0 += nl->edge_rows) {
+            const int64_t rows = std::min(nl->edge_rows, nr - r0);
+            if (!keep_edges)
+                if (int rc = edges(r0, rows)) return rc;
+            if (int rc = pass(r0, rows)) return rc;
+        }
+        return REANN_OK;
+    };
+    if (keep_edges)
+        if (int rc = edges(0, nr)) return rc;
     const bool pairs = ctx->model.pairs;
     const size_t lw = (size_t)(LMAX + 1) * NPHI * ctx->model.n_orb();
     const int64_t nf = nl->n_feat;
@@ -938,10 +982,13 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
             ProfScope p(ctx, PR_GATHER);  // ghost slots receive their owners' coefficients (Fig. 4a)
             REANN_CUDA_TRY(ctx, launch_gather_ghost_rows(s, nl, coef_t, NPHI));
         }
-        {
-            ProfScope p(ctx, PR_DENSITY_FWD);
-            REANN_CUDA_TRY(ctx, launch_density_fwd(s, nl, ctx->radial, ctx->d_W + t * lw, coef_t, rho_t, bck_t, pairs));
-        }
+        if (int rc = edge_pass([&](int64_t r0, int64_t rows) -> int {
+                ProfScope p(ctx, PR_DENSITY_FWD);
+                REANN_CUDA_TRY(ctx, launch_density_fwd(s, nl, ctx->radial, r0, rows, ctx->d_W + t * lw, coef_t, rho_t,
+                                                       bck_t, pairs));
+                return REANN_OK;
+            }))
+            return rc;
         ProfScope p(ctx, PR_MLP_FWD);
         const bool energy_net = t == T - 1;
         // the FP32 energy network also sums the tiles' energies (unless per-structure sums are wanted)
@@ -993,10 +1040,14 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
             ProfScope p(ctx, PR_GATHER);  // ghost slots receive their owners' adjoints (vector-Jacobian product)
             REANN_CUDA_TRY(ctx, launch_gather_ghost_rows(s, nl, nl->bbar, NREC));
         }
-        ProfScope p(ctx, PR_DENSITY_ADJ);
-        REANN_CUDA_TRY(ctx, launch_density_adj(s, nl, ctx->radial, nl->bbar, nl->cbar, nl->grad, t >= 1,
-                                               ctx->d_flags, vir, t == 0 ? forces : nullptr,
-                                               t == 0 ? atom_energy : nullptr, t == T - 1));
+        if (int rc = edge_pass([&](int64_t r0, int64_t rows) -> int {
+                ProfScope p(ctx, PR_DENSITY_ADJ);
+                REANN_CUDA_TRY(ctx, launch_density_adj(s, nl, ctx->radial, r0, rows, nl->bbar, bck_t, nl->cbar,
+                                                       nl->grad, t >= 1, vir, t == 0 ? forces : nullptr,
+                                                       t == 0 ? atom_energy : nullptr, t == T - 1));
+                return REANN_OK;
+            }))
+            return rc;
     }
     ProfScope p(ctx, PR_OUTPUT);
     if (vir) {
@@ -1553,8 +1604,7 @@ extern "C" int reann_serve_create(reann_ctx* ctx, int64_t max_atoms, int64_t max
               cudaMemset(p->nbr_cnt, 0, sizeof(int32_t) * max_atoms) == cudaSuccess &&
               cudaMemset(p->species, 0, sizeof(int32_t) * max_atoms) == cudaSuccess &&
               cudaMemset(p->g_owner, 0, sizeof(int32_t) * std::max<int64_t>(max_ghosts, 1)) == cudaSuccess &&
-              cudaMemset(p->pos_hi, 0, sizeof(float4) * (max_atoms + max_ghosts)) == cudaSuccess &&
-              cudaMemset(p->pos_lo, 0, sizeof(float4) * (max_atoms + max_ghosts)) == cudaSuccess &&
+              cudaMemset(p->pos, 0, sizeof(float4) * 2 * (max_atoms + max_ghosts)) == cudaSuccess &&
               cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) return fail(REANN_E_CUDA, "serving pool: initialisation failed");
     *out = srv;
@@ -1762,5 +1812,13 @@ extern "C" int reann_serve_usage(reann_serve* srv, int64_t* free_atoms, int64_t*
     if (free_atoms) *free_atoms = fa;
     if (free_ghosts) *free_ghosts = fg;
     if (free_slots) *free_slots = fs;
+    return REANN_OK;
+}
+
+// Not part of the ABI: keep the edge records of at most `rows` rows, as when device memory
+// has no room for all of them (call it before the list's first evaluation).
+extern "C" int reann_test_limit_edge_rows(reann_nlist* nl, int64_t rows) {
+    if (!nl || rows < 1) return REANN_E_ARG;
+    nl->edge_rows = std::min(nl->edge_rows, rows);
     return REANN_OK;
 }

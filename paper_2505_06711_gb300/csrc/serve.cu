@@ -53,7 +53,7 @@ struct PackDst {
     int64_t no, ob, gb;  // pool owned size, owned base, ghost base
     int stride;
     int32_t *nbr, *cnt, *species, *perm, *owner;
-    float4 *hi, *lo;
+    float4* pos_out;  // hi, lo parts of each slot, interleaved
 };
 
 // owned atoms: rows (remapped), species, destination, positions
@@ -76,7 +76,7 @@ __global__ void k_pack_owned(PackSrc s, PackDst d) {
     shift_vec(s.geom, s.wrapm[3 * i], s.wrapm[3 * i + 1], s.wrapm[3 * i + 2], sm);
 #pragma unroll
     for (int k = 0; k < 3; ++k) x[k] = s.pos[3 * ci + k] - sm[k];
-    hilo(x, d.hi[d.ob + i], d.lo[d.ob + i]);
+    hilo(x, d.pos_out[2 * (d.ob + i)], d.pos_out[2 * (d.ob + i) + 1]);
 }
 
 // ghost slots: owner (pool index) and image position
@@ -94,7 +94,7 @@ __global__ void k_pack_ghosts(PackSrc s, PackDst d) {
     shift_vec(s.geom, a, b, c, sv);
 #pragma unroll
     for (int k = 0; k < 3; ++k) x[k] = (s.pos[3 * co + k] - sm[k]) + sv[k];
-    hilo(x, d.hi[d.no + d.gb + q], d.lo[d.no + d.gb + q]);
+    hilo(x, d.pos_out[2 * (d.no + d.gb + q)], d.pos_out[2 * (d.no + d.gb + q) + 1]);
 }
 
 // a released owned range: no neighbours, outputs to the sink row
@@ -144,7 +144,7 @@ cudaError_t launch_pack(cudaStream_t s, const reann_nlist* src, const double* ca
     PackSrc a{src->n,       src->g,     src->stride, src->nbr,      src->nbr_cnt, src->species,
               src->perm,    src->wrapm, src->g_owner, src->g_shift, caller_pos,   src->geom};
     PackDst b{pool->n, ob, gb, pool->stride, pool->nbr, pool->nbr_cnt, pool->species, pool->perm, pool->g_owner,
-              pool->pos_hi, pool->pos_lo};
+              pool->pos};
     launch_pdl(k_pack_owned, blocks_for(src->n, 128), 128, 0, s, a, b);
     if (src->g > 0) launch_pdl(k_pack_ghosts, blocks_for(src->g, 256), 256, 0, s, a, b);
     return cudaGetLastError();
