@@ -526,10 +526,19 @@ cudaError_t launch_unpermute_rows(cudaStream_t s, const reann_nlist* nl, const f
 
 // atomic networks, FP32 SIMT (mlp_fp32.cu)
 // dsave (N x 128, optional): the forward keeps SiLU'(z1), SiLU'(z2) of every row for the backward;
-// epart (energy network, optional): one FP64 energy partial sum per tile (reann_nlist::tiles order)
+// epart (energy network, optional): one FP64 energy partial sum per block (in reann_nlist::tiles order);
+// the 48-feature energy network has its own launcher
 cudaError_t launch_mlp_fwd_f32(cudaStream_t s, const reann_nlist* nl, const NetTable& nets, int t, bool energy,
                                const float* rho, float* out, int out_stride, bool pairs, GhostOut gh, float* dsave,
                                double* epart, int* flags);
+// blocks per 64-row tile of the FP32 networks (1, 2 or 4, by the number of tiles); epart holds
+// one partial sum per block
+int mlp_parts_f32(const reann_nlist* nl);
+// the 48-feature energy network, forward and backward, and its bbar step: eps, epart (nullable)
+// and the adjoint records
+cudaError_t launch_mlp_energy_f32(cudaStream_t s, const reann_nlist* nl, const NetTable& nets, int t, const float* rho,
+                                  float* eps, double* epart, const float* Wt, const float* bck, const float* coef,
+                                  float* rec, GhostOut gh, int* flags);
 // total energy from np partial sums, in a fixed order
 cudaError_t launch_energy_final(cudaStream_t s, const double* partial, int np, double* energy);
 // atomic networks on tcgen05 tensor cores (mlp_tc.cu), precision REANN_MLP_BF16,

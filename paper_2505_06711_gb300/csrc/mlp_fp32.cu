@@ -8,14 +8,24 @@
 // gradients.
 //
 // Atoms are stored element-major, so a tile of 64 consecutive rows uses one
-// element's weights.  A block of 256 threads computes a 64x64 layer output as
-// 16x16 threads x (4 rows x 4 columns), reading float4 fragments of the
-// row-major activations and weights from shared memory.  The forward keeps one
+// element's weights.  A block of 256 threads takes 16 RPT rows of a tile (RPT = 4:
+// the whole tile; RPT = 1: a quarter of it, so that the few tiles of a small system
+// occupy four times the SMs and each thread's chain is a quarter as long) and
+// computes a 64-wide layer output as 16 x 16 threads x (RPT rows x 4 columns),
+// reading float4 fragments of the row-major activations and weights from shared
+// memory.  A row's arithmetic is the same for every RPT.  The forward keeps one
 // activation buffer (48 KB of shared memory: four blocks per SM) and writes
 // SiLU'(z1), SiLU'(z2) of every row; the backward reads them instead of
 // recomputing the forward, and with the 48-feature networks also takes the
 // bbar step of Eq. 1's squares and writes the adjoint records (69 KB: three
-// blocks per SM).
+// blocks per SM).  The energy network (48 features) is one kernel, forward and
+// backward: its output adjoint is 1, so nothing waits for another layer, the SiLU'
+// values stay in registers and the tile's weights are staged by one launch (24,576
+// atoms: 15.3 + 23.8 us in two launches, 34.6 us in one; 1,048,576: 407 + 712, 1,071).
+//   Bound by issue: 7,680 FMAs per row forward and 10,240 with the bbar step
+// backward, beside a quarter as many instructions for SiLU and a fifth for the
+// shared-memory fragments (1,048,576 atoms: 436 and 744 us, about 70 % of the issue
+// slots; fma.rn.f32x2 was measured at 0.8 x the FMA rate of single fmas).
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -26,15 +36,26 @@
 namespace reann {
 namespace {
 
-constexpr int kT = 256;       // threads per block
-constexpr int kR = MLP_TILE;  // 64 rows per tile
-constexpr int LDH = H1 + 4;     // 68
+constexpr int kT = 256;      // threads per block
+constexpr int LDH = H1 + 4;  // 68
+static_assert(MLP_TILE == 64, "a block takes 16, 32 or 64 rows of a tile");
 // input rows of FIN features are held with stride FIN (one bulk copy of the
 // tile's contiguous rows) in the buffer that later holds h1 (stride LDH)
 template <int FIN>
 __host__ __device__ constexpr int ldx() { return FIN; }
-template <int FIN>
-__host__ __device__ constexpr int abuf() { return kR * (ldx<FIN>() > LDH ? ldx<FIN>() : LDH); }
+template <int FIN, int RPT>
+__host__ __device__ constexpr int abuf() { return 16 * RPT * (ldx<FIN>() > LDH ? ldx<FIN>() : LDH); }
+
+// the 16 RPT rows of a tile that this block takes (nrows <= 0: none)
+template <int RPT>
+__device__ __forceinline__ Tile block_rows(const Tile* __restrict__ tiles) {
+    constexpr int PARTS = 4 / RPT;
+    Tile t = tiles[blockIdx.x / PARTS];
+    const int skip = 16 * RPT * (int)(blockIdx.x % PARTS);
+    t.row0 += skip;
+    t.nrows = min(t.nrows - skip, 16 * RPT);
+    return t;
+}
 
 struct NetsOfLayer {
     NetDev e[MAX_ELEM];
@@ -62,24 +83,18 @@ __device__ __forceinline__ bool staged(uint64_t* bar, int* flags) {
     return false;
 }
 
-__device__ __forceinline__ void copy_f4(float* dst, const float* src, int count, int tid) {
-    const float4* s = reinterpret_cast<const float4*>(src);
-    float4* d = reinterpret_cast<float4*>(dst);
-    for (int i = tid; i < count / 4; i += kT) d[i] = s[i];
-}
-
-// acc[i][j] += sum_k A[(4ty+i)*LDA + k] * B[k*LDB + 4tx + j], K multiple of 4
-template <int K, int LDA, int LDB>
-__device__ __forceinline__ void mma_4x4(const float* A, const float* B, int ty, int tx, float acc[4][4]) {
+// acc[i][j] += sum_k A[(RPT ty+i)*LDA + k] * B[k*LDB + 4tx + j], K multiple of 4
+template <int K, int LDA, int LDB, int RPT>
+__device__ __forceinline__ void mma_rx4(const float* A, const float* B, int ty, int tx, float acc[RPT][4]) {
 #pragma unroll 4
     for (int k = 0; k < K; k += 4) {
-        float4 a[4], b[4];
+        float4 a[RPT], b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(A + (4 * ty + i) * LDA + k);
+        for (int i = 0; i < RPT; ++i) a[i] = *reinterpret_cast<const float4*>(A + (RPT * ty + i) * LDA + k);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) b[kk] = *reinterpret_cast<const float4*>(B + (k + kk) * LDB + 4 * tx);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < RPT; ++i) {
             const float av[4] = {a[i].x, a[i].y, a[i].z, a[i].w};
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
@@ -92,20 +107,25 @@ __device__ __forceinline__ void mma_4x4(const float* A, const float* B, int ty, 
     }
 }
 
-template <int FIN>
-__device__ __forceinline__ void load_rows(float* sX, const float* src, int row0, int nrows, int tid) {
-    // 64 rows x FIN floats -> sX[r][FIN + 4]
-    for (int t = tid; t < kR * (FIN / 4); t += kT) {
-        const int r = t / (FIN / 4), c = t % (FIN / 4);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < nrows) v = *reinterpret_cast<const float4*>(src + (size_t)(row0 + r) * FIN + 4 * c);
-        *reinterpret_cast<float4*>(sX + r * ldx<FIN>() + 4 * c) = v;
-    }
+template <int RPT>
+__device__ __forceinline__ void set_bias(const float* b, int tx, float acc[RPT][4]) {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = b ? b[4 * tx + j] : 0.f;
+}
+// a thread's RPT x 4 values to rows of shared memory (stride LDH)
+template <int RPT>
+__device__ __forceinline__ void put_rows(float* S, int ty, int tx, const float v[RPT][4]) {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+        *reinterpret_cast<float4*>(S + (RPT * ty + i) * LDH + 4 * tx) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
 }
 
-// Sum of 4 * OUT partial values over the 16 lanes of a half-warp (the tx of one
-// ty), as a butterfly reduce-scatter: with NV = 32 lane tx ends with values
-// 2 tx and 2 tx + 1, with NV = 4 every lane ends with value tx / 4.
+// Sum of NV partial values over the 16 lanes of a half-warp (the tx of one ty), as
+// a butterfly reduce-scatter: with NV = 32 lane tx ends with values 2 tx and
+// 2 tx + 1, with fewer every lane ends with value tx / (16 / NV).  The order of a
+// value's additions does not depend on NV.
 template <int NV>
 __device__ __forceinline__ void reduce16(float v[NV], int tx) {
     int cnt = NV;
@@ -136,19 +156,36 @@ __device__ __forceinline__ int w3_row(int k) {
     return (k & 3) * 16 + (k >> 2);
 }
 
+// The tile part's atomic energies (rows r, lanes with `own`) summed in FP64 in a
+// fixed order into *out; sE: 16 RPT doubles of shared memory.
+template <int RPT>
+__device__ __forceinline__ void sum_energies(double* sE, int r, bool own, double e, double* out) {
+    __syncthreads();  // every thread is done with the buffer
+    if (own) sE[r] = e;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int l = threadIdx.x;
+        double x = RPT == 4 ? sE[l] + sE[l + 32] : (RPT == 2 || l < 16 ? sE[l] : 0.0);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (l == 0) *out = x;
+    }
+}
+
 // ----------------------------------------------------------- forward ---
-// Shared memory: weights (31 KB) and one 64 x 68 activation buffer that holds
-// the input rows, then h1; h2 stays in registers and the output layer is a
-// half-warp reduction, so four blocks fit on an SM.  With dsave, the row's
-// SiLU derivatives are kept for the reverse pass: dsave[row][0..63] =
+// Shared memory: weights (31 KB) and one activation buffer that holds the input
+// rows, then h1 (64 x 68 floats at RPT = 4); h2 stays in registers and the output
+// layer is a half-warp reduction, so four blocks fit on an SM.  With dsave, the
+// row's SiLU derivatives are kept for the reverse pass: dsave[row][0..63] =
 // SiLU'(z1), dsave[row][64..127] = SiLU'(z2).
 constexpr int kSave = H1 + H2;
-template <int OUT, int FIN>
+template <int OUT, int FIN, int RPT>
 __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
                                                const float* __restrict__ rho, float* __restrict__ out,
                                                int out_stride, GhostOut gh, float* __restrict__ dsave,
                                                double* __restrict__ epart, int* __restrict__ flags) {
     pdl_enter();
+    constexpr int R = 16 * RPT;
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
     float* sW1 = sm;                 // FIN x 64
@@ -157,15 +194,15 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
     float* sb1 = sW3 + H2 * 8;       // 64
     float* sb2 = sb1 + H1;           // 64
     float* sb3 = sb2 + H2;           // 8
-    float* sA = sb3 + 8;             // input rows (stride FIN + 4), then h1 (stride LDH)
+    float* sA = sb3 + 8;             // input rows (stride FIN), then h1 (stride LDH)
     const int tid = threadIdx.x;
-    const Tile tl = tiles[blockIdx.x];
-    if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list
+    const Tile tl = block_rows<RPT>(tiles);
+    if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
         if (OUT == 1 && epart && tid == 0) epart[blockIdx.x] = 0.0;
         return;
     }
     const NetDev& w = nets.e[tl.elem];
-    if (tid == 0) {  // W1, W2 and the tile's input rows by bulk copies (TMA engine)
+    if (tid == 0) {  // W1, W2 and the input rows by bulk copies (TMA engine)
         bulk::mbar_init(&bar, 1);
         bulk::mbar_init_fence();
         const uint32_t xb = (uint32_t)tl.nrows * FIN * 4;
@@ -178,53 +215,45 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
     for (int i = tid; i < H1; i += kT) sb1[i] = w.b1[i];
     for (int i = tid; i < H2; i += kT) sb2[i] = w.b2[i];
     if (tid < OUT) sb3[tid] = w.b3[tid];
-    for (int i = tl.nrows * FIN + tid; i < kR * FIN; i += kT) sA[i] = 0.f;  // rows past the tile's end
+    for (int i = tl.nrows * FIN + tid; i < R * FIN; i += kT) sA[i] = 0.f;  // rows past the end
     if (!staged(&bar, flags)) return;
     const int ty = tid >> 4, tx = tid & 15;
-    float acc[4][4];
+    float acc[RPT][4];
     // layer 1
+    set_bias<RPT>(sb1, tx, acc);
+    mma_rx4<FIN, ldx<FIN>(), H1, RPT>(sA, sW1, ty, tx, acc);
+    float ds[RPT][4];  // SiLU'(z1) (acc becomes h1)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = sb1[4 * tx + j];
-    mma_4x4<FIN, ldx<FIN>(), H1>(sA, sW1, ty, tx, acc);
-    float ds[4][4];  // SiLU'(z1) (acc becomes h1)
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RPT; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ds[i][j] = silu_d(acc[i][j], acc[i][j]);
     if (dsave)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (4 * ty + i < tl.nrows)
-                *reinterpret_cast<float4*>(dsave + (size_t)(tl.row0 + 4 * ty + i) * kSave + 4 * tx) =
+        for (int i = 0; i < RPT; ++i)
+            if (RPT * ty + i < tl.nrows)
+                *reinterpret_cast<float4*>(dsave + (size_t)(tl.row0 + RPT * ty + i) * kSave + 4 * tx) =
                     make_float4(ds[i][0], ds[i][1], ds[i][2], ds[i][3]);
     __syncthreads();  // every thread is done reading the input rows
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4*>(sA + (4 * ty + i) * LDH + 4 * tx) =
-            make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    put_rows<RPT>(sA, ty, tx, acc);
     __syncthreads();
     // layer 2 (h2 stays in registers)
+    set_bias<RPT>(sb2, tx, acc);
+    mma_rx4<H1, LDH, H2, RPT>(sA, sW2, ty, tx, acc);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = sb2[4 * tx + j];
-    mma_4x4<H1, LDH, H2>(sA, sW2, ty, tx, acc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RPT; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ds[i][j] = silu_d(acc[i][j], acc[i][j]);  // acc becomes h2
     if (dsave)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (4 * ty + i < tl.nrows)
-                *reinterpret_cast<float4*>(dsave + (size_t)(tl.row0 + 4 * ty + i) * kSave + H1 + 4 * tx) =
+        for (int i = 0; i < RPT; ++i)
+            if (RPT * ty + i < tl.nrows)
+                *reinterpret_cast<float4*>(dsave + (size_t)(tl.row0 + RPT * ty + i) * kSave + H1 + 4 * tx) =
                     make_float4(ds[i][0], ds[i][1], ds[i][2], ds[i][3]);
     // layer 3: per-thread partial dot products over its 4 columns, reduced over tx
-    float v[4 * OUT];
+    constexpr int NV = RPT * OUT, PER = NV > 16 ? NV / 16 : 1, DUP = NV < 16 ? 16 / NV : 1;
+    float v[NV];
 #pragma unroll
-    for (int q = 0; q < 4 * OUT; ++q) v[q] = 0.f;
+    for (int q = 0; q < NV; ++q) v[q] = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const float* w3 = sW3 + (j * 16 + tx) * OUT;
@@ -232,146 +261,56 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
         for (int o = 0; o < OUT; ++o) {
             const float wv = w3[o];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i * OUT + o] = fmaf(acc[i][j], wv, v[i * OUT + o]);
+            for (int i = 0; i < RPT; ++i) v[i * OUT + o] = fmaf(acc[i][j], wv, v[i * OUT + o]);
         }
     }
-    reduce16<4 * OUT>(v, tx);
+    reduce16<NV>(v, tx);
+    const int q0 = tx / DUP * PER, r = RPT * ty + q0 / OUT, o = q0 % OUT;  // this lane's value(s): row r, outputs o ..
+    const bool own = tx % DUP == 0;
     if (OUT == 1) {
-        const int r = 4 * ty + (tx >> 2);
         const float e = v[0] + sb3[0];
-        if ((tx & 3) == 0 && r < tl.nrows) out[(size_t)(tl.row0 + r) * out_stride] = e;
-        if (epart) {  // the tile's energy in FP64, summed in a fixed order
-            __syncthreads();  // every thread is done with the activation buffer
-            double* sE = reinterpret_cast<double*>(sA);
-            if ((tx & 3) == 0) sE[r] = r < tl.nrows ? (double)e : 0.0;
-            __syncthreads();
-            if (tid < 32) {
-                double x = sE[tid] + sE[tid + 32];
+        if (own && r < tl.nrows) out[(size_t)(tl.row0 + r) * out_stride] = e;
+        if (epart)
+            sum_energies<RPT>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
+    } else if (own && r < tl.nrows) {
+        const int64_t i = tl.row0 + r;
+        float y[PER];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                if (tid == 0) epart[blockIdx.x] = x;
-            }
+        for (int k = 0; k < PER; ++k) {
+            y[k] = v[k] + sb3[o + k];
+            out[(size_t)i * out_stride + o + k] = y[k];
         }
-    } else {
-        const int r = 4 * ty + (tx >> 2), o = 2 * (tx & 3);
-        if (r < tl.nrows) {
-            const int64_t i = tl.row0 + r;
-            const float y0 = v[0] + sb3[o], y1 = v[1] + sb3[o + 1];
-            float* dst = out + (size_t)i * out_stride + o;
-            dst[0] = y0;
-            dst[1] = y1;
-            if (gh.goff)  // the row's ghost images get the same coefficients (Fig. 4a)
-                for (int64_t g = gh.goff[i]; g < gh.goff[i + 1] && g < gh.gcap; ++g) {
-                    float* gd = out + (size_t)(gh.base + g) * out_stride + o;
-                    gd[0] = y0;
-                    gd[1] = y1;
-                }
-        }
+        if (gh.goff)  // the row's ghost images get the same coefficients (Fig. 4a)
+            for (int64_t g = gh.goff[i]; g < gh.goff[i + 1] && g < gh.gcap; ++g)
+#pragma unroll
+                for (int k = 0; k < PER; ++k) out[(size_t)(gh.base + g) * out_stride + o + k] = y[k];
     }
 }
 
 // ---------------------------------------------------------- backward ---
 // rhobar = W1 (s1 * (W2 (s2 * (W3 ybar))))   per row, with s1 = SiLU'(z1) and
 // s2 = SiLU'(z2) kept by the forward (dsave), so nothing is recomputed.
-// Shared memory: the transposed weights, ybar, one 64 x 68 buffer (z2bar, then
+// Shared memory: the transposed weights, ybar, one activation buffer (z2bar, then
 // z1bar) and, with BBAR, the rhobar rows and the contraction weights.
 //
 // BBAR (Eq. 1's squares only): instead of writing rhobar, go on to the density
-// adjoint's first step for the tile's rows, bbar_{a,m} = sum_k 2 w_a g_{a,k}
-// rhobar_{l,k} W_{l,m,k} with g = b W recomputed from the b checkpoint (bck), and
-// write the rows' adjoint records, bbar with the layer's c (the separate bbar
-// kernel's work, without the rhobar round trip).
+// adjoint's first step for the rows (bbar_records).
 __device__ __forceinline__ float4 ld_save(const float* dsave, const Tile& tl, int r, int col) {
     if (r >= tl.nrows) return make_float4(0.f, 0.f, 0.f, 0.f);
     return __ldg(reinterpret_cast<const float4*>(dsave + (size_t)(tl.row0 + r) * kSave + col));
 }
 
-template <int OUT, int FIN, bool BBAR>
-__global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
-                                               const float* __restrict__ dsave, const float* __restrict__ ybar,
-                                               float* __restrict__ rhobar, const float* __restrict__ Wt,
-                                               const float* __restrict__ bck, const float* __restrict__ coef,
-                                               float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
-    pdl_enter();
-    __shared__ __align__(8) uint64_t bar;
-    extern __shared__ __align__(16) float sm[];
-    float* sW1t = sm;                 // W1^T: 64 x FIN
-    float* sW2t = sW1t + H1 * FIN;    // W2^T: 64 x 64
-    float* sW3t = sW2t + H1 * H2;     // W3^T: OUT x 64 (8 rows reserved)
-    float* sY = sW3t + 8 * H2;        // 64 x 8
-    float* sG = sY + kR * 8;          // z2bar, then z1bar (stride LDH)
-    float* sR = sG + kR * LDH;        // rhobar rows (BBAR, stride LDH)
-    float* sWc = sR + kR * LDH;       // (L+1) x N_orb x N_phi contraction W^t, transposed per l (BBAR)
-    const int tid = threadIdx.x;
-    const Tile tl = tiles[blockIdx.x];
-    if (tl.nrows <= 0) return;  // padding entry of a fixed-size tile list
-    const int ty = tid >> 4, tx = tid & 15;
-    // the thread's SiLU'(z2), in flight while the weights are staged
-    float4 s2[4];
+// rhobar = z1bar W1^T for the block's rows (z1bar in sG): into sR (stride LDH) with BBAR, else to memory
+template <int FIN, bool BBAR, int RPT>
+__device__ __forceinline__ void rhobar_rows(const float* sG, const float* sW1t, float* sR, float* __restrict__ rhobar,
+                                            const Tile& tl, int ty, int tx) {
+    for (int cg = tx; cg < FIN / 4; cg += 16) {  // FIN / 4 column groups of 4 over the 16 tx
+        float acc[RPT][4];
+        set_bias<RPT>(nullptr, tx, acc);
+        mma_rx4<H1, LDH, FIN, RPT>(sG, sW1t, ty, cg, acc);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s2[i] = ld_save(dsave, tl, 4 * ty + i, H1 + 4 * tx);
-    const NetDev& w = nets.e[tl.elem];
-    if (tid == 0) {  // W1^T, W2^T, W3^T by bulk copies (TMA engine)
-        bulk::mbar_init(&bar, 1);
-        bulk::mbar_init_fence();
-        bulk::mbar_expect_tx(&bar, (H1 * FIN + H1 * H2 + OUT * H2) * 4);
-        bulk::bulk_g2s(sW1t, w.W1t, H1 * FIN * 4, &bar);
-        bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
-        bulk::bulk_g2s(sW3t, w.W3t, OUT * H2 * 4, &bar);
-    }
-    if (BBAR)  // transposed per l: sWc[(l N_orb + k) N_phi + m] = W_{l,m,k}
-        for (int i = tid; i < (LMAX + 1) * NPHI * NORB; i += kT) {
-            const int l = i / (NPHI * NORB), m = (i / NORB) % NPHI, k = i % NORB;
-            sWc[(l * NORB + k) * NPHI + m] = Wt[i];
-        }
-    for (int i = tid; i < kR * OUT; i += kT) {
-        const int r = i / OUT, o = i % OUT;
-        sY[r * 8 + o] = (OUT == 1) ? 1.f : (r < tl.nrows ? ybar[(size_t)(tl.row0 + r) * OUT + o] : 0.f);
-    }
-    if (!staged(&bar, flags)) return;
-    // z2bar = (ybar W3^T) * s2 -> sG
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int o = 0; o < OUT; ++o) {
-            const float y = sY[(4 * ty + i) * 8 + o];
-            const float4 wv = *reinterpret_cast<const float4*>(sW3t + o * H2 + 4 * tx);
-            v[0] = fmaf(y, wv.x, v[0]);
-            v[1] = fmaf(y, wv.y, v[1]);
-            v[2] = fmaf(y, wv.z, v[2]);
-            v[3] = fmaf(y, wv.w, v[3]);
-        }
-        *reinterpret_cast<float4*>(sG + (4 * ty + i) * LDH + 4 * tx) =
-            make_float4(v[0] * s2[i].x, v[1] * s2[i].y, v[2] * s2[i].z, v[3] * s2[i].w);
-    }
-    float4 s1[4];  // SiLU'(z1), in flight during the z1bar product
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s1[i] = ld_save(dsave, tl, 4 * ty + i, 4 * tx);
-    __syncthreads();
-    // z1bar = (z2bar W2^T) * s1
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    mma_4x4<H2, LDH, H1>(sG, sW2t, ty, tx, acc);
-    __syncthreads();  // everyone is done reading z2bar
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4*>(sG + (4 * ty + i) * LDH + 4 * tx) = make_float4(
-            acc[i][0] * s1[i].x, acc[i][1] * s1[i].y, acc[i][2] * s1[i].z, acc[i][3] * s1[i].w);
-    __syncthreads();
-    // rhobar = z1bar W1^T  (64 x FIN): FIN / 4 column groups of 4 over the 16 tx
-    for (int cg = tx; cg < FIN / 4; cg += 16) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-        mma_4x4<H1, LDH, FIN>(sG, sW1t, ty, cg, acc);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = 4 * ty + i;
+        for (int i = 0; i < RPT; ++i) {
+            const int r = RPT * ty + i;
             if (BBAR) {
                 *reinterpret_cast<float4*>(sR + r * LDH + 4 * cg) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
             } else if (r < tl.nrows) {
@@ -380,16 +319,30 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
             }
         }
     }
-    if (!BBAR) return;
-    __syncthreads();
-    // four threads per row, record values v = q, q + 4, q + 8 (angular terms, then c and 0),
-    // staged in shared memory (W1^T, W2^T are no longer needed) and stored as whole lines
-    float* sRec = sW1t;
-    const int r = tid >> 2, q = tid & 3;
+}
+
+// contraction weights transposed per l: sWc[(l N_orb + k) N_phi + m] = W_{l,m,k}
+__device__ __forceinline__ void stage_wc(float* sWc, const float* __restrict__ Wt, int tid) {
+    for (int i = tid; i < (LMAX + 1) * NPHI * NORB; i += kT) {
+        const int l = i / (NPHI * NORB), m = (i / NORB) % NPHI, k = i % NORB;
+        sWc[(l * NORB + k) * NPHI + m] = Wt[i];
+    }
+}
+
+// bbar_{a,m} = sum_k 2 w_a g_{a,k} rhobar_{l,k} W_{l,m,k} of the block's rows, g = b W
+// recomputed from the b checkpoint (bck), written as their adjoint records (bbar with the
+// layer's c, ghost images too) through sRec.  16 / RPT threads per row take the record
+// values v = q, q + 16 / RPT, ... (angular terms, then c and 0).
+template <int RPT>
+__device__ __forceinline__ void bbar_records(const float* sR, const float* sWc, float* sRec, const Tile& tl,
+                                             const float* __restrict__ bck, const float* __restrict__ coef,
+                                             float* __restrict__ rec, const GhostOut& gh, int tid) {
+    constexpr int TPR = 16 / RPT;
+    const int r = tid / TPR, q = tid % TPR;
     const size_t row = (size_t)(tl.row0 + r);
     const float* rb = sR + r * LDH;
 #pragma unroll 1
-    for (int v = q; v < NREC / NPHI && r < tl.nrows; v += 4) {
+    for (int v = q; v < NREC / NPHI && r < tl.nrows; v += TPR) {
         float o[NPHI];
         if (v >= NANG) {
             rec_tail(coef, row, v, o);
@@ -422,14 +375,212 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
     flush_rec(sRec, tl.nrows, tl.row0, rec, gh, tid, kT);  // ghost images get the rows' records too (reverse exchange)
 }
 
-static_assert(NFEAT * H1 + H1 * H2 >= kR * kRecLd, "record staging must fit in the W1, W2 region");
+template <int OUT, int FIN, bool BBAR, int RPT>
+__global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
+                                               const float* __restrict__ dsave, const float* __restrict__ ybar,
+                                               float* __restrict__ rhobar, const float* __restrict__ Wt,
+                                               const float* __restrict__ bck, const float* __restrict__ coef,
+                                               float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
+    pdl_enter();
+    constexpr int R = 16 * RPT;
+    __shared__ __align__(8) uint64_t bar;
+    extern __shared__ __align__(16) float sm[];
+    float* sW1t = sm;                 // W1^T: 64 x FIN
+    float* sW2t = sW1t + H1 * FIN;    // W2^T: 64 x 64
+    float* sW3t = sW2t + H1 * H2;     // W3^T: OUT x 64 (8 rows reserved)
+    float* sY = sW3t + 8 * H2;        // R x 8
+    float* sG = sY + R * 8;           // z2bar, then z1bar (stride LDH)
+    float* sR = sG + R * LDH;         // rhobar rows (BBAR, stride LDH)
+    float* sWc = sR + R * LDH;        // (L+1) x N_orb x N_phi contraction W^t, transposed per l (BBAR)
+    const int tid = threadIdx.x;
+    const Tile tl = block_rows<RPT>(tiles);
+    if (tl.nrows <= 0) return;  // padding entry of a fixed-size tile list, or nothing left of the tile
+    const int ty = tid >> 4, tx = tid & 15;
+    // the thread's SiLU'(z2), in flight while the weights are staged
+    float4 s2[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) s2[i] = ld_save(dsave, tl, RPT * ty + i, H1 + 4 * tx);
+    const NetDev& w = nets.e[tl.elem];
+    if (tid == 0) {  // W1^T, W2^T, W3^T by bulk copies (TMA engine)
+        bulk::mbar_init(&bar, 1);
+        bulk::mbar_init_fence();
+        bulk::mbar_expect_tx(&bar, (H1 * FIN + H1 * H2 + OUT * H2) * 4);
+        bulk::bulk_g2s(sW1t, w.W1t, H1 * FIN * 4, &bar);
+        bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
+        bulk::bulk_g2s(sW3t, w.W3t, OUT * H2 * 4, &bar);
+    }
+    if (BBAR) stage_wc(sWc, Wt, tid);
+    for (int i = tid; i < R * OUT; i += kT) {
+        const int r = i / OUT, o = i % OUT;
+        sY[r * 8 + o] = (OUT == 1) ? 1.f : (r < tl.nrows ? ybar[(size_t)(tl.row0 + r) * OUT + o] : 0.f);
+    }
+    if (!staged(&bar, flags)) return;
+    // z2bar = (ybar W3^T) * s2 -> sG
+    float acc[RPT][4];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int o = 0; o < OUT; ++o) {
+            const float y = sY[(RPT * ty + i) * 8 + o];
+            const float4 wv = *reinterpret_cast<const float4*>(sW3t + o * H2 + 4 * tx);
+            v[0] = fmaf(y, wv.x, v[0]);
+            v[1] = fmaf(y, wv.y, v[1]);
+            v[2] = fmaf(y, wv.z, v[2]);
+            v[3] = fmaf(y, wv.w, v[3]);
+        }
+        acc[i][0] = v[0] * s2[i].x, acc[i][1] = v[1] * s2[i].y, acc[i][2] = v[2] * s2[i].z, acc[i][3] = v[3] * s2[i].w;
+    }
+    put_rows<RPT>(sG, ty, tx, acc);
+    float4 s1[RPT];  // SiLU'(z1), in flight during the z1bar product
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) s1[i] = ld_save(dsave, tl, RPT * ty + i, 4 * tx);
+    __syncthreads();
+    // z1bar = (z2bar W2^T) * s1
+    set_bias<RPT>(nullptr, tx, acc);
+    mma_rx4<H2, LDH, H1, RPT>(sG, sW2t, ty, tx, acc);
+    __syncthreads();  // everyone is done reading z2bar
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        acc[i][0] *= s1[i].x, acc[i][1] *= s1[i].y, acc[i][2] *= s1[i].z, acc[i][3] *= s1[i].w;
+    }
+    put_rows<RPT>(sG, ty, tx, acc);
+    __syncthreads();
+    rhobar_rows<FIN, BBAR, RPT>(sG, sW1t, sR, rhobar, tl, ty, tx);
+    if (!BBAR) return;
+    __syncthreads();
+    // records staged where W1^T, W2^T, no longer needed, were
+    bbar_records<RPT>(sR, sWc, sW1t, tl, bck, coef, rec, gh, tid);
+}
 
-template <int FIN>
-constexpr size_t fwd_smem() { return sizeof(float) * (FIN * H1 + H1 * H2 + H2 * 8 + H1 + H2 + 8 + abuf<FIN>()); }
-template <int FIN, bool BBAR>
+static_assert(NFEAT * H1 + H1 * H2 >= MLP_TILE * kRecLd, "record staging must fit in the W1, W2 region");
+
+// ------------------------------------------------------ energy network ---
+// Forward and backward of the energy network (48 -> 64 -> 64 -> 1) of the block's
+// rows, then the bbar step: eps, the tile's FP64 energy and the adjoint records.
+// ybar = 1, so z2bar = W3 * SiLU'(z2) and nothing but rho is read.  Shared memory: W1,
+// W2 (later rhobar) and W1^T, W2^T (later the records), one activation buffer, the
+// contraction weights: 76 KB, three blocks per SM.
+template <int RPT>
+__global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Tile* __restrict__ tiles,
+                                                      const float* __restrict__ rho, float* __restrict__ eps,
+                                                      double* __restrict__ epart, const float* __restrict__ Wt,
+                                                      const float* __restrict__ bck, const float* __restrict__ coef,
+                                                      float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
+    pdl_enter();
+    constexpr int R = 16 * RPT, F = NFEAT;
+    static_assert(F * H1 + H1 * H2 >= R * LDH, "rhobar rows must fit in the W1, W2 region");
+    __shared__ __align__(8) uint64_t bar;
+    extern __shared__ __align__(16) float sm[];
+    float* sW1 = sm;                // 48 x 64
+    float* sW2 = sW1 + F * H1;      // 64 x 64
+    float* sW1t = sW2 + H1 * H2;    // 64 x 48
+    float* sW2t = sW1t + H1 * F;    // 64 x 64
+    float* sA = sW2t + H1 * H2;     // input rows (stride 48), then h1, z2bar, z1bar (stride LDH)
+    float* sWc = sA + R * LDH;      // contraction weights, transposed per l
+    const int tid = threadIdx.x;
+    const Tile tl = block_rows<RPT>(tiles);
+    if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
+        if (epart && tid == 0) epart[blockIdx.x] = 0.0;
+        return;
+    }
+    const NetDev& w = nets.e[tl.elem];
+    if (tid == 0) {
+        bulk::mbar_init(&bar, 1);
+        bulk::mbar_init_fence();
+        const uint32_t xb = (uint32_t)tl.nrows * F * 4;
+        bulk::mbar_expect_tx(&bar, 2 * (F * H1 + H1 * H2) * 4 + xb);
+        bulk::bulk_g2s(sW1, w.W1, F * H1 * 4, &bar);
+        bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * F, xb, &bar);
+        bulk::bulk_g2s(sW2, w.W2, H1 * H2 * 4, &bar);
+        bulk::bulk_g2s(sW1t, w.W1t, F * H1 * 4, &bar);
+        bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
+    }
+    stage_wc(sWc, Wt, tid);
+    for (int i = tl.nrows * F + tid; i < R * F; i += kT) sA[i] = 0.f;  // rows past the end
+    const int ty = tid >> 4, tx = tid & 15;
+    const float4 b1 = __ldg(reinterpret_cast<const float4*>(w.b1) + tx), b2 = __ldg(reinterpret_cast<const float4*>(w.b2) + tx);
+    const float4 w3 = __ldg(reinterpret_cast<const float4*>(w.W3) + tx);
+    const float b3 = __ldg(w.b3);
+    if (!staged(&bar, flags)) return;
+    float acc[RPT][4], s1[RPT][4];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) acc[i][0] = b1.x, acc[i][1] = b1.y, acc[i][2] = b1.z, acc[i][3] = b1.w;
+    mma_rx4<F, F, H1, RPT>(sA, sW1, ty, tx, acc);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s1[i][j] = silu_d(acc[i][j], acc[i][j]);  // acc becomes h1
+    __syncthreads();  // every thread is done reading the input rows
+    put_rows<RPT>(sA, ty, tx, acc);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) acc[i][0] = b2.x, acc[i][1] = b2.y, acc[i][2] = b2.z, acc[i][3] = b2.w;
+    mma_rx4<H1, LDH, H2, RPT>(sA, sW2, ty, tx, acc);
+    float v[RPT];  // this thread's share of eps (the sum's order is k_mlp_fwd's)
+    const float wv[4] = {w3.x, w3.y, w3.z, w3.w};
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        v[i] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float h;
+            const float d = silu_d(acc[i][j], h);
+            v[i] = fmaf(h, wv[j], v[i]);
+            acc[i][j] = wv[j] * d;  // z2bar
+        }
+    }
+    reduce16<RPT>(v, tx);
+    constexpr int DUP = 16 / RPT;
+    const int r = RPT * ty + tx / DUP;
+    const bool own = tx % DUP == 0;
+    const float e = v[0] + b3;
+    if (own && r < tl.nrows) eps[tl.row0 + r] = e;
+    if (epart)
+        sum_energies<RPT>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
+    __syncthreads();  // h1 and the energies have been read
+    put_rows<RPT>(sA, ty, tx, acc);
+    __syncthreads();
+    set_bias<RPT>(nullptr, tx, acc);
+    mma_rx4<H2, LDH, H1, RPT>(sA, sW2t, ty, tx, acc);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] *= s1[i][j];  // z1bar
+    __syncthreads();
+    put_rows<RPT>(sA, ty, tx, acc);
+    __syncthreads();
+    rhobar_rows<F, true, RPT>(sA, sW1t, sW1, nullptr, tl, ty, tx);
+    __syncthreads();
+    bbar_records<RPT>(sW1, sWc, sW1t, tl, bck, coef, rec, gh, tid);
+}
+
+template <int FIN, int RPT>
+constexpr size_t fwd_smem() { return sizeof(float) * (FIN * H1 + H1 * H2 + H2 * 8 + H1 + H2 + 8 + abuf<FIN, RPT>()); }
+template <int FIN, bool BBAR, int RPT>
 constexpr size_t bwd_smem() {
-    return sizeof(float) * (H1 * FIN + H1 * H2 + 8 * H2 + kR * 8 + kR * LDH +
-                            (BBAR ? kR * LDH + (LMAX + 1) * NPHI * NORB : 0));
+    return sizeof(float) * (H1 * FIN + H1 * H2 + 8 * H2 + 16 * RPT * 8 + 16 * RPT * LDH +
+                            (BBAR ? 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB : 0));
+}
+template <int RPT>
+constexpr size_t energy_smem() {
+    return sizeof(float) * (2 * (NFEAT * H1 + H1 * H2) + 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB);
+}
+static_assert(3 * (energy_smem<4>() + 16 + 1024) <= 228 * 1024, "three blocks of the energy network per SM");
+
+template <typename K>
+void allow_smem(K* k, size_t bytes) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <int RPT>
+void set_attrs() {
+    allow_smem(k_mlp_fwd<NPHI, NFEAT, RPT>, fwd_smem<NFEAT, RPT>());
+    allow_smem(k_mlp_fwd<1, NFEAT_P, RPT>, fwd_smem<NFEAT_P, RPT>());
+    allow_smem(k_mlp_fwd<NPHI, NFEAT_P, RPT>, fwd_smem<NFEAT_P, RPT>());
+    allow_smem(k_mlp_bwd<NPHI, NFEAT, true, RPT>, bwd_smem<NFEAT, true, RPT>());
+    allow_smem(k_mlp_bwd<1, NFEAT_P, false, RPT>, bwd_smem<NFEAT_P, false, RPT>());
+    allow_smem(k_mlp_bwd<NPHI, NFEAT_P, false, RPT>, bwd_smem<NFEAT_P, false, RPT>());
+    allow_smem(k_mlp_energy<RPT>, energy_smem<RPT>());
 }
 void ensure_attrs() {
     // once per device, safe under concurrent first calls
@@ -439,18 +590,9 @@ void ensure_attrs() {
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 64 && ((done >> dev) & 1)) return;
-#define REANN_SMEM(K, BYTES) cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(BYTES))
-    REANN_SMEM((k_mlp_fwd<1, NFEAT>), fwd_smem<NFEAT>());
-    REANN_SMEM((k_mlp_fwd<NPHI, NFEAT>), fwd_smem<NFEAT>());
-    REANN_SMEM((k_mlp_fwd<1, NFEAT_P>), fwd_smem<NFEAT_P>());
-    REANN_SMEM((k_mlp_fwd<NPHI, NFEAT_P>), fwd_smem<NFEAT_P>());
-    REANN_SMEM((k_mlp_bwd<1, NFEAT, false>), (bwd_smem<NFEAT, false>()));
-    REANN_SMEM((k_mlp_bwd<NPHI, NFEAT, false>), (bwd_smem<NFEAT, false>()));
-    REANN_SMEM((k_mlp_bwd<1, NFEAT, true>), (bwd_smem<NFEAT, true>()));
-    REANN_SMEM((k_mlp_bwd<NPHI, NFEAT, true>), (bwd_smem<NFEAT, true>()));
-    REANN_SMEM((k_mlp_bwd<1, NFEAT_P, false>), (bwd_smem<NFEAT_P, false>()));
-    REANN_SMEM((k_mlp_bwd<NPHI, NFEAT_P, false>), (bwd_smem<NFEAT_P, false>()));
-#undef REANN_SMEM
+    set_attrs<1>();
+    set_attrs<2>();
+    set_attrs<4>();
     if (dev < 64) done |= (uint64_t)1 << dev;
 }
 
@@ -462,26 +604,42 @@ NetsOfLayer layer_nets(const NetTable& t, int layer) {
 
 }  // namespace
 
+// Parts while they still fit the 152 SMs in one wave.  us per launch of the coefficient
+// network's forward / energy network / backward with 1, 2 and 4 parts: 4 tiles (192 atoms)
+// 8.7 / 18.5 / 13.5, 6.3 / 13.6 / 9.8, 5.4 / 10.4 / 7.5; 63 tiles 8.4 / 17.7 / 12.6, 6.3 / 13.6 / 9.9,
+// 7.8 / 15.8 / 11.4; 96 tiles 8.5 / 17.5 / 12.2, 9.3 / 19.8 / 14.5, 10.2 / 21.7 / 15.2.
+int mlp_parts_f32(const reann_nlist* nl) {
+    const int64_t nt = tiles_of(nl);
+    return nt <= 38 ? 4 : (nt <= 76 ? 2 : 1);
+}
+
 cudaError_t launch_mlp_fwd_f32(cudaStream_t s, const reann_nlist* nl, const NetTable& nets, int t, bool energy,
                                const float* rho, float* out, int out_stride, bool pairs, GhostOut gh, float* dsave,
                                double* epart, int* flags) {
-    const int nt = (int)tiles_of(nl);
+    const int nt = (int)tiles_of(nl), parts = mlp_parts_f32(nl);
     if (nt == 0) return cudaSuccess;
+    if (energy && !pairs) return cudaErrorInvalidValue;  // launch_mlp_energy_f32
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
-#define REANN_FWD(O, F) \
-    k_mlp_fwd<O, F><<<nt, kT, fwd_smem<F>(), s>>>(ln, nl->tiles, rho, out, out_stride, gh, dsave, epart, flags)
-    if (pairs) {
-        if (energy)
-            REANN_FWD(1, NFEAT_P);
-        else
-            REANN_FWD(NPHI, NFEAT_P);
-    } else {
-        if (energy)
-            REANN_FWD(1, NFEAT);
-        else
-            REANN_FWD(NPHI, NFEAT);
-    }
+#define REANN_FWD(O, F, RPT)                                                                                         \
+    k_mlp_fwd<O, F, RPT><<<nt * (4 / RPT), kT, fwd_smem<F, RPT>(), s>>>(ln, nl->tiles, rho, out, out_stride, gh, dsave, \
+                                                                        epart, flags)
+#define REANN_FWD_R(O, F)        \
+    do {                         \
+        if (parts == 4)          \
+            REANN_FWD(O, F, 1);  \
+        else if (parts == 2)     \
+            REANN_FWD(O, F, 2);  \
+        else                     \
+            REANN_FWD(O, F, 4);  \
+    } while (0)
+    if (!pairs)
+        REANN_FWD_R(NPHI, NFEAT);
+    else if (energy)
+        REANN_FWD_R(1, NFEAT_P);
+    else
+        REANN_FWD_R(NPHI, NFEAT_P);
+#undef REANN_FWD_R
 #undef REANN_FWD
     return cudaGetLastError();
 }
@@ -489,31 +647,52 @@ cudaError_t launch_mlp_fwd_f32(cudaStream_t s, const reann_nlist* nl, const NetT
 cudaError_t launch_mlp_bwd_f32(cudaStream_t s, const reann_nlist* nl, const NetTable& nets, int t, bool energy,
                                const float* dsave, const float* ybar, float* rhobar, int* flags, bool pairs,
                                const float* Wt, const float* bck, const float* coef, float* rec, GhostOut gh) {
-    const int nt = (int)tiles_of(nl);
+    const int nt = (int)tiles_of(nl), parts = mlp_parts_f32(nl);
+    if (nt == 0) return cudaSuccess;
+    if (energy && !pairs) return cudaErrorInvalidValue;  // launch_mlp_energy_f32
+    ensure_attrs();
+    const NetsOfLayer ln = layer_nets(nets, t);
+#define REANN_BWD(O, F, B, RPT)                                                                                    \
+    k_mlp_bwd<O, F, B, RPT><<<nt * (4 / RPT), kT, bwd_smem<F, B, RPT>(), s>>>(                                     \
+        ln, nl->tiles, dsave, ybar, rhobar, B ? Wt : nullptr, B ? bck : nullptr, B ? coef : nullptr,              \
+        B ? rec : nullptr, B ? gh : GhostOut{}, flags)
+#define REANN_BWD_R(O, F, B)        \
+    do {                            \
+        if (parts == 4)             \
+            REANN_BWD(O, F, B, 1);  \
+        else if (parts == 2)        \
+            REANN_BWD(O, F, B, 2);  \
+        else                        \
+            REANN_BWD(O, F, B, 4);  \
+    } while (0)
+    if (!pairs)
+        REANN_BWD_R(NPHI, NFEAT, true);
+    else if (energy)
+        REANN_BWD_R(1, NFEAT_P, false);
+    else
+        REANN_BWD_R(NPHI, NFEAT_P, false);
+#undef REANN_BWD_R
+#undef REANN_BWD
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_energy_f32(cudaStream_t s, const reann_nlist* nl, const NetTable& nets, int t, const float* rho,
+                                  float* eps, double* epart, const float* Wt, const float* bck, const float* coef,
+                                  float* rec, GhostOut gh, int* flags) {
+    const int nt = (int)tiles_of(nl), parts = mlp_parts_f32(nl);
     if (nt == 0) return cudaSuccess;
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
-#define REANN_BWD(O, F, B)                                                                                      \
-    k_mlp_bwd<O, F, B><<<nt, kT, bwd_smem<F, B>(), s>>>(ln, nl->tiles, dsave, ybar, rhobar, B ? Wt : nullptr, \
-                                                        B ? bck : nullptr, B ? coef : nullptr, B ? rec : nullptr, \
-                                                        B ? gh : GhostOut{}, flags)
-    if (pairs) {
-        if (energy)
-            REANN_BWD(1, NFEAT_P, false);
-        else
-            REANN_BWD(NPHI, NFEAT_P, false);
-    } else if (rec) {
-        if (energy)
-            REANN_BWD(1, NFEAT, true);
-        else
-            REANN_BWD(NPHI, NFEAT, true);
-    } else {
-        if (energy)
-            REANN_BWD(1, NFEAT, false);
-        else
-            REANN_BWD(NPHI, NFEAT, false);
-    }
-#undef REANN_BWD
+#define REANN_EN(RPT)                                                                                              \
+    k_mlp_energy<RPT><<<nt * (4 / RPT), kT, energy_smem<RPT>(), s>>>(ln, nl->tiles, rho, eps, epart, Wt, bck, coef, \
+                                                                     rec, gh, flags)
+    if (parts == 4)
+        REANN_EN(1);
+    else if (parts == 2)
+        REANN_EN(2);
+    else
+        REANN_EN(4);
+#undef REANN_EN
     return cudaGetLastError();
 }
 

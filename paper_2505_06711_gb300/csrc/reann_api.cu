@@ -183,7 +183,7 @@ int alloc_eval_buffers(reann_ctx* ctx, reann_nlist* nl, const std::vector<std::a
     }
     nl->tiles = nl_alloc<Tile>(nl, nl->tiles_h.size());
     // energy partial sums: per 2048 atoms, or per network tile when the energy network sums them
-    nl->n_partial = (int)std::max<int64_t>((n + 2047) / 2048, (int64_t)nl->tiles_h.size());
+    nl->n_partial = (int)std::max<int64_t>((n + 2047) / 2048, 4 * (int64_t)nl->tiles_h.size());
     nl->partial = nl_alloc<double>(nl, nl->n_partial);
     nl->tiles128 = nl_alloc<Tile>(nl, nl->tiles128_h.size());
     if (!nl->tiles128) return set_error(ctx, REANN_E_NOMEM, "evaluation buffers: out of device memory");
@@ -972,6 +972,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
     const size_t lw = (size_t)(LMAX + 1) * NPHI * ctx->model.n_orb();
     const int64_t nf = nl->n_feat;
     // single-domain lists: owners write their ghost rows (no gather launches); otherwise gather
+    const bool fused_energy = ctx->precision == REANN_MLP_FP32 && !pairs;  // energy network: one launch both ways
     const GhostOut gh = nl->ghosts_by_owner ? GhostOut{nl->w.goff, n, nl->g_cap} : GhostOut{};
     // forward: Eq. 1 then Eq. 2, re-using the same list in every layer (Sec. 2.2)
     for (int t = 0; t < T; ++t) {
@@ -999,6 +1000,9 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
             REANN_CUDA_TRY(ctx, launch_mlp_fwd_tc(s, nl, ctx->tc, t, energy_net, ctx->precision, rho_t, out,
                                                   out_stride, ctx->d_flags, gh,
                                                   nl->dsave + (size_t)t * n * (H1 + H2), epart));
+        else if (fused_energy && energy_net)  // and its backward
+            REANN_CUDA_TRY(ctx, launch_mlp_energy_f32(s, nl, ctx->nets, t, rho_t, out, epart, ctx->d_W + t * lw, bck_t,
+                                                      coef_t, nl->bbar, gh, ctx->d_flags));
         else
             REANN_CUDA_TRY(ctx, launch_mlp_fwd_f32(s, nl, ctx->nets, t, energy_net, rho_t, out, out_stride, pairs, gh,
                                                   nl->dsave + (size_t)t * n * (H1 + H2), epart, ctx->d_flags));
@@ -1007,10 +1011,11 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
         ProfScope p(ctx, PR_ENERGY);
         if (seg)
             REANN_CUDA_TRY(ctx, launch_segment_energy(s, seg, nseg, nl->eps, energy));
-        else  // the energy network summed its tiles (64-row FP32 tiles or 128-row tensor-core tiles)
+        else  // the energy network summed its blocks (parts of 64-row FP32 tiles, or 128-row tensor-core tiles)
             REANN_CUDA_TRY(ctx, launch_energy_final(s, nl->partial,
-                                                    (int)(ctx->precision == REANN_MLP_FP32 ? tiles_of(nl)
-                                                                                           : tiles128_of(nl)),
+                                                    (int)(ctx->precision == REANN_MLP_FP32
+                                                              ? tiles_of(nl) * mlp_parts_f32(nl)
+                                                              : tiles128_of(nl)),
                                                     energy));
     }
     // reverse: Eqs. 3-5, one vector-Jacobian product per layer
@@ -1020,7 +1025,9 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
         const float* dsave_t = nl->dsave + (size_t)t * n * (H1 + H2);
         {
             ProfScope p(ctx, PR_MLP_BWD);
-            if (ctx->precision != REANN_MLP_FP32)  // the tensor-core backward networks also take the bbar step
+            if (fused_energy && t == T - 1)
+                ;  // done by the energy network's forward launch (its time is in that region)
+            else if (ctx->precision != REANN_MLP_FP32)  // the tensor-core backward networks also take the bbar step
                 REANN_CUDA_TRY(ctx, launch_mlp_bwd_tc(s, nl, ctx->tc, t, t == T - 1, ctx->precision, dsave_t,
                                                       nl->cbar, ctx->d_W + t * lw, bck_t, coef_t, nl->bbar, gh,
                                                       ctx->d_flags));
