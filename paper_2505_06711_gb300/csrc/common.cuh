@@ -288,12 +288,14 @@ struct GraphSlot {
 // unmapping memory for each of its ~45 buffers (cudaMalloc + cudaFree of a
 // 4,000-atom list: 0.8 ms of a 1.37 ms build + evaluation).  It keeps at most
 // kKeep unused bytes and gives everything back with the last of its context and
-// lists (each holds a reference).  Blocks are taken on the building context's
+// lists (each holds a reference).  Blocks from kBig bytes on come from cudaMalloc as
+// before (the pool maps them more slowly: preparing a 1,048,576-atom list took 226
+// instead of 174 ms).  Blocks are taken on the building context's
 // stream.  They go back on the pool's own stream after a device synchronisation (as
 // cudaFree implies one), so that no stream of the caller needs to outlive a list
 // and a block is never handed on while work of any stream may still use it.
 struct ListPool {
-    static constexpr uint64_t kKeep = 512ull << 20;
+    static constexpr uint64_t kKeep = 512ull << 20, kBig = 64ull << 20;
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
     static std::shared_ptr<ListPool> create();  // null when the device has no memory pools
@@ -382,7 +384,7 @@ struct reann_nlist {
     bool ghosts_by_owner = false;  // ghost slots of owned row i are [goff[i], goff[i+1]) (single-domain build)
     int rank_grid[3] = {1, 1, 1};
     std::vector<int64_t> rank_local, rank_ghost, rank_remote;
-    std::vector<void*> allocs;
+    std::vector<void*> allocs, big_allocs;  // blocks of mem_pool (null: cudaMalloc); cudaMalloc blocks beside a list_pool
     // stream-ordered allocation: blocks come from mem_pool on alloc_stream.  Serving
     // builds return them with cudaFreeAsync on the same stream, so neither side waits
     // for unrelated device work; other lists as described at ListPool (list_pool set).
@@ -478,6 +480,7 @@ cudaError_t launch_moved(cudaStream_t s, const reann_nlist* nl, const double* po
 cudaError_t launch_pack(cudaStream_t s, const reann_nlist* src, const double* caller_pos, reann_nlist* pool,
                         int64_t ob, int64_t gb);
 void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes);
+void nlist_free_block(reann_nlist* nl, void* p);  // a block that nothing on the device uses yet
 template <typename T>
 inline T* nlist_alloc(reann_nlist* nl, size_t count) {
     return static_cast<T*>(nlist_alloc_bytes(nl, count * sizeof(T)));

@@ -711,8 +711,9 @@ static cudaError_t counting_sort(cudaStream_t s, const int* gate, int64_t n, int
 void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes) {
     void* p = nullptr;
     bytes = std::max<size_t>(bytes, 1);
+    const bool big = nl->list_pool && bytes >= ListPool::kBig;
     auto take = [&] {
-        return nl->mem_pool ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream) : cudaMalloc(&p, bytes);
+        return nl->mem_pool && !big ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream) : cudaMalloc(&p, bytes);
     };
     cudaError_t e = take();
     if (e != cudaSuccess && nl->list_pool) {  // give the pool's unused blocks back and try again
@@ -721,14 +722,27 @@ void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes) {
         e = take();
     }
     // after the build the block may be used on any stream
-    if (e == cudaSuccess && nl->list_pool && nl->alloc_stream == nl->list_pool->stream)
+    if (e == cudaSuccess && !big && nl->list_pool && nl->alloc_stream == nl->list_pool->stream)
         e = cudaStreamSynchronize(nl->alloc_stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    nl->allocs.push_back(p);
+    (big ? nl->big_allocs : nl->allocs).push_back(p);
     return p;
+}
+
+void nlist_free_block(reann_nlist* nl, void* p) {
+    for (auto* list : {&nl->allocs, &nl->big_allocs}) {
+        const auto it = std::find(list->begin(), list->end(), p);
+        if (it == list->end()) continue;
+        list->erase(it);
+        if (nl->mem_pool && list == &nl->allocs)
+            cudaFreeAsync(p, nl->alloc_stream);
+        else
+            cudaFree(p);
+        return;
+    }
 }
 
 template <typename T>

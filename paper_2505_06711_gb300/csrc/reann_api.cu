@@ -135,20 +135,14 @@ T* nl_alloc(reann_nlist* nl, size_t count) {
 // the records of one run of rows at a time in every pass instead of keeping all of them.
 bool alloc_edge_records(reann_nlist* nl, int64_t rows) {
     for (;;) {
-        const size_t count = (size_t)rows * nl->stride, first = nl->allocs.size();
+        const size_t count = (size_t)rows * nl->stride;
         nl->edge_xyzj = nl_alloc<float4>(nl, count);
         nl->edge_phi = nl->edge_xyzj ? nl_alloc<float2>(nl, count) : nullptr;
         nl->edge_der = nl->edge_phi ? nl_alloc<float2>(nl, count) : nullptr;
         nl->edge_rows = rows;
         if (nl->edge_der) return true;
-        while (nl->allocs.size() > first) {
-            void* p = nl->allocs.back();
-            nl->allocs.pop_back();
-            if (nl->mem_pool)
-                cudaFreeAsync(p, nl->alloc_stream);
-            else
-                cudaFree(p);
-        }
+        if (nl->edge_phi) nlist_free_block(nl, nl->edge_phi);
+        if (nl->edge_xyzj) nlist_free_block(nl, nl->edge_xyzj);
         if (rows <= 1024) return false;
         rows = std::max<int64_t>(1024, (rows + 1) / 2);
     }
@@ -223,6 +217,7 @@ void free_nlist(reann_nlist* nl) {
         else
             cudaFree(p);
     }
+    for (void* p : nl->big_allocs) cudaFree(p);
     delete nl;
 }
 
