@@ -443,7 +443,7 @@ int reann_ctx_profile_read(reann_ctx* ctx, double* total_ms, int64_t* launches);
  *   mass   dev, N FP64 (amu)
  *   e_pot  dev, n_steps FP64: E after each step (eV), or NULL
  *   e_kin  dev, n_steps FP64: kinetic energy after each step (eV), or NULL
- * The first call (and any call whose pointers, dt, n_steps or network
+ * The first call (and any call whose pos, vel or mass pointer, dt or network
  * precision differ from the previous one) evaluates the starting forces and
  * captures one step as a CUDA graph on a library-owned stream, ordered after
  * the context stream; every step is then one graph launch, the rebuild being

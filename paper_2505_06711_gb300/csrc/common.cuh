@@ -283,6 +283,11 @@ struct GraphSlot {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
+// Output arrays of an MD call (null: not recorded), one entry per step
+struct MdOut {
+    double *e_pot, *e_kin, *e_bath;
+    int n_steps;
+};
 // Device memory of a context's lists: a stream-ordered pool, so that building and
 // freeing one structure after another re-uses blocks instead of mapping and
 // unmapping memory for each of its ~45 buffers (cudaMalloc + cudaFree of a
@@ -368,16 +373,18 @@ struct reann_nlist {
     float* md_forces = nullptr;    // N x 3 (caller order)
     double* md_scalars = nullptr;  // [0] E_pot, [1] E_kin, [2] xi, [3] eta, [4] velocity scale
     double* md_partial = nullptr;
-    int* md_ints = nullptr;        // [0] rebuild gate, [1] step counter, [2] rebuild count
+    int* md_ints = nullptr;        // [0] rebuild gate, [1] step counter, [2] rebuild count, [3] ticket
+    reann::MdOut* md_out = nullptr;  // the current call's output arrays
     bool md_forces_valid = false;
     const double* md_forces_at = nullptr;  // positions the forces belong to
     cudaGraph_t md_graph = nullptr;
     cudaGraphExec_t md_exec = nullptr;
     reann::GraphSlot graphs[reann::GS_COUNT];  // rebuild / evaluation calls replayed as graphs
-    const void* md_key[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    const void* md_key[3] = {nullptr, nullptr, nullptr};  // pos, vel, mass of the captured step
     double md_dt = 0.0;
     double md_kt = 0.0, md_tau = 0.0;  // thermostat of the captured step (tau 0: NVE)
-    int md_precision = -1, md_nsteps = -1;
+    int md_precision = -1;         // network precision of md_forces
+    int md_step_precision = -1;    // and of the captured step
     // spatial decomposition into virtual ranks (reann_build_nlist_decomposed):
     // per rank its local atoms, ghost slots, and ghost slots owned by another rank
     bool decomposed = false;
@@ -490,15 +497,18 @@ cudaError_t launch_retire(cudaStream_t s, const int4* seg, int nseg, reann_nlist
 cudaError_t launch_segment_energy(cudaStream_t s, const int4* seg, int nseg, const float* eps, double* energies);
 
 // velocity Verlet (md.cu)
-cudaError_t launch_kick(cudaStream_t s, int64_t n, double* vel, const float* forces, const double* mass,
-                        double half_dt, const double* scale = nullptr);
+int64_t md_partials(int64_t n);  // kinetic-energy partial sums of launch_second_half
+cudaError_t launch_md_begin(cudaStream_t s, MdOut* dst, const MdOut& out, int* ints);
+cudaError_t launch_first_half(cudaStream_t s, int64_t n, double* pos, double* vel, const float* forces,
+                              const double* mass, double dt, const double* scale, const double* ref, double skin,
+                              int* gate);
+cudaError_t launch_second_half(cudaStream_t s, int64_t n, double* vel, const float* forces, const double* mass,
+                               double dt, double* partial, double* scalars, const MdOut* out, int* ints, double tau,
+                               double gkt, double q);
 cudaError_t launch_scale(cudaStream_t s, int64_t n, double* vel, const double* scale);
 cudaError_t launch_nh_half(cudaStream_t s, double* scalars, double dt, double gkt, double q);
-cudaError_t launch_drift(cudaStream_t s, int64_t n, double* pos, const double* vel, double dt);
 cudaError_t launch_ekin(cudaStream_t s, int64_t n, const double* vel, const double* mass, double* partial,
                         double* out);
-cudaError_t launch_record(cudaStream_t s, int* counter, const double* scalars, double* epot_out, double* ekin_out,
-                          double* bath_out, double gkt, double q, int n_steps, const int* gate, int* rebuilds);
 const int32_t* ghost_count_ptr(const reann_nlist* nl);
 // with c0: also the first layer's coefficients of every slot (k_init_coef's work)
 cudaError_t launch_refresh_positions(cudaStream_t s, const reann_nlist* nl, const double* pos,

@@ -12,6 +12,12 @@
 //   xi += (dt/4) G(K);  eta += (dt/2) xi;  s = exp(-(dt/2) xi);  K *= s^2;
 //   xi += (dt/4) G(K),  with G(K) = (2K - g kT)/Q, Q = g kT tau^2, g = 3N - 3.
 // The conserved quantity is E + K + Q xi^2 / 2 + g kT eta.
+// The integration around the rebuild and the forces is two kernels (a small system's
+// step is a chain of launches of about 2 us each): k_first_half also makes the
+// skin/2 test, k_second_half also sums K, takes the thermostat's half step and
+// records (NVT scales the velocities afterwards).  The recording kernel finds the
+// call's output arrays in device memory (MdOut, written once per call), so the
+// captured step serves calls with other output arrays and step counts.
 // Units: A, fs, amu, eV; 1 eV/(A amu) = 9.648533212e-3 A/fs^2.
 #include <cuda_runtime.h>
 
@@ -23,14 +29,37 @@ namespace {
 constexpr double kAccel = 9.648533212e-3;  // (eV/A)/amu -> A/fs^2
 constexpr int kThreads = 256, kPer = 8;
 
-// v = s v + (dt/2) F/m, s read from the device (1 without a thermostat)
-__global__ void k_kick(int64_t n, double* __restrict__ vel, const float* __restrict__ forces,
-                       const double* __restrict__ mass, double half_dt, const double* __restrict__ scale) {
+// once per call: the output arrays, and the step counter and rebuild gate at zero
+__global__ void k_md_begin(MdOut* __restrict__ dst, MdOut out, int* __restrict__ ints) {
     pdl_enter();
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 3 * n) return;
-    const double v = scale ? vel[t] * *scale : vel[t];
-    vel[t] = v + half_dt * kAccel * (double)forces[t] / mass[t / 3];
+    *dst = out;
+    ints[0] = ints[1] = 0;
+}
+
+// v = s v + (dt/2) F/m (s read from the device; 1 without a thermostat), x += dt v, and
+// the gate of the rebuild: set when the atom is more than skin/2 from where it was at
+// the last build
+__global__ void __launch_bounds__(64) k_first_half(int64_t n, double* __restrict__ pos, double* __restrict__ vel,
+                                                   const float* __restrict__ forces, const double* __restrict__ mass,
+                                                   double half_dt, double dt, const double* __restrict__ scale,
+                                                   const double* __restrict__ ref, double thr2, int* __restrict__ gate) {
+    pdl_enter();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double m = mass[i];
+    double d2 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int64_t t = 3 * i + k;
+        const double v0 = scale ? vel[t] * *scale : vel[t];
+        const double v = v0 + half_dt * kAccel * (double)forces[t] / m;
+        const double x = pos[t] + dt * v;
+        vel[t] = v;
+        pos[t] = x;
+        const double d = x - ref[t];
+        d2 += d * d;
+    }
+    if (!(d2 <= thr2)) atomicOr(gate, 1);
 }
 
 __global__ void k_scale(int64_t n, double* __restrict__ vel, const double* __restrict__ scale) {
@@ -40,8 +69,7 @@ __global__ void k_scale(int64_t n, double* __restrict__ vel, const double* __res
 }
 
 // thermostat half step on the device scalars: sc[1] K, sc[2] xi, sc[3] eta, sc[4] s
-__global__ void k_nh_half(double* __restrict__ sc, double dt, double gkt, double q) {
-    pdl_enter();
+__device__ __forceinline__ void nh_half(double* sc, double dt, double gkt, double q) {
     double K = sc[1], xi = sc[2], eta = sc[3];
     xi += 0.25 * dt * (2.0 * K - gkt) / q;
     eta += 0.5 * dt * xi;
@@ -54,10 +82,9 @@ __global__ void k_nh_half(double* __restrict__ sc, double dt, double gkt, double
     sc[4] = s;
 }
 
-__global__ void k_drift(int64_t n, double* __restrict__ pos, const double* __restrict__ vel, double dt) {
+__global__ void k_nh_half(double* __restrict__ sc, double dt, double gkt, double q) {
     pdl_enter();
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < 3 * n) pos[t] += dt * vel[t];
+    nh_half(sc, dt, gkt, q);
 }
 
 // kinetic energy in eV, two-level FP64 tree (fixed order, deterministic)
@@ -100,29 +127,97 @@ __global__ void __launch_bounds__(kThreads) k_ekin_final(int np, const double* _
     if (threadIdx.x == 0) out[0] = sm[0];
 }
 
-// append this step's energies at the device step counter, count rebuilds; the
-// bath energy Q xi^2 / 2 + g kT eta from the thermostat scalars
-__global__ void k_record(int* __restrict__ counter, const double* __restrict__ sc, double* __restrict__ epot_out,
-                         double* __restrict__ ekin_out, double* __restrict__ bath_out, double gkt, double q,
-                         int n_steps, const int* __restrict__ gate, int* __restrict__ rebuilds) {
+// v += (dt/2) F/m and the step's end: the kinetic energy (FP64, per block of
+// kHalfThreads atoms in a fixed tree, then the blocks' sums by the block that finishes
+// last, in a fixed order), with tau > 0 the thermostat's half step, the step's energies
+// and the bath energy Q xi^2 / 2 + g kT eta into the call's arrays at the step counter,
+// and the count of rebuilds.  ints: rebuild gate (left at zero), step counter, rebuild
+// count, ticket (atomicInc wraps it to zero).
+constexpr int kHalfThreads = 128;
+__global__ void __launch_bounds__(kHalfThreads) k_second_half(int64_t n, double* __restrict__ vel,
+                                                              const float* __restrict__ forces,
+                                                              const double* __restrict__ mass, double half_dt,
+                                                              double* __restrict__ partial, double* __restrict__ sc,
+                                                              const MdOut* __restrict__ outp, int* __restrict__ ints,
+                                                              double dt, double tau, double gkt, double q) {
     pdl_enter();
-    const int k = *counter;
-    if (k < n_steps) {
-        if (epot_out) epot_out[k] = sc[0];
-        if (ekin_out) ekin_out[k] = sc[1];
-        if (bath_out) bath_out[k] = 0.5 * q * sc[2] * sc[2] + gkt * sc[3];
+    __shared__ double sm[kHalfThreads];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * kHalfThreads + tid;
+    double s = 0.0;
+    if (i < n) {
+        const double m = mass[i];
+        double v2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int64_t t = 3 * i + k;
+            const double v = vel[t] + half_dt * kAccel * (double)forces[t] / m;
+            vel[t] = v;
+            v2 += v * v;
+        }
+        s = 0.5 * m * v2 / kAccel;
     }
-    *counter = k + 1;
-    if (*gate) *rebuilds += 1;
+    auto tree = [&] {
+        sm[tid] = s;
+        __syncthreads();
+        for (int o = kHalfThreads / 2; o > 0; o >>= 1) {
+            if (tid < o) sm[tid] += sm[tid + o];
+            __syncthreads();
+        }
+    };
+    tree();
+    if (tid == 0) {
+        partial[blockIdx.x] = sm[0];
+        __threadfence();
+        last = atomicInc(reinterpret_cast<unsigned*>(ints + 3), gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    s = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += kHalfThreads) s += __ldcg(partial + b);
+    tree();
+    if (tid != 0) return;
+    sc[1] = sm[0];
+    if (tau > 0.0) nh_half(sc, dt, gkt, q);
+    const MdOut out = *outp;
+    const int k = ints[1];
+    if (k < out.n_steps) {
+        if (out.e_pot) out.e_pot[k] = sc[0];
+        if (out.e_kin) out.e_kin[k] = sc[1];
+        if (out.e_bath) out.e_bath[k] = 0.5 * q * sc[2] * sc[2] + gkt * sc[3];
+    }
+    ints[1] = k + 1;
+    if (ints[0]) ints[2] += 1;
+    ints[0] = 0;
 }
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
-cudaError_t launch_kick(cudaStream_t s, int64_t n, double* vel, const float* forces, const double* mass,
-                        double half_dt, const double* scale) {
-    launch_pdl(k_kick, blocks_for(3 * n, 256), 256, 0, s, n, vel, forces, mass, half_dt, scale);
+int64_t md_partials(int64_t n) { return blocks_for(n, kHalfThreads); }
+
+cudaError_t launch_md_begin(cudaStream_t s, MdOut* dst, const MdOut& out, int* ints) {
+    launch_pdl(k_md_begin, 1, 1, 0, s, dst, out, ints);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_first_half(cudaStream_t s, int64_t n, double* pos, double* vel, const float* forces,
+                              const double* mass, double dt, const double* scale, const double* ref, double skin,
+                              int* gate) {
+    const double half = 0.5 * skin;
+    launch_pdl(k_first_half, blocks_for(n, 64), 64, 0, s, n, pos, vel, forces, mass, 0.5 * dt, dt, scale, ref,
+               half * half, gate);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_second_half(cudaStream_t s, int64_t n, double* vel, const float* forces, const double* mass,
+                               double dt, double* partial, double* scalars, const MdOut* out, int* ints, double tau,
+                               double gkt, double q) {
+    launch_pdl(k_second_half, blocks_for(n, kHalfThreads), kHalfThreads, 0, s, n, vel, forces, mass, 0.5 * dt, partial,
+               scalars, out, ints, dt, tau, gkt, q);
     return cudaGetLastError();
 }
 
@@ -136,22 +231,11 @@ cudaError_t launch_nh_half(cudaStream_t s, double* scalars, double dt, double gk
     return cudaGetLastError();
 }
 
-cudaError_t launch_drift(cudaStream_t s, int64_t n, double* pos, const double* vel, double dt) {
-    launch_pdl(k_drift, blocks_for(3 * n, 256), 256, 0, s, n, pos, vel, dt);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_ekin(cudaStream_t s, int64_t n, const double* vel, const double* mass, double* partial,
                         double* out) {
     const int np = (int)blocks_for(n, kThreads * kPer);
     launch_pdl(k_ekin_partial, np, kThreads, 0, s, n, vel, mass, partial);
     launch_pdl(k_ekin_final, 1, kThreads, 0, s, np, partial, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_record(cudaStream_t s, int* counter, const double* scalars, double* epot_out, double* ekin_out,
-                          double* bath_out, double gkt, double q, int n_steps, const int* gate, int* rebuilds) {
-    launch_pdl(k_record, 1, 1, 0, s, counter, scalars, epot_out, ekin_out, bath_out, gkt, q, n_steps, gate, rebuilds);
     return cudaGetLastError();
 }
 

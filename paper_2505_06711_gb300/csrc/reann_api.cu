@@ -1220,7 +1220,6 @@ extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const d
 
 namespace {
 
-// enqueue one velocity-Verlet step on ctx->stream (captured into the step graph)
 // Nose-Hoover parameters: kT (eV), Q = g kT tau^2, g = 3N - 3; tau = 0: NVE
 struct Thermo {
     double kt = 0.0, tau = 0.0, gkt = 0.0, q = 0.0;
@@ -1238,28 +1237,22 @@ Thermo make_thermo(int64_t n, double temperature_k, double tau_fs) {
     return th;
 }
 
+// enqueue one velocity-Verlet step on ctx->stream (captured into the step graph)
 int md_step_body(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const double* mass, double dt,
-                 int n_steps, double* e_pot, double* e_kin, const Thermo& th, double* e_bath) {
+                 const Thermo& th) {
     cudaStream_t s = ctx->stream;
     const int64_t n = nl->n;
     int* gate = nl->md_ints;
     double* sc = nl->md_scalars;
     if (th.on()) REANN_CUDA_TRY(ctx, launch_nh_half(s, sc, dt, th.gkt, th.q));
-    REANN_CUDA_TRY(ctx, launch_kick(s, n, vel, nl->md_forces, mass, 0.5 * dt, th.on() ? sc + 4 : nullptr));
-    REANN_CUDA_TRY(ctx, launch_drift(s, n, pos, vel, dt));
-    REANN_CUDA_TRY(ctx, cudaMemsetAsync(gate, 0, sizeof(int), s));
-    REANN_CUDA_TRY(ctx, launch_moved(s, nl, pos, gate));
+    REANN_CUDA_TRY(ctx, launch_first_half(s, n, pos, vel, nl->md_forces, mass, dt, th.on() ? sc + 4 : nullptr,
+                                          nl->pos_ref, nl->skin, gate));
     REANN_CUDA_TRY(ctx, launch_rebuild(s, nl, pos, ctx->d_flags, gate));  // kernels return at once unless gate != 0
     int rc = run_energy_forces(ctx, nl, pos, nl->T, nl->md_scalars, nl->md_forces, nullptr);
     if (rc) return rc;
-    REANN_CUDA_TRY(ctx, launch_kick(s, n, vel, nl->md_forces, mass, 0.5 * dt));
-    REANN_CUDA_TRY(ctx, launch_ekin(s, n, vel, mass, nl->md_partial, sc + 1));
-    if (th.on()) {
-        REANN_CUDA_TRY(ctx, launch_nh_half(s, sc, dt, th.gkt, th.q));
-        REANN_CUDA_TRY(ctx, launch_scale(s, n, vel, sc + 4));
-    }
-    REANN_CUDA_TRY(ctx, launch_record(s, nl->md_ints + 1, sc, e_pot, e_kin, e_bath, th.gkt, th.q, n_steps, gate,
-                                      nl->md_ints + 2));
+    REANN_CUDA_TRY(ctx, launch_second_half(s, n, vel, nl->md_forces, mass, dt, nl->md_partial, sc, nl->md_out,
+                                           nl->md_ints, th.tau, th.gkt, th.q));
+    if (th.on()) REANN_CUDA_TRY(ctx, launch_scale(s, n, vel, sc + 4));
     return REANN_OK;
 }
 
@@ -1270,11 +1263,14 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
     if (!nl->md_forces) {
         nl->md_forces = nl_alloc<float>(nl, 3 * n);
         nl->md_scalars = nl_alloc<double>(nl, 8);
-        nl->md_partial = nl_alloc<double>(nl, (n + 2047) / 2048);
-        nl->md_ints = nl_alloc<int>(nl, 3);
-        if (!nl->md_forces || !nl->md_scalars || !nl->md_partial || !nl->md_ints)
+        nl->md_partial = nl_alloc<double>(nl, std::max<int64_t>((n + 2047) / 2048, md_partials(n)));
+        nl->md_ints = nl_alloc<int>(nl, 4);
+        nl->md_out = nl_alloc<MdOut>(nl, 1);
+        if (!nl->md_forces || !nl->md_scalars || !nl->md_partial || !nl->md_ints || !nl->md_out) {
+            nl->md_forces = nullptr;  // (what was allocated goes with the list)
             return set_error(ctx, REANN_E_NOMEM, "MD buffers: out of device memory");
-        REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_ints, 0, 3 * sizeof(int), s));
+        }
+        REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_ints, 0, 4 * sizeof(int), s));
         REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_scalars, 0, 8 * sizeof(double), s));  // xi = eta = 0
     }
     int* gate = nl->md_ints;
@@ -1287,20 +1283,20 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
         if (rc) return rc;
         nl->md_forces_valid = true;
         nl->md_forces_at = pos;
+        nl->md_precision = ctx->precision;
     }
     // the thermostat's first half step needs K of the current velocities
     if (th.on()) REANN_CUDA_TRY(ctx, launch_ekin(s, n, vel, mass, nl->md_partial, nl->md_scalars + 1));
-    const void* key[6] = {pos, vel, mass, e_pot, e_kin, e_bath};
+    const void* key[3] = {pos, vel, mass};
     const bool same = nl->md_exec && std::memcmp(key, nl->md_key, sizeof(key)) == 0 && nl->md_dt == dt &&
-                      nl->md_precision == ctx->precision && nl->md_nsteps == n_steps && nl->md_kt == th.kt &&
-                      nl->md_tau == th.tau;
+                      nl->md_step_precision == ctx->precision && nl->md_kt == th.kt && nl->md_tau == th.tau;
     if (!same) {
         if (nl->md_exec) cudaGraphExecDestroy(nl->md_exec);
         if (nl->md_graph) cudaGraphDestroy(nl->md_graph);
         nl->md_exec = nullptr;
         nl->md_graph = nullptr;
         REANN_CUDA_TRY(ctx, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-        const int rc = md_step_body(ctx, nl, pos, vel, mass, dt, n_steps, e_pot, e_kin, th, e_bath);
+        const int rc = md_step_body(ctx, nl, pos, vel, mass, dt, th);
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(s, &g);
         if (rc || ec != cudaSuccess) {
@@ -1311,12 +1307,11 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
         REANN_CUDA_TRY(ctx, cudaGraphInstantiate(&nl->md_exec, g, 0));
         std::memcpy(nl->md_key, key, sizeof(key));
         nl->md_dt = dt;
-        nl->md_precision = ctx->precision;
-        nl->md_nsteps = n_steps;
+        nl->md_step_precision = ctx->precision;
         nl->md_kt = th.kt;
         nl->md_tau = th.tau;
     }
-    REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_ints + 1, 0, sizeof(int), s));
+    REANN_CUDA_TRY(ctx, launch_md_begin(s, nl->md_out, MdOut{e_pot, e_kin, e_bath, n_steps}, nl->md_ints));
     for (int k = 0; k < n_steps; ++k) REANN_CUDA_TRY(ctx, cudaGraphLaunch(nl->md_exec, s));
     return REANN_OK;
 }

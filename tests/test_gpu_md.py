@@ -178,3 +178,36 @@ def test_nvt_holds_temperature_and_conserves_extended_energy():
     assert abs(late.mean() - T0) < 0.03 * T0
     assert e_bath.cpu().numpy()[-1] / n > 0.5  # the bath took up the released potential energy
     sy.close()
+
+
+def test_calls_with_other_output_arrays_continue_one_trajectory():
+    """Blocks of steps recorded into new arrays (or not at all) give the trajectory of one call."""
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    s = water_box(43, seed=9)  # 129 atoms: one more than a block of the integrator's kernels
+    pot = Potential(make_model(T=2))
+    got = []
+    for blocks in ((12,), (1, 4, 7)):
+        for temperature in (None, 250.0):
+            sy = pot.system(s.pos, s.species, s.cell)
+            mass = torch.as_tensor(MASS_AMU[s.species], device="cuda")
+            vel = torch.as_tensor(maxwell_boltzmann(MASS_AMU[s.species], 300.0, seed=2), device="cuda").contiguous()
+            e, keep = [], []
+            for k, n in enumerate(blocks):
+                record = k != 1
+                r = sy.md(vel, mass, 0.5, n, record=record, temperature_k=temperature)
+                keep.append(r)  # every block has its own arrays
+                e.append(torch.stack(r) if record else torch.full((2 if temperature is None else 3, n), float("nan"),
+                                                                  dtype=torch.float64, device="cuda"))
+            sy.check()
+            torch.cuda.synchronize()
+            assert sy.md_info()[0] == blocks[-1]
+            got.append((sy.pos.cpu().numpy().copy(), vel.cpu().numpy().copy(), torch.cat(e, 1).cpu().numpy()))
+            sy.close()
+    pot.close()
+    for one, many in ((got[0], got[2]), (got[1], got[3])):
+        assert np.allclose(one[0], many[0], rtol=0, atol=1e-9) and np.allclose(one[1], many[1], rtol=0, atol=1e-9)
+        rec = ~np.isnan(many[2])
+        assert rec.any() and np.allclose(one[2][rec], many[2][rec], rtol=1e-9, atol=1e-9)
