@@ -445,30 +445,57 @@ inline int64_t tiles128_of(const reann_nlist* nl) {
 
 int set_error(reann_ctx* ctx, int code, const std::string& msg);
 
-// Launches k with the programmatic-stream-serialization attribute; every
-// kernel of the library calls pdl_enter() first.  In a captured graph the
-// attribute becomes a programmatic edge.  The network kernels and the two edge
-// passes are launched without it.  Blocks of the networks' one-wave grids that
-// become resident while the previous kernel drains pile up on the SMs that freed
-// first (measured: FP32 step 0.489 -> 0.502 ms with them).  Blocks of an edge pass
-// that become resident beside a network kernel keep that kernel's split of the
-// SM's 256 KB into shared memory and L1, up to 207 KB of shared memory, and leave
-// the gathers of the whole pass little L1 (1,048,576 atoms: reverse pass 1.17 -> 1.62 ms
-// with the attribute; 24,576: evaluation 0.342 -> 0.349 ms; 192: no difference).
+// Kernel launches with two optional attributes.  Programmatic stream serialization
+// (`pdl`): the kernel's blocks may become resident while the previous kernel drains
+// (every kernel of the library calls pdl_enter() before it touches memory that
+// another kernel writes; in a captured graph the attribute becomes a programmatic
+// edge).  `carve` >= 0: preferred share (percent) of the SM's 256 KB for shared memory.
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_with(bool pdl, int carve, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               A... args) {
+    cudaLaunchAttribute at[2];
+    unsigned na = 0;
+    if (pdl) {
+        at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carve >= 0) {
+        at[na].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[na++].val.sharedMemCarveout = (unsigned)carve;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = na;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    return launch_with(true, -1, k, grid, block, smem, s, args...);
+}
+
+// How an evaluation's kernels are launched.  A small system's evaluation is a chain of
+// kernels of 4 to 10 us that leave most of the GPU idle: all of them are launched
+// programmatically, so that a kernel's blocks are in place (and the networks' weights
+// staged) when the previous one ends, and all with the same preferred carveout, since
+// kernels that want different ones wait for the SM to drain between them (evaluation of
+// 192 atoms 82 -> 74 us, of 4,000 102 -> 93 us; with the driver's own carveouts the
+// programmatic network launches took 55 us longer from 3,000 atoms on).  Above that the
+// networks and the two edge passes are launched plainly: blocks of the networks'
+// one-wave grids that become resident while the previous kernel drains pile up on the
+// SMs that freed first (24,576 atoms: 333 -> 340 us), and an edge pass whose blocks
+// become resident beside a network kernel keeps that kernel's carveout, up to 207 KB of
+// shared memory, which leaves its gathers little L1 (1,048,576 atoms: reverse pass 1.17
+// -> 1.62 ms).
+constexpr int64_t kChainRows = 6144;
+struct EvalLaunch {
+    bool chain;  // programmatic, one carveout
+    int carve(int plain = -1) const { return chain ? 25 : plain; }
+};
+inline EvalLaunch eval_launch(const reann_nlist* nl) { return EvalLaunch{rows_of(nl) <= kChainRows}; }
 
 #define REANN_CUDA_TRY(ctx, expr)                                                                   \
     do {                                                                                            \
@@ -553,7 +580,7 @@ cudaError_t launch_mlp_energy_f32(cudaStream_t s, const reann_nlist* nl, const N
                                   float* eps, double* epart, const float* Wt, const float* bck, const float* coef,
                                   float* rec, GhostOut gh, int* flags);
 // total energy from np partial sums, in a fixed order
-cudaError_t launch_energy_final(cudaStream_t s, const double* partial, int np, double* energy);
+cudaError_t launch_energy_final(cudaStream_t s, const double* partial, int np, double* energy, int carve = -1);
 // atomic networks on tcgen05 tensor cores (mlp_tc.cu), precision REANN_MLP_BF16,
 // REANN_MLP_BF16X3 or REANN_MLP_FP8.  The forward keeps SiLU'(z1), SiLU'(z2) of every
 // row in dsave (128 floats per row) and, for the energy network, writes one FP64

@@ -479,6 +479,10 @@ __global__ void __launch_bounds__(4 * kBbarAtoms) k_bbar(int64_t n, const float*
 // Summed over the edges, the term c_j phi grad Q_k needs only the moments sum_j
 // c_j phi A_a = b_{k,a} that the forward pass kept (grad Q_k is linear in r), so
 // it is added once per atom from the checkpoint b instead of once per edge.
+// Preferred shared memory of the reverse pass: 75 % holds the blocks its registers allow;
+// the driver's choice was 2 % slower (1,048,576 atoms 1,160 -> 1,138 us, 24,576 40.8 -> 39.8),
+// 25 % and 100 % 14 to 38 %.
+constexpr int kAdjCarveout = 75;
 // Small blocks: the block scheduler balances the SMs at fine grain.
 constexpr int kAdjWarps = 4;
 // With forces set (the last reverse layer), the kernel also writes F = -dE/dr
@@ -825,7 +829,7 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 cudaError_t launch_init_coef(cudaStream_t s, const reann_nlist* nl, const float* c0) {
     const int64_t nr = rows_of(nl), gr = ghost_rows_of(nl);
     if (nr + gr == 0) return cudaSuccess;
-    launch_pdl(k_init_coef, blocks_for(nr + gr, 256), 256, 0, s, nl->n, nr, gr, ghost_count_ptr(nl), nl->g_cap,
+    launch_with(true, eval_launch(nl).carve(), k_init_coef, blocks_for(nr + gr, 256), 256, 0, s, nl->n, nr, gr, ghost_count_ptr(nl), nl->g_cap,
                nl->species, nl->g_owner, c0, nl->coef);
     return cudaGetLastError();
 }
@@ -834,7 +838,7 @@ cudaError_t launch_gather_ghost_rows(cudaStream_t s, const reann_nlist* nl, floa
     const int64_t gr = ghost_rows_of(nl);
     if (gr == 0) return cudaSuccess;
     const int w4 = width / 4;
-    launch_pdl(k_gather_rows, blocks_for(gr * w4, 256), 256, 0, s, nl->n, ghost_count_ptr(nl), gr, w4, nl->g_owner,
+    launch_with(true, eval_launch(nl).carve(), k_gather_rows, blocks_for(gr * w4, 256), 256, 0, s, nl->n, ghost_count_ptr(nl), gr, w4, nl->g_owner,
                base);
     return cudaGetLastError();
 }
@@ -842,7 +846,7 @@ cudaError_t launch_gather_ghost_rows(cudaStream_t s, const reann_nlist* nl, floa
 cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
                          int* flags) {
     if (rows == 0) return cudaSuccess;
-    launch_pdl(k_edges, blocks_for(rows, kEdgeWarps), kEdgeWarps * 32, 0, s, row0, rows, nl->stride, r, nl->nbr,
+    launch_with(true, eval_launch(nl).carve(), k_edges, blocks_for(rows, kEdgeWarps), kEdgeWarps * 32, 0, s, row0, rows, nl->stride, r, nl->nbr,
                nl->nbr_cnt, nl->pos, nl->edge_xyzj, nl->edge_phi, nl->edge_der, nl->live_cnt, flags);
     return cudaGetLastError();
 }
@@ -853,13 +857,14 @@ cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radi
     // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer need
     // less reduction work per atom (many).  us per launch with 16 / 8 / 4 lanes: 192 atoms 4.5 / 5.6 /
     // 7.9, 4,000 5.5 / 5.8 / 7.1, 10,976 11.8 / 10.8 / 9.1, 24,576 25 / 20 / 20, 1,048,576 914 / 670 / 536.
+    const EvalLaunch how = eval_launch(nl);
     const int lpa = rows <= 4096 ? 16 : (rows <= 8192 ? 8 : 4);
     // records of more rows than this outgrow L2 between the passes: prefetch each atom's when it
     // starts (1,048,576 atoms: 580 -> 541 us; 24,576 atoms: 19.9 -> 20.2 us, so not there)
     const bool far = rows > (int64_t)1 << 16;
 #define REANN_FWD(P, L)                                                                                              \
-    k_density_fwd<P, L><<<blocks_for(rows, kFwdWarps * (32 / L)), kFwdWarps * 32, 0, s>>>(                             \
-        row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, coef, W, rho, bck, far)
+    launch_with(how.chain, how.carve(), k_density_fwd<P, L>, blocks_for(rows, kFwdWarps * (32 / L)), kFwdWarps * 32, 0, s, \
+                row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, coef, W, rho, bck, far)
     if (pairs) {
         if (lpa == 16)
             REANN_FWD(true, 16);
@@ -884,7 +889,7 @@ cudaError_t launch_bbar(cudaStream_t s, const reann_nlist* nl, const float* W, c
     const int64_t nr = rows_of(nl);
     if (nr == 0) return cudaSuccess;
     if (pairs)
-        launch_pdl(k_bbar<true>, blocks_for(nr, kBbarAtoms), 4 * kBbarAtoms, 0, s, nr, W, bck, rhobar, coef, rec, gh);
+        launch_with(true, eval_launch(nl).carve(), k_bbar<true>, blocks_for(nr, kBbarAtoms), 4 * kBbarAtoms, 0, s, nr, W, bck, rhobar, coef, rec, gh);
     else
         launch_pdl(k_bbar<false>, blocks_for(nr, kBbarAtoms), 4 * kBbarAtoms, 0, s, nr, W, bck, rhobar, coef, rec, gh);
     return cudaGetLastError();
@@ -911,10 +916,11 @@ cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radi
     // Lanes per atom, as in the forward pass.  us per launch with 32 / 16 / 8 lanes: 192 atoms 7.2 /
     // 10.6 / 18.3, 4,000 8.6 / 11.1 / 16.1, 24,576 43.5 / 41.1 / 49, 32,000 53 / 47.0 / 45.6,
     // 1,048,576 1,644 / 1,242 / 1,161.
+    const EvalLaunch how = eval_launch(nl);
     const int lpa = rows <= 16384 ? 32 : (rows <= 28672 ? 16 : 8);
 #define REANN_ADJ_L(C, V, L)                                                                                       \
-    k_density_adj<C, V, L><<<blocks_for(rows, kAdjWarps * (32 / L)), kAdjWarps * 32, 0, s>>>(                          \
-        row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, nl->edge_der, rec, bck, cbar, grad, vir, out)
+    launch_with(how.chain, how.carve(kAdjCarveout), k_density_adj<C, V, L>, blocks_for(rows, kAdjWarps * (32 / L)),     \
+                kAdjWarps * 32, 0, s, row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, nl->edge_der, rec, bck, cbar, grad, vir, out)
 #define REANN_ADJ(C, V)              \
     do {                             \
         if (lpa == 32)               \
@@ -951,8 +957,8 @@ cudaError_t launch_energy_sum(cudaStream_t s, const reann_nlist* nl, double* ene
     return cudaGetLastError();
 }
 
-cudaError_t launch_energy_final(cudaStream_t s, const double* partial, int np, double* energy) {
-    launch_pdl(k_energy_final, 1, kSumThreads, 0, s, np, partial, energy);
+cudaError_t launch_energy_final(cudaStream_t s, const double* partial, int np, double* energy, int carve) {
+    launch_with(true, carve, k_energy_final, 1, kSumThreads, 0, s, np, partial, energy);
     return cudaGetLastError();
 }
 

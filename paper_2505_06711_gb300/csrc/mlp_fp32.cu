@@ -22,6 +22,9 @@
 // backward: its output adjoint is 1, so nothing waits for another layer, the SiLU'
 // values stay in registers and the tile's weights are staged by one launch (24,576
 // atoms: 15.3 + 23.8 us in two launches, 34.6 us in one; 1,048,576: 407 + 712, 1,071).
+// Before pdl_enter() the networks read only what no kernel of the stream writes after the
+// previous kernel began: the tile list and the weights, whose copies are then under way
+// while the previous kernel ends.
 //   Bound by issue: 7,680 FMAs per row forward and 10,240 with the bbar step
 // backward, beside a quarter as many instructions for SiLU and a fifth for the
 // shared-memory fragments (1,048,576 atoms: 436 and 744 us, about 70 % of the issue
@@ -184,7 +187,6 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
                                                const float* __restrict__ rho, float* __restrict__ out,
                                                int out_stride, GhostOut gh, float* __restrict__ dsave,
                                                double* __restrict__ epart, int* __restrict__ flags) {
-    pdl_enter();
     constexpr int R = 16 * RPT;
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
@@ -198,24 +200,26 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
     const int tid = threadIdx.x;
     const Tile tl = block_rows<RPT>(tiles);
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
+        pdl_enter();
         if (OUT == 1 && epart && tid == 0) epart[blockIdx.x] = 0.0;
         return;
     }
     const NetDev& w = nets.e[tl.elem];
+    const uint32_t xb = (uint32_t)tl.nrows * FIN * 4;
     if (tid == 0) {  // W1, W2 and the input rows by bulk copies (TMA engine)
         bulk::mbar_init(&bar, 1);
         bulk::mbar_init_fence();
-        const uint32_t xb = (uint32_t)tl.nrows * FIN * 4;
         bulk::mbar_expect_tx(&bar, (FIN * H1 + H1 * H2) * 4 + xb);
         bulk::bulk_g2s(sW1, w.W1, FIN * H1 * 4, &bar);
         bulk::bulk_g2s(sW2, w.W2, H1 * H2 * 4, &bar);
-        bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * FIN, xb, &bar);
     }
     for (int i = tid; i < H2 * OUT; i += kT) sW3[w3_row<OUT>(i / OUT) * OUT + i % OUT] = w.W3[i];
     for (int i = tid; i < H1; i += kT) sb1[i] = w.b1[i];
     for (int i = tid; i < H2; i += kT) sb2[i] = w.b2[i];
     if (tid < OUT) sb3[tid] = w.b3[tid];
     for (int i = tl.nrows * FIN + tid; i < R * FIN; i += kT) sA[i] = 0.f;  // rows past the end
+    pdl_enter();
+    if (tid == 0) bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * FIN, xb, &bar);
     if (!staged(&bar, flags)) return;
     const int ty = tid >> 4, tx = tid & 15;
     float acc[RPT][4];
@@ -381,7 +385,6 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
                                                float* __restrict__ rhobar, const float* __restrict__ Wt,
                                                const float* __restrict__ bck, const float* __restrict__ coef,
                                                float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
-    pdl_enter();
     constexpr int R = 16 * RPT;
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
@@ -394,12 +397,11 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
     float* sWc = sR + R * LDH;        // (L+1) x N_orb x N_phi contraction W^t, transposed per l (BBAR)
     const int tid = threadIdx.x;
     const Tile tl = block_rows<RPT>(tiles);
-    if (tl.nrows <= 0) return;  // padding entry of a fixed-size tile list, or nothing left of the tile
+    if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
+        pdl_enter();
+        return;
+    }
     const int ty = tid >> 4, tx = tid & 15;
-    // the thread's SiLU'(z2), in flight while the weights are staged
-    float4 s2[RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) s2[i] = ld_save(dsave, tl, RPT * ty + i, H1 + 4 * tx);
     const NetDev& w = nets.e[tl.elem];
     if (tid == 0) {  // W1^T, W2^T, W3^T by bulk copies (TMA engine)
         bulk::mbar_init(&bar, 1);
@@ -410,6 +412,11 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
         bulk::bulk_g2s(sW3t, w.W3t, OUT * H2 * 4, &bar);
     }
     if (BBAR) stage_wc(sWc, Wt, tid);
+    pdl_enter();
+    // the thread's SiLU'(z2), in flight while ybar and the weights arrive
+    float4 s2[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) s2[i] = ld_save(dsave, tl, RPT * ty + i, H1 + 4 * tx);
     for (int i = tid; i < R * OUT; i += kT) {
         const int r = i / OUT, o = i % OUT;
         sY[r * 8 + o] = (OUT == 1) ? 1.f : (r < tl.nrows ? ybar[(size_t)(tl.row0 + r) * OUT + o] : 0.f);
@@ -467,7 +474,6 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
                                                       double* __restrict__ epart, const float* __restrict__ Wt,
                                                       const float* __restrict__ bck, const float* __restrict__ coef,
                                                       float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
-    pdl_enter();
     constexpr int R = 16 * RPT, F = NFEAT;
     static_assert(F * H1 + H1 * H2 >= R * LDH, "rhobar rows must fit in the W1, W2 region");
     __shared__ __align__(8) uint64_t bar;
@@ -481,17 +487,17 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
     const int tid = threadIdx.x;
     const Tile tl = block_rows<RPT>(tiles);
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
+        pdl_enter();
         if (epart && tid == 0) epart[blockIdx.x] = 0.0;
         return;
     }
     const NetDev& w = nets.e[tl.elem];
+    const uint32_t xb = (uint32_t)tl.nrows * F * 4;
     if (tid == 0) {
         bulk::mbar_init(&bar, 1);
         bulk::mbar_init_fence();
-        const uint32_t xb = (uint32_t)tl.nrows * F * 4;
         bulk::mbar_expect_tx(&bar, 2 * (F * H1 + H1 * H2) * 4 + xb);
         bulk::bulk_g2s(sW1, w.W1, F * H1 * 4, &bar);
-        bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * F, xb, &bar);
         bulk::bulk_g2s(sW2, w.W2, H1 * H2 * 4, &bar);
         bulk::bulk_g2s(sW1t, w.W1t, F * H1 * 4, &bar);
         bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
@@ -502,6 +508,8 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
     const float4 b1 = __ldg(reinterpret_cast<const float4*>(w.b1) + tx), b2 = __ldg(reinterpret_cast<const float4*>(w.b2) + tx);
     const float4 w3 = __ldg(reinterpret_cast<const float4*>(w.W3) + tx);
     const float b3 = __ldg(w.b3);
+    pdl_enter();
+    if (tid == 0) bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * F, xb, &bar);
     if (!staged(&bar, flags)) return;
     float acc[RPT][4], s1[RPT][4];
 #pragma unroll
@@ -621,9 +629,10 @@ cudaError_t launch_mlp_fwd_f32(cudaStream_t s, const reann_nlist* nl, const NetT
     if (energy && !pairs) return cudaErrorInvalidValue;  // launch_mlp_energy_f32
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
+    const EvalLaunch how = eval_launch(nl);
 #define REANN_FWD(O, F, RPT)                                                                                         \
-    k_mlp_fwd<O, F, RPT><<<nt * (4 / RPT), kT, fwd_smem<F, RPT>(), s>>>(ln, nl->tiles, rho, out, out_stride, gh, dsave, \
-                                                                        epart, flags)
+    launch_with(how.chain, how.carve(), k_mlp_fwd<O, F, RPT>, nt * (4 / RPT), kT, fwd_smem<F, RPT>(), s, ln, nl->tiles, \
+                rho, out, out_stride, gh, dsave, epart, flags)
 #define REANN_FWD_R(O, F)        \
     do {                         \
         if (parts == 4)          \
@@ -652,10 +661,11 @@ cudaError_t launch_mlp_bwd_f32(cudaStream_t s, const reann_nlist* nl, const NetT
     if (energy && !pairs) return cudaErrorInvalidValue;  // launch_mlp_energy_f32
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
+    const EvalLaunch how = eval_launch(nl);
 #define REANN_BWD(O, F, B, RPT)                                                                                    \
-    k_mlp_bwd<O, F, B, RPT><<<nt * (4 / RPT), kT, bwd_smem<F, B, RPT>(), s>>>(                                     \
-        ln, nl->tiles, dsave, ybar, rhobar, B ? Wt : nullptr, B ? bck : nullptr, B ? coef : nullptr,              \
-        B ? rec : nullptr, B ? gh : GhostOut{}, flags)
+    launch_with(how.chain, how.carve(), k_mlp_bwd<O, F, B, RPT>, nt * (4 / RPT), kT, bwd_smem<F, B, RPT>(), s, ln,  \
+                nl->tiles, dsave, ybar, rhobar, B ? Wt : nullptr, B ? bck : nullptr, B ? coef : nullptr,           \
+                B ? rec : nullptr, B ? gh : GhostOut{}, flags)
 #define REANN_BWD_R(O, F, B)        \
     do {                            \
         if (parts == 4)             \
@@ -683,9 +693,10 @@ cudaError_t launch_mlp_energy_f32(cudaStream_t s, const reann_nlist* nl, const N
     if (nt == 0) return cudaSuccess;
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
+    const EvalLaunch how = eval_launch(nl);
 #define REANN_EN(RPT)                                                                                              \
-    k_mlp_energy<RPT><<<nt * (4 / RPT), kT, energy_smem<RPT>(), s>>>(ln, nl->tiles, rho, eps, epart, Wt, bck, coef, \
-                                                                     rec, gh, flags)
+    launch_with(how.chain, how.carve(), k_mlp_energy<RPT>, nt * (4 / RPT), kT, energy_smem<RPT>(), s, ln, nl->tiles, \
+                rho, eps, epart, Wt, bck, coef, rec, gh, flags)
     if (parts == 4)
         REANN_EN(1);
     else if (parts == 2)

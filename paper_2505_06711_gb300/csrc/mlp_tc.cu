@@ -468,7 +468,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
                                                        const float* __restrict__ rho, float* __restrict__ out,
                                                        int out_stride, int* __restrict__ flags, GhostOut gh,
                                                        float* __restrict__ dsave, double* __restrict__ epart) {
-    pdl_enter();
     using L = FwdL<P>;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::BAR);
@@ -483,6 +482,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
     const int r = 32 * q + lane, c0 = 16 * cq;
     const Tile tl = tiles[blockIdx.x];
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list (before any TMEM allocation)
+        pdl_enter();
         if (OUT == 1 && epart && tid == 0) epart[blockIdx.x] = 0.0;
         return;
     }
@@ -490,19 +490,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
     const int64_t row = tl.row0 + r;
     const float inv_n = 1.f / (float)tl.nrows;
     const TcImg& w = nets.e[tl.elem];
-    int64_t g_lo = 0, g_hi = 0;  // the row's ghost images (loaded now, used by the output stage)
-    if (OUT > 1 && gh.goff && valid) {
-        g_lo = gh.goff[row];
-        g_hi = min((int64_t)gh.goff[row + 1], gh.gcap);
-    }
     const uint32_t tmem = setup(tslot, bar);
+    const uint32_t xb = (uint32_t)tl.nrows * NFEAT * 4;
     if (tid == 0) {
-        const uint32_t xb = (uint32_t)tl.nrows * NFEAT * 4;
         const uint8_t* img = P == P_FP8 ? w.wf8 : w.wf;
         mbar_expect_tx(&bar[0], L::WB * L::NS + xb);
         bulk_g2s(smem + L::W, img, L::WB, &bar[0]);
         if (P == P_SPLIT) bulk_g2s(smem + L::W + L::WB, img + L::WB, L::WB, &bar[0]);
-        bulk_g2s(smem + L::X, rho + (size_t)tl.row0 * NFEAT, xb, &bar[0]);
     }
     if (tid < 64) {
         par[F_B1 + tid] = w.b1[tid];
@@ -516,6 +510,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
     for (int i = tid; i < H2 * OUT; i += kThreads) par[F_W3 + (i / OUT) * 8 + i % OUT] = w.W3[i];
     WQ<NFEAT> wq1;  // this thread's eighth of W1 for the anchor zhat1 = rho-bar W1 + b1
     wq_load<NFEAT>(wq1, w.W1, H1, H1);
+    pdl_enter();  // so far only the tile list and the weights were read
+    if (tid == 0) bulk_g2s(smem + L::X, rho + (size_t)tl.row0 * NFEAT, xb, &bar[0]);
+    int64_t g_lo = 0, g_hi = 0;  // the row's ghost images (loaded now, used by the output stage)
+    if (OUT > 1 && gh.goff && valid) {
+        g_lo = gh.goff[row];
+        g_hi = min((int64_t)gh.goff[row + 1], gh.gcap);
+    }
     bool ok = wait_all(&bar[0], 0);
     if (!ok) fail(flags, bar, false);
     float sx = 1.f, sh = 1.f;
@@ -677,7 +678,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
                                                        const float* __restrict__ Wc, const float* __restrict__ bck,
                                                        const float* __restrict__ coef, float* __restrict__ rec,
                                                        GhostOut gh, int* __restrict__ flags) {
-    pdl_enter();
     using L = BwdL<P>;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::BAR);
@@ -690,7 +690,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = warp & 3, cq = warp >> 2;
     const int r = 32 * q + lane, c0 = 16 * cq;
     const Tile tl = tiles[blockIdx.x];
-    if (tl.nrows <= 0) return;  // padding entry of a fixed-size tile list (before any TMEM allocation)
+    if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list (before any TMEM allocation)
+        pdl_enter();
+        return;
+    }
     const bool valid = r < tl.nrows;
     const int64_t row = tl.row0 + r;
     const float inv_n = 1.f / (float)tl.nrows;
@@ -713,6 +716,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     }
     WQ<H2> wq;  // this thread's eighth of W2^T for the anchor u2-hat = v2-bar W2^T
     wq_load<H2>(wq, w.W2t, H1, H1);
+    pdl_enter();  // so far only the tile list and the weights were read
     float yb[OUT];
 #pragma unroll
     for (int o = 0; o < OUT; ++o)  // d eps_i / d eps_i = 1 for the energy network
@@ -884,15 +888,17 @@ int prec_of(int precision) {
 }
 
 template <int OUT, int P>
-void fwd_launch(cudaStream_t s, int nt, const TcLayer& l, const Tile* tiles, const float* rho, float* out,
+void fwd_launch(cudaStream_t s, const EvalLaunch& how, int nt, const TcLayer& l, const Tile* tiles, const float* rho, float* out,
                 int out_stride, int* flags, GhostOut gh, float* dsave, double* epart) {
-    k_tc_fwd<OUT, P><<<nt, kThreads, FwdL<P>::BYTES, s>>>(l, tiles, rho, out, out_stride, flags, gh, dsave, epart);
+    launch_with(how.chain, how.carve(), k_tc_fwd<OUT, P>, nt, kThreads, FwdL<P>::BYTES, s, l, tiles, rho, out, out_stride,
+                flags, gh, dsave, epart);
 }
 
 template <int OUT, int P>
-void bwd_launch(cudaStream_t s, int nt, const TcLayer& l, const Tile* tiles, const float* dsave, const float* ybar,
+void bwd_launch(cudaStream_t s, const EvalLaunch& how, int nt, const TcLayer& l, const Tile* tiles, const float* dsave, const float* ybar,
                 const float* Wc, const float* bck, const float* coef, float* rec, GhostOut gh, int* flags) {
-    k_tc_bwd<OUT, P><<<nt, kThreads, BwdL<P>::BYTES, s>>>(l, tiles, dsave, ybar, Wc, bck, coef, rec, gh, flags);
+    launch_with(how.chain, how.carve(), k_tc_bwd<OUT, P>, nt, kThreads, BwdL<P>::BYTES, s, l, tiles, dsave, ybar, Wc, bck,
+                coef, rec, gh, flags);
 }
 
 }  // namespace
@@ -905,11 +911,11 @@ cudaError_t launch_mlp_fwd_tc(cudaStream_t s, const reann_nlist* nl, const TcTab
     if (!dsave) return cudaErrorInvalidValue;
     ensure_tc_attrs();
     const TcLayer l = layer_of(nets, t);
-    using F = void (*)(cudaStream_t, int, const TcLayer&, const Tile*, const float*, float*, int, int*, GhostOut,
+    using F = void (*)(cudaStream_t, const EvalLaunch&, int, const TcLayer&, const Tile*, const float*, float*, int, int*, GhostOut,
                        float*, double*);
     static const F table[2][3] = {{fwd_launch<NPHI, P_BF16>, fwd_launch<NPHI, P_SPLIT>, fwd_launch<NPHI, P_FP8>},
                                   {fwd_launch<1, P_BF16>, fwd_launch<1, P_SPLIT>, fwd_launch<1, P_FP8>}};
-    table[energy ? 1 : 0][prec_of(precision)](s, nt, l, nl->tiles128, rho, out, out_stride, flags, gh, dsave,
+    table[energy ? 1 : 0][prec_of(precision)](s, eval_launch(nl), nt, l, nl->tiles128, rho, out, out_stride, flags, gh, dsave,
                                               energy ? epart : nullptr);
     return cudaGetLastError();
 }
@@ -922,11 +928,11 @@ cudaError_t launch_mlp_bwd_tc(cudaStream_t s, const reann_nlist* nl, const TcTab
     if (!dsave) return cudaErrorInvalidValue;  // the backward reads the forward's SiLU' values
     ensure_tc_attrs();
     const TcLayer l = layer_of(nets, t);
-    using F = void (*)(cudaStream_t, int, const TcLayer&, const Tile*, const float*, const float*, const float*,
+    using F = void (*)(cudaStream_t, const EvalLaunch&, int, const TcLayer&, const Tile*, const float*, const float*, const float*,
                        const float*, const float*, float*, GhostOut, int*);
     static const F table[2][3] = {{bwd_launch<NPHI, P_BF16>, bwd_launch<NPHI, P_SPLIT>, bwd_launch<NPHI, P_FP8>},
                                   {bwd_launch<1, P_BF16>, bwd_launch<1, P_SPLIT>, bwd_launch<1, P_FP8>}};
-    table[energy ? 1 : 0][prec_of(precision)](s, nt, l, nl->tiles128, dsave, ybar, Wc, bck, coef, rec, gh, flags);
+    table[energy ? 1 : 0][prec_of(precision)](s, eval_launch(nl), nt, l, nl->tiles128, dsave, ybar, Wc, bck, coef, rec, gh, flags);
     return cudaGetLastError();
 }
 

@@ -922,7 +922,7 @@ const int32_t* ghost_count_ptr(const reann_nlist* nl) { return nl->w.goff + nl->
 
 cudaError_t launch_refresh_positions(cudaStream_t s, const reann_nlist* nl, const double* pos, const float* c0) {
     const int64_t total = nl->n + nl->g_cap;
-    launch_pdl(k_refresh, blocks_for(total, kFp64Threads), kFp64Threads, 0, s, nl->n, ghost_count_ptr(nl), nl->g_cap,
+    launch_with(true, eval_launch(nl).carve(), k_refresh, blocks_for(total, kFp64Threads), kFp64Threads, 0, s, nl->n, ghost_count_ptr(nl), nl->g_cap,
                nl->geom, pos, nl->perm, nl->wrapm, nl->g_owner, nl->g_shift, nl->pos, nl->species, c0,
                nl->coef);
     return cudaGetLastError();

@@ -1011,7 +1011,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
                                                     (int)(ctx->precision == REANN_MLP_FP32
                                                               ? tiles_of(nl) * mlp_parts_f32(nl)
                                                               : tiles128_of(nl)),
-                                                    energy));
+                                                    energy, eval_launch(nl).carve()));
     }
     // reverse: Eqs. 3-5, one vector-Jacobian product per layer
     for (int t = T - 1; t >= 0; --t) {
