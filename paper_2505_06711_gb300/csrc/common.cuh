@@ -136,6 +136,43 @@ __device__ __forceinline__ void bbar_term(const float bm[NPHI], float two_w, con
     }
 }
 
+// The bbar step of N angular terms a0 .. a0 + N - 1 of one l: bbar_{a,m} = sum_k 2 w_a g_{a,k}
+// rhobar_{l,k} W_{l,m,k}, g = b W from the b checkpoint row b.  The terms share each weight fragment
+// wl[k] (N_phi floats) and rhobar value rb[k] read from shared memory.  Only the first `keep` are staged.
+template <int N>
+__device__ __forceinline__ void bbar_terms(const float* __restrict__ b, const float* wl, const float* rb, int a0,
+                                           int keep, float* sRec, int r) {
+    float bm[N][NPHI], o[N][NPHI], two_w[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const float4 b0 = __ldg(reinterpret_cast<const float4*>(b + (a0 + i) * NPHI));
+        const float4 b1 = __ldg(reinterpret_cast<const float4*>(b + (a0 + i) * NPHI + 4));
+        const float x[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int m = 0; m < NPHI; ++m) bm[i][m] = x[m], o[i][m] = 0.f;
+        two_w[i] = 2.f * rec_scale(a0 + i) * ang_w(a0 + i);
+    }
+#pragma unroll 2
+    for (int k = 0; k < NORB; ++k) {
+        const float4 w0 = *reinterpret_cast<const float4*>(wl + k * NPHI);
+        const float4 w1 = *reinterpret_cast<const float4*>(wl + k * NPHI + 4);
+        const float wm[NPHI] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        const float rv = rb[k];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float g = 0.f;
+#pragma unroll
+            for (int m = 0; m < NPHI; ++m) g = fmaf(bm[i][m], wm[m], g);
+            const float gb = two_w[i] * g * rv;
+#pragma unroll
+            for (int m = 0; m < NPHI; ++m) o[i][m] = fmaf(gb, wm[m], o[i][m]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (i < keep) stage_rec(sRec, r, a0 + i, o[i]);
+}
+
 // Values 10 and 11 of the record: the layer's coefficients c_m of `row`, and zero.
 __device__ __forceinline__ void rec_tail(const float* __restrict__ coef, int64_t row, int v, float val[NPHI]) {
     if (v == NANG) {

@@ -333,47 +333,43 @@ __device__ __forceinline__ void stage_wc(float* sWc, const float* __restrict__ W
     }
 }
 
-// bbar_{a,m} = sum_k 2 w_a g_{a,k} rhobar_{l,k} W_{l,m,k} of the block's rows, g = b W
-// recomputed from the b checkpoint (bck), written as their adjoint records (bbar with the
-// layer's c, ghost images too) through sRec.  16 / RPT threads per row take the record
-// values v = q, q + 16 / RPT, ... (angular terms, then c and 0).
+// The bbar step of the block's rows, written as their adjoint records (bbar with the layer's c, ghost
+// images too) through sRec.  RPT = 4: four threads per row, up to three terms of one l each; fewer rows: 16 / RPT threads per row, one record value at a time.
 template <int RPT>
 __device__ __forceinline__ void bbar_records(const float* sR, const float* sWc, float* sRec, const Tile& tl,
                                              const float* __restrict__ bck, const float* __restrict__ coef,
                                              float* __restrict__ rec, const GhostOut& gh, int tid) {
-    constexpr int TPR = 16 / RPT;
+    constexpr int TPR = kT / (16 * RPT);
     const int r = tid / TPR, q = tid % TPR;
-    const size_t row = (size_t)(tl.row0 + r);
-    const float* rb = sR + r * LDH;
+    if (r < tl.nrows) {
+        const size_t row = (size_t)(tl.row0 + r);
+        const float* rb = sR + r * LDH;
+        const float* b = bck + row * NB;
+        if constexpr (RPT == 4) {
+            // q = 0: term 0 (and two that are not kept, in step with its neighbours), c and 0;
+            // q = 1, 2, 3: terms 1-3, 4-6, 7-9
+            const int l = q == 0 ? 0 : (q == 1 ? 1 : 2);
+            bbar_terms<3>(b, sWc + l * NORB * NPHI, rb + l * NORB, q == 0 ? 0 : 3 * q - 2, q == 0 ? 1 : 3, sRec, r);
+            if (q == 0) {
+                float o[NPHI];
+                rec_tail(coef, row, NANG, o);
+                stage_rec(sRec, r, NANG, o);
+                rec_tail(coef, row, NANG + 1, o);
+                stage_rec(sRec, r, NANG + 1, o);
+            }
+        } else {
 #pragma unroll 1
-    for (int v = q; v < NREC / NPHI && r < tl.nrows; v += TPR) {
-        float o[NPHI];
-        if (v >= NANG) {
-            rec_tail(coef, row, v, o);
-            stage_rec(sRec, r, v, o);
-            continue;
+            for (int v = q; v < NREC / NPHI; v += TPR) {
+                if (v >= NANG) {
+                    float o[NPHI];
+                    rec_tail(coef, row, v, o);
+                    stage_rec(sRec, r, v, o);
+                } else {
+                    const int l = ang_l(v);
+                    bbar_terms<1>(b, sWc + l * NORB * NPHI, rb + l * NORB, v, 1, sRec, r);
+                }
+            }
         }
-        const int a = v, l = ang_l(a);
-        const float4 b0 = __ldg(reinterpret_cast<const float4*>(bck + row * NB + a * NPHI));
-        const float4 b1 = __ldg(reinterpret_cast<const float4*>(bck + row * NB + a * NPHI + 4));
-        const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int m = 0; m < NPHI; ++m) o[m] = 0.f;
-        const float two_w = 2.f * rec_scale(a) * ang_w(a);
-        const float* wl = sWc + l * NORB * NPHI;
-#pragma unroll 4
-        for (int k = 0; k < NORB; ++k) {
-            const float4 w0 = *reinterpret_cast<const float4*>(wl + k * NPHI);
-            const float4 w1 = *reinterpret_cast<const float4*>(wl + k * NPHI + 4);
-            const float wm[NPHI] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-            float g = 0.f;
-#pragma unroll
-            for (int m = 0; m < NPHI; ++m) g = fmaf(bm[m], wm[m], g);
-            const float gb = two_w * g * rb[l * NORB + k];
-#pragma unroll
-            for (int m = 0; m < NPHI; ++m) o[m] = fmaf(gb, wm[m], o[m]);
-        }
-        stage_rec(sRec, r, v, o);
     }
     __syncthreads();
     flush_rec(sRec, tl.nrows, tl.row0, rec, gh, tid, kT);  // ghost images get the rows' records too (reverse exchange)

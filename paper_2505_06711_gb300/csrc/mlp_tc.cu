@@ -803,37 +803,21 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         float* sRec = reinterpret_cast<float*>(smem + L::REC);
         if (valid) {
             const float* rb = sRB + r * L::kLdR;
-            // record values v = cq, cq + 4, cq + 8: angular terms a < 10, then c (10) and zero (11)
-#pragma unroll 1
-            for (int vv = cq; vv < NREC / NPHI; vv += 4) {
+            // column quarter 0: term 0, c and zero; 1, 2, 3: terms 1-3, 4-6, 7-9, of one l each (two
+            // and one at a time: three would not fit 64 registers)
+            const float* b = bck + (size_t)row * NB;
+            if (cq == 0) {
+                bbar_terms<1>(b, par + B_WC, rb, 0, 1, sRec, r);
                 float o[NPHI];
-                if (vv >= NANG) {
-                    rec_tail(coef, row, vv, o);
-                    stage_rec(sRec, r, vv, o);
-                    continue;
-                }
-                const int a_ = vv, l = ang_l(a_);
-                const float4 b0 = __ldg(reinterpret_cast<const float4*>(bck + (size_t)row * NB + a_ * NPHI));
-                const float4 b1 = __ldg(reinterpret_cast<const float4*>(bck + (size_t)row * NB + a_ * NPHI + 4));
-                const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                for (int m = 0; m < NPHI; ++m) o[m] = 0.f;
-                const float two_w = 2.f * rec_scale(a_) * ang_w(a_);
-                const float* wl = par + B_WC + l * NORB * NPHI;
-                const float* rl = rb + l * NORB;
-#pragma unroll 4
-                for (int k = 0; k < NORB; ++k) {
-                    const float4 w0 = *reinterpret_cast<const float4*>(wl + k * NPHI);
-                    const float4 w1 = *reinterpret_cast<const float4*>(wl + k * NPHI + 4);
-                    const float wm[NPHI] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-                    float g = 0.f;
-#pragma unroll
-                    for (int m = 0; m < NPHI; ++m) g = fmaf(bm[m], wm[m], g);
-                    const float gb = two_w * g * rl[k];
-#pragma unroll
-                    for (int m = 0; m < NPHI; ++m) o[m] = fmaf(gb, wm[m], o[m]);
-                }
-                stage_rec(sRec, r, a_, o);
+                rec_tail(coef, row, NANG, o);
+                stage_rec(sRec, r, NANG, o);
+                rec_tail(coef, row, NANG + 1, o);
+                stage_rec(sRec, r, NANG + 1, o);
+            } else {
+                const int l = cq == 1 ? 1 : 2;
+                const float *wl = par + B_WC + l * NORB * NPHI, *rl = rb + l * NORB;
+                bbar_terms<2>(b, wl, rl, 3 * cq - 2, 2, sRec, r);
+                bbar_terms<1>(b, wl, rl, 3 * cq, 1, sRec, r);
             }
         }
         __syncthreads();
