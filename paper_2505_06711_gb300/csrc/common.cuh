@@ -302,7 +302,7 @@ struct NlistScratch {
     int32_t *gcnt = nullptr, *goff = nullptr;  // ghosts per atom and offsets; goff[n] = ghost count
     int32_t* halo = nullptr;                    // per atom and axis: the image interval (pack_halo)
     int32_t* species_c = nullptr;              // caller-order species
-    int32_t *ekey = nullptr, *ecounts = nullptr, *estart = nullptr, *eorder = nullptr;
+    int32_t *ekey = nullptr, *ecounts = nullptr, *estart = nullptr;
     int32_t *scat = nullptr, *escat = nullptr;  // atomic-order scatter before the in-bucket ranking
     int32_t *tsum = nullptr, *etsum = nullptr;  // look-back status words of the scans (owned / extended)
     int32_t* rb_state = nullptr;  // rebuilds since the last sort, sort gate, keep-order gate

@@ -13,8 +13,9 @@
 //   2. counting sort by key -> internal order (element-major so the atomic
 //      networks see contiguous per-element tiles, spatially sorted inside an
 //      element so neighbour gathers stay local);
-//   3. enumerate ghost images (count while gathering, scan, fill while keying);
-//   4. bin owned + ghost slots into an extended cell grid (counting sort);
+//   3. enumerate ghost images (count while gathering, scan, fill while keying, a
+//      warp's lanes sharing its 32 atoms' images);
+//   4. bin owned + used ghost slots into an extended cell grid (counting sort);
 //   5. warp per owned atom: scan the stencil bins (in a rectangular cell each
 //      column trimmed to the sphere), FP32 pre-test with a margin, FP64 exact
 //      test for pairs near r_c + skin, ballot-compacted writes into a
@@ -57,7 +58,15 @@ __device__ __forceinline__ double smul(int n, double h) {
     return dmul((double)n, h);
 }
 
+// In a rectangular cell only the diagonal counts: the other terms are zeros, and adding them
+// changes at most the sign of a zero
 __device__ __forceinline__ void shift_vec(const CellGeom& g, int n0, int n1, int n2, double s[3]) {
+    if (g.ortho) {
+        s[0] = smul(n0, g.h[0]);
+        s[1] = smul(n1, g.h[4]);
+        s[2] = smul(n2, g.h[8]);
+        return;
+    }
 #pragma unroll
     for (int d = 0; d < 3; ++d) s[d] = dadd(dadd(smul(n0, g.h[d]), smul(n1, g.h[3 + d])), smul(n2, g.h[6 + d]));
 }
@@ -95,7 +104,8 @@ __device__ __forceinline__ void wrap_one(const CellGeom& g, const double x_in[3]
     bad = !(isfinite(x[0]) && isfinite(x[1]) && isfinite(x[2]));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        fr[k] = dadd(dadd(dmul(x[0], g.hinv[k]), dmul(x[1], g.hinv[3 + k])), dmul(x[2], g.hinv[6 + k]));
+        fr[k] = g.ortho ? dmul(x[k], g.hinv[4 * k])  // (the other terms are zeros)
+                        : dadd(dadd(dmul(x[0], g.hinv[k]), dmul(x[1], g.hinv[3 + k])), dmul(x[2], g.hinv[6 + k]));
         if (!isfinite(fr[k]) || fabs(fr[k]) > 1e9) bad = true;
     }
     if (bad) {
@@ -276,6 +286,70 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ g
     }
 }
 
+// The same scan of up to kDirectMax entries without communication: every block adds up
+// all entries before its tile itself (at most 256 KB from L2), so no block waits for
+// another.  24,576 entries, traced within the chain: 7.7 -> 6.1 us, 192: 7.1 -> 5.6 us (the
+// look-back's ticket, polls and reset); past 64 Ki entries the re-reading grows quadratically.
+constexpr int kDirectThreads = 1024, kDirectTile = 4 * kDirectThreads;
+constexpr int64_t kDirectMax = 1 << 16;
+__global__ void __launch_bounds__(kDirectThreads) k_scan_direct(const int* __restrict__ gate, int64_t n,
+                                                                const int32_t* __restrict__ in,
+                                                                int32_t* __restrict__ out) {
+    pdl_enter();
+    if (gate && *gate == 0) return;  // rebuild not needed this step
+    __shared__ int32_t warp_sums[32], warp_before[32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kDirectTile, i0 = base + 4 * tid;
+    int4 v = make_int4(0, 0, 0, 0);
+    if (i0 + 3 < n) {
+        v = *reinterpret_cast<const int4*>(in + i0);
+    } else {
+        if (i0 < n) v.x = in[i0];
+        if (i0 + 1 < n) v.y = in[i0 + 1];
+        if (i0 + 2 < n) v.z = in[i0 + 2];
+    }
+    int32_t before = 0;  // this thread's share of the entries before the tile
+    const int4* p = reinterpret_cast<const int4*>(in);
+#pragma unroll 4
+    for (int64_t q = tid; q < base / 4; q += kDirectThreads) {
+        const int4 x = p[q];
+        before += (x.x + x.y) + (x.z + x.w);
+    }
+    const int32_t local = (v.x + v.y) + (v.z + v.w);
+    int32_t incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31) warp_sums[w] = incl;
+    if (lane == 0) warp_before[w] = before;
+    __syncthreads();
+    if (w == 0) {
+        int32_t t = warp_sums[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        const int32_t all = __reduce_add_sync(0xffffffffu, warp_before[lane]);
+        warp_sums[lane] = t + all;  // entries up to the end of this warp
+        if (lane == 0) warp_before[0] = all;
+    }
+    __syncthreads();
+    const int32_t run = (w > 0 ? warp_sums[w - 1] : warp_before[0]) + incl - local;
+    const int4 e = make_int4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
+    if (i0 + 3 < n) {
+        *reinterpret_cast<int4*>(out + i0) = e;
+    } else {
+        if (i0 < n) out[i0] = e.x;
+        if (i0 + 1 < n) out[i0 + 1] = e.y;
+        if (i0 + 2 < n) out[i0 + 2] = e.z;
+    }
+    if (blockIdx.x == gridDim.x - 1 && tid == kDirectThreads - 1) out[n] = run + local;
+}
+
 inline int64_t scan_tiles(int64_t n) { return n > 0 ? (n + kScanTile - 1) / kScanTile : 1; }
 inline int64_t scan_status_words(int64_t n) { return scan_tiles(n) + 2; }
 
@@ -283,16 +357,28 @@ inline int64_t scan_status_words(int64_t n) { return scan_tiles(n) + 2; }
 // zeroed words
 static void scan_exclusive(cudaStream_t s, const int* gate, int64_t n, const int32_t* in, int32_t* out,
                            int32_t* status, int* flags) {
+    if (n <= kDirectMax) {
+        launch_pdl(k_scan_direct, (unsigned)std::max<int64_t>(1, (n + kDirectTile - 1) / kDirectTile), kDirectThreads, 0,
+                   s, gate, n, in, out);
+        return;
+    }
     launch_pdl(k_scan, (unsigned)scan_tiles(n), kScanThreads, 0, s, gate, n, in, out, status, flags);
 }
 
-__global__ void k_scatter(const int* __restrict__ gate, int64_t n, const int32_t* __restrict__ key,
-                          const int32_t* __restrict__ start, int32_t* __restrict__ counts,
-                          int32_t* __restrict__ order) {
+// The sorts cover n entries, of which the last g_cap are ghost slots that are in use up to
+// *g_count (null: all n).  Unused slots take no part (counted like the others, all of them
+// would queue at one address).
+__device__ __forceinline__ int64_t entries_in_use(int64_t n, const int32_t* g_count, int64_t g_cap) {
+    return g_count ? n - g_cap + (*g_count < g_cap ? *g_count : g_cap) : n;
+}
+
+__global__ void k_scatter(const int* __restrict__ gate, int64_t n, const int32_t* __restrict__ g_count, int64_t g_cap,
+                          const int32_t* __restrict__ key, const int32_t* __restrict__ start,
+                          int32_t* __restrict__ counts, int32_t* __restrict__ order) {
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= entries_in_use(n, g_count, g_cap)) return;
     int k = key[i];
     // counting the histogram back down: the bucket's entries take its slots from the top,
     // and the counts end at zero, ready for the next sort's histogram
@@ -303,30 +389,26 @@ __global__ void k_scatter(const int* __restrict__ gate, int64_t n, const int32_t
 // Deterministic placement inside each bucket: the entry at position p of the
 // atomic-order scatter moves to start[b] + (number of entries of its bucket with
 // a smaller index).  One thread per entry, each scanning its own bucket (buckets
-// hold tens of entries); entries of buckets >= sorted_keys keep their position.
-// With `pin`, the entry's FP32 position follows it into sorted order, its index
-// carried in .w (bit pattern), so that the search reads candidates contiguously.
-__global__ void k_bucket_rank(const int* __restrict__ gate, int64_t n, const int32_t* __restrict__ key,
-                              const int32_t* __restrict__ start, const int32_t* __restrict__ scattered,
-                              int64_t sorted_keys, int32_t* __restrict__ order, const float4* __restrict__ pin,
-                              float4* __restrict__ pout) {
+// hold tens of entries).  With `order` its index is stored there; with `pin` its
+// FP32 position follows it into sorted order, the index carried in .w (bit
+// pattern), so that the search reads candidates contiguously.
+__global__ void k_bucket_rank(const int* __restrict__ gate, int64_t n, const int32_t* __restrict__ g_count,
+                              int64_t g_cap, const int32_t* __restrict__ key, const int32_t* __restrict__ start,
+                              const int32_t* __restrict__ scattered, int32_t* __restrict__ order,
+                              const float4* __restrict__ pin, float4* __restrict__ pout) {
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+    if (p >= entries_in_use(n, g_count, g_cap)) return;
     const int32_t v = scattered[p];
     const int32_t b = key[v];
-    int64_t dst = p;
-    if (b < sorted_keys) {
-        const int lo = start[b], hi = start[b + 1];
-        int rank = 0;
-        for (int q = lo; q < hi; ++q) rank += scattered[q] < v;
-        dst = lo + rank;
-    }
-    order[dst] = v;
+    const int lo = start[b], hi = start[b + 1];
+    int rank = 0;
+    for (int q = lo; q < hi; ++q) rank += scattered[q] < v;
+    if (order) order[lo + rank] = v;
     if (pin) {
         const float4 x = pin[v];
-        pout[dst] = make_float4(x.x, x.y, x.z, __int_as_float(v));
+        pout[lo + rank] = make_float4(x.x, x.y, x.z, __int_as_float(v));
     }
 }
 
@@ -463,54 +545,78 @@ __device__ __forceinline__ void ext_slot_self(const CellGeom& g, const double* _
     p32[o] = make_float4((float)xw[3 * o], (float)xw[3 * o + 1], (float)xw[3 * o + 2], 0.f);
 }
 
-// 3-4. ghost images and the extended binning, one thread per slot of [0, n + g_cap):
-// owned slot i keys itself and fills its images' slots [goff[i], goff[i+1])
-// (owner, shift, key, FP32 position) in the order a, b, c of the per-axis
-// intervals; unused ghost capacity sorts last.
+// 3-4. ghost images and the extended binning.  A warp takes 32 atoms: each lane keys its
+// own atom, then the warp walks its atoms' images 32 at a time (slots goff[first] ..
+// goff[last + 1], in order; the order of an atom's images is a, b, c over the per-axis
+// intervals without the zero shift), so that the images of the few atoms near the
+// cell's faces, up to 7 in a large cell and 26 or more in a small one, are shared
+// by all lanes instead of keyed one after another by their owner's.  Bound by the FP64
+// pipe and the histogram's atomics; 24,576 atoms: 15.7 -> 9.6 us, 1,048,576: 74 -> 49 us
+// against one thread per slot with the unused ones keyed to a bucket of their own (whose
+// sort took another 28 us there).
 __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g, const double* __restrict__ xw,
                              const double* __restrict__ fw, const int32_t* __restrict__ goff, int64_t g_cap,
                              int32_t* __restrict__ owner, int32_t* __restrict__ shift, int32_t* __restrict__ key,
-                             int32_t* __restrict__ counts, float4* __restrict__ p32, int32_t dead_key,
-                             const int32_t* __restrict__ halo, int* __restrict__ flags) {
+                             int32_t* __restrict__ counts, float4* __restrict__ p32, const int32_t* __restrict__ halo,
+                             int* __restrict__ flags) {
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
+    const unsigned FULL = 0xffffffffu;
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n + g_cap) return;
-    if (s >= n) {
-        if (s >= n + ghosts_in_use(goff + n, g_cap)) {
-            key[s] = dead_key;
-            atomicAdd(&counts[dead_key], 1);
-            p32[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        return;  // slots in use are written by their owners
-    }
-    ext_slot_self(g, xw, fw, s, key, counts, p32);
-    int lo[3], hi[3];  // the intervals the wrap computed
+    const int lane = threadIdx.x & 31;
+    if (s - lane >= n) return;  // whole warps
+    // this lane's atom: where its images end (lanes past n have none), its intervals
+    int32_t end = INT32_MAX, low = 0, extent = 0;
+    if (s < n) {
+        ext_slot_self(g, xw, fw, s, key, counts, p32);
+        int lo[3], hi[3];  // as the wrap computed them
 #pragma unroll
-    for (int k = 0; k < 3; ++k) unpack_halo(halo[3 * s + k], lo[k], hi[k]);
-    int64_t q = goff[s];
-    for (int a = lo[0]; a <= hi[0]; ++a)
-        for (int b = lo[1]; b <= hi[1]; ++b)
-            for (int c = lo[2]; c <= hi[2]; ++c) {
-                if (a == 0 && b == 0 && c == 0) continue;
-                if (q < g_cap) {
-                    owner[q] = (int32_t)s;
-                    shift[q] = pack_shift(a, b, c);
-                    ext_slot(g, xw, fw, s, a, b, c, key, counts, p32, n + q);
-                } else {
-                    atomicOr(&flags[FLAG_GHOST_OVERFLOW], 1);
-                }
-                ++q;
-            }
+        for (int k = 0; k < 3; ++k) unpack_halo(halo[3 * s + k], lo[k], hi[k]);
+        low = pack_shift(lo[0], lo[1], lo[2]);
+        extent = (hi[0] - lo[0] + 1) | ((hi[1] - lo[1] + 1) << 8) | ((hi[2] - lo[2] + 1) << 16);
+        end = goff[s + 1];
+    }
+    const int32_t first = goff[s - lane], last = goff[s - lane + 32 < n ? s - lane + 32 : n];
+    if (last > g_cap && lane == 0) atomicOr(&flags[FLAG_GHOST_OVERFLOW], 1);
+    for (int32_t q0 = first; q0 < last; q0 += 32) {
+        const int32_t q = q0 + lane;
+        // the image's atom: the first lane whose images end beyond q
+        int lo = 0, hi = 31;
+#pragma unroll
+        for (int step = 0; step < 5; ++step) {
+            const int mid = (lo + hi) >> 1;
+            if (__shfl_sync(FULL, end, mid) > q) hi = mid;
+            else lo = mid + 1;
+        }
+        const int r = min(lo, 31);
+        const int32_t prev = __shfl_sync(FULL, end, max(r - 1, 0));
+        const int32_t low_r = __shfl_sync(FULL, low, r), ext_r = __shfl_sync(FULL, extent, r);
+        if (q < last && q < g_cap) {
+            int l0, l1, l2;
+            unpack_shift(low_r, l0, l1, l2);
+            const int d1 = (ext_r >> 8) & 255, d2 = (ext_r >> 16) & 255;
+            int e = q - (r > 0 ? prev : first);           // its number among the atom's images
+            e += e >= (-l0 * d1 - l1) * d2 - l2 ? 1 : 0;  // and among all shifts, the zero shift included
+            const int ab = e / d2, a = ab / d1, b = ab - a * d1, c = e - ab * d2;
+            const int64_t o = s - lane + r;
+            owner[q] = (int32_t)o;
+            shift[q] = pack_shift(l0 + a, l1 + b, l2 + c);
+            ext_slot(g, xw, fw, o, l0 + a, l1 + b, l2 + c, key, counts, p32, n + q);
+        }
+    }
 }
 
 // 5. neighbour search: one warp per owned atom.  For each (x, y) column of the
 // stencil the z-run of bins is one contiguous range of the bin-sorted slots;
 // lane l takes column l of a batch of 32, a warp scan of the run lengths
 // concatenates them, and the warp walks the concatenation 32 candidates at a
-// time (a binary search over the scanned lengths maps a candidate to its
-// column), reading the sorted FP32 positions with their slot index in .w.
+// time, reading the sorted FP32 positions with their slot index in .w.  The
+// columns that start among the 32 candidates are gathered as a bit mask (one
+// warp-wide OR); counting the mask's bits up to a candidate gives its column.
 // Candidates come in the same order as a bin-by-bin walk (x, then y, then z).
+// Bound by issue (70 % of the slots).  24,576 atoms: 34.1 -> 32.3 us, 1,048,576: 1,128 ->
+// 1,091 us, 192: 8.5 -> 7.9 us against a binary search by shuffles for the column,
+// integer divisions for the bins and one atomic per atom for the longest row.
 __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate, int64_t n, CellGeom g,
                                                    const double* __restrict__ xw, const int32_t* __restrict__ owner,
                                                    const int32_t* __restrict__ shift, const float4* __restrict__ p32,
@@ -521,7 +627,9 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
     const unsigned FULL = 0xffffffffu;
+    __shared__ int s_bases[8][32];
     const int lane = threadIdx.x & 31;
+    int* s_base = s_bases[threadIdx.x >> 5];
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= n) return;
     const float4 pi = p32[i];
@@ -530,23 +638,30 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
     // every lane here, kept a third of GB300's narrow FP64 pipe busy)
     int b[3];
     {
-        const int key = ekey[i];
-        b[2] = key % g.nbx[2];
-        b[1] = (key / g.nbx[2]) % g.nbx[1];
-        b[0] = key / (g.nbx[2] * g.nbx[1]);
+        // FP32 quotients, put right where they are off (by one, below 2^20 bins an axis)
+        const int key = ekey[i], plane = g.nbx[1] * g.nbx[2];
+        b[0] = (int)(__fdividef((float)key, (float)plane));
+        int rem = key - b[0] * plane;
+        while (rem < 0) --b[0], rem += plane;
+        while (rem >= plane) ++b[0], rem -= plane;
+        b[1] = (int)(__fdividef((float)rem, (float)g.nbx[2]));
+        b[2] = rem - b[1] * g.nbx[2];
+        while (b[2] < 0) --b[1], b[2] += g.nbx[2];
+        while (b[2] >= g.nbx[2]) ++b[1], b[2] -= g.nbx[2];
     }
     const int x0 = max(0, b[0] - g.sw[0]), x1 = min(g.nbx[0] - 1, b[0] + g.sw[0]);
     const int y0 = max(0, b[1] - g.sw[1]), y1 = min(g.nbx[1] - 1, b[1] + g.sw[1]);
     const int z0 = max(0, b[2] - g.sw[2]), z1 = min(g.nbx[2] - 1, b[2] + g.sw[2]);
     const int ny = y1 - y0 + 1, ncol = (x1 - x0 + 1) * ny;
+    const float inv_ny = __fdividef(1.f, (float)ny);
     const float lo2 = g.rcut2_f - g.margin, hi2 = g.rcut2_f + g.margin;
     int count = 0;
     int32_t* row = nbr + (size_t)i * stride;
     for (int cb = 0; cb < ncol; cb += 32) {
         int st = 0, len = 0;
         if (cb + lane < ncol) {
-            const int col = cb + lane;
-            const int bx = x0 + col / ny, by = y0 + col % ny;
+            const int col = cb + lane, cx = (int)((col + 0.5f) * inv_ny);  // col / ny: half a step from any integer
+            const int bx = x0 + cx, by = y0 + col - cx * ny;
             const int bin0 = (bx * g.nbx[1] + by) * g.nbx[2];
             int za = z0, zb = z1;
             if (g.ortho) {
@@ -579,18 +694,17 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
             if (lane >= o) pref += y;
         }
         const int total = __shfl_sync(FULL, pref, 31);
+        const int excl = pref - len;
+        const unsigned filled = __ballot_sync(FULL, len > 0), upto = (2u << lane) - 1u;
+        if (len > 0) s_base[__popc(filled & (upto >> 1))] = st - excl;  // of the non-empty columns, in order
+        __syncwarp();
+        int before = 0;  // non-empty columns that start before t0
         for (int t0 = 0; t0 < total; t0 += 32) {
             const int t = t0 + lane;
-            // column r of candidate t: the first lane whose inclusive prefix exceeds t
-            int lo = 0, hi = 31;
-#pragma unroll
-            for (int step = 0; step < 5; ++step) {
-                const int mid = (lo + hi) >> 1;
-                if (__shfl_sync(FULL, pref, mid) > t) hi = mid;
-                else lo = mid + 1;
-            }
-            const int r = min(lo, 31);
-            const int c = __shfl_sync(FULL, st, r) + t - (__shfl_sync(FULL, pref, r) - __shfl_sync(FULL, len, r));
+            const int rel = excl - t0;
+            const unsigned starts = __reduce_or_sync(FULL, len > 0 && rel >= 0 && rel < 32 ? 1u << rel : 0u);
+            const int c = s_base[before + __popc(starts & upto) - 1] + t;
+            before += __popc(starts);
             bool hit = false;
             int j = -1;
             if (t < total) {
@@ -627,11 +741,13 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
             }
             count += __popc(m);
         }
+        __syncwarp();  // s_base is rewritten for the next 32 columns
     }
     if (lane == 0) {
         cnt_out[i] = min(count, stride);
         if (count > stride) atomicOr(&flags[FLAG_NBR_OVERFLOW], 1);
-        atomicMax(&flags[FLAG_MAXNBR], count);
+        // (every atom's atomic at one address would serialise the kernel's end)
+        if (count > __ldcg(&flags[FLAG_MAXNBR])) atomicMax(&flags[FLAG_MAXNBR], count);
     }
 }
 
@@ -690,19 +806,19 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 
 }  // namespace
 
-// Counting sort of n keys in [0, nkeys) whose histogram `counts` the kernel that
-// produced the keys has filled: order = indices sorted by (key, index) within the
-// first `sorted_keys` buckets (later buckets hold unused capacity whose order does
-// not matter); start = bucket offsets.  The scatter counts the histogram back down
-// to zero for the next sort.
-static cudaError_t counting_sort(cudaStream_t s, const int* gate, int64_t n, int64_t nkeys, const int32_t* key,
-                                 int32_t* counts, int32_t* start, int32_t* scattered, int32_t* order,
-                                 int64_t sorted_keys, int32_t* tsum, int* flags, const float4* pin = nullptr,
-                                 float4* pout = nullptr) {
+// Counting sort of n entries (the ghost slots among them in use up to *g_count, null: all;
+// see entries_in_use) with keys in [0, nkeys) whose histogram `counts` the kernel that
+// produced the keys has filled: order (nullable) = indices sorted by (key, index), pout =
+// their FP32 positions pin; start = bucket offsets.  The scatter counts the histogram back
+// down to zero for the next sort.
+static cudaError_t counting_sort(cudaStream_t s, const int* gate, int64_t n, const int32_t* g_count, int64_t g_cap,
+                                 int64_t nkeys, const int32_t* key, int32_t* counts, int32_t* start,
+                                 int32_t* scattered, int32_t* order, int32_t* tsum, int* flags,
+                                 const float4* pin = nullptr, float4* pout = nullptr) {
     scan_exclusive(s, gate, nkeys, counts, start, tsum, flags);
     if (n > 0) {
-        launch_pdl(k_scatter, blocks_for(n, 256), 256, 0, s, gate, n, key, start, counts, scattered);
-        launch_pdl(k_bucket_rank, blocks_for(n, 256), 256, 0, s, gate, n, key, start, scattered, sorted_keys, order,
+        launch_pdl(k_scatter, blocks_for(n, 256), 256, 0, s, gate, n, g_count, g_cap, key, start, counts, scattered);
+        launch_pdl(k_bucket_rank, blocks_for(n, 256), 256, 0, s, gate, n, g_count, g_cap, key, start, scattered, order,
                    pin, pout);
     }
     return cudaGetLastError();
@@ -768,8 +884,7 @@ static cudaError_t stage_sort_and_count(cudaStream_t s, reann_nlist* nl, const d
     NlistScratch& w = nl->w;
     launch_pdl(k_wrap_key, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, sort_gate, n, pos, w.species_c,
                nl->n_elem, nl->geom, w.xw_c, w.fw_c, w.mw_c, w.key, w.counts, flags, nl->pos_ref);
-    counting_sort(s, sort_gate, n, owned_keys(nl), w.key, w.counts, w.start, w.scat, nl->perm, owned_keys(nl),
-                  w.tsum, flags);
+    counting_sort(s, sort_gate, n, nullptr, 0, owned_keys(nl), w.key, w.counts, w.start, w.scat, nl->perm, w.tsum, flags);
     launch_pdl(k_gather_internal, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, sort_gate, n, nl->geom, nl->perm,
                w.xw_c, w.fw_c, w.mw_c, w.species_c, w.xw, w.fw, nl->wrapm, nl->species, w.gcnt, w.halo);
     if (keep_gate)
@@ -784,10 +899,10 @@ static cudaError_t stage_ghosts_and_bins(cudaStream_t s, reann_nlist* nl, int* f
     const int64_t n = nl->n, next = n + nl->g_cap;
     NlistScratch& w = nl->w;
     const int64_t nx = ext_bins(nl);
-    launch_pdl(k_ghosts_ext, blocks_for(next, kFp64Threads), kFp64Threads, 0, s, gate, n, nl->geom, w.xw, w.fw,
-               w.goff, nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, (int32_t)nx, w.halo, flags);
-    counting_sort(s, gate, next, nx + 1, w.ekey, w.ecounts, w.estart, w.escat, w.eorder, nx, w.etsum, flags,
-                  w.p32, w.p32s);
+    launch_pdl(k_ghosts_ext, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, gate, n, nl->geom, w.xw, w.fw, w.goff,
+               nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, w.halo, flags);
+    counting_sort(s, gate, next, w.goff + n, nl->g_cap, nx, w.ekey, w.ecounts, w.estart, w.escat, nullptr, w.etsum,
+                  flags, w.p32, w.p32s);
     return cudaGetLastError();
 }
 
@@ -864,16 +979,15 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
     w.ekey = dalloc<int32_t>(nl, next);
     w.p32 = dalloc<float4>(nl, next);
     w.p32s = dalloc<float4>(nl, next);
-    w.ecounts = dalloc<int32_t>(nl, nx + 1);
-    w.estart = dalloc<int32_t>(nl, nx + 2);
-    w.eorder = dalloc<int32_t>(nl, next);
+    w.ecounts = dalloc<int32_t>(nl, nx);
+    w.estart = dalloc<int32_t>(nl, nx + 1);
     w.escat = dalloc<int32_t>(nl, next);
-    w.etsum = dalloc<int32_t>(nl, scan_status_words(nx + 1));
-    if (!nl->g_owner || !nl->g_shift || !w.ekey || !w.p32 || !w.p32s || !w.ecounts || !w.estart || !w.eorder ||
+    w.etsum = dalloc<int32_t>(nl, scan_status_words(nx));
+    if (!nl->g_owner || !nl->g_shift || !w.ekey || !w.p32 || !w.p32s || !w.ecounts || !w.estart ||
         !w.escat || !w.etsum)
         return set_error(ctx, REANN_E_NOMEM, "ghost allocation failed");
-    REANN_CUDA_TRY(ctx, cudaMemsetAsync(w.ecounts, 0, sizeof(int32_t) * (nx + 1), s));  // kept zero between sorts
-    REANN_CUDA_TRY(ctx, cudaMemsetAsync(w.etsum, 0, sizeof(int32_t) * scan_status_words(nx + 1), s));
+    REANN_CUDA_TRY(ctx, cudaMemsetAsync(w.ecounts, 0, sizeof(int32_t) * nx, s));  // kept zero between sorts
+    REANN_CUDA_TRY(ctx, cudaMemsetAsync(w.etsum, 0, sizeof(int32_t) * scan_status_words(nx), s));
     REANN_CUDA_TRY(ctx, stage_ghosts_and_bins(s, nl, ctx->d_flags, nullptr));
     // row capacity: expected neighbours from the number density, with headroom
     const CellGeom& g = nl->geom;
