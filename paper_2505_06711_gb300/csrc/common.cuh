@@ -393,7 +393,7 @@ struct reann_nlist {
     float* bck = nullptr;          // T x N x 80
     float* eps = nullptr;          // N
     float* rhobar = nullptr;       // N x 48
-    float* dsave = nullptr;        // T x N x 128 SiLU'(z1), SiLU'(z2) of the FP32 networks
+    float* dsave = nullptr;        // T x N x 128 SiLU'(z1), SiLU'(z2) of the networks (by rows; tensor-core: by tiles)
     float* bbar = nullptr;         // (N + g_cap) x 96 adjoint records (bbar, c)
     float* cbar = nullptr;         // N x 8
     float* grad = nullptr;         // N x 3

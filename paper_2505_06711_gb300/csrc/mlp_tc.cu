@@ -408,11 +408,20 @@ __device__ __forceinline__ void lds16(const float* p, float* v) {
     }
 }
 
-// 16 consecutive floats of global memory (16 B aligned) into registers, zeros when !ok
-__device__ __forceinline__ void ldg16(const float* p, bool ok, float* v) {
+// The saved SiLU' values of a tile: values 4 c .. 4 c + 3 of its rows side by side (block c nrows + r
+// from the tile's first row), since a warp's lanes are 32 rows.  Row by row each 16 B access
+// touched its own line: 8,192 of the forward's and backward's 28,000 L1 cycles per tile.  With
+// bbar_three, 1,048,576 rows of split BF16: forward 393 -> 296 us, backward 612 -> 516 us;
+// 24,576 rows of BF16: 15.4 -> 11.8 and 25.3 -> 21.2 us.
+__device__ __forceinline__ size_t save_at(const Tile& tl, int r, int c) {
+    return (size_t)tl.row0 * ((H1 + H2) / 4) + (size_t)(c * tl.nrows + r);
+}
+// blocks c .. c + 3 of row r, zeros for rows past the tile's end
+__device__ __forceinline__ void ld_save16(const float* dsave, const Tile& tl, int r, int c, float* v) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 x = ok ? __ldg(reinterpret_cast<const float4*>(p) + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 x = r < tl.nrows ? __ldg(reinterpret_cast<const float4*>(dsave) + save_at(tl, r, c + k))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
         v[4 * k] = x.x, v[4 * k + 1] = x.y, v[4 * k + 2] = x.z, v[4 * k + 3] = x.w;
     }
 }
@@ -570,9 +579,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
             if (!valid) v[i] = 0.f;
         }
         if (valid && dsave) {
-            float4* d = reinterpret_cast<float4*>(dsave + (size_t)row * (H1 + H2) + c0);
+            float4* d = reinterpret_cast<float4*>(dsave) + save_at(tl, r, c0 / 4);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
+            for (int k = 0; k < 4; ++k) d[k * tl.nrows] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
         }
         WQ<H1> wq2;  // this thread's eighth of W2 for zhat2 = h1-bar W2 + b2
         wq_load<H1>(wq2, w.W2, H2, H2);
@@ -604,9 +613,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
             a[i] = silu_fast(z, v[i]);  // a: SiLU'(z2), v: h2
         }
         if (valid && dsave) {
-            float4* d = reinterpret_cast<float4*>(dsave + (size_t)row * (H1 + H2) + H1 + c0);
+            float4* d = reinterpret_cast<float4*>(dsave) + save_at(tl, r, (H1 + c0) / 4);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
+            for (int k = 0; k < 4; ++k) d[k * tl.nrows] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
         }
         // output layer in FP32: this quarter row's partial dot products, then the four quarters
         float y[OUT];
@@ -668,6 +677,58 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
 }
 
 // ------------------------------------------------------------ backward ---
+// The bbar step of terms a0, a0 + 1, a0 + 2, of one l: with the symmetric
+//   M_{m,m'} = sum_k rhobar_{l,k} W_{l,m,k} W_{l,m',k}
+// of the row, bbar_{a,m} = 2 w_a sum_m' M_{m,m'} b_{a,m'}.  The weights are read from shared memory
+// once for the three terms (which side by side would need 48 sums, more than fit 64 registers;
+// in two passes they were read twice: 1,024 L1 cycles of a tile more).
+__device__ __forceinline__ void bbar_three(const float* __restrict__ b, const float* wl, const float* rb, int a0,
+                                           float* sRec, int r) {
+    float M[NPHI * (NPHI + 1) / 2];
+#pragma unroll
+    for (int i = 0; i < NPHI * (NPHI + 1) / 2; ++i) M[i] = 0.f;
+    float4 b0 = __ldg(reinterpret_cast<const float4*>(b + a0 * NPHI));
+    float4 b1 = __ldg(reinterpret_cast<const float4*>(b + a0 * NPHI) + 1);
+#pragma unroll 1
+    for (int k = 0; k < NORB; ++k) {
+        const float4 w0 = *reinterpret_cast<const float4*>(wl + k * NPHI);
+        const float4 w1 = *reinterpret_cast<const float4*>(wl + k * NPHI + 4);
+        const float wm[NPHI] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        const float rv = rb[k];
+        int p = 0;
+#pragma unroll
+        for (int m = 0; m < NPHI; ++m) {
+            const float t = rv * wm[m];
+#pragma unroll
+            for (int q = m; q < NPHI; ++q, ++p) M[p] = fmaf(t, wm[q], M[p]);
+        }
+    }
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+        const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        const int a = a0 + i;
+        if (i < 2) {  // the next term's
+            const float4* next = reinterpret_cast<const float4*>(b + (a + 1) * NPHI);
+            b0 = __ldg(next), b1 = __ldg(next + 1);
+        }
+        float o[NPHI];
+#pragma unroll
+        for (int m = 0; m < NPHI; ++m) o[m] = 0.f;
+        int p = 0;
+#pragma unroll
+        for (int m = 0; m < NPHI; ++m)
+#pragma unroll
+            for (int q = m; q < NPHI; ++q, ++p) {
+                o[m] = fmaf(M[p], bm[q], o[m]);
+                if (q > m) o[q] = fmaf(M[p], bm[m], o[q]);
+            }
+        const float two_w = 2.f * rec_scale(a) * ang_w(a);
+#pragma unroll
+        for (int m = 0; m < NPHI; ++m) o[m] *= two_w;
+        stage_rec(sRec, r, a, o);
+    }
+}
+
 // rhobar = J^T ybar of the tile's rows (ybar: c-bar rows, or 1 for the energy
 // network), then the bbar step of Eq. 1's squares for the same rows,
 //   bbar_{a,m} = sum_k 2 w_a g_{a,k} rhobar_{l(a),k} W_{l,m,k},  g = b W (b: checkpoint bck),
@@ -722,7 +783,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     for (int o = 0; o < OUT; ++o)  // d eps_i / d eps_i = 1 for the energy network
         yb[o] = OUT == 1 ? 1.f : (valid ? __ldg(ybar + (size_t)row * OUT + o) : 0.f);
     float sd[16], v[16], a[16];
-    ldg16(dsave + (size_t)row * (H1 + H2) + H1 + c0, valid, sd);  // SiLU'(z2) of this quarter row
+    ld_save16(dsave, tl, r, (H1 + c0) / 4, sd);  // SiLU'(z2) of this quarter row
     __syncthreads();
     // v2 = (ybar W3^T) * SiLU'(z2) in FP32
 #pragma unroll
@@ -753,7 +814,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
             issue<P>(tmem, sA, sAlo, 64, sW, P == P_SPLIT ? sW + L::WB : nullptr, H1);
             mma_commit(&bar[1]);
         }
-        ldg16(dsave + (size_t)row * (H1 + H2) + c0, valid, sd);  // SiLU'(z1), while the product runs
+        ld_save16(dsave, tl, r, c0 / 4, sd);  // SiLU'(z1), while the product runs
         // u2-hat = v2-bar W2^T: sum_q W2[u][q] v2-bar[q] = sum_q W2t[q][u] v2-bar[q]
         wq_sum(par + B_ZP, nullptr, par + B_U2, H1);
         ok = wait_all(&bar[1], 0);
@@ -803,8 +864,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         float* sRec = reinterpret_cast<float*>(smem + L::REC);
         if (valid) {
             const float* rb = sRB + r * L::kLdR;
-            // column quarter 0: term 0, c and zero; 1, 2, 3: terms 1-3, 4-6, 7-9, of one l each (two
-            // and one at a time: three would not fit 64 registers)
+            // column quarter 0: term 0, c and zero; 1, 2, 3: terms 1-3, 4-6, 7-9, of one l each
             const float* b = bck + (size_t)row * NB;
             if (cq == 0) {
                 bbar_terms<1>(b, par + B_WC, rb, 0, 1, sRec, r);
@@ -815,9 +875,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
                 stage_rec(sRec, r, NANG + 1, o);
             } else {
                 const int l = cq == 1 ? 1 : 2;
-                const float *wl = par + B_WC + l * NORB * NPHI, *rl = rb + l * NORB;
-                bbar_terms<2>(b, wl, rl, 3 * cq - 2, 2, sRec, r);
-                bbar_terms<1>(b, wl, rl, 3 * cq, 1, sRec, r);
+                bbar_three(b, par + B_WC + l * NORB * NPHI, rb + l * NORB, 3 * cq - 2, sRec, r);
             }
         }
         __syncthreads();
