@@ -56,33 +56,7 @@ struct PackDst {
     float4* pos_out;  // hi, lo parts of each slot, interleaved
 };
 
-// owned atoms: rows (remapped), species, destination, positions
-__global__ void k_pack_owned(PackSrc s, PackDst d) {
-    pdl_enter();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= s.n) return;
-    const int c = s.cnt[i];
-    const int32_t* src = s.nbr + (size_t)i * s.stride;
-    int32_t* dst = d.nbr + (size_t)(d.ob + i) * d.stride;
-    for (int e = 0; e < c; ++e) {
-        const int64_t j = src[e];
-        dst[e] = (int32_t)(j < s.n ? d.ob + j : d.no + d.gb + (j - s.n));
-    }
-    d.cnt[d.ob + i] = c;
-    d.species[d.ob + i] = s.species[i];
-    d.perm[d.ob + i] = (int32_t)(d.ob + s.perm[i]);
-    const int64_t ci = s.perm[i];
-    double sm[3], x[3];
-    shift_vec(s.geom, s.wrapm[3 * i], s.wrapm[3 * i + 1], s.wrapm[3 * i + 2], sm);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) x[k] = s.pos[3 * ci + k] - sm[k];
-    hilo(x, d.pos_out[2 * (d.ob + i)], d.pos_out[2 * (d.ob + i) + 1]);
-}
-
-// ghost slots: owner (pool index) and image position
-__global__ void k_pack_ghosts(PackSrc s, PackDst d) {
-    pdl_enter();
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void pack_ghost(const PackSrc& s, const PackDst& d, int64_t q) {
     if (q >= s.g) return;
     const int64_t o = s.owner[q];
     const int p = s.shift[q];
@@ -95,6 +69,38 @@ __global__ void k_pack_ghosts(PackSrc s, PackDst d) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) x[k] = (s.pos[3 * co + k] - sm[k]) + sv[k];
     hilo(x, d.pos_out[2 * (d.no + d.gb + q)], d.pos_out[2 * (d.no + d.gb + q) + 1]);
+}
+
+// The first own_blocks blocks take the owned atoms, a warp each (rows remapped, species,
+// destination, positions), the others a ghost per thread.  Bound by latency (13 us for a
+// structure of a few hundred atoms; with a thread walking each row and the ghosts in a
+// second launch 26 us).
+__global__ void __launch_bounds__(256) k_pack(PackSrc s, PackDst d, unsigned own_blocks) {
+    pdl_enter();
+    if (blockIdx.x >= own_blocks) {
+        pack_ghost(s, d, (int64_t)(blockIdx.x - own_blocks) * blockDim.x + threadIdx.x);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= s.n) return;
+    const int c = s.cnt[i];
+    const int32_t* src = s.nbr + (size_t)i * s.stride;
+    int32_t* dst = d.nbr + (size_t)(d.ob + i) * d.stride;
+    for (int e = lane; e < c; e += 32) {
+        const int64_t j = src[e];
+        dst[e] = (int32_t)(j < s.n ? d.ob + j : d.no + d.gb + (j - s.n));
+    }
+    if (lane != 0) return;
+    d.cnt[d.ob + i] = c;
+    d.species[d.ob + i] = s.species[i];
+    const int64_t ci = s.perm[i];
+    d.perm[d.ob + i] = (int32_t)(d.ob + ci);
+    double sm[3], x[3];
+    shift_vec(s.geom, s.wrapm[3 * i], s.wrapm[3 * i + 1], s.wrapm[3 * i + 2], sm);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[k] = s.pos[3 * ci + k] - sm[k];
+    hilo(x, d.pos_out[2 * (d.ob + i)], d.pos_out[2 * (d.ob + i) + 1]);
 }
 
 // a released owned range: no neighbours, outputs to the sink row
@@ -145,8 +151,8 @@ cudaError_t launch_pack(cudaStream_t s, const reann_nlist* src, const double* ca
               src->perm,    src->wrapm, src->g_owner, src->g_shift, caller_pos,   src->geom};
     PackDst b{pool->n, ob, gb, pool->stride, pool->nbr, pool->nbr_cnt, pool->species, pool->perm, pool->g_owner,
               pool->pos};
-    launch_pdl(k_pack_owned, blocks_for(src->n, 128), 128, 0, s, a, b);
-    if (src->g > 0) launch_pdl(k_pack_ghosts, blocks_for(src->g, 256), 256, 0, s, a, b);
+    const unsigned own = blocks_for(src->n * 32, 256);
+    launch_pdl(k_pack, own + (src->g > 0 ? blocks_for(src->g, 256) : 0), 256, 0, s, a, b, own);
     return cudaGetLastError();
 }
 
