@@ -545,7 +545,7 @@ __device__ __forceinline__ void ext_slot_self(const CellGeom& g, const double* _
     p32[o] = make_float4((float)xw[3 * o], (float)xw[3 * o + 1], (float)xw[3 * o + 2], 0.f);
 }
 
-// 3-4. ghost images and the extended binning.  A warp takes 32 atoms: each lane keys its
+// 3-4. ghost images and the extended binning.  A warp takes apw atoms: each lane keys its
 // own atom, then the warp walks its atoms' images 32 at a time (slots goff[first] ..
 // goff[last + 1], in order; the order of an atom's images is a, b, c over the per-axis
 // intervals without the zero shift), so that the images of the few atoms near the
@@ -558,16 +558,16 @@ __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g
                              const double* __restrict__ fw, const int32_t* __restrict__ goff, int64_t g_cap,
                              int32_t* __restrict__ owner, int32_t* __restrict__ shift, int32_t* __restrict__ key,
                              int32_t* __restrict__ counts, float4* __restrict__ p32, const int32_t* __restrict__ halo,
-                             int* __restrict__ flags) {
+                             int apw, int* __restrict__ flags) {
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
     const unsigned FULL = 0xffffffffu;
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
-    if (s - lane >= n) return;  // whole warps
-    // this lane's atom: where its images end (lanes past n have none), its intervals
+    const int64_t s0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * apw, s = s0 + lane;
+    if (s0 >= n) return;  // whole warps
+    // this lane's atom: where its images end (lanes without one have none), its intervals
     int32_t end = INT32_MAX, low = 0, extent = 0;
-    if (s < n) {
+    if (lane < apw && s < n) {
         ext_slot_self(g, xw, fw, s, key, counts, p32);
         int lo[3], hi[3];  // as the wrap computed them
 #pragma unroll
@@ -576,7 +576,7 @@ __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g
         extent = (hi[0] - lo[0] + 1) | ((hi[1] - lo[1] + 1) << 8) | ((hi[2] - lo[2] + 1) << 16);
         end = goff[s + 1];
     }
-    const int32_t first = goff[s - lane], last = goff[s - lane + 32 < n ? s - lane + 32 : n];
+    const int32_t first = goff[s0], last = goff[s0 + apw < n ? s0 + apw : n];
     if (last > g_cap && lane == 0) atomicOr(&flags[FLAG_GHOST_OVERFLOW], 1);
     for (int32_t q0 = first; q0 < last; q0 += 32) {
         const int32_t q = q0 + lane;
@@ -598,7 +598,7 @@ __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g
             int e = q - (r > 0 ? prev : first);           // its number among the atom's images
             e += e >= (-l0 * d1 - l1) * d2 - l2 ? 1 : 0;  // and among all shifts, the zero shift included
             const int ab = e / d2, a = ab / d1, b = ab - a * d1, c = e - ab * d2;
-            const int64_t o = s - lane + r;
+            const int64_t o = s0 + r;
             owner[q] = (int32_t)o;
             shift[q] = pack_shift(l0 + a, l1 + b, l2 + c);
             ext_slot(g, xw, fw, o, l0 + a, l1 + b, l2 + c, key, counts, p32, n + q);
@@ -935,8 +935,12 @@ static cudaError_t stage_ghosts_and_bins(cudaStream_t s, reann_nlist* nl, int* f
     const int64_t n = nl->n, next = n + nl->g_cap;
     NlistScratch& w = nl->w;
     const int64_t nx = ext_bins(nl);
-    launch_pdl(k_ghosts_ext, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, gate, n, nl->geom, w.xw, w.fw, w.goff,
-               nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, w.halo, flags);
+    // Atoms per warp: in a small cell most atoms have several images, and a warp's chain of 32-image
+    // batches is what the launch lasts.  us with 4 / 8 / 16 / 32: 192 atoms 4.2 / 5.2 / 7.7 / 11.5,
+    // 3,069 4.7 / 5.7 / 7.8 / 9.2, 8,100 7.0 / 6.4 / 8.2 / 10.6, 24,576 14.6 / 11.5 / 9.8 / 10.0.
+    const int apw = n <= 8192 ? 4 : 32;
+    launch_pdl(k_ghosts_ext, blocks_for((n + apw - 1) / apw * 32, kFp64Threads), kFp64Threads, 0, s, gate, n, nl->geom,
+               w.xw, w.fw, w.goff, nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, w.halo, apw, flags);
     counting_sort(s, gate, next, w.goff + n, nl->g_cap, nx, w.ekey, w.ecounts, w.estart, w.escat, nullptr, w.etsum,
                   flags, w.p32, w.p32s);
     return cudaGetLastError();
