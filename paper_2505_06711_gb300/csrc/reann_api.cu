@@ -1053,8 +1053,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
     }
     ProfScope p(ctx, PR_OUTPUT);
     if (vir) {
-        REANN_CUDA_TRY(ctx, launch_virial_sum(s, nl, vir, nl->vir_partial, virial));
-        if (atom_virial) REANN_CUDA_TRY(ctx, launch_unpermute_rows(s, nl, vir, 9, atom_virial, 9));
+        REANN_CUDA_TRY(ctx, launch_virial_sum(s, nl, vir, nl->vir_partial, virial, atom_virial));
     }
     return REANN_OK;
 }
@@ -1062,7 +1061,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
 int ensure_virial(reann_ctx* ctx, reann_nlist* nl) {
     if (nl->vir) return REANN_OK;
     nl->vir = nl_alloc<float>(nl, (size_t)nl->n * 9);
-    nl->vir_partial = nl_alloc<double>(nl, (size_t)9 * ((nl->n + 2047) / 2048 + 1));
+    nl->vir_partial = nl_alloc<double>(nl, (size_t)virial_partials(nl->n));
     if (!nl->vir || !nl->vir_partial) return set_error(ctx, REANN_E_NOMEM, "virial buffers: out of device memory");
     return REANN_OK;
 }

@@ -92,3 +92,19 @@ def test_virial_bf16x3_within_bound():
     W, _, _ = _virial(spec, s, precision=2)
     ref = oracle.energy_forces(spec, s.pos, s.species, s.cell)["virial"]
     assert float(np.abs(W - ref).max()) / s.n_atoms <= W_TOL_PER_ATOM
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 256, 257, 545])
+def test_virial_sums_over_rows(n):
+    # block and warp edges of the sums: the total is the FP64 sum of the rows, and the rows come in caller order
+    from synth import Structure
+
+    spec = make_model(T=1)
+    full = water_box(200, seed=3)
+    s = Structure(full.pos[:n], full.species[:n], full.cell)
+    W, Wa, _ = _virial(spec, s)
+    np.testing.assert_allclose(W, Wa.sum(0).reshape(3, 3), rtol=1e-12, atol=1e-12 * n)
+    p = np.random.default_rng(n).permutation(n)
+    _, Wp, _ = _virial(spec, Structure(s.pos[p], s.species[p], s.cell))
+    # another order of the atoms changes the order of each row's sums only: FP32 roundings of ~200 terms
+    np.testing.assert_allclose(Wp, Wa[p], rtol=0, atol=2e-5 * max(1e-3, np.abs(Wa).max()))
