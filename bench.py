@@ -532,17 +532,17 @@ def measured_peaks() -> tuple[float, str]:
         return 6800.0, "fallback"
 
 
-def launches_per_step(T: int, fused_energy: bool = False) -> int:
+def launches_per_step(T: int, fused_energy: bool = False, rebuild: int = 13) -> int:
     """Library kernel launches per step (single-domain list):
-    rebuild 13 (sort-or-keep gate; wrap + keys + histogram, 3 sort kernels (scan,
-    scatter, rank) and the gather, which return at once on rebuilds that keep the
-    atom order; the keep-order wrap; ghost-count scan; ghosts + extended keys +
-    histogram, 3 sort kernels, search), evaluation 2 (positions with c0, live
-    edges) + 2T forward (density, network; the energy network also sums its
-    tiles) + 1 (total energy) + 2T reverse (network with bbar, density adjoint;
-    the last one writes forces and atomic energies).  ``fused_energy``: the 48-feature
-    FP32 energy network is one launch forward and backward."""
-    return 13 + 2 + 2 * T + 1 + 2 * T - (1 if fused_energy else 0)
+    ``rebuild`` for the list, evaluation 2 (positions with c0, live edges) + 2T forward
+    (density, network; the energy network also sums its tiles) + 1 (total energy) + 2T
+    reverse (network with bbar, density adjoint; the last one writes forces and atomic
+    energies).  ``fused_energy``: the 48-feature FP32 energy network is one launch forward
+    and backward.  A rebuild is 11 launches above 2,048 atoms (wrap + keys + histogram, 3
+    sort kernels (scan, scatter, rank) and the gather, which return at once on rebuilds
+    that keep the atom order; ghost-count scan; ghosts + extended keys + histogram, 3 sort
+    kernels, search) and 7 up to there (one block sorts, gathers and scans)."""
+    return rebuild + 2 + 2 * T + 1 + 2 * T - (1 if fused_energy else 0)
 
 
 def cpu_baseline(structure, spec):
@@ -814,7 +814,7 @@ def run_ours(args):
         line["pair_features"] = pairs
         line["e2e"] = e2e
         line["roofline"] = roof
-        line["gpu_launches"] = launches_per_step(T_LAYERS, fused_energy=True) * args.steps
+        line["gpu_launches"] = launches_per_step(T_LAYERS, fused_energy=True, rebuild=11) * args.steps
         line["clocks"] = clk
         line["wall_s_timed_region"] = wall
         line["breakdown_ms_per_step"] = breakdown

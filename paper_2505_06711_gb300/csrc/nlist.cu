@@ -9,7 +9,7 @@
 // Build (all deterministic):
 //   1. wrap positions into the cell in FP64 and key every atom by
 //      (element, cell bin) -- on the first build and every 8th rebuild; the
-//      rebuilds in between keep the previous internal order (k_wrap_keep);
+//      rebuilds in between keep the previous internal order;
 //   2. counting sort by key -> internal order (element-major so the atomic
 //      networks see contiguous per-element tiles, spatially sorted inside an
 //      element so neighbour gathers stay local);
@@ -121,43 +121,6 @@ __device__ __forceinline__ void wrap_one(const CellGeom& g, const double x_in[3]
         xw[k] = dsub(x[k], s[k]);
         fw[k] = dsub(fr[k], (double)m[k]);
     }
-}
-
-__global__ void k_wrap_key(const int* __restrict__ gate, int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ species, int n_elem,
-                           CellGeom g, double* __restrict__ xw, double* __restrict__ fw, int32_t* __restrict__ mw,
-                           int32_t* __restrict__ key, int32_t* __restrict__ counts, int* __restrict__ flags,
-                           double* __restrict__ ref) {
-    pdl_enter();
-    if (gate && *gate == 0) return;  // rebuild (or this rebuild's sort) not needed
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double x[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]};
-    // the positions of this build, for the moved-by-more-than-skin/2 test
-    ref[3 * i] = x[0];
-    ref[3 * i + 1] = x[1];
-    ref[3 * i + 2] = x[2];
-    int sp = species[i];
-    if (sp < 0 || sp >= n_elem) {
-        atomicOr(&flags[FLAG_SPECIES], 1);
-        sp = 0;
-    }
-    double xwi[3], f[3];
-    int m[3];
-    bool bad;
-    wrap_one(g, x, xwi, f, m, bad);
-    if (bad) atomicOr(&flags[FLAG_GEOM], 1);
-    int b[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        xw[3 * i + k] = xwi[k];
-        fw[3 * i + k] = f[k];
-        mw[3 * i + k] = m[k];
-        b[k] = clampi((int)floor(f[k] * g.nb[k]), 0, g.nb[k] - 1);
-    }
-    int nbins = g.nb[0] * g.nb[1] * g.nb[2];
-    const int k = sp * nbins + (b[0] * g.nb[1] + b[1]) * g.nb[2] + b[2];
-    key[i] = k;
-    atomicAdd(&counts[k], 1);  // the counting sort's histogram
 }
 
 // ---- deterministic counting sort ------------------------------------------
@@ -350,6 +313,38 @@ __global__ void __launch_bounds__(kDirectThreads) k_scan_direct(const int* __res
     if (blockIdx.x == gridDim.x - 1 && tid == kDirectThreads - 1) out[n] = run + local;
 }
 
+// out = exclusive scan of in, out[n] = the sum, by one block of kDirectThreads threads
+__device__ __forceinline__ void block_scan(int n, const int32_t* in, int32_t* out, int32_t* warp_sums) {
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int32_t carry = 0;
+    for (int base = 0; base < n; base += kDirectTile) {
+        int32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = base + 4 * tid + k < n ? in[base + 4 * tid + k] : 0;
+        const int32_t local = (v[0] + v[1]) + (v[2] + v[3]);
+        int32_t incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_sums[w] = incl;
+        __syncthreads();
+        const int32_t s = warp_sums[lane];
+        const int32_t before = __reduce_add_sync(0xffffffffu, lane < w ? s : 0);
+        int32_t run = carry + before + incl - local;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (base + 4 * tid + k < n) out[base + 4 * tid + k] = run;
+            run += v[k];
+        }
+        carry += __reduce_add_sync(0xffffffffu, s);
+        __syncthreads();  // warp_sums is written again
+    }
+    if (tid == 0) out[n] = carry;
+    __syncthreads();
+}
+
 inline int64_t scan_tiles(int64_t n) { return n > 0 ? (n + kScanTile - 1) / kScanTile : 1; }
 inline int64_t scan_status_words(int64_t n) { return scan_tiles(n) + 2; }
 
@@ -433,64 +428,36 @@ __device__ __forceinline__ void halo_interval(const CellGeom& g, int k, double f
     }
 }
 
-// 2. gather per-atom arrays into internal order
-// (also each atom's number of ghost images: the product of its per-axis intervals
-// minus the zero shift, which wrapped coordinates in [0, 1) always admit)
-__global__ void k_gather_internal(const int* __restrict__ gate, int64_t n, CellGeom g, const int32_t* __restrict__ perm,
-                                  const double* __restrict__ xw_c, const double* __restrict__ fw_c,
-                                  const int32_t* __restrict__ mw_c, const int32_t* __restrict__ sp_c,
-                                  double* __restrict__ xw, double* __restrict__ fw, int32_t* __restrict__ mw,
-                                  int32_t* __restrict__ sp, int32_t* __restrict__ gcnt, int32_t* __restrict__ halo) {
-    pdl_enter();
-    if (gate && *gate == 0) return;  // rebuild not needed this step
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int c = perm[i];
-    int cnt = 1;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        xw[3 * i + k] = xw_c[3 * (int64_t)c + k];
-        const double f = fw_c[3 * (int64_t)c + k];
-        fw[3 * i + k] = f;
-        mw[3 * i + k] = mw_c[3 * (int64_t)c + k];
-        int lo, hi;
-        halo_interval(g, k, f, lo, hi);
-        halo[3 * i + k] = pack_halo(lo, hi);
-        cnt *= hi - lo + 1;
-    }
-    sp[i] = sp_c[c];
-    gcnt[i] = cnt - 1;
-}
+// an atom's wrapped coordinates, the integer shifts and its image intervals (pack_halo)
+struct WrappedAtoms {
+    double *xw, *fw;
+    int32_t *mw, *halo;
+};
 
 // Rebuilds between sorts: every kResortPeriod-th rebuild sorts the owned atoms
 // again; the others keep the internal order of the last sort, and only wrap the
 // new positions (straight into internal order) and count their ghost images.
 // The list itself (ghosts, extended bins, search) is rebuilt in full either way.
-// state[0] counts rebuilds since the last sort; state[1] gates the sort path and
-// state[2] the keep-order path for this rebuild (both 0 when it is gated off).
+// state[0] counts rebuilds since the last sort (k_ghosts_ext counts on);
+// state[1] gates the sort's kernels, 0 when the rebuild is gated off.
 constexpr int kResortPeriod = 8;
 
-__global__ void k_rebuild_gates(const int* __restrict__ gate, int* __restrict__ state) {
+// 1. wrap: caller-order atom i with its sort key and the sort's histogram when this
+// rebuild sorts (first: always), else the caller's position of internal atom i
+__global__ void k_wrap(const int* __restrict__ gate, int* __restrict__ state, bool first, int64_t n, CellGeom g,
+                       const double* __restrict__ pos, const int32_t* __restrict__ species, int n_elem,
+                       WrappedAtoms caller, int32_t* __restrict__ key, int32_t* __restrict__ counts,
+                       WrappedAtoms internal, const int32_t* __restrict__ perm, int32_t* __restrict__ gcnt,
+                       int* __restrict__ flags, double* __restrict__ ref) {
     pdl_enter();
     const bool run = !gate || *gate != 0;
-    const bool sort = run && state[0] >= kResortPeriod;
-    if (run) state[0] = sort ? 1 : state[0] + 1;
-    state[1] = sort ? 1 : 0;
-    state[2] = run && !sort ? 1 : 0;
-}
-
-// the keep-order path: wrap the caller-order positions of the internal atoms i
-// (the same arithmetic as k_wrap_key) and count their ghost images
-__global__ void k_wrap_keep(const int* __restrict__ gate, int64_t n, CellGeom g, const double* __restrict__ pos,
-                            const int32_t* __restrict__ perm, double* __restrict__ xw, double* __restrict__ fw,
-                            int32_t* __restrict__ mw, int32_t* __restrict__ gcnt, int32_t* __restrict__ halo,
-                            int* __restrict__ flags, double* __restrict__ ref) {
-    pdl_enter();
-    if (gate && *gate == 0) return;
+    const bool sort = run && (first || state[0] >= kResortPeriod);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t c = perm[i];
+    if (i == 0) state[1] = sort ? 1 : 0;
+    if (!run || i >= n) return;
+    const int64_t c = sort ? i : perm[i];
     const double x[3] = {pos[3 * c], pos[3 * c + 1], pos[3 * c + 2]};
+    // the positions of this build, for the moved-by-more-than-skin/2 test
     ref[3 * c] = x[0];
     ref[3 * c + 1] = x[1];
     ref[3 * c + 2] = x[2];
@@ -499,18 +466,101 @@ __global__ void k_wrap_keep(const int* __restrict__ gate, int64_t n, CellGeom g,
     bool bad;
     wrap_one(g, x, xwi, f, m, bad);
     if (bad) atomicOr(&flags[FLAG_GEOM], 1);
+    const WrappedAtoms& o = sort ? caller : internal;
     int cnt = 1;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        xw[3 * i + k] = xwi[k];
-        fw[3 * i + k] = f[k];
-        mw[3 * i + k] = m[k];
+        o.xw[3 * i + k] = xwi[k];
+        o.fw[3 * i + k] = f[k];
+        o.mw[3 * i + k] = m[k];
         int lo, hi;
         halo_interval(g, k, f[k], lo, hi);
-        halo[3 * i + k] = pack_halo(lo, hi);
+        o.halo[3 * i + k] = pack_halo(lo, hi);
         cnt *= hi - lo + 1;
     }
-    gcnt[i] = cnt - 1;
+    if (!sort) {
+        // ghost images: the product of the intervals minus the zero shift, which wrapped coordinates
+        // in [0, 1) always admit
+        gcnt[i] = cnt - 1;
+        return;
+    }
+    int sp = species[i];
+    if (sp < 0 || sp >= n_elem) {
+        atomicOr(&flags[FLAG_SPECIES], 1);
+        sp = 0;
+    }
+    int b[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) b[k] = clampi((int)floor(f[k] * g.nb[k]), 0, g.nb[k] - 1);
+    const int nbins = g.nb[0] * g.nb[1] * g.nb[2];
+    const int k = sp * nbins + (b[0] * g.nb[1] + b[1]) * g.nb[2] + b[2];
+    key[i] = k;
+    atomicAdd(&counts[k], 1);  // the counting sort's histogram
+}
+
+// 2. per-atom arrays into internal order, with each atom's number of ghost images
+struct GatherAtoms {
+    WrappedAtoms caller, internal;
+    const int32_t* species_c;
+    int32_t *species, *gcnt;
+};
+__device__ __forceinline__ void gather_atom(const GatherAtoms& a, int64_t i, int64_t c) {
+    int cnt = 1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        a.internal.xw[3 * i + k] = a.caller.xw[3 * c + k];
+        a.internal.fw[3 * i + k] = a.caller.fw[3 * c + k];
+        a.internal.mw[3 * i + k] = a.caller.mw[3 * c + k];
+        const int32_t h = a.caller.halo[3 * c + k];
+        a.internal.halo[3 * i + k] = h;
+        int lo, hi;
+        unpack_halo(h, lo, hi);
+        cnt *= hi - lo + 1;
+    }
+    a.species[i] = a.species_c[c];
+    a.gcnt[i] = cnt - 1;
+}
+__global__ void k_gather_internal(const int* __restrict__ gate, int64_t n, const int32_t* __restrict__ perm,
+                                  GatherAtoms a) {
+    pdl_enter();
+    if (*gate == 0) return;  // the order is kept
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) gather_atom(a, i, perm[i]);
+}
+
+// Sort (if state[1] says so), gather and ghost-count scan of a small system by one block:
+// one launch instead of five, which return at once on most rebuilds, and on the steps of a
+// trajectory that need none, at 0.85 us each.  Step with rebuild before and with it, us: 192
+// atoms 108.0 -> 103.0, 1,536 115.0 -> 112.7, 3,069 131.0 -> 131.3, 4,095 133.0 -> 137.9 (one
+// block's sort grows past what the launches cost); with k_wrap's merge alone 4,098 atoms
+// 139.9 -> 136.4.  20 trajectory steps of 1,536 atoms 2,050 -> 1,967.
+constexpr int64_t kSmallOrder = 2048, kSmallKeys = 1 << 15;
+__global__ void __launch_bounds__(kDirectThreads) k_order_small(const int* gate, const int* state, int n, int nkeys,
+                                                                const int32_t* key, int32_t* counts, int32_t* start,
+                                                                int32_t* scattered, int32_t* perm, GatherAtoms a,
+                                                                int32_t* goff) {
+    pdl_enter();
+    if (gate && *gate == 0) return;  // rebuild not needed this step
+    __shared__ int32_t warp_sums[32];
+    const int tid = threadIdx.x;
+    if (state[1] != 0) {
+        block_scan(nkeys, counts, start, warp_sums);
+        for (int i = tid; i < n; i += kDirectThreads) {
+            const int k = key[i];
+            scattered[start[k] + atomicSub(&counts[k], 1) - 1] = i;
+        }
+        __syncthreads();
+        for (int p = tid; p < n; p += kDirectThreads) {
+            const int v = scattered[p], b = key[v], lo = start[b], hi = start[b + 1];
+            int rank = 0;
+            for (int q = lo; q < hi; ++q) rank += scattered[q] < v;
+            perm[lo + rank] = v;
+        }
+        __syncthreads();
+        for (int i = tid; i < n; i += kDirectThreads) gather_atom(a, i, perm[i]);
+        __syncthreads();
+    }
+    block_scan(n, a.gcnt, goff, warp_sums);
 }
 
 // 3-4. ghost images (fractional coordinate within (-reach, 1 + reach) on every
@@ -558,9 +608,10 @@ __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g
                              const double* __restrict__ fw, const int32_t* __restrict__ goff, int64_t g_cap,
                              int32_t* __restrict__ owner, int32_t* __restrict__ shift, int32_t* __restrict__ key,
                              int32_t* __restrict__ counts, float4* __restrict__ p32, const int32_t* __restrict__ halo,
-                             int apw, int* __restrict__ flags) {
+                             int apw, int* __restrict__ state, int* __restrict__ flags) {
     pdl_enter();
     if (gate && *gate == 0) return;  // rebuild not needed this step
+    if (state && blockIdx.x == 0 && threadIdx.x == 0) state[0] = state[1] ? 1 : state[0] + 1;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t s0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * apw, s = s0 + lane;
@@ -914,24 +965,28 @@ static int64_t ext_bins(const reann_nlist* nl) {
 // steps 1-3a: wrap, sort, gather, ghost count + scan (goff[n] = ghost count on the device)
 // sort_gate: the sort path (nullptr: always); keep_gate: the keep-order path (nullptr:
 // never); gate: the rest of the rebuild (nullptr: always)
+// first: the list's first build, which sorts
 static cudaError_t stage_sort_and_count(cudaStream_t s, reann_nlist* nl, const double* pos, int* flags,
-                                        const int* sort_gate, const int* keep_gate, const int* gate) {
-    const int64_t n = nl->n;
+                                        const int* gate, bool first) {
+    const int64_t n = nl->n, nkeys = owned_keys(nl);
     NlistScratch& w = nl->w;
-    launch_pdl(k_wrap_key, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, sort_gate, n, pos, w.species_c,
-               nl->n_elem, nl->geom, w.xw_c, w.fw_c, w.mw_c, w.key, w.counts, flags, nl->pos_ref);
-    counting_sort(s, sort_gate, n, nullptr, 0, owned_keys(nl), w.key, w.counts, w.start, w.scat, nl->perm, w.tsum, flags);
-    launch_pdl(k_gather_internal, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, sort_gate, n, nl->geom, nl->perm,
-               w.xw_c, w.fw_c, w.mw_c, w.species_c, w.xw, w.fw, nl->wrapm, nl->species, w.gcnt, w.halo);
-    if (keep_gate)
-        launch_pdl(k_wrap_keep, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, keep_gate, n, nl->geom, pos,
-                   nl->perm, w.xw, w.fw, nl->wrapm, w.gcnt, w.halo, flags, nl->pos_ref);
+    const WrappedAtoms caller{w.xw_c, w.fw_c, w.mw_c, w.halo_c}, internal{w.xw, w.fw, nl->wrapm, w.halo};
+    const GatherAtoms gather{caller, internal, w.species_c, nl->species, w.gcnt};
+    launch_pdl(k_wrap, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, gate, w.rb_state, first, n, nl->geom, pos,
+               w.species_c, nl->n_elem, caller, w.key, w.counts, internal, nl->perm, w.gcnt, flags, nl->pos_ref);
+    if (n <= kSmallOrder && nkeys <= kSmallKeys) {
+        launch_pdl(k_order_small, 1, kDirectThreads, 0, s, gate, w.rb_state, (int)n, (int)nkeys, w.key, w.counts,
+                   w.start, w.scat, nl->perm, gather, w.goff);
+        return cudaGetLastError();
+    }
+    const int* sort_gate = w.rb_state + 1;
+    counting_sort(s, sort_gate, n, nullptr, 0, nkeys, w.key, w.counts, w.start, w.scat, nl->perm, w.tsum, flags);
+    launch_pdl(k_gather_internal, blocks_for(n, kFp64Threads), kFp64Threads, 0, s, sort_gate, n, nl->perm, gather);
     scan_exclusive(s, gate, n, w.gcnt, w.goff, w.tsum, flags);
     return cudaGetLastError();
 }
 
-// steps 3b-4: ghost fill and the extended bins (needs the ghost capacity)
-static cudaError_t stage_ghosts_and_bins(cudaStream_t s, reann_nlist* nl, int* flags, const int* gate) {
+static cudaError_t stage_ghosts_and_bins(cudaStream_t s, reann_nlist* nl, int* flags, const int* gate, bool first) {
     const int64_t n = nl->n, next = n + nl->g_cap;
     NlistScratch& w = nl->w;
     const int64_t nx = ext_bins(nl);
@@ -940,7 +995,8 @@ static cudaError_t stage_ghosts_and_bins(cudaStream_t s, reann_nlist* nl, int* f
     // 3,069 4.7 / 5.7 / 7.8 / 9.2, 8,100 7.0 / 6.4 / 8.2 / 10.6, 24,576 14.6 / 11.5 / 9.8 / 10.0.
     const int apw = n <= 8192 ? 4 : 32;
     launch_pdl(k_ghosts_ext, blocks_for((n + apw - 1) / apw * 32, kFp64Threads), kFp64Threads, 0, s, gate, n, nl->geom,
-               w.xw, w.fw, w.goff, nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, w.halo, apw, flags);
+               w.xw, w.fw, w.goff, nl->g_cap, nl->g_owner, nl->g_shift, w.ekey, w.ecounts, w.p32, w.halo, apw,
+               first ? nullptr : w.rb_state, flags);
     counting_sort(s, gate, next, w.goff + n, nl->g_cap, nx, w.ekey, w.ecounts, w.estart, w.escat, nullptr, w.etsum,
                   flags, w.p32, w.p32s);
     return cudaGetLastError();
@@ -975,6 +1031,7 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
     w.xw = dalloc<double>(nl, 3 * n);
     w.fw = dalloc<double>(nl, 3 * n);
     w.gcnt = dalloc<int32_t>(nl, n);
+    w.halo_c = dalloc<int32_t>(nl, 3 * n);
     w.halo = dalloc<int32_t>(nl, 3 * n);
     w.goff = dalloc<int32_t>(nl, n + 1);
     w.species_c = dalloc<int32_t>(nl, n);
@@ -986,14 +1043,14 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
     nl->wrapm = dalloc<int32_t>(nl, 3 * n);
     nl->pos_ref = dalloc<double>(nl, 3 * n);
     if (!w.xw_c || !w.fw_c || !w.mw_c || !w.key || !w.counts || !w.start || !w.xw || !w.fw || !w.gcnt || !w.goff ||
-        !w.halo ||
+        !w.halo_c || !w.halo ||
         !w.species_c || !w.scat || !nl->perm || !nl->species || !nl->wrapm || !nl->pos_ref || !w.rb_state ||
         !w.tsum)
         return set_error(ctx, REANN_E_NOMEM, "neighbour-list allocation failed");
     // counts and tsum are kept zero between sorts; this build sorts, rebuilds count from 1
     launch_begin(s, {n, species, w.species_c, nkeys, w.counts, std::max(scan_status_words(nkeys), scan_status_words(n)),
                      w.tsum, ctx->d_flags, w.rb_state});
-    REANN_CUDA_TRY(ctx, stage_sort_and_count(s, nl, pos, ctx->d_flags, nullptr, nullptr, nullptr));
+    REANN_CUDA_TRY(ctx, stage_sort_and_count(s, nl, pos, ctx->d_flags, nullptr, true));
     // sizes: element ranges of the internal order and the ghost count, read back with the flags
     const int32_t* es = ctx->h_flags + NFLAGS;
     launch_pdl(k_read_sizes, 1, 64, 0, s, nl->n_elem, nkeys / nl->n_elem, w.start, w.goff + n, ctx->d_flags,
@@ -1023,7 +1080,7 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
         !w.escat || !w.etsum)
         return set_error(ctx, REANN_E_NOMEM, "ghost allocation failed");
     launch_begin(s, {0, nullptr, nullptr, nx, w.ecounts, scan_status_words(nx), w.etsum, ctx->d_flags, nullptr});
-    REANN_CUDA_TRY(ctx, stage_ghosts_and_bins(s, nl, ctx->d_flags, nullptr));
+    REANN_CUDA_TRY(ctx, stage_ghosts_and_bins(s, nl, ctx->d_flags, nullptr, true));
     // row capacity: expected neighbours from the number density, with headroom
     const CellGeom& g = nl->geom;
     const double vol = std::fabs(g.h[0] * (g.h[4] * g.h[8] - g.h[5] * g.h[7]) -
@@ -1053,9 +1110,8 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
 
 // gate == nullptr: always rebuild; otherwise every kernel returns at once unless *gate != 0
 cudaError_t launch_rebuild(cudaStream_t s, reann_nlist* nl, const double* pos, int* flags, const int* gate) {
-    launch_pdl(k_rebuild_gates, 1, 1, 0, s, gate, nl->w.rb_state);
-    cudaError_t e = stage_sort_and_count(s, nl, pos, flags, nl->w.rb_state + 1, nl->w.rb_state + 2, gate);
-    if (e == cudaSuccess) e = stage_ghosts_and_bins(s, nl, flags, gate);
+    cudaError_t e = stage_sort_and_count(s, nl, pos, flags, gate, false);
+    if (e == cudaSuccess) e = stage_ghosts_and_bins(s, nl, flags, gate, false);
     if (e == cudaSuccess) e = stage_search(s, nl, flags, gate);
     return e;
 }
