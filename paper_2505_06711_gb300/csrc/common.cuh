@@ -482,15 +482,15 @@ inline int64_t tiles128_of(const reann_nlist* nl) {
 
 int set_error(reann_ctx* ctx, int code, const std::string& msg);
 
-// Kernel launches with two optional attributes.  Programmatic stream serialization
+// Kernel launches with optional attributes, in clusters of `cluster` blocks.  Programmatic stream serialization
 // (`pdl`): the kernel's blocks may become resident while the previous kernel drains
 // (every kernel of the library calls pdl_enter() before it touches memory that
 // another kernel writes; in a captured graph the attribute becomes a programmatic
 // edge).  `carve` >= 0: preferred share (percent) of the SM's 256 KB for shared memory.
 template <typename... P, typename... A>
-inline cudaError_t launch_with(bool pdl, int carve, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                               A... args) {
-    cudaLaunchAttribute at[2];
+inline cudaError_t launch_clusters(int cluster, bool pdl, int carve, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                                   cudaStream_t s, A... args) {
+    cudaLaunchAttribute at[3];
     unsigned na = 0;
     if (pdl) {
         at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -500,6 +500,12 @@ inline cudaError_t launch_with(bool pdl, int carve, void (*k)(P...), dim3 grid, 
         at[na].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
         at[na++].val.sharedMemCarveout = (unsigned)carve;
     }
+    if (cluster > 1) {
+        at[na].id = cudaLaunchAttributeClusterDimension;
+        at[na].val.clusterDim.x = (unsigned)cluster;
+        at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+        ++na;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -508,6 +514,11 @@ inline cudaError_t launch_with(bool pdl, int carve, void (*k)(P...), dim3 grid, 
     cfg.attrs = at;
     cfg.numAttrs = na;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_with(bool pdl, int carve, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               A... args) {
+    return launch_clusters(1, pdl, carve, k, grid, block, smem, s, args...);
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {

@@ -332,6 +332,54 @@ __device__ __forceinline__ void fail(int* flags, uint64_t* bar, bool copies_land
     if (!__syncthreads_and(drained) && threadIdx.x == 0) atomicOr(&flags[FLAG_TIMEOUT_DRAIN], 1);
 }
 
+// A tile's rows split over a cluster of `parts` blocks (SPLIT; 2 or 4): block p takes the row
+// quarters p nq .. (p + 1) nq - 1, and column sums are exchanged through distributed shared
+// memory, twice in the backward.  A block writes to its peers only after all have started
+// and before the barrier that ends the exchange, so none exits while another writes to
+// it; a block that gives up takes the remaining barriers (finish).
+template <bool SPLIT>
+struct Part {
+    int parts, p, nq;
+    __device__ explicit Part(int n) : parts(SPLIT ? n : 1), p(SPLIT ? (int)(blockIdx.x % n) : 0), nq(SPLIT ? 4 / n : 4) {}
+    __device__ int row0() const { return 32 * nq * p; }
+    __device__ int rows_of(const Tile& t) const { return SPLIT ? max(0, min(t.nrows - row0(), 32 * nq)) : t.nrows; }
+    __device__ static void arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+    __device__ static void wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+    __device__ static void begin() {
+        if (SPLIT) arrive();
+    }
+    __device__ static void started() {
+        if (SPLIT) wait();
+    }
+    // one value into the same place of every block's shared memory
+    __device__ void share(float* place, float x) const {
+        *place = x;
+        for (int peer = 0; SPLIT && peer < parts; ++peer) {
+            if (peer == p) continue;
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(place)), "r"(peer));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory");
+        }
+    }
+    __device__ static void sync() {
+        if (SPLIT) {
+            arrive();
+            wait();
+        } else {
+            __syncthreads();
+        }
+    }
+    // after `done` of the two exchanges
+    __device__ static void finish(int done) {
+        if (!SPLIT) return;
+        if (done == 0) wait();
+        for (; done < 2; ++done) {
+            arrive();
+            wait();
+        }
+    }
+};
+
 // One butterfly reduce-scatter stage over CNT values: lanes with bit CNT/2 set
 // keep the upper half, and each kept value adds its partner lane's.
 template <int CNT>
@@ -350,19 +398,24 @@ __device__ __forceinline__ void rs_stage(float* v, int lane) {
 // thread (rows past the tile's end must hold zeros).  In each warp the stages
 // 16, 8, 4, 2 leave lane l with column c0 + (l % 16) summed over its half-warp,
 // one more shuffle adds the other half; the 4 row quarters are then added in a
-// fixed order, so the result is deterministic.
-__device__ __forceinline__ void tile_mean64(const float* v, float* psum, float* mean, int q, int c0, int lane,
-                                            float inv_n) {
-    float t[16];
+// fixed order, so the result is deterministic and the same however many blocks the tile
+// is split over.  psum: one buffer per mean, since the cluster's blocks write to each other's.
+template <bool SPLIT>
+__device__ __forceinline__ void tile_mean64(const float* v, const Part<SPLIT>& part, int which, float* psum,
+                                            float* mean, int q, int c0, int lane, float inv_n) {
+    if (which == 0) part.started();
+    if (q < part.nq) {
+        float t[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) t[i] = v[i];
-    rs_stage<16>(t, lane);
-    rs_stage<8>(t, lane);
-    rs_stage<4>(t, lane);
-    rs_stage<2>(t, lane);
-    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 16);
-    if (lane < 16) psum[q * 64 + c0 + lane] = t[0];
-    __syncthreads();
+        for (int i = 0; i < 16; ++i) t[i] = v[i];
+        rs_stage<16>(t, lane);
+        rs_stage<8>(t, lane);
+        rs_stage<4>(t, lane);
+        rs_stage<2>(t, lane);
+        t[0] += __shfl_xor_sync(0xffffffffu, t[0], 16);
+        if (lane < 16) part.share(psum + (part.p * part.nq + q) * 64 + c0 + lane, t[0]);
+    }
+    part.sync();
     const int c = threadIdx.x;
     if (c < 64) mean[c] = ((psum[c] + psum[64 + c]) + (psum[128 + c] + psum[192 + c])) * inv_n;
     __syncthreads();
@@ -416,12 +469,11 @@ __device__ __forceinline__ void lds16(const float* p, float* v) {
 __device__ __forceinline__ size_t save_at(const Tile& tl, int r, int c) {
     return (size_t)tl.row0 * ((H1 + H2) / 4) + (size_t)(c * tl.nrows + r);
 }
-// blocks c .. c + 3 of row r, zeros for rows past the tile's end
-__device__ __forceinline__ void ld_save16(const float* dsave, const Tile& tl, int r, int c, float* v) {
+// blocks c .. c + 3 of row r, zeros when !ok
+__device__ __forceinline__ void ld_save16(const float* dsave, const Tile& tl, int r, bool ok, int c, float* v) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 x = r < tl.nrows ? __ldg(reinterpret_cast<const float4*>(dsave) + save_at(tl, r, c + k))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 x = ok ? __ldg(reinterpret_cast<const float4*>(dsave) + save_at(tl, r, c + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
         v[4 * k] = x.x, v[4 * k + 1] = x.y, v[4 * k + 2] = x.z, v[4 * k + 3] = x.w;
     }
 }
@@ -434,7 +486,7 @@ enum FwdPar {
 };
 enum BwdPar {
     B_W3 = 0, B_WC = 512, B_S2 = 896, B_S1 = 960, B_VB2 = 1024, B_U2 = 1088, B_VB1 = 1152, B_RA = 1216,
-    B_PS = 1280, B_RM = 1536, B_ZP = 2048, B_END = 2560
+    B_PS = 1280, B_PS2 = 1536, B_RM = 1792, B_ZP = 2304, B_END = 2816
 };
 
 constexpr uint32_t img_bytes(int P) { return P == P_FP8 ? 8192u : 14336u; }  // W1^T | W2^T  (bwd: W2 | W1)
@@ -539,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
                                                : make_float4(0.f, 0.f, 0.f, 0.f);
             v[4 * k] = x.x, v[4 * k + 1] = x.y, v[4 * k + 2] = x.z, v[4 * k + 3] = x.w;
         }
-        tile_mean64(v, par + F_PS, par + F_RB, q, c0, lane, inv_n);
+        tile_mean64(v, Part<false>(1), 0, par + F_PS, par + F_RB, q, c0, lane, inv_n);
         // A0 = rho - rho-bar: BF16 tiles have K = 48 (the fourth quarter writes nothing),
         // E4M3 tiles K = 64 (48 + zeros)
         float xb[16];
@@ -585,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_fwd(TcLayer nets, const Tile
         }
         WQ<H1> wq2;  // this thread's eighth of W2 for zhat2 = h1-bar W2 + b2
         wq_load<H1>(wq2, w.W2, H2, H2);
-        tile_mean64(v, par + F_PS, par + F_HB, q, c0, lane, inv_n);  // h1-bar
+        tile_mean64(v, Part<false>(1), 0, par + F_PS, par + F_HB, q, c0, lane, inv_n);  // h1-bar
         lds16(par + F_HB + c0, zb);
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = valid ? v[i] - zb[i] : 0.f;
@@ -733,9 +785,10 @@ __device__ __forceinline__ void bbar_three(const float* __restrict__ b, const fl
 // network), then the bbar step of Eq. 1's squares for the same rows,
 //   bbar_{a,m} = sum_k 2 w_a g_{a,k} rhobar_{l(a),k} W_{l,m,k},  g = b W (b: checkpoint bck),
 // written as the rows' adjoint records (bbar with the layer's c; ghost images too).
-template <int OUT, int P>
+template <int OUT, int P, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile* __restrict__ tiles,
-                                                       const float* __restrict__ dsave, const float* __restrict__ ybar,
+                                                       int parts, const float* __restrict__ dsave,
+                                                       const float* __restrict__ ybar,
                                                        const float* __restrict__ Wc, const float* __restrict__ bck,
                                                        const float* __restrict__ coef, float* __restrict__ rec,
                                                        GhostOut gh, int* __restrict__ flags) {
@@ -749,16 +802,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     uint8_t* sAlo = P == P_SPLIT ? smem + L::A + L::AB : nullptr;
     const uint8_t* sW = smem + L::W;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = warp & 3, cq = warp >> 2;
-    const int r = 32 * q + lane, c0 = 16 * cq;
-    const Tile tl = tiles[blockIdx.x];
+    const Part<SPLIT> part(parts);
+    const int r = 32 * q + lane, c0 = 16 * cq;  // r: the thread's row in the block
+    const Tile tl = tiles[SPLIT ? blockIdx.x / parts : blockIdx.x];
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list (before any TMEM allocation)
         pdl_enter();
         return;
     }
-    const bool valid = r < tl.nrows;
-    const int64_t row = tl.row0 + r;
+    const int rt = part.row0() + r, nrows = part.rows_of(tl);  // in the tile; the block's rows
+    const bool live = q < part.nq && 32 * q < nrows, valid = q < part.nq && r < nrows;  // live: some row of the warp is valid
+    const int64_t row = tl.row0 + rt;
     const float inv_n = 1.f / (float)tl.nrows;
     const TcImg& w = nets.e[tl.elem];
+    part.begin();
     const uint32_t tmem = setup(tslot, bar);
     if (tid == 0) {
         const uint8_t* img = P == P_FP8 ? w.wb8 : w.wb;
@@ -783,13 +839,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     for (int o = 0; o < OUT; ++o)  // d eps_i / d eps_i = 1 for the energy network
         yb[o] = OUT == 1 ? 1.f : (valid ? __ldg(ybar + (size_t)row * OUT + o) : 0.f);
     float sd[16], v[16], a[16];
-    ld_save16(dsave, tl, r, (H1 + c0) / 4, sd);  // SiLU'(z2) of this quarter row
+    ld_save16(dsave, tl, rt, valid, (H1 + c0) / 4, sd);  // SiLU'(z2) of this quarter row
     __syncthreads();
     // v2 = (ybar W3^T) * SiLU'(z2) in FP32
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         float u = 0.f;
-        if (OUT == 1) {
+        if (!live) {
+        } else if (OUT == 1) {
             u = yb[0] * par[B_W3 + (c0 + i) * 8];
         } else {
             const float4 wa = *reinterpret_cast<const float4*>(par + B_W3 + (c0 + i) * 8);
@@ -800,7 +857,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         }
         v[i] = valid ? u * sd[i] : 0.f;
     }
-    tile_mean64(v, par + B_PS, par + B_VB2, q, c0, lane, inv_n);
+    tile_mean64(v, part, 0, par + B_PS, par + B_VB2, q, c0, lane, inv_n);
+    int means = 1;
     wq_part<H2>(wq, par + B_VB2, par + B_ZP);  // u2-hat partials (summed after the next barrier)
     lds16(par + B_VB2 + c0, a);
 #pragma unroll
@@ -814,7 +872,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
             issue<P>(tmem, sA, sAlo, 64, sW, P == P_SPLIT ? sW + L::WB : nullptr, H1);
             mma_commit(&bar[1]);
         }
-        ld_save16(dsave, tl, r, c0 / 4, sd);  // SiLU'(z1), while the product runs
+        ld_save16(dsave, tl, rt, valid, c0 / 4, sd);  // SiLU'(z1), while the product runs
         // u2-hat = v2-bar W2^T: sum_q W2[u][q] v2-bar[q] = sum_q W2t[q][u] v2-bar[q]
         wq_sum(par + B_ZP, nullptr, par + B_U2, H1);
         ok = wait_all(&bar[1], 0);
@@ -822,18 +880,22 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     }
     if (ok) {
         tc_fence_after();
-        tmem_ld16(lane_addr(tmem, q, c0), a);
-        float ub[16], sc[16];
-        lds16(par + B_U2 + c0, ub);
-        if (P == P_FP8) lds16(par + B_S2 + c0, sc);
+        float ub[16];
+        if (live) {
+            float sc[16];
+            tmem_ld16(lane_addr(tmem, q, c0), a);
+            lds16(par + B_U2 + c0, ub);
+            if (P == P_FP8) lds16(par + B_S2 + c0, sc);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float u = (P == P_FP8 ? a[i] * (sa * sc[i]) : a[i]) + ub[i];
-            v[i] = valid ? u * sd[i] : 0.f;  // v1 = u2 * SiLU'(z1)
+            for (int i = 0; i < 16; ++i) {
+                const float u = (P == P_FP8 ? a[i] * (sa * sc[i]) : a[i]) + ub[i];
+                v[i] = valid ? u * sd[i] : 0.f;  // v1 = u2 * SiLU'(z1)
+            }
         }
         WQ<H1> wq1;  // this thread's eighth of W1^T for rhobar-hat = v1-bar W1^T
         wq_load<H1>(wq1, w.W1t, NFEAT, NFEAT);
-        tile_mean64(v, par + B_PS, par + B_VB1, q, c0, lane, inv_n);
+        tile_mean64(v, part, 1, par + B_PS2, par + B_VB1, q, c0, lane, inv_n);
+        ++means;
         wq_part<H1>(wq1, par + B_VB1, par + B_ZP);
         lds16(par + B_VB1 + c0, ub);
 #pragma unroll
@@ -852,7 +914,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
     if (ok) {
         tc_fence_after();
         // rhobar of the row, features [16 cq, 16 cq + 16) from the first three column quarters
-        if (cq < 3) {
+        if (cq < 3 && live) {
             tmem_ld16(lane_addr(tmem, q, 64 + c0), a);
             float ra[16], sc[16];
             lds16(par + B_RA + c0, ra);
@@ -879,8 +941,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
             }
         }
         __syncthreads();
-        flush_rec(sRec, tl.nrows, tl.row0, rec, gh, tid, kThreads);  // ghost images get the rows' records too
+        flush_rec(sRec, nrows, tl.row0 + part.row0(), rec, gh, tid, kThreads);  // ghost images get the rows' records too
     }
+    part.finish(means);
     teardown(tmem);
 }
 
@@ -905,7 +968,8 @@ TcLayer layer_of(const TcTable& t, int layer) {
 template <int OUT, int P>
 void set_attrs() {
     cudaFuncSetAttribute(k_tc_fwd<OUT, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdL<P>::BYTES);
-    cudaFuncSetAttribute(k_tc_bwd<OUT, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdL<P>::BYTES);
+    cudaFuncSetAttribute(k_tc_bwd<OUT, P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdL<P>::BYTES);
+    cudaFuncSetAttribute(k_tc_bwd<OUT, P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdL<P>::BYTES);
 }
 
 void ensure_tc_attrs() {
@@ -936,11 +1000,20 @@ void fwd_launch(cudaStream_t s, const EvalLaunch& how, int nt, const TcLayer& l,
                 flags, gh, dsave, epart);
 }
 
+// Blocks (a cluster) per tile in the backward.  A tile takes one block 14 us, mostly the rows' own
+// work at one block per SM, and a small system has few tiles.  us per evaluation with 1 / 2 / 4: 3
+// layers of BF16, 256 atoms (2 tiles) 106 / 97 / 93, 1,372 (11) 105 / 98 / 95, 4,800 (38) 138 / 130 /
+// 162, 6,600 (52) 149 / 144 / 155, 9,600 (76) 177 / 173 / 213; 5 of FP8, 4,000 (32) 190 / 179 / 176.  More
+// than about 128 blocks in clusters of four no longer find room at once.  (Splitting the forward the same
+// way gave 1 to 4 us up to 11 tiles and nothing at 32.)
+int bwd_parts(int64_t nt) { return nt <= 32 ? 4 : (nt <= 76 ? 2 : 1); }
+
 template <int OUT, int P>
 void bwd_launch(cudaStream_t s, const EvalLaunch& how, int nt, const TcLayer& l, const Tile* tiles, const float* dsave, const float* ybar,
                 const float* Wc, const float* bck, const float* coef, float* rec, GhostOut gh, int* flags) {
-    launch_with(how.chain, how.carve(), k_tc_bwd<OUT, P>, nt, kThreads, BwdL<P>::BYTES, s, l, tiles, dsave, ybar, Wc, bck,
-                coef, rec, gh, flags);
+    const int parts = bwd_parts(nt);
+    launch_clusters(parts, how.chain, how.carve(), parts > 1 ? k_tc_bwd<OUT, P, true> : k_tc_bwd<OUT, P, false>, nt * parts,
+                    kThreads, BwdL<P>::BYTES, s, l, tiles, parts, dsave, ybar, Wc, bck, coef, rec, gh, flags);
 }
 
 }  // namespace
