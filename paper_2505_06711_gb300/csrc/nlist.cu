@@ -672,9 +672,12 @@ __global__ void k_ghosts_ext(const int* __restrict__ gate, int64_t n, CellGeom g
 // columns that start among the 32 candidates are gathered as a bit mask (one
 // warp-wide OR); counting the mask's bits up to a candidate gives its column.
 // Candidates come in the same order as a bin-by-bin walk (x, then y, then z).
-// Bound by issue (70 % of the slots).  24,576 atoms: 34.1 -> 32.3 us, 1,048,576: 1,128 ->
-// 1,091 us, 192: 8.5 -> 7.9 us against a binary search by shuffles for the column,
-// integer divisions for the bins and one atomic per atom for the longest row.
+// Bound by latency and issue (57 % of the slots before the next batch's positions were
+// fetched ahead; 722 warp instructions per atom).  24,576 atoms: 34.1 -> 27.2 us, 1,048,576: 1,128 ->
+// 830 us against a binary search by shuffles for the column, integer divisions for
+// the bins, one atomic per atom for the longest row, the atom's FP64 position held
+// in registers (rarely needed, read there) and each batch fetched when its turn came.
+// Two batches ahead take 971 us, 128-thread blocks 853, five blocks per SM 910.
 __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate, int64_t n, CellGeom g,
                                                    const double* __restrict__ xw, const int32_t* __restrict__ owner,
                                                    const int32_t* __restrict__ shift, const float4* __restrict__ p32,
@@ -691,7 +694,6 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= n) return;
     const float4 pi = p32[i];
-    const double xi[3] = {xw[3 * i], xw[3 * i + 1], xw[3 * i + 2]};
     // the atom's own bin, as the extended keying computed it (its FP64 floor, evaluated by
     // every lane here, kept a third of GB300's narrow FP64 pipe busy)
     int b[3];
@@ -757,16 +759,22 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
         if (len > 0) s_base[__popc(filled & (upto >> 1))] = st - excl;  // of the non-empty columns, in order
         __syncwarp();
         int before = 0;  // non-empty columns that start before t0
-        for (int t0 = 0; t0 < total; t0 += 32) {
-            const int t = t0 + lane;
+        auto fetch = [&](int t0) {  // candidate t0 + lane
             const int rel = excl - t0;
             const unsigned starts = __reduce_or_sync(FULL, len > 0 && rel >= 0 && rel < 32 ? 1u << rel : 0u);
-            const int c = s_base[before + __popc(starts & upto) - 1] + t;
+            const int c = s_base[before + __popc(starts & upto) - 1] + t0 + lane;
             before += __popc(starts);
+            return t0 + lane < total ? p32s[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (total > 0) next = fetch(0);
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            const float4 pj = next;
+            if (t0 + 32 < total) next = fetch(t0 + 32);  // on its way while this batch is decided
             bool hit = false;
             int j = -1;
             if (t < total) {
-                const float4 pj = p32s[c];
                 j = __float_as_int(pj.w);
                 if (j != (int)i) {
                     const float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
@@ -785,7 +793,7 @@ __global__ void __launch_bounds__(256) k_nbr_search(const int* __restrict__ gate
                         shift_vec_mul(g, a0, a1, a2, sv);
                         double rr[3];
 #pragma unroll
-                        for (int k = 0; k < 3; ++k) rr[k] = dadd(dsub(xw[3 * o + k], xi[k]), sv[k]);
+                        for (int k = 0; k < 3; ++k) rr[k] = dadd(dsub(xw[3 * o + k], xw[3 * i + k]), sv[k]);
                         const double dd = dadd(dadd(dmul(rr[0], rr[0]), dmul(rr[1], rr[1])), dmul(rr[2], rr[2]));
                         hit = dd < g.rcut2;
                         if (dd < 1e-16) atomicOr(&flags[FLAG_GEOM], 2);
