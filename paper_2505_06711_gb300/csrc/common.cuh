@@ -611,7 +611,6 @@ int64_t virial_partials(int64_t n);  // launch_virial_sum's partial sums
 // with atom_virial: also the per-atom rows in caller order
 cudaError_t launch_virial_sum(cudaStream_t s, const reann_nlist* nl, const float* vir, double* partial, double* out,
                               float* atom_virial);
-cudaError_t launch_energy_sum(cudaStream_t s, const reann_nlist* nl, double* energy);
 cudaError_t launch_unpermute_rows(cudaStream_t s, const reann_nlist* nl, const float* src, int src_stride, float* dst,
                                   int width);
 

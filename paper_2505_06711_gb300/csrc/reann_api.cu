@@ -1002,16 +1002,9 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
             REANN_CUDA_TRY(ctx, launch_mlp_fwd_f32(s, nl, ctx->nets, t, energy_net, rho_t, out, out_stride, pairs, gh,
                                                   nl->dsave + (size_t)t * n * (H1 + H2), epart, ctx->d_flags));
     }
-    {
+    if (seg) {
         ProfScope p(ctx, PR_ENERGY);
-        if (seg)
-            REANN_CUDA_TRY(ctx, launch_segment_energy(s, seg, nseg, nl->eps, energy));
-        else  // the energy network summed its blocks (parts of 64-row FP32 tiles, or 128-row tensor-core tiles)
-            REANN_CUDA_TRY(ctx, launch_energy_final(s, nl->partial,
-                                                    (int)(ctx->precision == REANN_MLP_FP32
-                                                              ? tiles_of(nl) * mlp_parts_f32(nl)
-                                                              : tiles128_of(nl)),
-                                                    energy, eval_launch(nl).carve()));
+        REANN_CUDA_TRY(ctx, launch_segment_energy(s, seg, nseg, nl->eps, energy));
     }
     // reverse: Eqs. 3-5, one vector-Jacobian product per layer
     for (int t = T - 1; t >= 0; --t) {
@@ -1050,6 +1043,13 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
                 return REANN_OK;
             }))
             return rc;
+    }
+    if (!seg) {  // the energy network summed its blocks (parts of 64-row FP32 tiles, or 128-row tensor-core tiles)
+        ProfScope p(ctx, PR_ENERGY);
+        REANN_CUDA_TRY(ctx, launch_energy_final(s, nl->partial,
+                                                (int)(ctx->precision == REANN_MLP_FP32 ? tiles_of(nl) * mlp_parts_f32(nl)
+                                                                                       : tiles128_of(nl)),
+                                                energy, eval_launch(nl).carve()));
     }
     ProfScope p(ctx, PR_OUTPUT);
     if (vir) {
