@@ -8,12 +8,13 @@
 // gradients.
 //
 // Atoms are stored element-major, so a tile of 64 consecutive rows uses one
-// element's weights.  A block of 256 threads takes 16 RPT rows of a tile (RPT = 4:
-// the whole tile; RPT = 1: a quarter of it, so that the few tiles of a small system
-// occupy four times the SMs and each thread's chain is a quarter as long) and
-// computes a 64-wide layer output as 16 x 16 threads x (RPT rows x 4 columns),
+// element's weights.  A block of NT threads takes NT / 16 x RPT rows of a tile: the whole
+// tile (256 threads, RPT = 4), or, so that the few tiles of a small system occupy two or
+// four times the SMs and each thread's chain is shorter, half of it (256 threads, RPT = 2;
+// backward 128, RPT = 4) or a quarter (128 threads, RPT = 2), and
+// computes a 64-wide layer output as NT / 16 x 16 threads x (RPT rows x 4 columns),
 // reading float4 fragments of the row-major activations and weights from shared
-// memory.  A row's arithmetic is the same for every RPT.  The forward keeps one
+// memory.  A row's arithmetic is the same for every split.  The forward keeps one
 // activation buffer (48 KB of shared memory: four blocks per SM) and writes
 // SiLU'(z1), SiLU'(z2) of every row; the backward reads them instead of
 // recomputing the forward, and with the 48-feature networks also takes the
@@ -25,10 +26,11 @@
 // Before pdl_enter() the networks read only what no kernel of the stream writes after the
 // previous kernel began: the tile list and the weights, whose copies are then under way
 // while the previous kernel ends.
-//   Bound by issue: 7,680 FMAs per row forward and 10,240 with the bbar step
-// backward, beside a quarter as many instructions for SiLU and a fifth for the
-// shared-memory fragments (1,048,576 atoms: 436 and 744 us, about 70 % of the issue
-// slots; fma.rn.f32x2 was measured at 0.8 x the FMA rate of single fmas).
+//   Bound by L1, the float4 fragments (a 16 B load writes 512 B of registers per warp whatever it
+// broadcasts), and issue: 7,680 FMAs per row forward and 10,240 with the bbar step
+// backward, beside a quarter as many instructions for SiLU.  1,048,576 atoms: 451 us forward (L1
+// 80 %, issue 77 %) and 735 us backward (89 %, 58 %); fma.rn.f32x2 was measured at 0.8 x the FMA
+// rate of single fmas.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -39,24 +41,23 @@
 namespace reann {
 namespace {
 
-constexpr int kT = 256;      // threads per block
 constexpr int LDH = H1 + 4;  // 68
 static_assert(MLP_TILE == 64, "a block takes 16, 32 or 64 rows of a tile");
 // input rows of FIN features are held with stride FIN (one bulk copy of the
 // tile's contiguous rows) in the buffer that later holds h1 (stride LDH)
 template <int FIN>
 __host__ __device__ constexpr int ldx() { return FIN; }
-template <int FIN, int RPT>
-__host__ __device__ constexpr int abuf() { return 16 * RPT * (ldx<FIN>() > LDH ? ldx<FIN>() : LDH); }
+template <int FIN, int RPT, int NT>
+__host__ __device__ constexpr int abuf() { return NT / 16 * RPT * (ldx<FIN>() > LDH ? ldx<FIN>() : LDH); }
 
 // the 16 RPT rows of a tile that this block takes (nrows <= 0: none)
-template <int RPT>
+template <int RPT, int NT>
 __device__ __forceinline__ Tile block_rows(const Tile* __restrict__ tiles) {
-    constexpr int PARTS = 4 / RPT;
+    constexpr int PARTS = MLP_TILE / (NT / 16 * RPT);
     Tile t = tiles[blockIdx.x / PARTS];
-    const int skip = 16 * RPT * (int)(blockIdx.x % PARTS);
+    const int skip = NT / 16 * RPT * (int)(blockIdx.x % PARTS);
     t.row0 += skip;
-    t.nrows = min(t.nrows - skip, 16 * RPT);
+    t.nrows = min(t.nrows - skip, NT / 16 * RPT);
     return t;
 }
 
@@ -160,15 +161,15 @@ __device__ __forceinline__ int w3_row(int k) {
 }
 
 // The tile part's atomic energies (rows r, lanes with `own`) summed in FP64 in a
-// fixed order into *out; sE: 16 RPT doubles of shared memory.
-template <int RPT>
+// fixed order into *out; sE: ROWS doubles of shared memory.
+template <int ROWS>
 __device__ __forceinline__ void sum_energies(double* sE, int r, bool own, double e, double* out) {
     __syncthreads();  // every thread is done with the buffer
     if (own) sE[r] = e;
     __syncthreads();
     if (threadIdx.x < 32) {
         const int l = threadIdx.x;
-        double x = RPT == 4 ? sE[l] + sE[l + 32] : (RPT == 2 || l < 16 ? sE[l] : 0.0);
+        double x = ROWS == 64 ? sE[l] + sE[l + 32] : (ROWS == 32 || l < 16 ? sE[l] : 0.0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (l == 0) *out = x;
@@ -182,12 +183,12 @@ __device__ __forceinline__ void sum_energies(double* sE, int r, bool own, double
 // row's SiLU derivatives are kept for the reverse pass: dsave[row][0..63] =
 // SiLU'(z1), dsave[row][64..127] = SiLU'(z2).
 constexpr int kSave = H1 + H2;
-template <int OUT, int FIN, int RPT>
-__global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
+template <int OUT, int FIN, int RPT, int NT>
+__global__ void __launch_bounds__(NT) k_mlp_fwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
                                                const float* __restrict__ rho, float* __restrict__ out,
                                                int out_stride, GhostOut gh, float* __restrict__ dsave,
                                                double* __restrict__ epart, int* __restrict__ flags) {
-    constexpr int R = 16 * RPT;
+    constexpr int R = NT / 16 * RPT;
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
     float* sW1 = sm;                 // FIN x 64
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
     float* sb3 = sb2 + H2;           // 8
     float* sA = sb3 + 8;             // input rows (stride FIN), then h1 (stride LDH)
     const int tid = threadIdx.x;
-    const Tile tl = block_rows<RPT>(tiles);
+    const Tile tl = block_rows<RPT, NT>(tiles);
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
         pdl_enter();
         if (OUT == 1 && epart && tid == 0) epart[blockIdx.x] = 0.0;
@@ -213,11 +214,11 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
         bulk::bulk_g2s(sW1, w.W1, FIN * H1 * 4, &bar);
         bulk::bulk_g2s(sW2, w.W2, H1 * H2 * 4, &bar);
     }
-    for (int i = tid; i < H2 * OUT; i += kT) sW3[w3_row<OUT>(i / OUT) * OUT + i % OUT] = w.W3[i];
-    for (int i = tid; i < H1; i += kT) sb1[i] = w.b1[i];
-    for (int i = tid; i < H2; i += kT) sb2[i] = w.b2[i];
+    for (int i = tid; i < H2 * OUT; i += NT) sW3[w3_row<OUT>(i / OUT) * OUT + i % OUT] = w.W3[i];
+    for (int i = tid; i < H1; i += NT) sb1[i] = w.b1[i];
+    for (int i = tid; i < H2; i += NT) sb2[i] = w.b2[i];
     if (tid < OUT) sb3[tid] = w.b3[tid];
-    for (int i = tl.nrows * FIN + tid; i < R * FIN; i += kT) sA[i] = 0.f;  // rows past the end
+    for (int i = tl.nrows * FIN + tid; i < R * FIN; i += NT) sA[i] = 0.f;  // rows past the end
     pdl_enter();
     if (tid == 0) bulk::bulk_g2s(sA, rho + (size_t)tl.row0 * FIN, xb, &bar);
     if (!staged(&bar, flags)) return;
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(kT) k_mlp_fwd(NetsOfLayer nets, const Tile* __
         const float e = v[0] + sb3[0];
         if (own && r < tl.nrows) out[(size_t)(tl.row0 + r) * out_stride] = e;
         if (epart)
-            sum_energies<RPT>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
+            sum_energies<R>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
     } else if (own && r < tl.nrows) {
         const int64_t i = tl.row0 + r;
         float y[PER];
@@ -326,26 +327,27 @@ __device__ __forceinline__ void rhobar_rows(const float* sG, const float* sW1t, 
 }
 
 // contraction weights transposed per l: sWc[(l N_orb + k) N_phi + m] = W_{l,m,k}
+template <int NT>
 __device__ __forceinline__ void stage_wc(float* sWc, const float* __restrict__ Wt, int tid) {
-    for (int i = tid; i < (LMAX + 1) * NPHI * NORB; i += kT) {
+    for (int i = tid; i < (LMAX + 1) * NPHI * NORB; i += NT) {
         const int l = i / (NPHI * NORB), m = (i / NORB) % NPHI, k = i % NORB;
         sWc[(l * NORB + k) * NPHI + m] = Wt[i];
     }
 }
 
 // The bbar step of the block's rows, written as their adjoint records (bbar with the layer's c, ghost
-// images too) through sRec.  RPT = 4: four threads per row, up to three terms of one l each; fewer rows: 16 / RPT threads per row, one record value at a time.
-template <int RPT>
+// images too) through sRec.  Four threads per row, up to three terms of one l each, or eight, up to two.
+template <int RPT, int NT>
 __device__ __forceinline__ void bbar_records(const float* sR, const float* sWc, float* sRec, const Tile& tl,
                                              const float* __restrict__ bck, const float* __restrict__ coef,
                                              float* __restrict__ rec, const GhostOut& gh, int tid) {
-    constexpr int TPR = kT / (16 * RPT);
+    constexpr int TPR = 16 / RPT;
     const int r = tid / TPR, q = tid % TPR;
     if (r < tl.nrows) {
         const size_t row = (size_t)(tl.row0 + r);
         const float* rb = sR + r * LDH;
         const float* b = bck + row * NB;
-        if constexpr (RPT == 4) {
+        if constexpr (TPR == 4) {
             // q = 0: term 0 (and two that are not kept, in step with its neighbours), c and 0;
             // q = 1, 2, 3: terms 1-3, 4-6, 7-9
             const int l = q == 0 ? 0 : (q == 1 ? 1 : 2);
@@ -358,30 +360,29 @@ __device__ __forceinline__ void bbar_records(const float* sR, const float* sWc, 
                 stage_rec(sRec, r, NANG + 1, o);
             }
         } else {
-#pragma unroll 1
-            for (int v = q; v < NREC / NPHI; v += TPR) {
-                if (v >= NANG) {
-                    float o[NPHI];
-                    rec_tail(coef, row, v, o);
-                    stage_rec(sRec, r, v, o);
-                } else {
-                    const int l = ang_l(v);
-                    bbar_terms<1>(b, sWc + l * NORB * NPHI, rb + l * NORB, v, 1, sRec, r);
-                }
+            // q = 0: term 0 (and one that is not kept); 1, 2: terms 1 and 2, 3; 3, 4, 5: two terms each; 6, 7: c and 0
+            static_assert(TPR == 8, "four or eight threads per row");
+            if (q >= 6) {
+                float o[NPHI];
+                rec_tail(coef, row, NANG + q - 6, o);
+                stage_rec(sRec, r, NANG + q - 6, o);
+            } else {
+                const int l = q == 0 ? 0 : (q <= 2 ? 1 : 2), a0 = q == 0 ? 0 : (q <= 2 ? 2 * q - 1 : 2 * q - 2);
+                bbar_terms<2>(b, sWc + l * NORB * NPHI, rb + l * NORB, a0, q == 0 || q == 2 ? 1 : 2, sRec, r);
             }
         }
     }
     __syncthreads();
-    flush_rec(sRec, tl.nrows, tl.row0, rec, gh, tid, kT);  // ghost images get the rows' records too (reverse exchange)
+    flush_rec(sRec, tl.nrows, tl.row0, rec, gh, tid, NT);  // ghost images get the rows' records too (reverse exchange)
 }
 
-template <int OUT, int FIN, bool BBAR, int RPT>
-__global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
+template <int OUT, int FIN, bool BBAR, int RPT, int NT>
+__global__ void __launch_bounds__(NT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile* __restrict__ tiles,
                                                const float* __restrict__ dsave, const float* __restrict__ ybar,
                                                float* __restrict__ rhobar, const float* __restrict__ Wt,
                                                const float* __restrict__ bck, const float* __restrict__ coef,
                                                float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
-    constexpr int R = 16 * RPT;
+    constexpr int R = NT / 16 * RPT;
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
     float* sW1t = sm;                 // W1^T: 64 x FIN
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
     float* sR = sG + R * LDH;         // rhobar rows (BBAR, stride LDH)
     float* sWc = sR + R * LDH;        // (L+1) x N_orb x N_phi contraction W^t, transposed per l (BBAR)
     const int tid = threadIdx.x;
-    const Tile tl = block_rows<RPT>(tiles);
+    const Tile tl = block_rows<RPT, NT>(tiles);
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
         pdl_enter();
         return;
@@ -407,13 +408,13 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
         bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
         bulk::bulk_g2s(sW3t, w.W3t, OUT * H2 * 4, &bar);
     }
-    if (BBAR) stage_wc(sWc, Wt, tid);
+    if (BBAR) stage_wc<NT>(sWc, Wt, tid);
     pdl_enter();
     // the thread's SiLU'(z2), in flight while ybar and the weights arrive
     float4 s2[RPT];
 #pragma unroll
     for (int i = 0; i < RPT; ++i) s2[i] = ld_save(dsave, tl, RPT * ty + i, H1 + 4 * tx);
-    for (int i = tid; i < R * OUT; i += kT) {
+    for (int i = tid; i < R * OUT; i += NT) {
         const int r = i / OUT, o = i % OUT;
         sY[r * 8 + o] = (OUT == 1) ? 1.f : (r < tl.nrows ? ybar[(size_t)(tl.row0 + r) * OUT + o] : 0.f);
     }
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_bwd(NetsOfLayer nets, const Tile*
     if (!BBAR) return;
     __syncthreads();
     // records staged where W1^T, W2^T, no longer needed, were
-    bbar_records<RPT>(sR, sWc, sW1t, tl, bck, coef, rec, gh, tid);
+    bbar_records<RPT, NT>(sR, sWc, sW1t, tl, bck, coef, rec, gh, tid);
 }
 
 static_assert(NFEAT * H1 + H1 * H2 >= MLP_TILE * kRecLd, "record staging must fit in the W1, W2 region");
@@ -464,13 +465,13 @@ static_assert(NFEAT * H1 + H1 * H2 >= MLP_TILE * kRecLd, "record staging must fi
 // ybar = 1, so z2bar = W3 * SiLU'(z2) and nothing but rho is read.  Shared memory: W1,
 // W2 (later rhobar) and W1^T, W2^T (later the records), one activation buffer, the
 // contraction weights: 76 KB, three blocks per SM.
-template <int RPT>
-__global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Tile* __restrict__ tiles,
+template <int RPT, int NT>
+__global__ void __launch_bounds__(NT, 3) k_mlp_energy(NetsOfLayer nets, const Tile* __restrict__ tiles,
                                                       const float* __restrict__ rho, float* __restrict__ eps,
                                                       double* __restrict__ epart, const float* __restrict__ Wt,
                                                       const float* __restrict__ bck, const float* __restrict__ coef,
                                                       float* __restrict__ rec, GhostOut gh, int* __restrict__ flags) {
-    constexpr int R = 16 * RPT, F = NFEAT;
+    constexpr int R = NT / 16 * RPT, F = NFEAT;
     static_assert(F * H1 + H1 * H2 >= R * LDH, "rhobar rows must fit in the W1, W2 region");
     __shared__ __align__(8) uint64_t bar;
     extern __shared__ __align__(16) float sm[];
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
     float* sA = sW2t + H1 * H2;     // input rows (stride 48), then h1, z2bar, z1bar (stride LDH)
     float* sWc = sA + R * LDH;      // contraction weights, transposed per l
     const int tid = threadIdx.x;
-    const Tile tl = block_rows<RPT>(tiles);
+    const Tile tl = block_rows<RPT, NT>(tiles);
     if (tl.nrows <= 0) {  // padding entry of a fixed-size tile list, or nothing left of the tile
         pdl_enter();
         if (epart && tid == 0) epart[blockIdx.x] = 0.0;
@@ -498,8 +499,8 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
         bulk::bulk_g2s(sW1t, w.W1t, F * H1 * 4, &bar);
         bulk::bulk_g2s(sW2t, w.W2t, H1 * H2 * 4, &bar);
     }
-    stage_wc(sWc, Wt, tid);
-    for (int i = tl.nrows * F + tid; i < R * F; i += kT) sA[i] = 0.f;  // rows past the end
+    stage_wc<NT>(sWc, Wt, tid);
+    for (int i = tl.nrows * F + tid; i < R * F; i += NT) sA[i] = 0.f;  // rows past the end
     const int ty = tid >> 4, tx = tid & 15;
     const float4 b1 = __ldg(reinterpret_cast<const float4*>(w.b1) + tx), b2 = __ldg(reinterpret_cast<const float4*>(w.b2) + tx);
     const float4 w3 = __ldg(reinterpret_cast<const float4*>(w.W3) + tx);
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
     const float e = v[0] + b3;
     if (own && r < tl.nrows) eps[tl.row0 + r] = e;
     if (epart)
-        sum_energies<RPT>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
+        sum_energies<R>(reinterpret_cast<double*>(sA), r, own, r < tl.nrows ? (double)e : 0.0, epart + blockIdx.x);
     __syncthreads();  // h1 and the energies have been read
     put_rows<RPT>(sA, ty, tx, acc);
     __syncthreads();
@@ -556,35 +557,38 @@ __global__ void __launch_bounds__(kT, 3) k_mlp_energy(NetsOfLayer nets, const Ti
     __syncthreads();
     rhobar_rows<F, true, RPT>(sA, sW1t, sW1, nullptr, tl, ty, tx);
     __syncthreads();
-    bbar_records<RPT>(sW1, sWc, sW1t, tl, bck, coef, rec, gh, tid);
+    bbar_records<RPT, NT>(sW1, sWc, sW1t, tl, bck, coef, rec, gh, tid);
 }
 
-template <int FIN, int RPT>
-constexpr size_t fwd_smem() { return sizeof(float) * (FIN * H1 + H1 * H2 + H2 * 8 + H1 + H2 + 8 + abuf<FIN, RPT>()); }
-template <int FIN, bool BBAR, int RPT>
+template <int FIN, int RPT, int NT>
+constexpr size_t fwd_smem() { return sizeof(float) * (FIN * H1 + H1 * H2 + H2 * 8 + H1 + H2 + 8 + abuf<FIN, RPT, NT>()); }
+template <int FIN, bool BBAR, int RPT, int NT>
 constexpr size_t bwd_smem() {
-    return sizeof(float) * (H1 * FIN + H1 * H2 + 8 * H2 + 16 * RPT * 8 + 16 * RPT * LDH +
-                            (BBAR ? 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB : 0));
+    return sizeof(float) * (H1 * FIN + H1 * H2 + 8 * H2 + NT / 16 * RPT * 8 + NT / 16 * RPT * LDH +
+                            (BBAR ? NT / 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB : 0));
 }
-template <int RPT>
+template <int RPT, int NT>
 constexpr size_t energy_smem() {
-    return sizeof(float) * (2 * (NFEAT * H1 + H1 * H2) + 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB);
+    return sizeof(float) * (2 * (NFEAT * H1 + H1 * H2) + NT / 16 * RPT * LDH + (LMAX + 1) * NPHI * NORB);
 }
-static_assert(3 * (energy_smem<4>() + 16 + 1024) <= 228 * 1024, "three blocks of the energy network per SM");
+static_assert(3 * (energy_smem<4, 256>() + 16 + 1024) <= 228 * 1024, "three blocks of the energy network per SM");
 
 template <typename K>
 void allow_smem(K* k, size_t bytes) {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-template <int RPT>
-void set_attrs() {
-    allow_smem(k_mlp_fwd<NPHI, NFEAT, RPT>, fwd_smem<NFEAT, RPT>());
-    allow_smem(k_mlp_fwd<1, NFEAT_P, RPT>, fwd_smem<NFEAT_P, RPT>());
-    allow_smem(k_mlp_fwd<NPHI, NFEAT_P, RPT>, fwd_smem<NFEAT_P, RPT>());
-    allow_smem(k_mlp_bwd<NPHI, NFEAT, true, RPT>, bwd_smem<NFEAT, true, RPT>());
-    allow_smem(k_mlp_bwd<1, NFEAT_P, false, RPT>, bwd_smem<NFEAT_P, false, RPT>());
-    allow_smem(k_mlp_bwd<NPHI, NFEAT_P, false, RPT>, bwd_smem<NFEAT_P, false, RPT>());
-    allow_smem(k_mlp_energy<RPT>, energy_smem<RPT>());
+template <int RPT, int NT>
+void set_fwd_attrs() {
+    allow_smem(k_mlp_fwd<NPHI, NFEAT, RPT, NT>, fwd_smem<NFEAT, RPT, NT>());
+    allow_smem(k_mlp_fwd<1, NFEAT_P, RPT, NT>, fwd_smem<NFEAT_P, RPT, NT>());
+    allow_smem(k_mlp_fwd<NPHI, NFEAT_P, RPT, NT>, fwd_smem<NFEAT_P, RPT, NT>());
+    allow_smem(k_mlp_energy<RPT, NT>, energy_smem<RPT, NT>());
+}
+template <int RPT, int NT>
+void set_bwd_attrs() {
+    allow_smem(k_mlp_bwd<NPHI, NFEAT, true, RPT, NT>, bwd_smem<NFEAT, true, RPT, NT>());
+    allow_smem(k_mlp_bwd<1, NFEAT_P, false, RPT, NT>, bwd_smem<NFEAT_P, false, RPT, NT>());
+    allow_smem(k_mlp_bwd<NPHI, NFEAT_P, false, RPT, NT>, bwd_smem<NFEAT_P, false, RPT, NT>());
 }
 void ensure_attrs() {
     // once per device, safe under concurrent first calls
@@ -594,9 +598,12 @@ void ensure_attrs() {
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 64 && ((done >> dev) & 1)) return;
-    set_attrs<1>();
-    set_attrs<2>();
-    set_attrs<4>();
+    set_fwd_attrs<2, 128>();
+    set_fwd_attrs<2, 256>();
+    set_fwd_attrs<4, 256>();
+    set_bwd_attrs<2, 128>();
+    set_bwd_attrs<4, 128>();
+    set_bwd_attrs<4, 256>();
     if (dev < 64) done |= (uint64_t)1 << dev;
 }
 
@@ -609,9 +616,13 @@ NetsOfLayer layer_nets(const NetTable& t, int layer) {
 }  // namespace
 
 // Parts while they still fit the 152 SMs in one wave.  us per launch of the coefficient
-// network's forward / energy network / backward with 1, 2 and 4 parts: 4 tiles (192 atoms)
-// 8.7 / 18.5 / 13.5, 6.3 / 13.6 / 9.8, 5.4 / 10.4 / 7.5; 63 tiles 8.4 / 17.7 / 12.6, 6.3 / 13.6 / 9.9,
-// 7.8 / 15.8 / 11.4; 96 tiles 8.5 / 17.5 / 12.2, 9.3 / 19.8 / 14.5, 10.2 / 21.7 / 15.2.
+// network's forward / energy network / backward with 1, 2 and 4 parts of 256 threads: 4 tiles (192
+// atoms) 8.7 / 18.5 / 13.5, 6.3 / 13.6 / 9.8, 5.4 / 10.4 / 7.5; 63 tiles 8.4 / 17.7 / 12.6, 6.3 / 13.6 / 9.9,
+// 7.8 / 15.8 / 11.4; 96 tiles 8.5 / 17.5 / 12.2, 9.3 / 19.8 / 14.5, 10.2 / 21.7 / 15.2.  A part's time is that of its
+// shared-memory fragments, of which two rows per thread need 40 % less per row than one: quarters with 128
+// threads instead of 256 took an evaluation of 192 atoms from 70.7 to 66.8 us, of 1,536 from 77.7 to 74.4
+// (with 64 threads and four rows each 74.0 and 82.2); halves with 128 threads in the backward
+// one of 4,500 from 108.5 to 105.4 (in the forward networks 108.6).
 int mlp_parts_f32(const reann_nlist* nl) {
     const int64_t nt = tiles_of(nl);
     return nt <= 38 ? 4 : (nt <= 76 ? 2 : 1);
@@ -626,17 +637,17 @@ cudaError_t launch_mlp_fwd_f32(cudaStream_t s, const reann_nlist* nl, const NetT
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
     const EvalLaunch how = eval_launch(nl);
-#define REANN_FWD(O, F, RPT)                                                                                         \
-    launch_with(how.chain, how.carve(), k_mlp_fwd<O, F, RPT>, nt * (4 / RPT), kT, fwd_smem<F, RPT>(), s, ln, nl->tiles, \
+#define REANN_FWD(O, F, RPT, NT)                                                                                         \
+    launch_with(how.chain, how.carve(), k_mlp_fwd<O, F, RPT, NT>, nt * parts, NT, fwd_smem<F, RPT, NT>(), s, ln, nl->tiles, \
                 rho, out, out_stride, gh, dsave, epart, flags)
 #define REANN_FWD_R(O, F)        \
     do {                         \
         if (parts == 4)          \
-            REANN_FWD(O, F, 1);  \
+            REANN_FWD(O, F, 2, 128);  \
         else if (parts == 2)     \
-            REANN_FWD(O, F, 2);  \
+            REANN_FWD(O, F, 2, 256);  \
         else                     \
-            REANN_FWD(O, F, 4);  \
+            REANN_FWD(O, F, 4, 256);  \
     } while (0)
     if (!pairs)
         REANN_FWD_R(NPHI, NFEAT);
@@ -658,18 +669,18 @@ cudaError_t launch_mlp_bwd_f32(cudaStream_t s, const reann_nlist* nl, const NetT
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
     const EvalLaunch how = eval_launch(nl);
-#define REANN_BWD(O, F, B, RPT)                                                                                    \
-    launch_with(how.chain, how.carve(), k_mlp_bwd<O, F, B, RPT>, nt * (4 / RPT), kT, bwd_smem<F, B, RPT>(), s, ln,  \
+#define REANN_BWD(O, F, B, RPT, NT)                                                                                    \
+    launch_with(how.chain, how.carve(), k_mlp_bwd<O, F, B, RPT, NT>, nt * parts, NT, bwd_smem<F, B, RPT, NT>(), s, ln,  \
                 nl->tiles, dsave, ybar, rhobar, B ? Wt : nullptr, B ? bck : nullptr, B ? coef : nullptr,           \
                 B ? rec : nullptr, B ? gh : GhostOut{}, flags)
 #define REANN_BWD_R(O, F, B)        \
     do {                            \
         if (parts == 4)             \
-            REANN_BWD(O, F, B, 1);  \
+            REANN_BWD(O, F, B, 2, 128);  \
         else if (parts == 2)        \
-            REANN_BWD(O, F, B, 2);  \
+            REANN_BWD(O, F, B, 4, 128);  \
         else                        \
-            REANN_BWD(O, F, B, 4);  \
+            REANN_BWD(O, F, B, 4, 256);  \
     } while (0)
     if (!pairs)
         REANN_BWD_R(NPHI, NFEAT, true);
@@ -690,15 +701,15 @@ cudaError_t launch_mlp_energy_f32(cudaStream_t s, const reann_nlist* nl, const N
     ensure_attrs();
     const NetsOfLayer ln = layer_nets(nets, t);
     const EvalLaunch how = eval_launch(nl);
-#define REANN_EN(RPT)                                                                                              \
-    launch_with(how.chain, how.carve(), k_mlp_energy<RPT>, nt * (4 / RPT), kT, energy_smem<RPT>(), s, ln, nl->tiles, \
+#define REANN_EN(RPT, NT)                                                                                            \
+    launch_with(how.chain, how.carve(), k_mlp_energy<RPT, NT>, nt * parts, NT, energy_smem<RPT, NT>(), s, ln, nl->tiles, \
                 rho, eps, epart, Wt, bck, coef, rec, gh, flags)
     if (parts == 4)
-        REANN_EN(1);
+        REANN_EN(2, 128);
     else if (parts == 2)
-        REANN_EN(2);
+        REANN_EN(2, 256);
     else
-        REANN_EN(4);
+        REANN_EN(4, 256);
 #undef REANN_EN
     return cudaGetLastError();
 }
