@@ -452,7 +452,7 @@ struct reann_ctx {
     void* d_fp8 = nullptr;         // FP8 E4M3 weight images for the tensor-core networks
     reann::TcTable tc{};
     int* d_flags = nullptr;        // reann::NFLAGS ints
-    int* h_flags = nullptr;        // pinned mirror, then kHostInts ints for the build's sizes
+    int* h_flags = nullptr;        // pinned mirror, then kHostInts ints: the build's sizes, or an energy
     static constexpr int kHostInts = reann::MAX_ELEM + 2;
     std::shared_ptr<reann::ListPool> list_pool;  // created by the first build
     std::string err;
@@ -555,6 +555,8 @@ inline EvalLaunch eval_launch(const reann_nlist* nl) { return EvalLaunch{rows_of
 // ---- launchers (defined in the .cu files) ----
 // neighbour list (nlist.cu)
 int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const int32_t* species);
+// flags (and energy, nullable) into pinned host memory, the flags zeroed
+cudaError_t launch_take_flags(cudaStream_t s, int* flags, const double* energy, int* host);
 cudaError_t launch_rebuild(cudaStream_t s, reann_nlist* nl, const double* pos, int* flags, const int* gate);
 cudaError_t launch_moved(cudaStream_t s, const reann_nlist* nl, const double* pos, int* moved);
 

@@ -906,6 +906,17 @@ __global__ void k_read_sizes(int n_elem, int64_t nbins, const int32_t* __restric
     if (t == 0) host[NFLAGS + MAX_ELEM + 1] = *ghosts;
 }
 
+// the flags into pinned host memory, zeroed for the next calls; with energy (nullable) it follows them
+__global__ void k_take_flags(int* __restrict__ flags, const double* __restrict__ energy, int* host) {
+    pdl_enter();
+    const int t = threadIdx.x;
+    if (t < NFLAGS) {
+        host[t] = flags[t];
+        flags[t] = 0;
+    }
+    if (t == 0 && energy) *reinterpret_cast<double*>(host + NFLAGS) = *energy;
+}
+
 }  // namespace
 
 // Counting sort of n entries (the ghost slots among them in use up to *g_count, null: all;
@@ -1121,6 +1132,14 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
         stride = ((ctx->h_flags[FLAG_MAXNBR] + ctx->h_flags[FLAG_MAXNBR] / 8 + 16 + 7) / 8) * 8;
     }
     return REANN_OK;
+}
+
+// one launch for what were a copy of the flags, their reset and a copy of the energy (host callback
+// of 24,576 atoms 414.7 -> 411.3 us)
+cudaError_t launch_take_flags(cudaStream_t s, int* flags, const double* energy, int* host) {
+    static_assert(NFLAGS % 2 == 0 && reann_ctx::kHostInts >= 2, "the energy follows the flags, 8 B aligned");
+    launch_pdl(k_take_flags, 1, 32, 0, s, flags, energy, host);
+    return cudaGetLastError();
 }
 
 // gate == nullptr: always rebuild; otherwise every kernel returns at once unless *gate != 0

@@ -540,10 +540,8 @@ extern "C" const char* reann_last_error(const reann_ctx* ctx) { return ctx ? ctx
 namespace {
 
 // enqueue the read-back of the device flags and their reset on the context stream
-int enqueue_flags_readback(reann_ctx* ctx) {
-    REANN_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(int) * NFLAGS, cudaMemcpyDeviceToHost,
-                                        ctx->stream));
-    REANN_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_flags, 0, sizeof(int) * NFLAGS, ctx->stream));
+int enqueue_flags_readback(reann_ctx* ctx, const double* energy = nullptr) {
+    REANN_CUDA_TRY(ctx, launch_take_flags(ctx->stream, ctx->d_flags, energy, ctx->h_flags));
     return REANN_OK;
 }
 
@@ -1211,9 +1209,9 @@ extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const d
     int rc = graphed_eval(ctx, nl, nl->h2d_pos, T, nl->d_energy, nl->d_forces, nullptr, nullptr, nullptr, GS_HOST_EVAL);
     if (rc) return rc;
     REANN_CUDA_TRY(ctx, cudaMemcpyAsync(forces, nl->d_forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
-    REANN_CUDA_TRY(ctx, cudaMemcpyAsync(energy, nl->d_energy, sizeof(double), cudaMemcpyDeviceToHost, s));
-    if (int rc2 = enqueue_flags_readback(ctx)) return rc2;  // the flags come back with the results:
-    REANN_CUDA_TRY(ctx, cudaStreamSynchronize(s));           // one synchronisation per call
+    if (int rc2 = enqueue_flags_readback(ctx, nl->d_energy)) return rc2;  // energy and flags come back with the forces:
+    REANN_CUDA_TRY(ctx, cudaStreamSynchronize(s));                         // one synchronisation per call
+    std::memcpy(energy, ctx->h_flags + NFLAGS, sizeof(double));
     return flags_status(ctx);
 }
 
