@@ -414,8 +414,7 @@ struct reann_nlist {
     reann::MdOut* md_out = nullptr;  // the current call's output arrays
     bool md_forces_valid = false;
     const double* md_forces_at = nullptr;  // positions the forces belong to
-    cudaGraph_t md_graph = nullptr;
-    cudaGraphExec_t md_exec = nullptr;
+    cudaGraphExec_t md_exec = nullptr, md_exec_many = nullptr;  // one MD step; several in a longer run
     reann::GraphSlot graphs[reann::GS_COUNT];  // rebuild / evaluation calls replayed as graphs
     const void* md_key[3] = {nullptr, nullptr, nullptr};  // pos, vel, mass of the captured step
     double md_dt = 0.0;

@@ -211,3 +211,26 @@ def test_calls_with_other_output_arrays_continue_one_trajectory():
         assert np.allclose(one[0], many[0], rtol=0, atol=1e-9) and np.allclose(one[1], many[1], rtol=0, atol=1e-9)
         rec = ~np.isnan(many[2])
         assert rec.any() and np.allclose(one[2][rec], many[2][rec], rtol=1e-9, atol=1e-9)
+
+
+def test_steps_captured_together_are_the_same_steps():
+    """Calls that replay graphs of four steps and of one (4, 9 = 2 x 4 + 1, 3, 8) against calls of three, which never do."""
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    s = water_box(43, seed=9)
+    pot = Potential(make_model(T=2))
+    got = []
+    for blocks in ((1, 4, 9, 3, 8, 2), (3,) * 9):
+        sy = pot.system(s.pos, s.species, s.cell)
+        mass = torch.as_tensor(MASS_AMU[s.species], device="cuda")
+        vel = torch.as_tensor(maxwell_boltzmann(MASS_AMU[s.species], 300.0, seed=2), device="cuda").contiguous()
+        e = [torch.stack(sy.md(vel, mass, 0.5, n)) for n in blocks]
+        sy.check()
+        torch.cuda.synchronize()
+        got.append((sy.pos.cpu().numpy().copy(), vel.cpu().numpy().copy(), torch.cat(e, 1).cpu().numpy()))
+        sy.close()
+    pot.close()
+    for one, many in zip(*got):
+        assert one.shape == many.shape and np.allclose(one, many, rtol=1e-9, atol=1e-9)
