@@ -106,36 +106,6 @@ __device__ __forceinline__ void flush_rec(const float* __restrict__ sRec, int nr
     }
 }
 
-// The bbar step of one angular term a of one atom (Eq. 1's squares):
-//   bbar_{a,m} = sum_k W_{l,m,k} gbar_{a,k},  gbar_{a,k} = 2 w_a rhobar_{l,k} sum_m' b_{a,m'} W_{l,m',k}
-// bm = b_{a,0..7}, Wl = W_{l} (N_phi x N_orb, row-major, 16 B aligned), rb = rhobar_{l,0..15}
-// (16 B aligned); blocked over 4 orbitals (W fragments are float4 loads, read again
-// for the second product rather than held in registers).
-__device__ __forceinline__ void bbar_term(const float bm[NPHI], float two_w, const float* Wl, const float* rb,
-                                          float out[NPHI]) {
-#pragma unroll
-    for (int m = 0; m < NPHI; ++m) out[m] = 0.f;
-#pragma unroll
-    for (int k4 = 0; k4 < NORB; k4 += 4) {
-        float g[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int m = 0; m < NPHI; ++m) {
-            const float4 w = *reinterpret_cast<const float4*>(Wl + m * NORB + k4);
-            g[0] = fmaf(bm[m], w.x, g[0]);
-            g[1] = fmaf(bm[m], w.y, g[1]);
-            g[2] = fmaf(bm[m], w.z, g[2]);
-            g[3] = fmaf(bm[m], w.w, g[3]);
-        }
-        const float4 r = *reinterpret_cast<const float4*>(rb + k4);
-        const float gb[4] = {two_w * g[0] * r.x, two_w * g[1] * r.y, two_w * g[2] * r.z, two_w * g[3] * r.w};
-#pragma unroll
-        for (int m = 0; m < NPHI; ++m) {
-            const float4 w = *reinterpret_cast<const float4*>(Wl + m * NORB + k4);
-            out[m] = fmaf(gb[0], w.x, fmaf(gb[1], w.y, fmaf(gb[2], w.z, fmaf(gb[3], w.w, out[m]))));
-        }
-    }
-}
-
 // The bbar step of N angular terms a0 .. a0 + N - 1 of one l: bbar_{a,m} = sum_k 2 w_a g_{a,k}
 // rhobar_{l,k} W_{l,m,k}, g = b W from the b checkpoint row b.  The terms share each weight fragment
 // wl[k] (N_phi floats) and rhobar value rb[k] read from shared memory.  Only the first `keep` are staged.
@@ -600,7 +570,7 @@ cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r,
 cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
                                const float* W, const float* coef, float* rho, float* bck, bool pairs = false);
 cudaError_t launch_bbar(cudaStream_t s, const reann_nlist* nl, const float* W, const float* bck, const float* rhobar,
-                        const float* coef, float* rec, bool pairs = false, GhostOut gh = {});
+                        const float* coef, float* rec, GhostOut gh);
 // forces / atom_energy (caller order): the last reverse layer writes the outputs itself;
 // first: the first reverse layer writes grad (and vir) instead of accumulating
 cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,

@@ -398,42 +398,48 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
 }
 
 // -------------------------------------------------------------- bbar -----
-// bbar_{a,m} = sum_k gbar_{a,k} W_{l(a),m,k}, g recomputed from the b checkpoint, with
-//   squares:  gbar_{a,k} = 2 w_a g_{a,k} rhobar_{l,k}
-//   pairs:    gbar_{a,k} = w_a sum_k' R_{kk'} g_{a,k'},  R_{kk'} = rhobar_{l,(min,max)} (x 2 on the diagonal)
+// bbar_{a,m} = sum_k gbar_{a,k} W_{l(a),m,k}, g recomputed from the b checkpoint, for the orbital-pair
+// features (Eq. 1's squares are taken by the backward networks):
+//   gbar_{a,k} = w_a sum_k' R_{kk'} g_{a,k'},  R_{kk'} = rhobar_{l,(min,max)} (x 2 on the diagonal)
 // written into the atom's adjoint record with the layer's c (values 10, 11 of
-// the record); 4 threads per atom take values q, q + 4, q + 8.  The block's
+// the record).  TPA = 12 threads per atom take a value each, 4 take values q, q + 4, q + 8: a chain
+// a third as long against fewer registers.  us per launch with 12 / 4: 192 atoms 6.2 / 8.8, 3,069 8.3 /
+// 11.7, 10,976 21.7 / 22.2, 16,200 24.7 / 22.9, 256,000 181 / 130.  The block's
 // kBbarAtoms records are staged in shared memory and stored as whole lines.
 constexpr int kBbarAtoms = 16;  // small blocks (64 threads): 4x finer balancing than 64 atoms, ~1.5 % per BF16 step
-template <bool PAIRS>
-__global__ void __launch_bounds__(4 * kBbarAtoms) k_bbar(int64_t n, const float* __restrict__ Wt, const float* __restrict__ bck,
-                                              const float* __restrict__ rhobar, const float* __restrict__ coef,
-                                              float* __restrict__ rec, GhostOut gh) {
-    pdl_enter();
-    constexpr int KO = PAIRS ? NORB_P : NORB;
+template <int TPA>
+__global__ void __launch_bounds__(TPA * kBbarAtoms) k_bbar(int64_t n, const float* __restrict__ Wt,
+                                                                const float* __restrict__ bck,
+                                                                const float* __restrict__ rhobar,
+                                                                const float* __restrict__ coef,
+                                                                float* __restrict__ rec, GhostOut gh) {
+    constexpr int KO = NORB_P, KP = NORB_P * (NORB_P + 1) / 2;
     __shared__ __align__(16) float sW[(LMAX + 1) * NPHI * KO];
     __shared__ __align__(16) float sRec[kBbarAtoms * kRecLd];
     for (int i = threadIdx.x; i < (LMAX + 1) * NPHI * KO; i += blockDim.x) sW[i] = Wt[i];
+    pdl_enter();  // so far only the weights were read
     __syncthreads();
     const int64_t atom0 = (int64_t)blockIdx.x * kBbarAtoms;
-    const int r = threadIdx.x >> 2, q = threadIdx.x & 3;
+    const int r = threadIdx.x / TPA;
     const int64_t atom = atom0 + r;
     const int nrows = n - atom0 < kBbarAtoms ? (int)(n - atom0) : kBbarAtoms;
 #pragma unroll 1
-    for (int v = q; v < NREC / NPHI && r < nrows; v += 4) {
+    for (int v = threadIdx.x % TPA; v < NREC / NPHI && r < nrows; v += TPA) {
         float out[NPHI];
         if (v >= NANG) {
             rec_tail(coef, atom, v, out);
-            stage_rec(sRec, r, v, out);
-            continue;
-        }
-        const int a = v, l = ang_l(a);
-        const float4 b0 = ldg4(bck + (size_t)atom * NB + a * NPHI), b1 = ldg4(bck + (size_t)atom * NB + a * NPHI + 4);
-        const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        } else {
+            const int a = v, l = ang_l(a);
+            const float4 b0 = ldg4(bck + (size_t)atom * NB + a * NPHI), b1 = ldg4(bck + (size_t)atom * NB + a * NPHI + 4);
+            const float* rb = rhobar + (size_t)atom * NFEAT_P + l * KP;
+            float pre[KP];  // few atoms: all in flight at once (many: the registers cost more warps)
+            if (TPA == 12)
 #pragma unroll
-        for (int m = 0; m < NPHI; ++m) out[m] = 0.f;
-        if constexpr (PAIRS) {
-            constexpr int KP = NORB_P * (NORB_P + 1) / 2;
+                for (int p = 0; p < KP / 4; ++p) {
+                    const float4 x = ldg4(rb + 4 * p);
+                    pre[4 * p] = x.x, pre[4 * p + 1] = x.y, pre[4 * p + 2] = x.z, pre[4 * p + 3] = x.w;
+                }
+            const float bm[NPHI] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
             float g[NORB_P], gb[NORB_P];
 #pragma unroll
             for (int k = 0; k < NORB_P; ++k) {
@@ -442,23 +448,22 @@ __global__ void __launch_bounds__(4 * kBbarAtoms) k_bbar(int64_t n, const float*
 #pragma unroll
                 for (int m = 0; m < NPHI; ++m) g[k] = fmaf(bm[m], sW[(l * NPHI + m) * KO + k], g[k]);
             }
-            const float* rb = rhobar + (size_t)atom * NFEAT_P + l * KP;
             int p = 0;
 #pragma unroll
             for (int k = 0; k < NORB_P; ++k)
 #pragma unroll
                 for (int k2 = k; k2 < NORB_P; ++k2, ++p) {
-                    const float rv = __ldg(rb + p);
+                    const float rv = TPA == 12 ? pre[p] : __ldg(rb + p);
                     gb[k] = fmaf(rv, g[k2], gb[k]);
                     gb[k2] = fmaf(rv, g[k], gb[k2]);
                 }
             const float wa = rec_scale(a) * ang_w(a);
 #pragma unroll
-            for (int m = 0; m < NPHI; ++m)
+            for (int m = 0; m < NPHI; ++m) {
+                out[m] = 0.f;
 #pragma unroll
                 for (int k = 0; k < NORB_P; ++k) out[m] = fmaf(wa * gb[k], sW[(l * NPHI + m) * KO + k], out[m]);
-        } else {
-            bbar_term(bm, 2.f * rec_scale(a) * ang_w(a), sW + l * NPHI * NORB, rhobar + (size_t)atom * NFEAT + l * NORB, out);
+            }
         }
         stage_rec(sRec, r, v, out);
     }
@@ -883,13 +888,12 @@ cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radi
 }
 
 cudaError_t launch_bbar(cudaStream_t s, const reann_nlist* nl, const float* W, const float* bck, const float* rhobar,
-                        const float* coef, float* rec, bool pairs, GhostOut gh) {
+                        const float* coef, float* rec, GhostOut gh) {
     const int64_t nr = rows_of(nl);
     if (nr == 0) return cudaSuccess;
-    if (pairs)
-        launch_with(true, eval_launch(nl).carve(), k_bbar<true>, blocks_for(nr, kBbarAtoms), 4 * kBbarAtoms, 0, s, nr, W, bck, rhobar, coef, rec, gh);
-    else
-        launch_pdl(k_bbar<false>, blocks_for(nr, kBbarAtoms), 4 * kBbarAtoms, 0, s, nr, W, bck, rhobar, coef, rec, gh);
+    const int tpa = nr <= kChainRows ? 12 : 4;
+    launch_with(true, eval_launch(nl).carve(), tpa == 12 ? k_bbar<12> : k_bbar<4>, blocks_for(nr, kBbarAtoms), tpa * kBbarAtoms, 0,
+                s, nr, W, bck, rhobar, coef, rec, gh);
     return cudaGetLastError();
 }
 

@@ -1032,7 +1032,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
         }
         if (pairs) {
             ProfScope p(ctx, PR_BBAR);
-            REANN_CUDA_TRY(ctx, launch_bbar(s, nl, ctx->d_W + t * lw, bck_t, nl->rhobar, coef_t, nl->bbar, pairs, gh));
+            REANN_CUDA_TRY(ctx, launch_bbar(s, nl, ctx->d_W + t * lw, bck_t, nl->rhobar, coef_t, nl->bbar, gh));
         }
         if (!gh.goff) {
             ProfScope p(ctx, PR_GATHER);  // ghost slots receive their owners' adjoints (vector-Jacobian product)

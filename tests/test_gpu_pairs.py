@@ -76,3 +76,11 @@ def test_pair_features_decomposed_virial_and_precision_guard():
             pot.set_precision(binding.REANN_MLP_BF16)  # tensor-core networks: 48 features only
     finally:
         pot.close()
+
+
+@pytest.mark.parametrize("n", [5, 6, 2048, 2049])
+def test_pair_adjoint_thread_layouts(n):
+    # 3 n atoms: a partly filled block of 16, and both sides of the 6,144 rows where 12 threads per atom become 4
+    s = water_box(n, seed=n)
+    spec = make_model(T=2, pairs=True)
+    assert_parity(gpu_eval(spec, s), oracle.energy_forces(spec, s.pos, s.species, s.cell), s.n_atoms)
