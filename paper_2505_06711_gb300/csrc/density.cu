@@ -259,12 +259,12 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
                                                             const float* __restrict__ coef,
                                                             const float* __restrict__ Wt, float* __restrict__ rho,
                                                             float* __restrict__ bck, bool far) {
-    pdl_enter();
     constexpr int KO = PAIRS ? NORB_P : NORB, APW = 32 / LPA;
     static_assert(LPA == 4 || LPA == 8 || LPA == 16, "80 sums split evenly");
     __shared__ __align__(16) float sW[(LMAX + 1) * NPHI * KO];
     __shared__ __align__(16) float sB[kFwdWarps * APW][kBStride];
     for (int i = threadIdx.x; i < (LMAX + 1) * NPHI * KO; i += blockDim.x) sW[i] = Wt[i];
+    pdl_enter();  // so far only the weights were read
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & (LPA - 1), slot = lane / LPA;
     const int64_t kr = ((int64_t)blockIdx.x * kFwdWarps + warp) * APW + slot;
