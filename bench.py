@@ -80,10 +80,10 @@ BYTES_PER_ATOM_EDGE_FIXED = {"density_fwd": 16 + 32 + 320 + 192, "density_adj": 
 # kernel, from one ncu capture of this workload; valid only for the kernel
 # source they were taken on (keyed by its hash), null otherwise.
 TRAFFIC = {  # {(region, source_sha of the kernel source): bytes per launch}
-    ("density_adj", "6e0a443d3c37"): 65194240,  # mean of the three launches of one step
+    ("density_adj", "bd83f08f9138"): 65194240,  # mean of the three launches of one step
 }
 L2_FRAC = {  # {(region, source_sha): lts__t_sectors throughput as a fraction of peak}
-    ("density_adj", "6e0a443d3c37"): 0.347,
+    ("density_adj", "bd83f08f9138"): 0.347,
 }
 
 
