@@ -349,8 +349,10 @@ int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const double* pos,
  *                       capacity divided by 1, 2, 4, ... 128, at least 2,048
  *                       rows), so its cost follows the work, not the pool's
  *                       size.  Every class is captured as a CUDA graph on the
- *                       first launch (per precision and output pointers; that
- *                       launch itself runs directly) and replayed afterwards;
+ *                       first launch (per precision and output pointers, and
+ *                       again for the first structure of more than 16,384
+ *                       atoms; that launch itself runs directly) and replayed
+ *                       afterwards;
  *                       submissions take the lowest free ranges, which keeps
  *                       the classes small.  Asynchronous: the
  *                       context stream waits for it.  A slot is evaluated

@@ -21,9 +21,9 @@
 // derivative (32 B per live edge, in the row order of the list).  The passes
 // stream the records of their atom (coalesced) and gather only what belongs to
 // the neighbour: its coefficients (forward) or its adjoint record (reverse).
-// Both passes give one warp to a centre atom: its lanes first expand 32 edges'
-// records, one edge per lane, into shared memory, then the four groups of 8
-// lanes (lane m of a group: radial channel m) take every fourth edge.
+// Both passes give 4 to 32 lanes to a centre atom, more where there are few atoms.
+// The order in which an atom's edges are summed does not depend on that choice nor
+// on how many rows a launch has (see the passes).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -221,14 +221,20 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
 }
 
 // ------------------------------------------------------------- forward ---
-// LPA lanes per centre atom (32 / LPA atoms per warp).  Lane q walks the edges
-// q, q + LPA, ... of its atom and accumulates the 80 products t_m A_a,
-// t_m = c_{j,m} phi_m, in registers; the record two edges ahead and the
-// coefficients one edge ahead are in flight meanwhile.  A butterfly
-// reduce-scatter over the LPA lanes leaves 80 / LPA of the sums in each lane
+// LPA lanes per centre atom (32 / LPA atoms per warp).  A row's edges fall into four
+// classes, e mod 4; a class's 80 sums of t_m A_a, t_m = c_{j,m} phi_m, are taken edge after
+// edge, and the classes' are added as (0 + 2) + (1 + 3): the result does not depend on LPA,
+// so that a structure's is the same alone and among others, whose number decides it.
+//   LPA = 4: lane q walks class q and keeps its 80 sums in registers; the record two
+// edges ahead and the coefficients one edge ahead are in flight meanwhile.
+//   LPA = 8, 16: lane (h, q) keeps the 80 / (LPA / 4) sums of channels CH h .. CH h + CH - 1 of
+// class q.  Per batch of LPA edges each lane first forms one edge's t_m into shared memory;
+// the records and coefficients of two or four batches are gathered together (192 atoms, 16 lanes: 6.8 us
+// with one batch's, 6.0 with four).
+// A butterfly reduce-scatter over the four classes leaves 80 / LPA of the sums in each lane
 // (stored as the b checkpoint), and lane q contracts its 16 / LPA orbitals.
 // Bound by the latency of the record stream and the coefficient gathers at 16
-// warps per SM (126 registers, 80 of them sums; issue slots 55 % busy).  Reading
+// warps per SM (LPA = 4: 126 registers, 80 of them sums; issue slots 55 % busy).  Reading
 // records instead of recomputing the edge's geometry took a launch from 29.7 to
 // 19.9 us (24,576 atoms) and from 692 to 541 us (1,048,576 atoms).  Eight lanes per
 // edge with the sums of one channel each (48 registers, 37 warps) were slower, 39
@@ -238,6 +244,7 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
 // k <= k' over 8 orbitals (108 features).
 constexpr int kFwdWarps = 4;
 constexpr int kBStride = 84;  // padded b row of an atom in shared memory (16 B aligned)
+constexpr int kEdgeLd = 12;   // a staged edge's t_0..7, x, y, z (stride 12: no bank conflicts in the stores)
 
 // one butterfly stage over CNT values: lanes with bit O set keep the upper half
 template <int CNT, int O>
@@ -260,7 +267,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
                                                             const float* __restrict__ Wt, float* __restrict__ rho,
                                                             float* __restrict__ bck, bool far) {
     constexpr int KO = PAIRS ? NORB_P : NORB, APW = 32 / LPA;
-    static_assert(LPA == 4 || LPA == 8 || LPA == 16, "80 sums split evenly");
+    static_assert(LPA == 4 || LPA == 8 || LPA == 16, "four classes of edges, 80 sums split evenly");
+    constexpr int CH = NPHI / (LPA / 4), NS = NANG * CH;  // channels and sums per lane
     __shared__ __align__(16) float sW[(LMAX + 1) * NPHI * KO];
     __shared__ __align__(16) float sB[kFwdWarps * APW][kBStride];
     for (int i = threadIdx.x; i < (LMAX + 1) * NPHI * KO; i += blockDim.x) sW[i] = Wt[i];
@@ -270,61 +278,117 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
     const int64_t kr = ((int64_t)blockIdx.x * kFwdWarps + warp) * APW + slot;
     const bool valid = kr < rows;
     const int64_t atom = row0 + kr;
-    float acc[NB];
+    const int cnt = valid ? live_cnt[atom] : 0;
+    const float4* ex = xyzj + (size_t)kr * stride;
+    const float2* ep = phi + (size_t)kr * stride;
+    float acc[NS];
 #pragma unroll
-    for (int v = 0; v < NB; ++v) acc[v] = 0.f;
-    if (valid) {
-        const int cnt = live_cnt[atom];
-        const float4* ex = xyzj + (size_t)kr * stride;
-        const float2* ep = phi + (size_t)kr * stride;
-        // the row's records start on their way to L2 at once (large systems stream them from HBM)
-        if (far) {
-            for (int e = 8 * q; e < cnt; e += 8 * LPA) prefetch_l2(ex + e);
-            for (int e = 16 * q; e < cnt; e += 16 * LPA) prefetch_l2(ep + e);
-        }
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 e1 = zero, c0 = zero, c1 = zero;
-        float2 p1 = make_float2(0.f, 0.f);
+    for (int v = 0; v < NS; ++v) acc[v] = 0.f;
+    // the row's records start on their way to L2 at once (large systems stream them from HBM)
+    if (far) {
+        for (int e = 8 * q; e < cnt; e += 8 * LPA) prefetch_l2(ex + e);
+        for (int e = 16 * q; e < cnt; e += 16 * LPA) prefetch_l2(ep + e);
+    }
+    auto terms = [&](const float2& p, const float4& c0, const float4& c1, float t[NPHI]) {
+        float ph[NPHI];
+        phi_chain(R, p.x, p.y, ph);
+        t[0] = c0.x * ph[0], t[1] = c0.y * ph[1], t[2] = c0.z * ph[2], t[3] = c0.w * ph[3];
+        t[4] = c1.x * ph[4], t[5] = c1.y * ph[5], t[6] = c1.z * ph[6], t[7] = c1.w * ph[7];
+    };
+    auto add = [&](float x, float y, float z, const float* t) {
+        const float A[NANG] = {1.f, x, y, z, x * x, y * y, z * z, x * y, x * z, y * z};
+#pragma unroll
+        for (int a = 0; a < NANG; ++a)
+#pragma unroll
+            for (int m = 0; m < CH; ++m) acc[a * CH + m] = fmaf(t[m], A[a], acc[a * CH + m]);
+    };
+    auto coefs = [&](const float4& e, float4& c0, float4& c1) { ldg8(coef + (size_t)__float_as_int(e.w) * NPHI, c0, c1); };
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (LPA == 4) {
+        float4 e1 = zero, c0 = zero, c1 = zero, e2 = zero;
+        float2 p1 = make_float2(0.f, 0.f), p2 = p1;
         if (q < cnt) {
-            e1 = ex[q];
-            p1 = ep[q];
-            ldg8(coef + (size_t)__float_as_int(e1.w) * NPHI, c0, c1);
+            e1 = ex[q], p1 = ep[q];
+            coefs(e1, c0, c1);
         }
-        float4 e2 = zero;
-        float2 p2 = make_float2(0.f, 0.f);
         if (q + LPA < cnt) e2 = ex[q + LPA], p2 = ep[q + LPA];
         for (int e = q; e < cnt; e += LPA) {
             const float x = e1.x, y = e1.y, z = e1.z;
-            float ph[NPHI];
-            phi_chain(R, p1.x, p1.y, ph);
-            const float t[NPHI] = {c0.x * ph[0], c0.y * ph[1], c0.z * ph[2], c0.w * ph[3],
-                                   c1.x * ph[4], c1.y * ph[5], c1.z * ph[6], c1.w * ph[7]};
-            e1 = e2;
-            p1 = p2;
-            if (e + LPA < cnt) ldg8(coef + (size_t)__float_as_int(e2.w) * NPHI, c0, c1);
+            float t[NPHI];
+            terms(p1, c0, c1, t);
+            e1 = e2, p1 = p2;
+            if (e + LPA < cnt) coefs(e2, c0, c1);
             if (e + 2 * LPA < cnt) e2 = ex[e + 2 * LPA], p2 = ep[e + 2 * LPA];
-            const float A[NANG] = {1.f, x, y, z, x * x, y * y, z * z, x * y, x * z, y * z};
+            add(x, y, z, t);
+        }
+    } else {
+        // batches of LPA edges of each of the warp's atoms, a lane one edge of each; the loads of kAhead batches at a time
+        constexpr int kAhead = LPA == 16 ? 4 : 2;
+        __shared__ __align__(16) float sT[kFwdWarps][32 * kEdgeLd];
+        const int c = q & 3, h = q >> 2;
+        int cmax = cnt;  // longest row of the warp's atoms
 #pragma unroll
-            for (int a = 0; a < NANG; ++a)
+        for (int o = LPA; o < 32; o <<= 1) cmax = max(cmax, __shfl_xor_sync(FULL, cmax, o));
+        float4 e[kAhead] = {};
+        float2 p[kAhead] = {};
+        auto records = [&](int e0) {
 #pragma unroll
-                for (int m = 0; m < NPHI; ++m) acc[a * NPHI + m] = fmaf(t[m], A[a], acc[a * NPHI + m]);
+            for (int u = 0; u < kAhead; ++u)
+                if (e0 + u * LPA + q < cnt) e[u] = ex[e0 + u * LPA + q], p[u] = ep[e0 + u * LPA + q];
+        };
+        records(0);
+#pragma unroll 1
+        for (int e0 = 0; e0 < cmax; e0 += kAhead * LPA) {
+            float4 c0[kAhead] = {}, c1[kAhead] = {};
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+                if (e0 + u * LPA + q < cnt) coefs(e[u], c0[u], c1[u]);
+            float t[kAhead][NPHI];
+            float4 r[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                r[u] = make_float4(e[u].x, e[u].y, e[u].z, 0.f);
+                terms(p[u], c0[u], c1[u], t[u]);
+            }
+            records(e0 + kAhead * LPA);
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                if (e0 + u * LPA >= cmax) break;
+                const bool in = e0 + u * LPA + q < cnt;  // past the row's end: an edge that adds zeros
+                float* d = sT[warp] + lane * kEdgeLd;
+                *reinterpret_cast<float4*>(d) = in ? make_float4(t[u][0], t[u][1], t[u][2], t[u][3]) : zero;
+                *reinterpret_cast<float4*>(d + 4) = in ? make_float4(t[u][4], t[u][5], t[u][6], t[u][7]) : zero;
+                *reinterpret_cast<float4*>(d + 8) = in ? r[u] : zero;
+                __syncwarp();
+                const float* st = sT[warp] + slot * LPA * kEdgeLd;
+#pragma unroll
+                for (int k = 0; k < LPA / 4; ++k) {
+                    const float* x = st + (4 * k + c) * kEdgeLd;
+                    const float4 xyz = ld4(x + 8);
+                    float tm[CH];
+                    ldk<CH>(x + CH * h, tm);
+                    add(xyz.x, xyz.y, xyz.z, tm);
+                }
+                __syncwarp();
+            }
         }
     }
-    // reduce-scatter: lane q keeps b[80 / LPA * rev(q) ..), rev the order the halves were taken in
+    // reduce-scatter over the classes: lane (h, c) keeps the sums NL c .. NL c + NL - 1 of its NS
     constexpr int NL = NB / LPA;
-    if constexpr (LPA == 16) rs_half<NB, 8>(acc, q);
-    if constexpr (LPA >= 8) rs_half<(LPA == 16 ? NB / 2 : NB), 4>(acc, q);
-    rs_half<NL * 4, 2>(acc, q);
-    rs_half<NL * 2, 1>(acc, q);
+    rs_half<NS, 2>(acc, q);
+    rs_half<NS / 2, 1>(acc, q);
     float* sb = sB[warp * APW + slot];
 #pragma unroll
     for (int v = 0; v < NL; ++v) acc[v] *= R.unscale;
-    if constexpr (LPA == 16) {
-#pragma unroll
-        for (int v = 0; v < NL; ++v) sb[NL * q + v] = acc[v];
-    } else {
+    if constexpr (LPA == 4) {
 #pragma unroll
         for (int v = 0; v < NL; v += 2) *reinterpret_cast<float2*>(sb + NL * q + v) = make_float2(acc[v], acc[v + 1]);
+    } else {
+#pragma unroll
+        for (int v = 0; v < NL; ++v) {
+            const int f = NL * (q & 3) + v;  // sum (a, m) of the lane at f = CH a + m
+            sb[f / CH * NPHI + CH * (q >> 2) + f % CH] = acc[v];
+        }
     }
     __syncwarp();
     if (valid)
@@ -474,12 +538,17 @@ __global__ void __launch_bounds__(TPA * kBbarAtoms) k_bbar(int64_t n, const floa
 // ---------------------------------------------------------- adjoint ------
 
 // Reverse pass (header formulas), LPA lanes per centre atom k (32 / LPA atoms per
-// warp), lane (g, m) owning radial channel m of the edges s = g mod LPA / 8.  Per
+// warp), lane (g, m) owning radial channel m of every (LPA / 8)th edge, g the lane's group of 8.  Per
 // batch of LPA edges each lane expands one edge's record into shared memory (the
 // next batch's record is on its way meanwhile).  Then, for its edges, lane (g, m)
 // gathers channel m of the neighbour's adjoint record (3 float4 loads; per load the
 // 8 lanes of a group read one full 128 B line) and accumulates its share of
-// dE/dr_k; cbar_{k,m} is summed over the groups.
+// dE/dr_k and of cbar_{k,m}.
+//   The shares are summed by NC LPA / 8 classes of edges, e mod (NC LPA / 8), edge after edge,
+// and the classes' sums added as (0 + 2) + (1 + 3).  How many classes is decided by the
+// atoms of the structure (adj_classes), never by how many rows a launch has, so that a structure's results
+// are the same alone and among others; a group keeps the sums of NC classes: four as (LPA, NC)
+// = (32, 1) or, in launches of many rows, (16, 2); two as (16, 1); one as (8, 1).
 //   Bound by the L2 latency and the L1 wavefronts of the record gathers (384 B per
 // edge; the L1 data stage is 70 % busy while blocks are resident, issue slots 56 %).
 // 59 -> 41 us per launch (24,576 atoms), 1,408 -> 1,166 us (1,048,576 atoms), 28 -> 7 us
@@ -512,7 +581,7 @@ struct Outputs {
 // WANT_VIR: also W -= (dE/dr_e) r_e^T over the atom's own edges (their
 // bbar_k c_j terms: every directed edge once) into vir (N x 9, accumulated
 // over the layers like grad); the part with grad Q_k again comes from b.
-template <bool WANT_CBAR, bool WANT_VIR, int LPA>
+template <bool WANT_CBAR, bool WANT_VIR, int LPA, int NC, bool POOL>
 __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_adj(int64_t row0, int64_t rows, int stride, Radial R,
                                                                 const int32_t* __restrict__ live_cnt,
                                                                 const float4* __restrict__ xyzj,
@@ -521,7 +590,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
                                                                 const float* __restrict__ rec,
                                                                 const float* __restrict__ bck,
                                                                 float* __restrict__ cbar, float* __restrict__ grad,
-                                                                float* __restrict__ vir, Outputs out) {
+                                                                float* __restrict__ vir,
+                                                                const int32_t* __restrict__ structure, Outputs out) {
     pdl_enter();
     constexpr int APW = 32 / LPA, G = LPA / 8;  // atoms per warp, groups of 8 lanes per atom
     // per atom, for its batch of LPA edges: (r, 1/d) [LPA][4], (j, r1) [LPA][2], phi [LPA][8]; an
@@ -531,8 +601,9 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
     __shared__ __align__(16) float sE[kAdjWarps * APW][LE + LJ + LP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane & 7, sub = lane & (LPA - 1), g = sub >> 3;
     const int64_t kr = ((int64_t)blockIdx.x * kAdjWarps + warp) * APW + lane / LPA;
-    const bool valid = kr < rows;
     const int64_t atom = row0 + kr;
+    // (of a serving pool's rows only those whose structure takes this many classes)
+    const bool valid = kr < rows && (!POOL || adj_classes(structure[atom]) == NC * G);
     float* s_e = sE[warp * APW + lane / LPA];
     float *s_j = s_e + LE, *s_phi = s_j + LJ;
     const float two_a_mu = R.two_a_mu[m];
@@ -571,16 +642,61 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
     const float4* ex = xyzj + (size_t)kr * stride;
     const float2* ep = phi + (size_t)kr * stride;
     const float2* ed = der + (size_t)kr * stride;
-    float gx = 0.f, gy = 0.f, gz = 0.f, cb = 0.f;
-    float w6[6];  // sum c_j psi Q_k r r^T: xx, yy, zz, xy, xz, yz
+    float gx[NC], gy[NC], gz[NC], cb[NC];
+    float w6[NC][6];  // sum c_j psi Q_k r r^T: xx, yy, zz, xy, xz, yz
 #pragma unroll
-    for (int q = 0; q < 6; ++q) w6[q] = 0.f;
+    for (int i = 0; i < NC; ++i) {
+        gx[i] = gy[i] = gz[i] = cb[i] = 0.f;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) w6[i][q] = 0.f;
+    }
     float w9[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) w9[q] = 0.f;
     float4 e_nx = make_float4(0.f, 0.f, 0.f, 0.f);  // the next batch's record of this lane
     float2 p_nx = make_float2(0.f, 0.f), d_nx = p_nx;
     if (sub < cnt) e_nx = ex[sub], p_nx = ep[sub], d_nx = ed[sub];
+    // one edge's shares: vx, vy, vz of -dE/dr_k, phi and Q_j (cbar += phi Q_j), a = c_j psi Q_k (virial)
+    struct Share {
+        float vx, vy, vz, ph, Qj, a;
+        float4 e;
+    };
+    auto share = [&](int s) {
+        const float2 jr = *reinterpret_cast<const float2*>(s_j + 2 * s);
+        float bj[12];
+        load_rec(__float_as_int(jr.x), bj);
+        const float4 e = ld4(s_e + 4 * s);
+        const float ph = s_phi[8 * s + m], ps = ph * fmaf(two_a_mu, e.w, jr.y);  // phi, phi' / d
+        const float x = e.x, y = e.y, z = e.z, cj = bj[NANG];
+        // grad Q_j; Q_j = q0 + (r . (l + grad Q_j)) / 2 for a quadratic with linear part l
+        const float gjx = fmaf(z, bj[8], fmaf(y, bj[7], fmaf(x, bj[4], -bj[1])));
+        const float gjy = fmaf(z, bj[9], fmaf(x, bj[7], fmaf(y, bj[5], -bj[2])));
+        const float gjz = fmaf(y, bj[9], fmaf(x, bj[8], fmaf(z, bj[6], -bj[3])));
+        const float Qj = fmaf(0.5f, fmaf(z, gjz - bj[3], fmaf(y, gjy - bj[2], x * (gjx - bj[1]))), bj[0]);
+        // Q_k by Horner's rule (bk's squares halved below)
+        const float Qk = fmaf(x, fmaf(z, bk[8], fmaf(y, bk[7], fmaf(x, bk[4], bk[1]))),
+                              fmaf(y, fmaf(z, bk[9], fmaf(y, bk[5], bk[2])), fmaf(z, fmaf(z, bk[6], bk[3]), bk[0])));
+        const float sk = cj * Qk;
+        const float sc = ps * fmaf(ck, Qj, sk);
+        const float qt = ck * ph;
+        return Share{fmaf(sc, x, qt * gjx), fmaf(sc, y, qt * gjy), fmaf(sc, z, qt * gjz), ph, Qj, ps * sk, e};
+    };
+    auto add_w6 = [](float* w, float a, const float4& e) {
+        const float ax = a * e.x, ay = a * e.y, az = a * e.z;
+        w[0] = fmaf(ax, e.x, w[0]);
+        w[1] = fmaf(ay, e.y, w[1]);
+        w[2] = fmaf(az, e.z, w[2]);
+        w[3] = fmaf(ax, e.y, w[3]);
+        w[4] = fmaf(ax, e.z, w[4]);
+        w[5] = fmaf(ay, e.z, w[5]);
+    };
+    auto add = [&](int i, const Share& v) {  // to class i's sums
+        gx[i] -= v.vx;
+        gy[i] -= v.vy;
+        gz[i] -= v.vz;
+        if (WANT_CBAR) cb[i] = fmaf(v.ph, v.Qj, cb[i]);
+        if (WANT_VIR) add_w6(w6[i], v.a, v.e);
+    };
     for (int e0 = 0; e0 < cmax; e0 += LPA) {
         const int ne = min(cnt - e0, LPA);
         if (sub < ne) {
@@ -599,53 +715,42 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
             if (e0 + LPA + sub < cnt) e_nx = ex[e0 + LPA + sub], p_nx = ep[e0 + LPA + sub], d_nx = ed[e0 + LPA + sub];
         }
         __syncwarp();
+        // the group's classes, one after the other
+#pragma unroll
+        for (int i = 0; i < NC; ++i)
 #pragma unroll 1
-        for (int s = g; s < ne; s += G) {
-            const float2 jr = *reinterpret_cast<const float2*>(s_j + 2 * s);
-            float bj[12];
-            load_rec(__float_as_int(jr.x), bj);
-            const float4 e = ld4(s_e + 4 * s);
-            const float ph = s_phi[8 * s + m], ps = ph * fmaf(two_a_mu, e.w, jr.y);  // phi, phi' / d
-            const float x = e.x, y = e.y, z = e.z, cj = bj[NANG];
-            // grad Q_j; Q_j = q0 + (r . (l + grad Q_j)) / 2 for a quadratic with linear part l
-            const float gjx = fmaf(z, bj[8], fmaf(y, bj[7], fmaf(x, bj[4], -bj[1])));
-            const float gjy = fmaf(z, bj[9], fmaf(x, bj[7], fmaf(y, bj[5], -bj[2])));
-            const float gjz = fmaf(y, bj[9], fmaf(x, bj[8], fmaf(z, bj[6], -bj[3])));
-            const float Qj = fmaf(0.5f, fmaf(z, gjz - bj[3], fmaf(y, gjy - bj[2], x * (gjx - bj[1]))), bj[0]);
-            // Q_k by Horner's rule (bk's squares halved below)
-            const float Qk = fmaf(x, fmaf(z, bk[8], fmaf(y, bk[7], fmaf(x, bk[4], bk[1]))),
-                                  fmaf(y, fmaf(z, bk[9], fmaf(y, bk[5], bk[2])), fmaf(z, fmaf(z, bk[6], bk[3]), bk[0])));
-            const float sk = cj * Qk;
-            const float sc = ps * fmaf(ck, Qj, sk);
-            const float qt = ck * ph;
-            gx -= fmaf(sc, x, qt * gjx);
-            gy -= fmaf(sc, y, qt * gjy);
-            gz -= fmaf(sc, z, qt * gjz);
-            if (WANT_CBAR) cb = fmaf(ph, Qj, cb);
-            if (WANT_VIR) {
-                const float a = ps * sk, ax = a * x, ay = a * y, az = a * z;
-                w6[0] = fmaf(ax, x, w6[0]);
-                w6[1] = fmaf(ay, y, w6[1]);
-                w6[2] = fmaf(az, z, w6[2]);
-                w6[3] = fmaf(ax, y, w6[3]);
-                w6[4] = fmaf(ax, z, w6[4]);
-                w6[5] = fmaf(ay, z, w6[5]);
-            }
-        }
+            for (int s = g + G * i; s < ne; s += G * NC) add(i, share(s));
         __syncwarp();
     }
-    gx *= R.unscale, gy *= R.unscale, gz *= R.unscale, cb *= R.unscale;
+    // the row's sums, in every group
+    auto total = [](const float* p) {
+        float v = NC == 2 ? p[0] + p[NC - 1] : p[0];
+        if (LPA == 32) v += __shfl_xor_sync(FULL, v, 16);
+        if (LPA >= 16) v += __shfl_xor_sync(FULL, v, 8);
+        return v;
+    };
+    gx[0] = total(gx), gy[0] = total(gy), gz[0] = total(gz), cb[0] = total(cb);
     if (WANT_VIR)
 #pragma unroll
-        for (int q = 0; q < 6; ++q) w6[q] *= R.unscale;
+        for (int q = 0; q < 6; ++q) {
+            float p[NC];
+#pragma unroll
+            for (int i = 0; i < NC; ++i) p[i] = w6[i][q];
+            w6[0][q] = total(p);
+        }
+    float sx = gx[0] * R.unscale, sy = gy[0] * R.unscale, sz = gz[0] * R.unscale;
+    if (WANT_CBAR && g == 0 && valid) cbar[(size_t)atom * NPHI + m] = cb[0] * R.unscale;
+    if (WANT_VIR)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) w6[0][q] *= R.unscale;
     if (g == 0 && valid) {
         // sum_j c_j phi grad Q_k (and, for the virial, times r) from the forward's moments b_{k,a,m}
         const float* b = bck + (size_t)atom * NB + m;
         const float h4 = 2.f * bk[4], h5 = 2.f * bk[5], h6 = 2.f * bk[6];
         const float b0 = __ldg(b), b1 = __ldg(b + NPHI), b2 = __ldg(b + 2 * NPHI), b3 = __ldg(b + 3 * NPHI);
-        gx -= fmaf(bk[1], b0, fmaf(h4, b1, fmaf(bk[7], b2, bk[8] * b3)));
-        gy -= fmaf(bk[2], b0, fmaf(bk[7], b1, fmaf(h5, b2, bk[9] * b3)));
-        gz -= fmaf(bk[3], b0, fmaf(bk[8], b1, fmaf(bk[9], b2, h6 * b3)));
+        sx -= fmaf(bk[1], b0, fmaf(h4, b1, fmaf(bk[7], b2, bk[8] * b3)));
+        sy -= fmaf(bk[2], b0, fmaf(bk[7], b1, fmaf(h5, b2, bk[9] * b3)));
+        sz -= fmaf(bk[3], b0, fmaf(bk[8], b1, fmaf(bk[9], b2, h6 * b3)));
         if (WANT_VIR) {
             const float b4 = __ldg(b + 4 * NPHI), b5 = __ldg(b + 5 * NPHI), b6 = __ldg(b + 6 * NPHI);
             const float b7 = __ldg(b + 7 * NPHI), b8 = __ldg(b + 8 * NPHI), b9 = __ldg(b + 9 * NPHI);
@@ -661,41 +766,37 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
         }
     }
 #pragma unroll
-    for (int o = 1; o < LPA; o <<= 1) {
-        gx += __shfl_xor_sync(FULL, gx, o);
-        gy += __shfl_xor_sync(FULL, gy, o);
-        gz += __shfl_xor_sync(FULL, gz, o);
+    for (int o = 1; o < NPHI; o <<= 1) {
+        sx += __shfl_xor_sync(FULL, sx, o);
+        sy += __shfl_xor_sync(FULL, sy, o);
+        sz += __shfl_xor_sync(FULL, sz, o);
     }
     if (WANT_VIR) {
-        w9[0] += w6[0], w9[4] += w6[1], w9[8] += w6[2];
-        w9[1] += w6[3], w9[3] += w6[3], w9[2] += w6[4], w9[6] += w6[4], w9[5] += w6[5], w9[7] += w6[5];
+        const float* w = w6[0];
+        w9[0] += w[0], w9[4] += w[1], w9[8] += w[2];
+        w9[1] += w[3], w9[3] += w[3], w9[2] += w[4], w9[6] += w[4], w9[5] += w[5], w9[7] += w[5];
 #pragma unroll
-        for (int o = 1; o < LPA; o <<= 1)
+        for (int o = 1; o < NPHI; o <<= 1)
 #pragma unroll
             for (int q = 0; q < 9; ++q) w9[q] += __shfl_xor_sync(FULL, w9[q], o);
-    }
-    if (WANT_CBAR) {
-#pragma unroll
-        for (int o = 8; o < LPA; o <<= 1) cb += __shfl_xor_sync(FULL, cb, o);
-        if (g == 0 && valid) cbar[(size_t)atom * NPHI + m] = cb;
     }
     if (sub == 0 && valid) {
         float* gr = grad + (size_t)atom * 3;
         if (!out.first) {  // the first reverse layer starts the sums (no memset)
-            gx += gr[0];
-            gy += gr[1];
-            gz += gr[2];
+            sx += gr[0];
+            sy += gr[1];
+            sz += gr[2];
         }
         if (out.forces) {  // the last layer: F = -dE/dr and eps_i in caller order
             const int64_t c = out.perm[atom];
-            out.forces[3 * c] = -gx;
-            out.forces[3 * c + 1] = -gy;
-            out.forces[3 * c + 2] = -gz;
+            out.forces[3 * c] = -sx;
+            out.forces[3 * c + 1] = -sy;
+            out.forces[3 * c + 2] = -sz;
             if (out.atom_energy) out.atom_energy[c] = out.eps[atom];
         } else {
-            gr[0] = gx;
-            gr[1] = gy;
-            gr[2] = gz;
+            gr[0] = sx;
+            gr[1] = sy;
+            gr[2] = sz;
         }
         if (WANT_VIR) {
             float* vr = vir + (size_t)atom * 9;
@@ -857,9 +958,10 @@ cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r,
 cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
                                const float* W, const float* coef, float* rho, float* bck, bool pairs) {
     if (rows == 0) return cudaSuccess;
-    // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer need
-    // less reduction work per atom (many).  us per launch with 16 / 8 / 4 lanes: 192 atoms 4.5 / 5.6 /
-    // 7.9, 4,000 5.5 / 5.8 / 7.1, 10,976 11.8 / 10.8 / 9.1, 24,576 25 / 20 / 20, 1,048,576 914 / 670 / 536.
+    // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer stage
+    // nothing (many).  us per launch within an evaluation with 16 / 8 / 4 lanes: 192 atoms 6.0 / 7.8 /
+    // 10.2, 4,000 9.1 / 10.7 / 11.9, 6,912 8.4 / 6.8 / 7.8, 10,976 10.5 / 12.4 / 8.8, 24,576 25 / 23 /
+    // 19.5, 1,048,576 859 / 757 / 537.
     const EvalLaunch how = eval_launch(nl);
     const int lpa = rows <= 4096 ? 16 : (rows <= 8192 ? 8 : 4);
     // records of more rows than this outgrow L2 between the passes: prefetch each atom's when it
@@ -917,29 +1019,51 @@ cudaError_t launch_density_adj(cudaStream_t s, const reann_nlist* nl, const Radi
     if (rows == 0) return cudaSuccess;
     // Lanes per atom, as in the forward pass.  us per launch with 32 / 16 / 8 lanes: 192 atoms 7.2 /
     // 10.6 / 18.3, 4,000 8.6 / 11.1 / 16.1, 24,576 43.5 / 41.1 / 49, 32,000 53 / 47.0 / 45.6,
-    // 1,048,576 1,644 / 1,242 / 1,161.
+    // 1,048,576 1,644 / 1,242 / 1,161.  The sums' classes follow: four with 32 lanes, two with 16, one with 8.
     const EvalLaunch how = eval_launch(nl);
-    const int lpa = rows <= 16384 ? 32 : (rows <= 28672 ? 16 : 8);
-#define REANN_ADJ_L(C, V, L)                                                                                       \
-    launch_with(how.chain, how.carve(kAdjCarveout), k_density_adj<C, V, L>, blocks_for(rows, kAdjWarps * (32 / L)),     \
-                kAdjWarps * 32, 0, s, row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, nl->edge_der, rec, bck, cbar, grad, vir, out)
-#define REANN_ADJ(C, V)              \
-    do {                             \
-        if (lpa == 32)               \
-            REANN_ADJ_L(C, V, 32);   \
-        else if (lpa == 16)          \
-            REANN_ADJ_L(C, V, 16);   \
-        else                         \
-            REANN_ADJ_L(C, V, 8);    \
+#define REANN_ADJ_L(C, V, L, N, P)                                                                                    \
+    launch_with(how.chain, how.carve(kAdjCarveout), k_density_adj<C, V, L, N, P>, blocks_for(rows, kAdjWarps * (32 / L)), \
+                kAdjWarps * 32, 0, s, row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, nl->edge_der, rec, bck, cbar, grad, vir, nl->structure, out)
+#define REANN_ADJ(C, V)                  \
+    do {                                 \
+        if (classes == 4)                \
+            REANN_ADJ_L(C, V, 32, 1, false); \
+        else if (classes == 2)           \
+            REANN_ADJ_L(C, V, 16, 1, false); \
+        else                             \
+            REANN_ADJ_L(C, V, 8, 1, false);  \
     } while (0)
-    if (want_cbar && vir)
-        REANN_ADJ(true, true);
-    else if (want_cbar)
-        REANN_ADJ(true, false);
-    else if (vir)
-        REANN_ADJ(false, true);
-    else
-        REANN_ADJ(false, false);
+    if (!nl->structure) {
+        const int classes = adj_classes(nl->n);
+        if (want_cbar && vir)
+            REANN_ADJ(true, true);
+        else if (want_cbar)
+            REANN_ADJ(true, false);
+        else if (vir)
+            REANN_ADJ(false, true);
+        else
+            REANN_ADJ(false, false);
+    }
+#undef REANN_ADJ
+#define REANN_ADJ(L, N)                            \
+    do {                                           \
+        if (want_cbar)                             \
+            REANN_ADJ_L(true, false, L, N, true);  \
+        else                                       \
+            REANN_ADJ_L(false, false, L, N, true); \
+    } while (0)
+    // A serving pool's rows belong to structures of their own: a launch for each number of classes that
+    // the evaluated structures take.  Many rows of four classes go with 16 lanes (24,576 rows: 41.8 us, with 32 51).
+    if (nl->structure) {
+        if (nl->adj_passes & 4) {
+            if (rows_of(nl) <= 16384)
+                REANN_ADJ(32, 1);
+            else
+                REANN_ADJ(16, 2);
+        }
+        if (nl->adj_passes & 2) REANN_ADJ(16, 1);
+        if (nl->adj_passes & 1) REANN_ADJ(8, 1);
+    }
 #undef REANN_ADJ
 #undef REANN_ADJ_L
     return cudaGetLastError();

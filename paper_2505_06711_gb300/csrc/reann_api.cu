@@ -1491,11 +1491,12 @@ struct reann_serve {
     cudaMemPool_t build_pool = nullptr;  // stream-ordered blocks of the per-submission lists
     cudaEvent_t staged = nullptr, done = nullptr, user_ready = nullptr;
     std::vector<std::pair<reann_nlist*, cudaEvent_t>> deferred;  // built lists freed once their pack has run
-    // one captured pass per size class k: owned rows [0, n >> k), ghost slots [0, g_cap >> k)
+    // one captured pass per size class k: owned rows [0, n >> k), ghost slots [0, g_cap >> k);
+    // [0] for launches whose structures all take one reverse edge pass (adj_classes 4), [1] for the others
     static constexpr int kClasses = 8;
     static constexpr int64_t kMinRows = 2048;
-    cudaGraph_t graph[kClasses] = {};
-    cudaGraphExec_t exec[kClasses] = {};
+    cudaGraph_t graph[2][kClasses] = {};
+    cudaGraphExec_t exec[2][kClasses] = {};
     int graph_precision = -1;
     const void* graph_out[2] = {nullptr, nullptr};
 };
@@ -1517,6 +1518,16 @@ void serve_reap(reann_serve* srv, bool wait) {
     }
 }
 
+void drop_serve_graphs(reann_serve* srv) {
+    for (int w = 0; w < 2; ++w)
+        for (int k = 0; k < reann_serve::kClasses; ++k) {
+            if (srv->exec[w][k]) cudaGraphExecDestroy(srv->exec[w][k]);
+            if (srv->graph[w][k]) cudaGraphDestroy(srv->graph[w][k]);
+            srv->exec[w][k] = nullptr;
+            srv->graph[w][k] = nullptr;
+        }
+}
+
 // one evaluation of every structure in the segment table, then their retirement
 int pool_pass(reann_ctx* ctx, reann_serve* srv, double* energies, float* forces) {
     reann_nlist* p = srv->pool;
@@ -1533,10 +1544,7 @@ extern "C" void reann_serve_free(reann_serve* srv) {
     serve_reap(srv, true);
     if (srv->stream) cudaStreamSynchronize(srv->stream);
     if (srv->build_pool) cudaMemPoolDestroy(srv->build_pool);
-    for (int k = 0; k < reann_serve::kClasses; ++k) {
-        if (srv->exec[k]) cudaGraphExecDestroy(srv->exec[k]);
-        if (srv->graph[k]) cudaGraphDestroy(srv->graph[k]);
-    }
+    drop_serve_graphs(srv);
     free_nlist(srv->pool);
     if (srv->d_seg) cudaFree(srv->d_seg);
     if (srv->h_seg) cudaFreeHost(srv->h_seg);
@@ -1579,8 +1587,9 @@ extern "C" int reann_serve_create(reann_ctx* ctx, int64_t max_atoms, int64_t max
     p->g_owner = nl_alloc<int32_t>(p, max_ghosts);
     p->nbr = nl_alloc<int32_t>(p, (size_t)max_atoms * stride);
     p->nbr_cnt = nl_alloc<int32_t>(p, max_atoms);
+    p->structure = nl_alloc<int32_t>(p, max_atoms);
     p->w.goff = nl_alloc<int32_t>(p, max_atoms + 1);
-    if (!p->perm || !p->species || !p->g_owner || !p->nbr || !p->nbr_cnt || !p->w.goff)
+    if (!p->perm || !p->species || !p->g_owner || !p->nbr || !p->nbr_cnt || !p->structure || !p->w.goff)
         return fail(REANN_E_NOMEM, "serving pool: out of device memory");
     if (alloc_eval_buffers(ctx, p)) return fail(REANN_E_NOMEM, "serving pool: out of device memory");
     // tile lists of fixed capacity (padding entries have nrows = 0)
@@ -1620,6 +1629,7 @@ extern "C" int reann_serve_create(reann_ctx* ctx, int64_t max_atoms, int64_t max
                   cudaSuccess &&
               cudaMemset(p->nbr_cnt, 0, sizeof(int32_t) * max_atoms) == cudaSuccess &&
               cudaMemset(p->species, 0, sizeof(int32_t) * max_atoms) == cudaSuccess &&
+              cudaMemset(p->structure, 0, sizeof(int32_t) * max_atoms) == cudaSuccess &&
               cudaMemset(p->g_owner, 0, sizeof(int32_t) * std::max<int64_t>(max_ghosts, 1)) == cudaSuccess &&
               cudaMemset(p->pos, 0, sizeof(float4) * 2 * (max_atoms + max_ghosts)) == cudaSuccess &&
               cudaDeviceSynchronize() == cudaSuccess;
@@ -1704,11 +1714,13 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
     size_t n64 = 0, n128 = 0;
     int nseg = 0;
     int64_t hi = 0, ghi = 0;  // owned rows and ghost slots the launched structures occupy
+    int passes = 0;           // the reverse edge passes they take
     for (int k = 0; k < srv->max_slots; ++k) {
         ServeSlot& sl = srv->slots[k];
         if (!sl.used || !sl.pending) continue;
         hi = std::max<int64_t>(hi, sl.ob + sl.n);
         ghi = std::max<int64_t>(ghi, sl.gb + sl.g);
+        passes |= adj_classes(sl.n);
         for (const Tile& t : sl.t64) srv->h_t64[n64++] = t;
         for (const Tile& t : sl.t128) srv->h_t128[n128++] = t;
         srv->h_seg[nseg] = make_int4((int)sl.ob, (int)sl.n, k, 0);
@@ -1733,7 +1745,10 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
     // One evaluation of the pool, sized to the work: size class k covers owned rows
     // [0, n >> k) and ghost slots [0, g_cap >> k), the smallest class holding every
     // launched structure (free and retired rows inside it have no neighbours).  Each
-    // class is captured once per (precision, outputs) and replayed.
+    // class is captured once per (precision, outputs) and replayed; again with the other
+    // reverse edge passes once a structure needs them.
+    const int wide = passes == 4 ? 0 : 1;
+    p->adj_passes = wide ? 7 : 4;
     int cls = 0, ncls = 1;
     while (ncls < reann_serve::kClasses && (p->n >> ncls) >= reann_serve::kMinRows) ++ncls;
     while (cls + 1 < ncls && (p->n >> (cls + 1)) >= hi && (p->g_cap >> (cls + 1)) >= ghi) ++cls;
@@ -1753,22 +1768,17 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
     ctx->prof_on = false;
     int rc = REANN_OK;
     if (srv->graph_precision != ctx->precision || srv->graph_out[0] != energies || srv->graph_out[1] != forces) {
-        for (int k = 0; k < reann_serve::kClasses; ++k) {  // another key: every class is captured again
-            if (srv->exec[k]) cudaGraphExecDestroy(srv->exec[k]);
-            if (srv->graph[k]) cudaGraphDestroy(srv->graph[k]);
-            srv->exec[k] = nullptr;
-            srv->graph[k] = nullptr;
-        }
+        drop_serve_graphs(srv);  // another key: every class is captured again
         srv->graph_precision = ctx->precision;
         srv->graph_out[0] = energies;
         srv->graph_out[1] = forces;
     }
-    if (!srv->exec[cls]) {
+    if (!srv->exec[wide][cls]) {
         // this launch runs directly (which also sets kernel attributes outside capture);
         // then every size class is captured, so that no later launch pays for a capture
         rc = pool_pass(ctx, srv, energies, forces);
         for (int k = 0; k < ncls && !rc; ++k) {
-            if (srv->exec[k]) continue;
+            if (srv->exec[wide][k]) continue;
             set_class(k);
             if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
                 rc = set_error(ctx, REANN_E_CUDA, "serving graph capture failed");
@@ -1777,15 +1787,15 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
             rc = pool_pass(ctx, srv, energies, forces);
             cudaGraph_t g = nullptr;
             const cudaError_t ec = cudaStreamEndCapture(s, &g);
-            if (!rc && ec == cudaSuccess && cudaGraphInstantiate(&srv->exec[k], g, 0) == cudaSuccess) {
-                srv->graph[k] = g;
+            if (!rc && ec == cudaSuccess && cudaGraphInstantiate(&srv->exec[wide][k], g, 0) == cudaSuccess) {
+                srv->graph[wide][k] = g;
             } else {
                 if (g) cudaGraphDestroy(g);
-                srv->exec[k] = nullptr;
+                srv->exec[wide][k] = nullptr;
                 if (!rc) rc = set_error(ctx, REANN_E_CUDA, "serving graph capture failed");
             }
         }
-    } else if (cudaGraphLaunch(srv->exec[cls], s) != cudaSuccess) {
+    } else if (cudaGraphLaunch(srv->exec[wide][cls], s) != cudaSuccess) {
         rc = set_error(ctx, REANN_E_CUDA, "serving graph launch failed");
     }
     p->n_rows = p->g_rows = p->tiles_active = p->tiles128_active = -1;

@@ -52,7 +52,7 @@ struct PackSrc {
 struct PackDst {
     int64_t no, ob, gb;  // pool owned size, owned base, ghost base
     int stride;
-    int32_t *nbr, *cnt, *species, *perm, *owner;
+    int32_t *nbr, *cnt, *species, *perm, *structure, *owner;
     float4* pos_out;  // hi, lo parts of each slot, interleaved
 };
 
@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(256) k_pack(PackSrc s, PackDst d, unsigned own
     if (lane != 0) return;
     d.cnt[d.ob + i] = c;
     d.species[d.ob + i] = s.species[i];
+    d.structure[d.ob + i] = (int32_t)s.n;
     const int64_t ci = s.perm[i];
     d.perm[d.ob + i] = (int32_t)(d.ob + ci);
     double sm[3], x[3];
@@ -149,7 +150,7 @@ cudaError_t launch_pack(cudaStream_t s, const reann_nlist* src, const double* ca
                         int64_t ob, int64_t gb) {
     PackSrc a{src->n,       src->g,     src->stride, src->nbr,      src->nbr_cnt, src->species,
               src->perm,    src->wrapm, src->g_owner, src->g_shift, caller_pos,   src->geom};
-    PackDst b{pool->n, ob, gb, pool->stride, pool->nbr, pool->nbr_cnt, pool->species, pool->perm, pool->g_owner,
+    PackDst b{pool->n, ob, gb, pool->stride, pool->nbr, pool->nbr_cnt, pool->species, pool->perm, pool->structure, pool->g_owner,
               pool->pos};
     const unsigned own = blocks_for(src->n * 32, 256);
     launch_pdl(k_pack, own + (src->g > 0 ? blocks_for(src->g, 256) : 0), 256, 0, s, a, b, own);

@@ -60,24 +60,44 @@ def test_narrow_gaussians_keep_their_range():
     pot.close()
 
 
-@pytest.mark.parametrize("virial", [False, True])
-def test_records_of_a_part_of_the_rows(virial):
+def _evaluated(s, T, rows, virial, precision=0):
     import torch
 
     from paper_2505_06711_gb300 import Potential, binding
 
-    s = water_box(400, seed=8)
-    pot = Potential(make_model(T=3))
-    got = []
-    for rows in (1 << 40, 1199, 512, 7):
-        sy = pot.system(s.pos, s.species, s.cell)
-        assert binding.lib().reann_test_limit_edge_rows(sy.nl, binding._i64(rows)) == 0
-        for _ in range(3):  # direct, captured, replayed
-            sy.evaluate(virial=virial)
-        sy.check()
-        torch.cuda.synchronize()
-        got.append((float(sy.energy), sy.forces.cpu().numpy().copy(), sy.info()[3]))
-        sy.close()
+    pot = Potential(make_model(T=T), precision=precision)
+    sy = pot.system(s.pos, s.species, s.cell)
+    assert binding.lib().reann_test_limit_edge_rows(sy.nl, binding._i64(rows)) == 0
+    for _ in range(3):  # direct, captured, replayed
+        sy.evaluate(virial=virial, atom_virial=virial)
+    sy.check()
+    torch.cuda.synchronize()
+    out = [np.array(sy.info()[3])] + [x.cpu().numpy().copy() for x in (sy.energy, sy.forces, sy.atom_energy)]
+    if virial:
+        out += [sy.virial.cpu().numpy().copy(), sy.atom_virial.cpu().numpy().copy()]
+    sy.close()
     pot.close()
-    for e, f, live in got[1:]:
-        assert e == got[0][0] and np.array_equal(f, got[0][1]) and live == got[0][2]
+    return out
+
+
+def _assert_same(a, b):
+    assert len(a) == len(b)
+    for k, (x, y) in enumerate(zip(a, b)):
+        assert np.array_equal(x, y), k
+
+
+@pytest.mark.parametrize("virial", [False, True])
+def test_records_of_a_part_of_the_rows(virial):
+    s = water_box(400, seed=8)
+    whole = _evaluated(s, 3, 1 << 40, virial)
+    for rows in (1199, 512, 7):
+        _assert_same(_evaluated(s, 3, rows, virial), whole)
+
+
+@pytest.mark.parametrize("virial,precision", [(False, 0), (True, 0), (False, 3)])
+@pytest.mark.parametrize("molecules,rows", [(1400, 3000), (2800, 4096), (5600, 9000), (9600, 20000), (9600, 700)])
+def test_sums_do_not_depend_on_the_lanes_per_atom(molecules, rows, virial, precision):
+    # the run's rows decide the lanes per atom (forward 16, 8, 4 up to 4,096, 8,192, beyond; reverse 32, 16,
+    # 8 up to 16,384, 28,672, beyond), on the other side of a line than the whole list's here
+    s = water_box(molecules, seed=9)
+    _assert_same(_evaluated(s, 2, rows, virial, precision), _evaluated(s, 2, 1 << 40, virial, precision))

@@ -128,6 +128,30 @@ def test_mix_is_bitwise_alone(spec, structs):
         srv.close()
 
 
+@pytest.mark.parametrize("precision", [0, 1, 3], ids=["fp32", "bf16", "fp8"])
+def test_mix_is_bitwise_alone_in_every_size_class(spec, precision):
+    # the size class of a launch (2,048 to 65,536 rows here) decides the lanes per atom of the edge
+    # passes, a System's own size its; neither may show in the results
+    srv = _server(spec, precision, max_atoms=65536, max_ghosts=300000, max_structures=8)
+    try:
+        mates = {k: fcc_box(k, seed=k) for k in (6, 9, 11, 14, 17, 18, 20)}
+        probe = water_box(200, seed=4)
+        _, want = _system(spec, probe, precision)
+        for mix in ([], [9], [11], [11, 9], [14], [14, 11, 6], [18, 14], [20, 17], [17], [6]):
+            slot = _submit(srv, probe)
+            others = {k: _submit(srv, mates[k]) for k in mix}
+            launched, _ = srv.launch()
+            res = srv.collect(launched)
+            assert np.array_equal(res[slot][1], want), mix
+            if mix in ([18, 14], [20, 17]):  # 4,000 to 32,000 atoms: every order of the sums
+                for k in mix:
+                    assert np.array_equal(res[others[k]][1], _system(spec, mates[k], precision)[1]), k
+            for sl in launched:
+                srv.release(sl)
+    finally:
+        srv.close()
+
+
 def test_lifecycle_retire_release_reuse(spec, structs):
     from paper_2505_06711_gb300 import binding
 
