@@ -101,13 +101,15 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 
 // 32 consecutive bytes (32 B aligned) in one load: one instruction and one tag lookup for a
-// neighbour's coefficients or position
+// neighbour's coefficients or position.  Volatile with a memory clobber, like every load written in
+// assembly here: kernels read what the one before wrote, and nothing else keeps such a load behind pdl_enter().
 __device__ __forceinline__ void ldg8(const void* p, float4& a, float4& b) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(p)
+                 : "memory");
 }
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
 
 // K = 1, 2 or 4 consecutive floats (aligned to their size)
 template <int K>
@@ -617,7 +619,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
                 "ld.global.nc.v4.f32 {%8, %9, %10, %11}, [%12 + 256];"
                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11])
-                : "l"(p));
+                : "l"(p)
+                : "memory");
         } else {
 #pragma unroll
             for (int line = 0; line < 3; ++line) {

@@ -103,3 +103,18 @@ def test_ctx_without_device_fails_cleanly(libpath):
     binding.reann_model_free(h)
     assert rc == binding.REANN_E_CUDA
     assert not out.value
+
+
+def test_loads_in_assembly_stay_behind_the_wait():
+    # the kernels' programmatic launches read what the previous kernel wrote once griddepcontrol.wait has
+    # returned: the compiler may move a load written in assembly ahead of it unless that is volatile
+    # and clobbers memory
+    csrc = os.path.join(ROOT, "paper_2505_06711_gb300", "csrc")
+    found = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for m in re.finditer(r"\basm\b(.*?)\);", text, flags=re.S):
+            if re.search(r"\b(ld|prefetch)\.global", m.group(1)):
+                found += 1
+                assert m.group(1).lstrip().startswith("volatile") and '"memory"' in m.group(1), (name, m.group(0))
+    assert found >= 3
