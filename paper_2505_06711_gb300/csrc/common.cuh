@@ -185,7 +185,6 @@ struct Radial {
     float alpha_hi, alpha_lo;  // alpha
     float tad_hi, tad_lo;      // 2 alpha Delta, Delta = r_c / (N_phi - 1)
     float mu_hi[NPHI], mu_lo[NPHI];      // Gaussian centres m Delta
-    float two_a_mu[NPHI];                // 2 alpha m Delta
     float kap_hi[NPHI], kap_lo[NPHI];    // exp(-alpha Delta^2 (2m+1)) for the Gaussian recurrence
     float scale, unscale;                // 2^s, 2^-s: s = 0 unless exp(-alpha r_c^2) f_c would leave the normal range
 };
@@ -359,7 +358,7 @@ struct reann_nlist {
     int64_t edge_rows = 0;
     float4* edge_xyzj = nullptr;   // r_j - r_i, j
     float2* edge_phi = nullptr;    // first Gaussian x cutoff, recurrence factor
-    float2* edge_der = nullptr;    // 1/d, radial derivative part
+    float2* edge_der = nullptr;    // d, the cutoff's logarithmic derivative
     reann::Tile* tiles = nullptr;  // MLP tiles (64 rows, FP32 networks)
     std::vector<reann::Tile> tiles128_h;
     reann::Tile* tiles128 = nullptr;  // 128-row tiles of the tensor-core networks

@@ -17,7 +17,7 @@
 // Edge records.  The list of live (d < r_c) edges and everything about an edge
 // that is the same in all 2T edge passes of an evaluation is computed once per
 // evaluation (k_edges): r = r_j - r_i and j, the first Gaussian times the cutoff
-// and the factor of the Gaussian recurrence, 1/d and the cutoff's logarithmic
+// and the factor of the Gaussian recurrence, d and the cutoff's logarithmic
 // derivative (32 B per live edge, in the row order of the list).  The passes
 // stream the records of their atom (coalesced) and gather only what belongs to
 // the neighbour: its coefficients (forward) or its adjoint record (reverse).
@@ -149,8 +149,7 @@ __constant__ unsigned char c_pair_k2[NORB_P * (NORB_P + 1) / 2];
 // 0.91 x for 1,048,576.)  Bound by the latency of the position gathers; with the next batch's
 // positions fetched ahead 192 atoms take 3.6 instead of 4.2 us, 24,576 20.4 instead of 21.9,
 // 1,048,576 720 instead of 787 (writing 2.8 GB of records there takes 410).
-//   xyzj = (r, j as bits); phi = (phi_0 R.scale, q) of phi_chain; der = (1/d, r1) with
-//   phi_m' / d = phi_m (r1 + 2 a mu_m / d), r1 = (f_c' / f_c) / d - 2 a
+//   xyzj = (r, j as bits); phi = (phi_0 R.scale, q) of phi_chain; der = (d, f_c' / f_c)
 __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t rows, int stride, Radial R,
                                                            const int32_t* __restrict__ nbr,
                                                            const int32_t* __restrict__ cnt,
@@ -173,7 +172,6 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
     auto emit = [&]() {      // the record of queue entry done + lane
         const float4 e = q[(done + lane) & 63];
         const float d = sqrtf(e.x * e.x + e.y * e.y + e.z * e.z);
-        const float inv_d = 1.f / d;
         float fc, dlog;
         cutoff(R, d, fc, dlog);
         // every radial function is that of the same rounded d (its rounding then acts like a
@@ -183,7 +181,7 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
         const float qf = exp_prod(1.f, d, 0.f, R.tad_hi, R.tad_lo);
         xyzj[out + done + lane] = e;
         phi[out + done + lane] = make_float2(g0 * R.scale * fc, qf);
-        der[out + done + lane] = make_float2(inv_d, fmaf(dlog, inv_d, -2.f * R.alpha_hi));
+        der[out + done + lane] = make_float2(d, dlog);
     };
     // the next batch's positions and the indices of the one after it are on their way meanwhile
     int j = lane < c ? row[lane] : 0, j1 = lane + 32 < c ? row[lane + 32] : 0;
@@ -583,8 +581,17 @@ struct Outputs {
 // WANT_VIR: also W -= (dE/dr_e) r_e^T over the atom's own edges (their
 // bbar_k c_j terms: every directed edge once) into vir (N x 9, accumulated
 // over the layers like grad); the part with grad Q_k again comes from b.
+// 8 values of a lane's edge to shared memory at f = base + 8 lane; lanes 4-7 of every 8 store the halves the
+// other way round: no bank conflicts
+__device__ __forceinline__ void store8(float* f, const float v[NPHI], int lane) {
+    const bool sw = lane & 4;
+    const int h0 = sw ? 4 : 0, h1 = 4 - h0;
+    *reinterpret_cast<float4*>(f + h0) = make_float4(sw ? v[4] : v[0], sw ? v[5] : v[1], sw ? v[6] : v[2], sw ? v[7] : v[3]);
+    *reinterpret_cast<float4*>(f + h1) = make_float4(sw ? v[0] : v[4], sw ? v[1] : v[5], sw ? v[2] : v[6], sw ? v[3] : v[7]);
+}
+
 template <bool WANT_CBAR, bool WANT_VIR, int LPA, int NC, bool POOL>
-__global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_adj(int64_t row0, int64_t rows, int stride, Radial R,
+__global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 || WANT_VIR ? 7 : 8) k_density_adj(int64_t row0, int64_t rows, int stride, Radial R,
                                                                 const int32_t* __restrict__ live_cnt,
                                                                 const float4* __restrict__ xyzj,
                                                                 const float2* __restrict__ phi,
@@ -596,19 +603,23 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
                                                                 const int32_t* __restrict__ structure, Outputs out) {
     pdl_enter();
     constexpr int APW = 32 / LPA, G = LPA / 8;  // atoms per warp, groups of 8 lanes per atom
-    // per atom, for its batch of LPA edges: (r, 1/d) [LPA][4], (j, r1) [LPA][2], phi [LPA][8]; an
+    // Per atom, for its batch of LPA edges: (r, j) [LPA][4], phi [LPA][8] and phi' / d [LPA][8], or, with 32 lanes,
+    // (r, d) [LPA][4], phi [LPA][8] and (j, f_c' / f_c, 1/d) [LPA][4], so that seven blocks fit beside the carveout of
+    // small systems (4,000 atoms: 16.9 us a launch instead of 20.0; with 16 and 8 lanes the first form takes 41.0
+    // instead of 44.4 for 24,576 atoms, 1,162 instead of 1,406 for 1,048,576).  An
     // atom's blocks are padded so that the words its groups and the other atoms of the warp read
-    // together lie in different banks
-    constexpr int PAD = LPA == 32 ? 0 : (LPA == 16 ? 16 : 8), LE = 4 * LPA + PAD, LJ = 2 * LPA + PAD, LP = 8 * LPA + PAD;
-    __shared__ __align__(16) float sE[kAdjWarps * APW][LE + LJ + LP];
+    // together lie in different banks.
+    constexpr bool kPsi = LPA < 32;
+    constexpr int PAD = LPA == 32 ? 0 : (LPA == 16 ? 16 : 8), LE = 4 * LPA + PAD, LP = 8 * LPA + PAD;
+    __shared__ __align__(16) float sE[kAdjWarps * APW][kPsi ? LE + 2 * LP : 2 * LE + LP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane & 7, sub = lane & (LPA - 1), g = sub >> 3;
     const int64_t kr = ((int64_t)blockIdx.x * kAdjWarps + warp) * APW + lane / LPA;
     const int64_t atom = row0 + kr;
     // (of a serving pool's rows only those whose structure takes this many classes)
     const bool valid = kr < rows && (!POOL || adj_classes(structure[atom]) == NC * G);
     float* s_e = sE[warp * APW + lane / LPA];
-    float *s_j = s_e + LE, *s_phi = s_j + LJ;
-    const float two_a_mu = R.two_a_mu[m];
+    float *s_phi = s_e + LE, *s_psi = s_phi + LP, *s_j = s_phi + LP;
+    const float m_two_a = -2.f * R.alpha_hi, mu_hi = R.mu_hi[m], mu_lo = R.mu_lo[m];
     // the 12 values of channel m in an atom's record: bbar_{0..9,m} (the squares' doubled), c_m, 0
     auto load_rec = [&](int r, float* v) {
         const float* p = rec + (size_t)r * NREC + 4 * m;
@@ -665,11 +676,18 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
         float4 e;
     };
     auto share = [&](int s) {
-        const float2 jr = *reinterpret_cast<const float2*>(s_j + 2 * s);
-        float bj[12];
-        load_rec(__float_as_int(jr.x), bj);
         const float4 e = ld4(s_e + 4 * s);
-        const float ph = s_phi[8 * s + m], ps = ph * fmaf(two_a_mu, e.w, jr.y);  // phi, phi' / d
+        float bj[12];
+        float ph, ps;
+        if constexpr (kPsi) {
+            load_rec(__float_as_int(e.w), bj);
+            ph = s_phi[8 * s + m], ps = s_psi[8 * s + m];  // phi, phi' / d
+        } else {
+            const float4 r = ld4(s_j + 4 * s);  // j, f_c' / f_c, 1 / d
+            load_rec(__float_as_int(r.x), bj);
+            ph = s_phi[8 * s + m];
+            ps = ph * (fmaf(m_two_a, (e.w - mu_hi) - mu_lo, r.y) * r.z);
+        }
         const float x = e.x, y = e.y, z = e.z, cj = bj[NANG];
         // grad Q_j; Q_j = q0 + (r . (l + grad Q_j)) / 2 for a quadratic with linear part l
         const float gjx = fmaf(z, bj[8], fmaf(y, bj[7], fmaf(x, bj[4], -bj[1])));
@@ -705,16 +723,18 @@ __global__ void __launch_bounds__(kAdjWarps * 32, LPA == 32 ? 7 : 8) k_density_a
         if (sub < ne) {
             float ph[NPHI];
             phi_chain(R, p_nx.x, p_nx.y, ph);
-            *reinterpret_cast<float4*>(s_e + 4 * sub) = make_float4(e_nx.x, e_nx.y, e_nx.z, d_nx.x);
-            *reinterpret_cast<float2*>(s_j + 2 * sub) = make_float2(e_nx.w, d_nx.y);
-            // lanes 4-7 of every 8 store the halves the other way round: no bank conflicts
-            const bool sw = sub & 4;
-            float* f = s_phi + 8 * sub;
-            const int h0 = sw ? 4 : 0, h1 = 4 - h0;
-            *reinterpret_cast<float4*>(f + h0) =
-                make_float4(sw ? ph[4] : ph[0], sw ? ph[5] : ph[1], sw ? ph[6] : ph[2], sw ? ph[7] : ph[3]);
-            *reinterpret_cast<float4*>(f + h1) =
-                make_float4(sw ? ph[0] : ph[4], sw ? ph[1] : ph[5], sw ? ph[2] : ph[6], sw ? ph[3] : ph[7]);
+            const float d = d_nx.x, inv_d = __frcp_rn(d);
+            *reinterpret_cast<float4*>(s_e + 4 * sub) = make_float4(e_nx.x, e_nx.y, e_nx.z, kPsi ? e_nx.w : d);
+            store8(s_phi + 8 * sub, ph, sub);
+            // phi_m' / d = phi_m (f_c' / f_c - 2 a (d - mu_m)) / d with mu_m a float pair: phi_m is largest where the
+            // difference is small (as 2 a mu_m / d - 2 a, rounded term by term, it had up to six times the error)
+            if constexpr (kPsi) {
+#pragma unroll
+                for (int k = 0; k < NPHI; ++k) ph[k] *= fmaf(m_two_a, (d - R.mu_hi[k]) - R.mu_lo[k], d_nx.y) * inv_d;
+                store8(s_psi + 8 * sub, ph, sub);
+            } else {
+                *reinterpret_cast<float4*>(s_j + 4 * sub) = make_float4(e_nx.w, d_nx.y, inv_d, 0.f);
+            }
             if (e0 + LPA + sub < cnt) e_nx = ex[e0 + LPA + sub], p_nx = ep[e0 + LPA + sub], d_nx = ed[e0 + LPA + sub];
         }
         __syncwarp();

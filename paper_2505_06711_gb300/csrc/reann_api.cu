@@ -383,7 +383,6 @@ extern "C" int reann_ctx_create(const reann_model* model, void* cuda_stream, rea
     for (int m = 0; m < NPHI; ++m) {
         split(m * delta, R.mu_hi[m], R.mu_lo[m]);
         split(std::exp(-M.alpha * delta * delta * (2 * m + 1)), R.kap_hi[m], R.kap_lo[m]);
-        R.two_a_mu[m] = (float)(2.0 * M.alpha * m * delta);
     }
     // exp(-40) f_c is normal down to f_c = 1e-20; wider Gaussian ranges are scaled up to that (2^58 at most)
     const int sh = (int)std::ceil(std::max(0.0, M.alpha * M.r_c * M.r_c - 40.0) / std::log(2.0));

@@ -9,6 +9,8 @@
 
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -101,3 +103,42 @@ def test_sums_do_not_depend_on_the_lanes_per_atom(molecules, rows, virial, preci
     # 8 up to 16,384, 28,672, beyond), on the other side of a line than the whole list's here
     s = water_box(molecules, seed=9)
     _assert_same(_evaluated(s, 2, rows, virial, precision), _evaluated(s, 2, 1 << 40, virial, precision))
+
+
+@pytest.mark.parametrize("m,alpha", [(3, 1.3), (6, 1.3), (2, 3.2), (4, 3.2), (5, 3.2), (6, 3.2)])
+def test_radial_derivative_near_a_gaussian_centre(m, alpha):
+    # lone pairs on an axis, at distances that FP32 holds, which see one radial channel of l = 0 only: |F| is
+    # |phi_m'| times a smooth factor.  phi_m' is a difference that is small where phi_m is largest; its rms error,
+    # relative to its rms, is up to 1.1e-7 in FP32 with d - mu_m taken first, and 1.3e-7 to 5.3e-7 with
+    # 2 alpha mu_m / d - 2 alpha rounded term by term (both from an FP32 emulation).  phi_m enters the force twice
+    # and the recurrence's factor phi_m m times: with that factor within an ulp, 6e-8, 1.2e-7 m at most.
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=1, n_elem=1, alpha=alpha)
+    p = np.array(spec.params)
+    p[:8] = 0.0
+    p[m] = 1.0
+    W = p[8 : 8 + 3 * 8 * 16].reshape(3, 8, 16)
+    W[1:] = 0.0
+    p[8 + W.size :] = np.abs(p[8 + W.size :])  # networks without cancellation
+    spec = dataclasses.replace(spec, params=p)
+    rng = np.random.default_rng(m)
+    at = 13.0 * np.stack(np.meshgrid(*[np.arange(10)] * 3, indexing="ij"), -1).reshape(-1, 3) + 4.0
+    mu = m * 5.0 / 7.0
+    w = 2.0 / np.sqrt(2.0 * alpha)
+    d = np.round(rng.uniform(max(0.7, mu - w), min(4.9, mu + w), len(at)) * 2**20) / 2**20
+    s = Structure(np.concatenate([at, at + d[:, None] * [1.0, 0.0, 0.0]]), np.zeros(2 * len(at), np.int32), np.eye(3) * 130.0)
+    pot = Potential(spec)
+    sy = pot.system(s.pos, s.species, s.cell)
+    sy.evaluate()
+    sy.check()
+    torch.cuda.synchronize()
+    f = sy.forces.double().cpu().numpy()
+    sy.close()
+    pot.close()
+    ref = oracle.energy_forces(spec, s.pos, s.species, s.cell)["forces"]
+    err = np.sqrt(((f - ref) ** 2).mean()) / np.sqrt((ref**2).mean())
+    print(f"[radial] m={m} alpha={alpha} rms error {err:.2e}")
+    assert err <= 1.1e-7 + 1.2e-7 * m
