@@ -283,10 +283,12 @@ struct NlistScratch {
     float4* p32s = nullptr;  // the same in bin-sorted order, slot index in .w
 };
 
-// A call replayed as a CUDA graph: the arguments it was captured with (key),
+// A call replayed as a CUDA graph: the context (its id: the graph holds the addresses of
+// the context's weights and flags) and arguments it was captured with (key),
 // and whether the same call has run once uncaptured (seen) or cannot be
 // captured (nograph).
 struct GraphSlot {
+    uint64_t ctx = 0;
     const void* key[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     int ikey[4] = {0, 0, 0, 0};
     bool seen = false, nograph = false;
@@ -390,10 +392,12 @@ struct reann_nlist {
     int* md_ints = nullptr;        // [0] rebuild gate, [1] step counter, [2] rebuild count, [3] ticket
     reann::MdOut* md_out = nullptr;  // the current call's output arrays
     bool md_forces_valid = false;
-    const double* md_forces_at = nullptr;  // positions the forces belong to
+    uint64_t md_forces_ctx = 0;            // context and positions the forces belong to
+    const double* md_forces_at = nullptr;
     cudaGraphExec_t md_exec = nullptr, md_exec_many = nullptr;  // one MD step; several in a longer run
     reann::GraphSlot graphs[reann::GS_COUNT];  // rebuild / evaluation calls replayed as graphs
-    const void* md_key[3] = {nullptr, nullptr, nullptr};  // pos, vel, mass of the captured step
+    uint64_t md_ctx = 0;                                  // context of the captured step
+    const void* md_key[3] = {nullptr, nullptr, nullptr};  // and its pos, vel, mass
     double md_dt = 0.0;
     double md_kt = 0.0, md_tau = 0.0;  // thermostat of the captured step (tau 0: NVE)
     int md_precision = -1;         // network precision of md_forces
@@ -415,6 +419,7 @@ struct reann_nlist {
 };
 
 struct reann_ctx {
+    uint64_t id = 0;  // never used again in the process, as an address may be
     reann::Model model;
     cudaStream_t stream = nullptr;
     int device = 0;

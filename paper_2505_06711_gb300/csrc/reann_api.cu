@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -359,6 +360,8 @@ extern "C" int reann_ctx_create(const reann_model* model, void* cuda_stream, rea
     *out = nullptr;
     reann_ctx* ctx = new (std::nothrow) reann_ctx;
     if (!ctx) return REANN_E_NOMEM;
+    static std::atomic<uint64_t> ids{0};
+    ctx->id = ++ids;
     ctx->model = model->m;
     ctx->stream = (cudaStream_t)cuda_stream;
     auto fail = [&](int code) {
@@ -1107,12 +1110,13 @@ int run_graphed(reann_ctx* ctx, reann_nlist* nl, GraphSlotId slot, const void* c
                 F body) {
     if (ctx->prof_on) return body();
     GraphSlot& gs = nl->graphs[slot];
-    const bool same = gs.seen && std::memcmp(gs.key, key, sizeof(gs.key)) == 0 &&
+    const bool same = gs.seen && gs.ctx == ctx->id && std::memcmp(gs.key, key, sizeof(gs.key)) == 0 &&
                       std::memcmp(gs.ikey, ikey, sizeof(gs.ikey)) == 0;
     if (!same) {
         if (gs.exec) cudaGraphExecDestroy(gs.exec);
         if (gs.graph) cudaGraphDestroy(gs.graph);
         gs = GraphSlot{};
+        gs.ctx = ctx->id;
         std::memcpy(gs.key, key, sizeof(gs.key));
         std::memcpy(gs.ikey, ikey, sizeof(gs.ikey));
         gs.seen = true;
@@ -1298,24 +1302,27 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
     }
     int* gate = nl->md_ints;
     // forces at the starting positions (rebuilding first if atoms moved beyond skin/2)
-    if (!nl->md_forces_valid || nl->md_forces_at != pos || nl->md_precision != ctx->precision) {
+    if (!nl->md_forces_valid || nl->md_forces_ctx != ctx->id || nl->md_forces_at != pos ||
+        nl->md_precision != ctx->precision) {
         REANN_CUDA_TRY(ctx, cudaMemsetAsync(gate, 0, sizeof(int), s));
         REANN_CUDA_TRY(ctx, launch_moved(s, nl, pos, gate));
         REANN_CUDA_TRY(ctx, launch_rebuild(s, nl, pos, ctx->d_flags, gate));
         int rc = run_energy_forces(ctx, nl, pos, nl->T, nl->md_scalars, nl->md_forces, nullptr);
         if (rc) return rc;
         nl->md_forces_valid = true;
+        nl->md_forces_ctx = ctx->id;
         nl->md_forces_at = pos;
         nl->md_precision = ctx->precision;
     }
     // the thermostat's first half step needs K of the current velocities
     if (th.on()) REANN_CUDA_TRY(ctx, launch_ekin(s, n, vel, mass, nl->md_partial, nl->md_scalars + 1));
     const void* key[3] = {pos, vel, mass};
-    const bool same = nl->md_exec && std::memcmp(key, nl->md_key, sizeof(key)) == 0 && nl->md_dt == dt &&
+    const bool same = nl->md_exec && nl->md_ctx == ctx->id && std::memcmp(key, nl->md_key, sizeof(key)) == 0 && nl->md_dt == dt &&
                       nl->md_step_precision == ctx->precision && nl->md_kt == th.kt && nl->md_tau == th.tau;
     if (!same) {
         drop_md_graphs(nl);
         if (const int rc = capture_md_steps(ctx, nl, pos, vel, mass, dt, th, 1, &nl->md_exec)) return rc;
+        nl->md_ctx = ctx->id;
         std::memcpy(nl->md_key, key, sizeof(key));
         nl->md_dt = dt;
         nl->md_step_precision = ctx->precision;

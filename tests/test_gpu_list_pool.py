@@ -71,6 +71,54 @@ def test_list_outlives_its_context_and_stream():
     other.close()
 
 
+@pytest.mark.parametrize("close_first", [False, True])
+def test_captured_calls_belong_to_their_context(close_first):
+    # a list's replayed rebuild, evaluation, host callback and MD step hold their context's weights
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+    from synth import MASS_AMU, maxwell_boltzmann
+
+    s = water_box(64, seed=6)
+    mass = torch.as_tensor(MASS_AMU[s.species], device="cuda")
+    vel0 = torch.as_tensor(maxwell_boltzmann(MASS_AMU[s.species], 300.0, seed=1), device="cuda")
+
+    def calls(sy, host, vel):
+        e, f = np.zeros(1), np.zeros((s.n_atoms, 3), np.float32)
+        pos0 = sy.pos.clone()
+        for _ in range(3):  # direct, captured, replayed
+            sy.rebuild()
+            sy.evaluate(virial=True)
+            sy.evaluate_host(host, e, f, rebuild=True)
+        out = [x.cpu().numpy().copy() for x in (sy.energy, sy.forces, sy.virial)] + [e.copy(), f.copy()]
+        for _ in range(2):
+            sy.pos.copy_(pos0)
+            vel.copy_(vel0)
+            e_pot, e_kin = sy.md(vel, mass, 0.25, 6)
+            out += [x.cpu().numpy().copy() for x in (e_pot, e_kin, sy.pos)]
+        sy.check()
+        sy.pos.copy_(pos0)
+        return out
+
+    first, second = (Potential(make_model(T=2, seed=k)) for k in (11, 12))
+    sy = second.system(s.pos, s.species, s.cell)
+    want = calls(sy, s.pos, vel0.clone())
+    sy.close()
+    sy = first.system(s.pos, s.species, s.cell)
+    vel = vel0.clone()
+    other = calls(sy, s.pos, vel)
+    assert not np.array_equal(other[0], want[0])
+    if close_first:
+        first.close()
+    sy.pot = second
+    got = calls(sy, s.pos, vel)
+    for k, (x, y) in enumerate(zip(got, want)):
+        assert np.array_equal(x, y), k
+    sy.close()
+    first.close()
+    second.close()
+
+
 def test_threads_build_and_free_together():
     from paper_2505_06711_gb300 import Potential
 
