@@ -50,7 +50,7 @@ extern "C" {
 
 #define REANN_OK 0
 #define REANN_E_ARG (-1)      /* invalid argument or unsupported model shape  */
-#define REANN_E_MISMATCH (-2) /* r_c or T differs from the model's            */
+#define REANN_E_MISMATCH (-2) /* r_c, T or the model's shape differs          */
 #define REANN_E_NOMEM (-3)    /* device or host allocation failed             */
 #define REANN_E_GEOM (-4)     /* non-finite position, coincident atoms, singular cell */
 #define REANN_E_CUDA (-5)     /* a CUDA runtime call failed                   */

@@ -342,6 +342,7 @@ struct reann_nlist {
     int max_count = 0;                // longest row found by the first build
     int n_elem = 0, T = 0;
     int n_feat = reann::NFEAT;        // features per atom of the model the buffers were sized for
+    int elem_end = 0;                 // 1 + the largest element among the atoms
     double r_c = 0, skin = 0;
     reann::CellGeom geom{};
     int elem_start[reann::MAX_ELEM + 1] = {0};

@@ -1087,6 +1087,8 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
     if (ctx->h_flags[FLAG_SPECIES]) return set_error(ctx, REANN_E_ARG, "species index out of range");
     if (ctx->h_flags[FLAG_GEOM]) return set_error(ctx, REANN_E_GEOM, "non-finite atom position");
     for (int e = 0; e <= nl->n_elem; ++e) nl->elem_start[e] = es[e];
+    for (int e = 0; e < nl->n_elem; ++e)
+        if (es[e + 1] > es[e]) nl->elem_end = e + 1;
     nl->g = G;
     nl->ghosts_by_owner = true;  // k_ghosts enumerates each atom's images contiguously at goff[i]
     // capacity with headroom so that rebuilds after atom motion fit

@@ -765,6 +765,7 @@ int build_decomposed(reann_ctx* ctx, reann_nlist* src, const int32_t ranks[3], r
     nl->r_c = src->r_c;
     nl->skin = src->skin;
     nl->geom = src->geom;
+    nl->elem_end = src->elem_end;
     for (int e = 0; e <= MAX_ELEM; ++e) nl->elem_start[e] = 0;
     nl->decomposed = true;
     for (int k = 0; k < 3; ++k) nl->rank_grid[k] = ranks[k];
@@ -1149,6 +1150,17 @@ int run_graphed(reann_ctx* ctx, reann_nlist* nl, GraphSlotId slot, const void* c
     });
 }
 
+// whether the context's model is one that the list can be evaluated with (its buffers are sized and its
+// elements counted at the build)
+int check_model(reann_ctx* ctx, const reann_nlist* nl, int T) {
+    if (T != ctx->model.T || T != nl->T) return set_error(ctx, REANN_E_MISMATCH, "T differs from the model");
+    if (ctx->model.n_feat() > nl->n_feat)
+        return set_error(ctx, REANN_E_MISMATCH, "the list was built for a model of fewer features");
+    if (ctx->model.n_elem < nl->elem_end)
+        return set_error(ctx, REANN_E_MISMATCH, "the list holds elements that the model does not have");
+    return REANN_OK;
+}
+
 int graphed_rebuild(reann_ctx* ctx, reann_nlist* nl, const double* pos, GraphSlotId slot) {
     if (nl->decomposed) return run_rebuild(ctx, nl, pos);  // refused, with its message
     const void* key[6] = {pos, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -1175,14 +1187,14 @@ extern "C" int reann_nlist_rebuild(reann_ctx* ctx, reann_nlist* nl, const double
 extern "C" int reann_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T, double* energy,
                                    float* forces, float* atom_energy) {
     if (!ctx || !nl || !pos || !energy || !forces) return set_error(ctx, REANN_E_ARG, "null argument");
-    if (T != ctx->model.T || T != nl->T) return set_error(ctx, REANN_E_MISMATCH, "T differs from the model");
+    if (int rc = check_model(ctx, nl, T)) return rc;
     return graphed_eval(ctx, nl, pos, T, energy, forces, atom_energy, nullptr, nullptr, GS_EVAL);
 }
 
 extern "C" int reann_energy_forces_virial(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T, double* energy,
                                           float* forces, float* atom_energy, double* virial, float* atom_virial) {
     if (!ctx || !nl || !pos || !energy || !forces || !virial) return set_error(ctx, REANN_E_ARG, "null argument");
-    if (T != ctx->model.T || T != nl->T) return set_error(ctx, REANN_E_MISMATCH, "T differs from the model");
+    if (int rc = check_model(ctx, nl, T)) return rc;
     if (int rc = ensure_virial(ctx, nl)) return rc;
     return graphed_eval(ctx, nl, pos, T, energy, forces, atom_energy, virial, atom_virial, GS_EVAL);
 }
@@ -1190,7 +1202,7 @@ extern "C" int reann_energy_forces_virial(reann_ctx* ctx, reann_nlist* nl, const
 extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T, double* energy,
                                         float* forces, int rebuild) {
     if (!ctx || !nl || !pos || !energy || !forces) return set_error(ctx, REANN_E_ARG, "null argument");
-    if (T != ctx->model.T || T != nl->T) return set_error(ctx, REANN_E_MISMATCH, "T differs from the model");
+    if (int rc = check_model(ctx, nl, T)) return rc;
     cudaStream_t s = ctx->stream;
     const int64_t n = nl->n;
     if (!nl->h2d_pos) {
@@ -1374,6 +1386,7 @@ int md_entry(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const do
     if (!ctx || !nl || !pos || !vel || !mass || !(dt_fs > 0) || !std::isfinite(dt_fs) || n_steps < 0)
         return set_error(ctx, REANN_E_ARG, "bad argument to reann_md_step");
     if (nl->decomposed) return set_error(ctx, REANN_E_ARG, "MD needs device rebuilds: use a single-domain list");
+    if (int rc = check_model(ctx, nl, nl->T)) return rc;
     if (n_steps == 0) return REANN_OK;
     // run on the graph stream, ordered after and before the caller's stream
     const bool prof = ctx->prof_on;

@@ -119,6 +119,35 @@ def test_captured_calls_belong_to_their_context(close_first):
     second.close()
 
 
+def test_lists_refuse_models_they_were_not_sized_for():
+    import torch
+
+    from paper_2505_06711_gb300 import Potential, binding
+
+    s = water_box(32, seed=7)  # elements 0 and 1
+    pot = Potential(make_model(T=2))
+    sy = pot.system(s.pos, s.species, s.cell)
+    sy.evaluate()
+    vel, mass = torch.zeros_like(sy.pos), torch.ones(s.n_atoms, dtype=torch.float64, device="cuda")
+    e, f = np.zeros(1), np.zeros((s.n_atoms, 3), np.float32)
+    for spec in (make_model(T=2, pairs=True), make_model(T=2, n_elem=1), make_model(T=3)):
+        other = Potential(spec)
+        sy.pot = other
+        for call in (lambda: sy.evaluate(), lambda: sy.evaluate(virial=True), lambda: sy.evaluate_host(s.pos, e, f),
+                     lambda: sy.md(vel, mass, 0.25, 1)):
+            with pytest.raises(binding.ReannError) as err:
+                call()
+            assert err.value.code == binding.REANN_E_MISMATCH
+        other.close()
+    fits = Potential(make_model(T=2, n_elem=2))  # the elements that the list holds
+    sy.pot = fits
+    sy.evaluate()
+    sy.check()
+    sy.close()
+    fits.close()
+    pot.close()
+
+
 def test_threads_build_and_free_together():
     from paper_2505_06711_gb300 import Potential
 
