@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -307,16 +308,30 @@ struct MdOut {
 // kKeep unused bytes and gives everything back with the last of its context and
 // lists (each holds a reference).  Blocks from kBig bytes on come from cudaMalloc as
 // before (the pool maps them more slowly: preparing a 1,048,576-atom list took 226
-// instead of 174 ms).  Blocks are taken on the building context's
-// stream.  They go back on the pool's own stream after a device synchronisation (as
-// cudaFree implies one), so that no stream of the caller needs to outlive a list
-// and a block is never handed on while work of any stream may still use it.
+// instead of 174 ms).  Blocks are taken on the stream of the context that asks
+// for them and go back on the pool's own stream, which first waits for the list's last use by
+// each context (ListUse): no stream of the caller needs to outlive a list, a block is
+// never handed on while a call's work may still use it, and freeing waits for nothing on the
+// host, so it may run while another thread captures a graph (a device synchronisation
+// would invalidate the capture).  Only a list that a caller captured into a graph of its own,
+// whose replays are not known here, is freed after a device synchronisation; where that is
+// refused its blocks wait for the next such try, the pool's end at the latest.
 struct ListPool {
     static constexpr uint64_t kKeep = 512ull << 20, kBig = 64ull << 20;
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
+    int device = 0;
+    std::mutex mu;
+    std::vector<void*> late;  // blocks still to be given back
+    bool wait_for_device();   // false when the device cannot be synchronised now
+    void give_late();
     static std::shared_ptr<ListPool> create();  // null when the device has no memory pools
     ~ListPool();
+};
+// The end of a list's last use by a context
+struct ListUse {
+    uint64_t ctx;
+    cudaEvent_t done;
 };
 enum GraphSlotId { GS_REBUILD = 0, GS_EVAL, GS_HOST_REBUILD, GS_HOST_EVAL, GS_COUNT };
 
@@ -412,11 +427,14 @@ struct reann_nlist {
     std::vector<void*> allocs, big_allocs;  // blocks of mem_pool (null: cudaMalloc); cudaMalloc blocks beside a list_pool
     // stream-ordered allocation: blocks come from mem_pool on alloc_stream.  Serving
     // builds return them with cudaFreeAsync on the same stream, so neither side waits
-    // for unrelated device work; other lists as described at ListPool (list_pool set).
+    // for unrelated device work; other lists as described at ListPool (list_pool set; alloc_stream is
+    // then the stream of the call that allocates).
     // Null mem_pool: cudaMalloc / cudaFree.
     std::shared_ptr<reann::ListPool> list_pool;
     cudaMemPool_t mem_pool = nullptr;
     cudaStream_t alloc_stream = nullptr;
+    std::vector<reann::ListUse> uses;  // with list_pool
+    bool unknown_use = false;          // used under a caller's capture, or in a way that could not be recorded
 };
 
 struct reann_ctx {
@@ -545,6 +563,7 @@ cudaError_t launch_moved(cudaStream_t s, const reann_nlist* nl, const double* po
 // serving pool (serve.cu)
 cudaError_t launch_pack(cudaStream_t s, const reann_nlist* src, const double* caller_pos, reann_nlist* pool,
                         int64_t ob, int64_t gb);
+bool capturing(cudaStream_t s);  // also when it cannot be told
 void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes);
 void nlist_free_block(reann_nlist* nl, void* p);  // a block that nothing on the device uses yet
 template <typename T>

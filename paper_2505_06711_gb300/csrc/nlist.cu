@@ -940,19 +940,18 @@ static cudaError_t counting_sort(cudaStream_t s, const int* gate, int64_t n, con
 void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes) {
     void* p = nullptr;
     bytes = std::max<size_t>(bytes, 1);
-    const bool big = nl->list_pool && bytes >= ListPool::kBig;
+    // (a block taken from the pool under capture would belong to the graph)
+    const bool big = nl->list_pool && (bytes >= ListPool::kBig || capturing(nl->alloc_stream));
     auto take = [&] {
         return nl->mem_pool && !big ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream) : cudaMalloc(&p, bytes);
     };
     cudaError_t e = take();
     if (e != cudaSuccess && nl->list_pool) {  // give the pool's unused blocks back and try again
         (void)cudaGetLastError();
+        cudaStreamSynchronize(nl->list_pool->stream);  // (what is on its way back)
         cudaMemPoolTrimTo(nl->mem_pool, 0);
         e = take();
     }
-    // after the build the block may be used on any stream
-    if (e == cudaSuccess && !big && nl->list_pool && nl->alloc_stream == nl->list_pool->stream)
-        e = cudaStreamSynchronize(nl->alloc_stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return nullptr;

@@ -41,6 +41,7 @@ std::shared_ptr<reann::ListPool> reann::ListPool::create() {
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     uint64_t keep = kKeep;
+    p->device = dev;
     if (cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMemPoolCreate(&p->pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
@@ -50,7 +51,42 @@ std::shared_ptr<reann::ListPool> reann::ListPool::create() {
     return p;
 }
 
+bool reann::ListPool::wait_for_device() {
+    int dev = 0;
+    const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != device;
+    if (other) cudaSetDevice(device);
+    const bool ok = cudaDeviceSynchronize() == cudaSuccess;
+    if (!ok) (void)cudaGetLastError();
+    if (other) cudaSetDevice(dev);
+    return ok;
+}
+
+void reann::ListPool::give_late() {
+    std::vector<void*> blocks;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        blocks.swap(late);
+    }
+    if (blocks.empty()) return;
+    if (wait_for_device()) {
+        for (void* p : blocks) cudaFreeAsync(p, stream);
+    } else {
+        std::lock_guard<std::mutex> lock(mu);
+        late.insert(late.end(), blocks.begin(), blocks.end());
+    }
+}
+
+bool reann::capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 reann::ListPool::~ListPool() {
+    give_late();
     if (stream) cudaStreamSynchronize(stream);
     if (pool) cudaMemPoolDestroy(pool);
     if (stream) cudaStreamDestroy(stream);
@@ -211,13 +247,23 @@ void free_nlist(reann_nlist* nl) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         if (g.graph) cudaGraphDestroy(g.graph);
     }
-    bool idle = true;  // (as with cudaFree, nothing is given back where the device cannot be waited for)
-    if (nl->list_pool) {
-        idle = cudaDeviceSynchronize() == cudaSuccess;
-        nl->alloc_stream = nl->list_pool->stream;
+    if (ListPool* pool = nl->list_pool.get()) {
+        bool ordered = !nl->unknown_use;
+        for (const ListUse& u : nl->uses) {
+            ordered = cudaStreamWaitEvent(pool->stream, u.done, 0) == cudaSuccess && ordered;
+            cudaEventDestroy(u.done);
+        }
+        nl->alloc_stream = pool->stream;
+        pool->give_late();
+        if (!ordered) {
+            (void)cudaGetLastError();
+            std::lock_guard<std::mutex> lock(pool->mu);
+            pool->late.insert(pool->late.end(), nl->allocs.begin(), nl->allocs.end());
+            nl->allocs.clear();
+        }
+        if (!ordered) pool->give_late();
     }
     for (void* p : nl->allocs) {
-        if (!idle) break;
         if (nl->mem_pool)
             cudaFreeAsync(p, nl->alloc_stream);
         else
@@ -546,6 +592,34 @@ extern "C" const char* reann_last_error(const reann_ctx* ctx) { return ctx ? ctx
 
 namespace {
 
+// Ends with the list's use by a call of the context: on its stream, everything that the call enqueued.
+// Also sets the stream that the call's blocks are taken on.
+struct UseScope {
+    reann_ctx* ctx;
+    reann_nlist* nl;
+    bool over = false;  // the call has waited for its stream
+    UseScope(reann_ctx* c, const reann_nlist* l) : ctx(c), nl(const_cast<reann_nlist*>(l)) {
+        if (nl->list_pool) nl->alloc_stream = ctx->stream;
+    }
+    ~UseScope() {
+        if (!nl->list_pool || over) return;
+        if (!capturing(ctx->stream)) {
+            for (const ListUse& u : nl->uses)
+                if (u.ctx == ctx->id) {
+                    nl->unknown_use |= cudaEventRecord(u.done, ctx->stream) != cudaSuccess;
+                    return;
+                }
+            ListUse u{ctx->id, nullptr};
+            if (cudaEventCreateWithFlags(&u.done, cudaEventDisableTiming) == cudaSuccess) {
+                nl->uses.push_back(u);
+                nl->unknown_use |= cudaEventRecord(u.done, ctx->stream) != cudaSuccess;
+                return;
+            }
+        }
+        nl->unknown_use = true;
+    }
+};
+
 // enqueue the read-back of the device flags and their reset on the context stream
 int enqueue_flags_readback(reann_ctx* ctx, const double* energy = nullptr) {
     REANN_CUDA_TRY(ctx, launch_take_flags(ctx->stream, ctx->d_flags, energy, ctx->h_flags));
@@ -611,10 +685,9 @@ int build_list(reann_ctx* ctx, int64_t n_atoms, const double* pos, const int32_t
     int rc = make_geometry(ctx, cell, r_c + skin, &nl->geom);
     if (!rc) rc = build_nlist_device(ctx, nl, pos, species);
     if (!rc && eval_buffers) rc = alloc_eval_buffers(ctx, nl);
-    if (!rc && nl->list_pool) {  // from here on the list's memory is valid on every stream
-        if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = set_error(ctx, REANN_E_CUDA, "list build failed");
-        nl->alloc_stream = nl->list_pool->stream;
-    }
+    // from here on the list's memory is valid on every stream
+    if (!rc && nl->list_pool && cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+        rc = set_error(ctx, REANN_E_CUDA, "list build failed");
     if (rc) {
         cudaStreamSynchronize(ctx->stream);
         free_nlist(nl);
@@ -878,6 +951,7 @@ extern "C" int reann_nlist_info(const reann_nlist* nl, int64_t* n_atoms, int64_t
 extern "C" int reann_nlist_export(reann_ctx* ctx, const reann_nlist* nl, int64_t cap, int32_t* i, int32_t* j,
                                   int32_t* n, int64_t* count) {
     if (!ctx || !nl || !count || cap < 0 || (cap > 0 && (!i || !j || !n))) return REANN_E_ARG;
+    UseScope use(ctx, nl);
     return export_nlist(ctx, nl, cap, i, j, n, count);
 }
 
@@ -1096,8 +1170,10 @@ int on_graph_stream(reann_ctx* ctx, F fn) {
     ctx->stream = ctx->md_stream;
     const int rc = fn();
     ctx->stream = user;
-    REANN_CUDA_TRY(ctx, cudaEventRecord(ctx->md_ev[1], ctx->md_stream));
-    REANN_CUDA_TRY(ctx, cudaStreamWaitEvent(user, ctx->md_ev[1], 0));
+    cudaError_t e = cudaEventRecord(ctx->md_ev[1], ctx->md_stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(user, ctx->md_ev[1], 0);
+    if (e != cudaSuccess) cudaStreamSynchronize(ctx->md_stream);  // nothing of the call stays unordered
+    REANN_CUDA_TRY(ctx, e);
     return rc;
 }
 
@@ -1181,6 +1257,7 @@ int graphed_eval(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T, doub
 
 extern "C" int reann_nlist_rebuild(reann_ctx* ctx, reann_nlist* nl, const double* pos) {
     if (!ctx || !nl || !pos) return set_error(ctx, REANN_E_ARG, "null argument");
+    UseScope use(ctx, nl);
     return graphed_rebuild(ctx, nl, pos, GS_REBUILD);
 }
 
@@ -1188,6 +1265,7 @@ extern "C" int reann_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double
                                    float* forces, float* atom_energy) {
     if (!ctx || !nl || !pos || !energy || !forces) return set_error(ctx, REANN_E_ARG, "null argument");
     if (int rc = check_model(ctx, nl, T)) return rc;
+    UseScope use(ctx, nl);
     return graphed_eval(ctx, nl, pos, T, energy, forces, atom_energy, nullptr, nullptr, GS_EVAL);
 }
 
@@ -1195,6 +1273,7 @@ extern "C" int reann_energy_forces_virial(reann_ctx* ctx, reann_nlist* nl, const
                                           float* forces, float* atom_energy, double* virial, float* atom_virial) {
     if (!ctx || !nl || !pos || !energy || !forces || !virial) return set_error(ctx, REANN_E_ARG, "null argument");
     if (int rc = check_model(ctx, nl, T)) return rc;
+    UseScope use(ctx, nl);
     if (int rc = ensure_virial(ctx, nl)) return rc;
     return graphed_eval(ctx, nl, pos, T, energy, forces, atom_energy, virial, atom_virial, GS_EVAL);
 }
@@ -1203,6 +1282,7 @@ extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const d
                                         float* forces, int rebuild) {
     if (!ctx || !nl || !pos || !energy || !forces) return set_error(ctx, REANN_E_ARG, "null argument");
     if (int rc = check_model(ctx, nl, T)) return rc;
+    UseScope use(ctx, nl);
     cudaStream_t s = ctx->stream;
     const int64_t n = nl->n;
     if (!nl->h2d_pos) {
@@ -1231,6 +1311,7 @@ extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const d
     REANN_CUDA_TRY(ctx, cudaMemcpyAsync(forces, nl->d_forces, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
     if (int rc2 = enqueue_flags_readback(ctx, nl->d_energy)) return rc2;  // energy and flags come back with the forces:
     REANN_CUDA_TRY(ctx, cudaStreamSynchronize(s));                         // one synchronisation per call
+    use.over = true;
     std::memcpy(energy, ctx->h_flags + NFLAGS, sizeof(double));
     return flags_status(ctx);
 }
@@ -1300,6 +1381,7 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
     cudaStream_t s = ctx->stream;
     const int64_t n = nl->n;
     if (!nl->md_forces) {
+        if (nl->list_pool) nl->alloc_stream = s;
         nl->md_forces = nl_alloc<float>(nl, 3 * n);
         nl->md_scalars = nl_alloc<double>(nl, 8);
         nl->md_partial = nl_alloc<double>(nl, std::max<int64_t>((n + 2047) / 2048, md_partials(n)));
@@ -1388,6 +1470,7 @@ int md_entry(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const do
     if (nl->decomposed) return set_error(ctx, REANN_E_ARG, "MD needs device rebuilds: use a single-domain list");
     if (int rc = check_model(ctx, nl, nl->T)) return rc;
     if (n_steps == 0) return REANN_OK;
+    UseScope use(ctx, nl);
     // run on the graph stream, ordered after and before the caller's stream
     const bool prof = ctx->prof_on;
     ctx->prof_on = false;
@@ -1440,6 +1523,7 @@ extern "C" int reann_ctx_profile_read(reann_ctx* ctx, double* total_ms, int64_t*
 
 extern "C" int reann_get_layer(reann_ctx* ctx, const reann_nlist* nl, int layer, float* rho, float* coef) {
     if (!ctx || !nl || layer < 0 || layer >= nl->T) return set_error(ctx, REANN_E_ARG, "bad layer");
+    UseScope use(ctx, nl);
     const int64_t n = nl->n, ne = nl->n + nl->g_cap;
     if (rho)
         REANN_CUDA_TRY(ctx, launch_unpermute_rows(ctx->stream, nl, nl->rho + (size_t)layer * n * nl->n_feat, nl->n_feat,

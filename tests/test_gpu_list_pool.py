@@ -16,11 +16,12 @@ from synth import fcc_box, make_model, water_box
 pytestmark = pytest.mark.gpu
 
 
-def _evaluate(pot, s):
+def _evaluate(pot, s, times=1):
     import torch
 
     sy = pot.system(s.pos, s.species, s.cell)
-    sy.evaluate(virial=True)
+    for _ in range(times):
+        sy.evaluate(virial=True)
     sy.check()
     out = float(sy.energy), sy.forces.cpu().numpy().copy(), sy.virial.cpu().numpy().copy()
     sy.close()
@@ -165,7 +166,7 @@ def test_threads_build_and_free_together():
         with torch.cuda.stream(stream):
             mine = Potential(spec, stream=stream)
             for _ in range(6):
-                got = _evaluate(mine, boxes[k])
+                got = _evaluate(mine, boxes[k], 4)  # direct, captured, replayed: while others free
                 if not _same(got, want[k]):
                     bad.append(k)
             mine.close()
@@ -176,3 +177,118 @@ def test_threads_build_and_free_together():
     for t in threads:
         t.join()
     assert not bad
+
+
+def test_freeing_while_another_thread_captures():
+    # freeing a list must neither invalidate the capture nor keep the list's memory
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=3)
+    s = fcc_box(20, seed=8)  # 32,000 atoms: about 0.4 GB in blocks of the pool and larger ones
+    warm = Potential(spec)
+    _evaluate(warm, fcc_box(3, seed=4))
+    warm.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    pot = Potential(spec)
+    sy = pot.system(s.pos, s.species, s.cell)
+    sy.evaluate()
+    x = torch.zeros(1000, device="cuda")
+    torch.cuda.synchronize()
+    begun, freed, errors = threading.Event(), threading.Event(), []
+    graph = torch.cuda.CUDAGraph()
+
+    def capture():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                graph.capture_begin(capture_error_mode="thread_local")
+                x.add_(1.0)
+                begun.set()
+                freed.wait(60)
+                x.mul_(2.0)
+                graph.capture_end()
+        except Exception as exc:  # pragma: no cover - the fault this test is for
+            errors.append(exc)
+            begun.set()
+
+    t = threading.Thread(target=capture)
+    t.start()
+    begun.wait(60)
+    sy.close()
+    freed.set()
+    t.join()
+    assert not errors, errors
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 2000.0
+    pot.close()
+    del sy, graph, x
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert torch.cuda.mem_get_info()[0] >= before - (64 << 20)
+
+
+def test_freeing_behind_work_in_flight():
+    # nothing waits on the host between a list's work, its release and the next list in the same blocks
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+    from synth import MASS_AMU
+
+    spec = make_model(T=3)
+    boxes = [water_box(400, seed=9), fcc_box(7, seed=10)]
+    pot = Potential(spec)
+
+    def run(s, steps):
+        sy = pot.system(s.pos, s.species, s.cell)
+        mass = torch.as_tensor(MASS_AMU[s.species], device="cuda")
+        vel = torch.zeros_like(sy.pos)
+        sy.evaluate(virial=True)
+        e_pot, _ = sy.md(vel, mass, 0.25, steps)
+        sy.evaluate()
+        out = e_pot, sy.energy, sy.forces, sy.virial, sy.pos
+        sy.close()
+        return out
+
+    want = []
+    for s in boxes:
+        got = run(s, 40)
+        torch.cuda.synchronize()
+        want.append([t.cpu().numpy() for t in got])
+    got = [run(s, 40) for _ in range(4) for s in boxes]
+    for k, g in enumerate(got):
+        assert all(np.array_equal(t.cpu().numpy(), w) for t, w in zip(g, want[k % 2])), k
+    pot.close()
+
+
+def test_list_in_a_callers_graph():
+    # replays of a caller's own graph are not known to the list: freeing it waits for the device
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+
+    spec = make_model(T=2)
+    s = water_box(300, seed=11)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        pot = Potential(spec, stream=stream)
+        want = _evaluate(pot, s)
+        sy = pot.system(s.pos, s.species, s.cell)
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        graph.capture_begin(capture_error_mode="thread_local")
+        sy.evaluate()
+        graph.capture_end()
+        for _ in range(20):
+            graph.replay()
+        energy, forces = sy.energy, sy.forces
+        sy.close()
+        other = pot.system(s.pos[::-1].copy(), s.species[::-1].copy(), s.cell)
+        other.evaluate()
+        torch.cuda.synchronize()
+        assert float(energy) == want[0] and np.array_equal(forces.cpu().numpy(), want[1])
+        other.close()
+        pot.close()
