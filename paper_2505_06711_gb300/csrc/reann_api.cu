@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "memory.h"
 
 using namespace reann;
 
@@ -167,21 +168,29 @@ T* nl_alloc(reann_nlist* nl, size_t count) {
     return nlist_alloc<T>(nl, count);
 }
 
-// Edge records (32 B per row entry) of `rows` rows, or of the largest half, quarter, ... of
-// them that device memory has room for (at least 1,024 rows): an evaluation then recomputes
-// the records of one run of rows at a time in every pass instead of keeping all of them.
+// Blocks of a list, all or none
+template <class MakeRoom>
+bool take_blocks(reann_nlist* nl, std::initializer_list<Block> want, MakeRoom make_room) {
+    return take_all(
+        want, [&](size_t bytes) { return nlist_alloc_bytes(nl, bytes); }, [&](void* p) { nlist_free_block(nl, p); },
+        make_room);
+}
+
+// Edge records (32 B per row entry) of `rows` rows, or of fewer where device memory is short (edge_rows_within;
+// false: not even the fewest)
 bool alloc_edge_records(reann_nlist* nl, int64_t rows) {
+    constexpr size_t kEntry = sizeof(float4) + 2 * sizeof(float2);
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess)
+        rows = edge_rows_within(rows, kEntry * nl->stride, kLaterBytesPerAtom * (uint64_t)nl->n, free_bytes);
     for (;;) {
         const size_t count = (size_t)rows * nl->stride;
-        nl->edge_xyzj = nl_alloc<float4>(nl, count);
-        nl->edge_phi = nl->edge_xyzj ? nl_alloc<float2>(nl, count) : nullptr;
-        nl->edge_der = nl->edge_phi ? nl_alloc<float2>(nl, count) : nullptr;
         nl->edge_rows = rows;
-        if (nl->edge_der) return true;
-        if (nl->edge_phi) nlist_free_block(nl, nl->edge_phi);
-        if (nl->edge_xyzj) nlist_free_block(nl, nl->edge_xyzj);
-        if (rows <= 1024) return false;
-        rows = std::max<int64_t>(1024, (rows + 1) / 2);
+        if (take_blocks(nl, {{&nl->edge_xyzj, count * sizeof(float4)}, {&nl->edge_phi, count * sizeof(float2)},
+                             {&nl->edge_der, count * sizeof(float2)}}, [] { return false; }))
+            return true;
+        if (rows <= kMinEdgeRows) return false;
+        rows = fewer_edge_rows(rows);
     }
 }
 
@@ -240,13 +249,35 @@ void drop_md_graphs(reann_nlist* nl) {
     nl->md_exec = nl->md_exec_many = nullptr;
 }
 
-void free_nlist(reann_nlist* nl) {
-    if (!nl) return;
+void drop_graphs(reann_nlist* nl) {
     drop_md_graphs(nl);
     for (GraphSlot& g : nl->graphs) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         if (g.graph) cudaGraphDestroy(g.graph);
+        g = GraphSlot{};
     }
+}
+
+// Room for a later block of the list: half of its edge records go, once their last use is over, and the
+// graphs that hold their addresses with them.  False: none to spare.
+bool halve_edge_records(reann_ctx* ctx, reann_nlist* nl) {
+    if (nl->edge_rows <= kMinEdgeRows || !nl->edge_der || nl->unknown_use || capturing(ctx->stream)) return false;
+    for (const ListUse& u : nl->uses)
+        if (cudaEventSynchronize(u.done) != cudaSuccess) return false;
+    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return false;
+    drop_graphs(nl);
+    for (void* p : {(void*)nl->edge_xyzj, (void*)nl->edge_phi, (void*)nl->edge_der}) nlist_free_block(nl, p);
+    return alloc_edge_records(nl, fewer_edge_rows(nl->edge_rows));
+}
+
+// blocks that a call needs after the build
+bool take_later(reann_ctx* ctx, reann_nlist* nl, std::initializer_list<Block> want) {
+    return take_blocks(nl, want, [&] { return halve_edge_records(ctx, nl); });
+}
+
+void free_nlist(reann_nlist* nl) {
+    if (!nl) return;
+    drop_graphs(nl);
     if (ListPool* pool = nl->list_pool.get()) {
         bool ordered = !nl->unknown_use;
         for (const ListUse& u : nl->uses) {
@@ -1025,6 +1056,7 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
     }
     // live edges and their records: once for all passes, or, when the records of only a part of
     // the rows fit, before each pass for one run of rows at a time
+    if (!nl->edge_der) return set_error(ctx, REANN_E_NOMEM, "edge records: out of device memory");
     const int64_t nr = rows_of(nl);
     const bool keep_edges = nr <= nl->edge_rows;
     auto edges = [&](int64_t row0, int64_t rows) -> int {
@@ -1140,9 +1172,9 @@ int run_energy_forces(reann_ctx* ctx, reann_nlist* nl, const double* pos, int T,
 
 int ensure_virial(reann_ctx* ctx, reann_nlist* nl) {
     if (nl->vir) return REANN_OK;
-    nl->vir = nl_alloc<float>(nl, (size_t)nl->n * 9);
-    nl->vir_partial = nl_alloc<double>(nl, (size_t)virial_partials(nl->n));
-    if (!nl->vir || !nl->vir_partial) return set_error(ctx, REANN_E_NOMEM, "virial buffers: out of device memory");
+    if (!take_later(ctx, nl, {{&nl->vir, sizeof(float) * 9 * nl->n},
+                              {&nl->vir_partial, sizeof(double) * virial_partials(nl->n)}}))
+        return set_error(ctx, REANN_E_NOMEM, "virial buffers: out of device memory");
     return REANN_OK;
 }
 
@@ -1285,12 +1317,10 @@ extern "C" int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const d
     UseScope use(ctx, nl);
     cudaStream_t s = ctx->stream;
     const int64_t n = nl->n;
-    if (!nl->h2d_pos) {
-        nl->h2d_pos = nl_alloc<double>(nl, 3 * n);
-        nl->d_forces = nl_alloc<float>(nl, 3 * n);
-        nl->d_energy = nl_alloc<double>(nl, 1);
-        if (!nl->h2d_pos || !nl->d_forces || !nl->d_energy) return set_error(ctx, REANN_E_NOMEM, "staging buffers");
-    }
+    if (!nl->h2d_pos && !take_later(ctx, nl, {{&nl->h2d_pos, sizeof(double) * 3 * n},
+                                              {&nl->d_forces, sizeof(float) * 3 * n},
+                                              {&nl->d_energy, sizeof(double)}}))
+        return set_error(ctx, REANN_E_NOMEM, "staging buffers");
     REANN_CUDA_TRY(ctx, cudaMemcpyAsync(nl->h2d_pos, pos, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s));
     if (rebuild) {
         int rc = graphed_rebuild(ctx, nl, nl->h2d_pos, GS_HOST_REBUILD);
@@ -1382,15 +1412,13 @@ int md_run(reann_ctx* ctx, reann_nlist* nl, double* pos, double* vel, const doub
     const int64_t n = nl->n;
     if (!nl->md_forces) {
         if (nl->list_pool) nl->alloc_stream = s;
-        nl->md_forces = nl_alloc<float>(nl, 3 * n);
-        nl->md_scalars = nl_alloc<double>(nl, 8);
-        nl->md_partial = nl_alloc<double>(nl, std::max<int64_t>((n + 2047) / 2048, md_partials(n)));
-        nl->md_ints = nl_alloc<int>(nl, 4);
-        nl->md_out = nl_alloc<MdOut>(nl, 1);
-        if (!nl->md_forces || !nl->md_scalars || !nl->md_partial || !nl->md_ints || !nl->md_out) {
-            nl->md_forces = nullptr;  // (what was allocated goes with the list)
+        if (!take_later(ctx, nl,
+                        {{&nl->md_forces, sizeof(float) * 3 * n},
+                         {&nl->md_scalars, sizeof(double) * 8},
+                         {&nl->md_partial, sizeof(double) * std::max<int64_t>((n + 2047) / 2048, md_partials(n))},
+                         {&nl->md_ints, sizeof(int) * 4},
+                         {&nl->md_out, sizeof(MdOut)}}))
             return set_error(ctx, REANN_E_NOMEM, "MD buffers: out of device memory");
-        }
         REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_ints, 0, 4 * sizeof(int), s));
         REANN_CUDA_TRY(ctx, cudaMemsetAsync(nl->md_scalars, 0, 8 * sizeof(double), s));  // xi = eta = 0
     }

@@ -292,3 +292,52 @@ def test_list_in_a_callers_graph():
         assert float(energy) == want[0] and np.array_equal(forces.cpu().numpy(), want[1])
         other.close()
         pot.close()
+
+
+def test_edge_records_leave_room():
+    # with little device memory left a list keeps fewer edge records: its later calls, and others, find room, and
+    # the results are the same
+    import torch
+
+    from paper_2505_06711_gb300 import Potential
+    from synth import MASS_AMU
+
+    spec = make_model(T=2)
+    s = fcc_box(24, seed=12)  # 55,296 atoms, about 0.25 GB of edge records
+    mass = torch.as_tensor(MASS_AMU[s.species], device="cuda")
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    def calls(sy):
+        out = []
+        for _ in range(3):
+            sy.evaluate(virial=True)
+        out += [x.cpu().numpy().copy() for x in (sy.energy, sy.forces, sy.virial)]
+        e, f = np.zeros(1), np.zeros((s.n_atoms, 3), np.float32)
+        sy.evaluate_host(s.pos, e, f)
+        e_pot, _ = sy.md(torch.zeros_like(sy.pos), mass, 0.25, 3)
+        sy.check()
+        return out + [e, f, e_pot.cpu().numpy()]
+
+    for _ in range(2):  # (the first list also loads the kernels)
+        pot = Potential(spec)
+        start = free()
+        sy = pot.system(s.pos, s.species, s.cell)
+        used = start - free()
+        want = calls(sy)
+        sy.close()
+        pot.close()
+    pot = Potential(spec)
+    fill = torch.empty(free() - used - (40 << 20), dtype=torch.uint8, device="cuda")
+    sy = pot.system(s.pos, s.species, s.cell)
+    left = free()
+    print(f"[room] used {used >> 20} MiB, left {left >> 20} MiB")
+    assert left >= 100 << 20
+    for k, (x, y) in enumerate(zip(calls(sy), want)):
+        assert np.array_equal(x, y), k
+    sy.close()
+    pot.close()
+    del fill
