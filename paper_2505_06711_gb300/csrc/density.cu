@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
 // a third as long against fewer registers.  us per launch with 12 / 4: 192 atoms 6.2 / 8.8, 3,069 8.3 /
 // 11.7, 10,976 21.7 / 22.2, 16,200 24.7 / 22.9, 256,000 181 / 130.  The block's
 // kBbarAtoms records are staged in shared memory and stored as whole lines.
-constexpr int kBbarAtoms = 16;  // small blocks (64 threads): 4x finer balancing than 64 atoms, ~1.5 % per BF16 step
+constexpr int kBbarAtoms = 16;  // small blocks (192 or 64 threads) balance better over the SMs than 64 atoms each
 template <int TPA>
 __global__ void __launch_bounds__(TPA * kBbarAtoms) k_bbar(int64_t n, const float* __restrict__ Wt,
                                                                 const float* __restrict__ bck,

@@ -156,22 +156,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 32 consecutive FP32 columns of this thread's TMEM lane (one load, one wait)
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // TMEM address of lane quarter q (a warp's w % 4), column col
 __device__ __forceinline__ uint32_t lane_addr(uint32_t tmem, int q, int col) {
     return tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)col;
@@ -369,14 +353,11 @@ struct Part {
             __syncthreads();
         }
     }
-    // after `done` of the two exchanges
-    __device__ static void finish(int done) {
-        if (!SPLIT) return;
-        if (done == 0) wait();
-        for (; done < 2; ++done) {
-            arrive();
-            wait();
-        }
+    // after the first of the two exchanges, or both
+    __device__ static void finish(bool both) {
+        if (!SPLIT || both) return;
+        arrive();
+        wait();
     }
 };
 
@@ -858,7 +839,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         v[i] = valid ? u * sd[i] : 0.f;
     }
     tile_mean64(v, part, 0, par + B_PS, par + B_VB2, q, c0, lane, inv_n);
-    int means = 1;
+    bool both_means = false;
     wq_part<H2>(wq, par + B_VB2, par + B_ZP);  // u2-hat partials (summed after the next barrier)
     lds16(par + B_VB2 + c0, a);
 #pragma unroll
@@ -895,7 +876,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         WQ<H1> wq1;  // this thread's eighth of W1^T for rhobar-hat = v1-bar W1^T
         wq_load<H1>(wq1, w.W1t, NFEAT, NFEAT);
         tile_mean64(v, part, 1, par + B_PS2, par + B_VB1, q, c0, lane, inv_n);
-        ++means;
+        both_means = true;
         wq_part<H1>(wq1, par + B_VB1, par + B_ZP);
         lds16(par + B_VB1 + c0, ub);
 #pragma unroll
@@ -943,7 +924,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tc_bwd(TcLayer nets, const Tile
         __syncthreads();
         flush_rec(sRec, nrows, tl.row0 + part.row0(), rec, gh, tid, kThreads);  // ghost images get the rows' records too
     }
-    part.finish(means);
+    part.finish(both_means);
     teardown(tmem);
 }
 

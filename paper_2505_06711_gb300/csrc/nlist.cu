@@ -988,8 +988,7 @@ static int64_t ext_bins(const reann_nlist* nl) {
 }
 
 // steps 1-3a: wrap, sort, gather, ghost count + scan (goff[n] = ghost count on the device)
-// sort_gate: the sort path (nullptr: always); keep_gate: the keep-order path (nullptr:
-// never); gate: the rest of the rebuild (nullptr: always)
+// gate: nothing is done where it is zero (nullptr: always run)
 // first: the list's first build, which sorts
 static cudaError_t stage_sort_and_count(cudaStream_t s, reann_nlist* nl, const double* pos, int* flags,
                                         const int* gate, bool first) {
@@ -1089,7 +1088,7 @@ int build_nlist_device(reann_ctx* ctx, reann_nlist* nl, const double* pos, const
     for (int e = 0; e < nl->n_elem; ++e)
         if (es[e + 1] > es[e]) nl->elem_end = e + 1;
     nl->g = G;
-    nl->ghosts_by_owner = true;  // k_ghosts enumerates each atom's images contiguously at goff[i]
+    nl->ghosts_by_owner = true;  // k_ghosts_ext enumerates each atom's images contiguously at goff[i]
     // capacity with headroom so that rebuilds after atom motion fit
     nl->g_cap = G + G / 4 + 64;
     const int64_t next = n + nl->g_cap;

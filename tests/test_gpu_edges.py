@@ -33,6 +33,18 @@ def test_lane_layouts(make):
     assert_parity(gpu_eval(spec, s), oracle.energy_forces(spec, s.pos, s.species, s.cell), s.n_atoms)
 
 
+def test_many_rows():
+    # beyond 65,536 rows the forward pass prefetches its records; a supercell repeats its cell's forces
+    spec = make_model(T=2)
+    one = fcc_box(13, seed=7)
+    shift = np.stack(np.meshgrid(*[np.arange(2)] * 3, indexing="ij"), -1).reshape(-1, 1, 3) @ one.cell
+    s = Structure((one.pos + shift).reshape(-1, 3), np.tile(one.species, 8), 2 * one.cell)
+    assert s.n_atoms > 1 << 16
+    ref = gpu_eval(spec, one)
+    assert_parity(gpu_eval(spec, s), {"energy": 8 * ref["energy"], "forces": np.tile(ref["forces"], (8, 1)),
+                                      "atom_energy": np.tile(ref["atom_energy"], 8)}, s.n_atoms)
+
+
 def test_short_rows():
     pos = np.array([[1.0, 1.0, 1.0], [1.0, 1.0, 5.9], [20.0, 20.0, 20.0], [30.0, 30.0, 30.0], [31.1, 30.2, 30.3],
                     [39.9, 10.0, 10.0], [0.4, 10.0, 10.0]])

@@ -26,6 +26,7 @@ CASES = {
     "cu4000-T3": (lambda: fcc_box(10, seed=0), 3, 3),
     "cu4000-T5": (lambda: fcc_box(10, seed=0), 5, 3),
     "hea4000-T3": (lambda: hea_box(10, seed=0), 3, 8),
+    "cu32000-T2": (lambda: fcc_box(20, seed=0), 2, 3),  # beyond 28,672 atoms the reverse pass has 8 lanes per atom
 }
 
 
