@@ -78,12 +78,12 @@ BYTES_PER_ATOM_EDGE_FIXED = {"density_fwd": 16 + 32 + 320 + 192, "density_adj": 
 
 # DRAM traffic and L2 throughput (share of peak) per launch of the dominant
 # kernel, from one ncu capture of this workload; valid only for the kernel
-# source they were taken on (keyed by its hash), null otherwise.
-TRAFFIC = {  # {(region, source_sha of the kernel source): bytes per launch}
-    ("density_adj", "bd83f08f9138"): 65194240,  # mean of the three launches of one step
+# they were taken on (keyed by the hash of its own text), null otherwise.
+TRAFFIC = {  # {(region, kernel_sha): bytes per launch}
+    ("density_adj", "544df997ffdb"): 65207040,  # mean of the three launches of one step
 }
-L2_FRAC = {  # {(region, source_sha): lts__t_sectors throughput as a fraction of peak}
-    ("density_adj", "bd83f08f9138"): 0.347,
+L2_FRAC = {  # {(region, kernel_sha): lts__t_sectors throughput as a fraction of peak}
+    ("density_adj", "544df997ffdb"): 0.341,
 }
 
 
@@ -474,21 +474,22 @@ class ClockSampler:
         }
 
 
-def source_sha(name: str) -> str:
-    """sha1[:12] of a kernel source's code: line comments and blank lines do not count."""
-    path = os.path.join(ROOT, "paper_2505_06711_gb300", "csrc", name)
-    code = []
-    for line in open(path, encoding="utf-8").read().splitlines():
-        line = line.split("//", 1)[0].rstrip()
-        if line:
-            code.append(line)
-    return hashlib.sha1("\n".join(code).encode()).hexdigest()[:12]
+def kernel_sha(kernel: str, source: str) -> str:
+    """sha1[:12] of one kernel's code in a CUDA source: from its template line or ``__global__`` to its closing
+    brace; line comments and blank lines do not count."""
+    code = [line for line in (raw.split("//", 1)[0].rstrip() for raw in source.splitlines()) if line]
+    at = next(k for k, line in enumerate(code) if "__global__" in line and kernel + "(" in line)
+    first = at - 1 if code[at - 1].startswith("template") else at
+    last = next(k for k in range(at, len(code)) if code[k] == "}")
+    return hashlib.sha1("\n".join(code[first : last + 1]).encode()).hexdigest()[:12]
 
 
-REGION_SOURCE = {
-    "density_fwd": "density.cu", "density_adj": "density.cu", "bbar": "density.cu", "mlp_fwd": "mlp_fp32.cu",
-    "mlp_bwd": "mlp_fp32.cu", "nlist_rebuild": "nlist.cu", "live_edges": "density.cu",
-}
+def region_key(region: str):
+    """Key of the counter tables: the region and the hash of its kernel (the tables hold one region)."""
+    if region != "density_adj":
+        return None
+    path = os.path.join(ROOT, "paper_2505_06711_gb300", "csrc", "density.cu")
+    return region, kernel_sha("k_density_adj", open(path, encoding="utf-8").read())
 
 
 def region_flops(region: str, n_atoms: int, n_live: int, T: int, launches: int) -> float | None:
@@ -769,7 +770,7 @@ def run_ours(args):
     if flops is not None and launches > 0:
         launch_s = per_step_ms / launches * 1e-3
         achieved = flops / launches / launch_s / 1e12
-        key = (region, source_sha(REGION_SOURCE.get(region, "density.cu")))
+        key = region_key(region)
         hbm_gbs, hbm_src = measured_peaks()
         coarse = region_flops_coarse(region, n_atoms, n_live, T_LAYERS)
         nbytes = region_bytes(region, n_atoms, n_pairs, T_LAYERS)
@@ -782,7 +783,7 @@ def run_ours(args):
             "frac": achieved / peak_tflops,
             "traffic": TRAFFIC.get(key),
             "peak_source": f"derived: {props.multi_processor_count} SMs x 128 FP32 lanes x 2 FLOP x {max_mhz:.0f} MHz",
-            "flop_count": "per live edge as the kernels' formulas need them (DESIGN section 6)",
+            "flop_count": "per live edge as the kernels' formulas need them",
             "frac_alu_survey": (coarse / launches / launch_s / 1e12 / peak_tflops) if coarse else None,
             "flop_count_survey": "scope table: 130 per live edge forward + 2560 per atom contraction, 260 reverse",
             "achieved_hbm_gbs": (nbytes / launches / launch_s / 1e9) if nbytes else None,

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/reann.h"
+#include "memory.h"
 
 namespace reann {
 
@@ -323,6 +324,8 @@ struct ListPool {
     int device = 0;
     std::mutex mu;
     std::vector<void*> late;  // blocks still to be given back
+    std::vector<cudaEvent_t> spare;  // events of freed lists, for others' uses
+    FreeMemory free_memory;          // asked by the context's builds
     bool wait_for_device();   // false when the device cannot be synchronised now
     void give_late();
     static std::shared_ptr<ListPool> create();  // null when the device has no memory pools
@@ -435,6 +438,7 @@ struct reann_nlist {
     cudaStream_t alloc_stream = nullptr;
     std::vector<reann::ListUse> uses;  // with list_pool
     bool unknown_use = false;          // used under a caller's capture, or in a way that could not be recorded
+    bool alloc_capturing = false;      // alloc_stream is being captured
 };
 
 struct reann_ctx {

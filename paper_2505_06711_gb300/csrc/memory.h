@@ -20,6 +20,17 @@ inline int64_t edge_rows_within(int64_t rows, uint64_t row_bytes, uint64_t later
     return rows;
 }
 
+// When the free memory is asked for: before records that, with those taken since the last answer, come to a
+// 64th of it (what others take meanwhile is seen at the next answer)
+struct FreeMemory {
+    uint64_t bytes = 0, since = 0;
+    bool ask(uint64_t want) {
+        since += want;
+        return since >= bytes / 64;
+    }
+    void told(uint64_t free_bytes) { bytes = free_bytes, since = 0; }
+};
+
 // Bytes per atom that a list may still take after its build: virials (36 + 9 / 32), host staging
 // (36), MD (12 + 1 / 16), rounded up
 constexpr uint64_t kLaterBytesPerAtom = 96;

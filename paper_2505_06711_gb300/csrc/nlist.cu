@@ -941,7 +941,7 @@ void* nlist_alloc_bytes(reann_nlist* nl, size_t bytes) {
     void* p = nullptr;
     bytes = std::max<size_t>(bytes, 1);
     // (a block taken from the pool under capture would belong to the graph)
-    const bool big = nl->list_pool && (bytes >= ListPool::kBig || capturing(nl->alloc_stream));
+    const bool big = nl->list_pool && (bytes >= ListPool::kBig || nl->alloc_capturing);
     auto take = [&] {
         return nl->mem_pool && !big ? cudaMallocFromPoolAsync(&p, bytes, nl->mem_pool, nl->alloc_stream) : cudaMalloc(&p, bytes);
     };

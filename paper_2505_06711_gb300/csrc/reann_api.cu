@@ -17,7 +17,6 @@
 #include <vector>
 
 #include "common.cuh"
-#include "memory.h"
 
 using namespace reann;
 
@@ -89,6 +88,7 @@ bool reann::capturing(cudaStream_t s) {
 reann::ListPool::~ListPool() {
     give_late();
     if (stream) cudaStreamSynchronize(stream);
+    for (cudaEvent_t e : spare) cudaEventDestroy(e);
     if (pool) cudaMemPoolDestroy(pool);
     if (stream) cudaStreamDestroy(stream);
 }
@@ -176,13 +176,26 @@ bool take_blocks(reann_nlist* nl, std::initializer_list<Block> want, MakeRoom ma
         make_room);
 }
 
+// whether to ask for the free memory before taking so many bytes of records (10 to 40 us among a build's allocations)
+bool records_should_ask(reann_nlist* nl, uint64_t bytes) {
+    ListPool* pool = nl->list_pool.get();
+    if (!pool) return true;
+    std::lock_guard<std::mutex> lock(pool->mu);
+    return pool->free_memory.ask(bytes);
+}
+
 // Edge records (32 B per row entry) of `rows` rows, or of fewer where device memory is short (edge_rows_within;
 // false: not even the fewest)
 bool alloc_edge_records(reann_nlist* nl, int64_t rows) {
     constexpr size_t kEntry = sizeof(float4) + 2 * sizeof(float2);
     size_t free_bytes = 0, total = 0;
-    if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess)
+    if (records_should_ask(nl, (uint64_t)rows * kEntry * nl->stride) && cudaMemGetInfo(&free_bytes, &total) == cudaSuccess) {
+        if (ListPool* pool = nl->list_pool.get()) {
+            std::lock_guard<std::mutex> lock(pool->mu);
+            pool->free_memory.told(free_bytes);
+        }
         rows = edge_rows_within(rows, kEntry * nl->stride, kLaterBytesPerAtom * (uint64_t)nl->n, free_bytes);
+    }
     for (;;) {
         const size_t count = (size_t)rows * nl->stride;
         nl->edge_rows = rows;
@@ -282,7 +295,8 @@ void free_nlist(reann_nlist* nl) {
         bool ordered = !nl->unknown_use;
         for (const ListUse& u : nl->uses) {
             ordered = cudaStreamWaitEvent(pool->stream, u.done, 0) == cudaSuccess && ordered;
-            cudaEventDestroy(u.done);
+            std::lock_guard<std::mutex> lock(pool->mu);
+            pool->spare.push_back(u.done);
         }
         nl->alloc_stream = pool->stream;
         pool->give_late();
@@ -630,18 +644,28 @@ struct UseScope {
     reann_nlist* nl;
     bool over = false;  // the call has waited for its stream
     UseScope(reann_ctx* c, const reann_nlist* l) : ctx(c), nl(const_cast<reann_nlist*>(l)) {
-        if (nl->list_pool) nl->alloc_stream = ctx->stream;
+        if (!nl->list_pool) return;
+        nl->alloc_stream = ctx->stream;
+        nl->alloc_capturing = capturing(ctx->stream);
     }
     ~UseScope() {
         if (!nl->list_pool || over) return;
-        if (!capturing(ctx->stream)) {
+        if (!nl->alloc_capturing) {
             for (const ListUse& u : nl->uses)
                 if (u.ctx == ctx->id) {
                     nl->unknown_use |= cudaEventRecord(u.done, ctx->stream) != cudaSuccess;
                     return;
                 }
             ListUse u{ctx->id, nullptr};
-            if (cudaEventCreateWithFlags(&u.done, cudaEventDisableTiming) == cudaSuccess) {
+            {
+                ListPool& pool = *nl->list_pool;
+                std::lock_guard<std::mutex> lock(pool.mu);
+                if (!pool.spare.empty()) {
+                    u.done = pool.spare.back();
+                    pool.spare.pop_back();
+                }
+            }
+            if (u.done || cudaEventCreateWithFlags(&u.done, cudaEventDisableTiming) == cudaSuccess) {
                 nl->uses.push_back(u);
                 nl->unknown_use |= cudaEventRecord(u.done, ctx->stream) != cudaSuccess;
                 return;

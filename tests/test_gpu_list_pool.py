@@ -332,12 +332,15 @@ def test_edge_records_leave_room():
         pot.close()
     pot = Potential(spec)
     fill = torch.empty(free() - used - (40 << 20), dtype=torch.uint8, device="cuda")
-    sy = pot.system(s.pos, s.species, s.cell)
-    left = free()
-    print(f"[room] used {used >> 20} MiB, left {left >> 20} MiB")
-    assert left >= 100 << 20
-    for k, (x, y) in enumerate(zip(calls(sy), want)):
-        assert np.array_equal(x, y), k
-    sy.close()
-    pot.close()
-    del fill
+    try:
+        sy = pot.system(s.pos, s.species, s.cell)
+        left = free()
+        print(f"[room] used {used >> 20} MiB, left {left >> 20} MiB")
+        assert left >= 100 << 20
+        for k, (x, y) in enumerate(zip(calls(sy), want)):
+            assert np.array_equal(x, y), k
+        sy.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+        pot.close()

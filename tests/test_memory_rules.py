@@ -2,7 +2,8 @@
 
 * a request for several blocks leaves none of them behind when one cannot be had, whichever it is, and
   can be made again;
-* edge records leave a quarter of the free memory, and what the list's later calls take, to everything else.
+* edge records leave a quarter of the free memory, and what the list's later calls take, to everything else; the
+  free memory is asked for again once a 64th of it has been taken.
 """
 
 from __future__ import annotations
@@ -55,6 +56,14 @@ int main() {
                     CHECK(got * row + later <= got_max || got == std::min(rows, kMinEdgeRows));
                     if (got < rows) CHECK(std::min<int64_t>(rows, 2 * got) * row + later + row > got_max);
                 }
+    FreeMemory m;
+    CHECK(m.ask(1));  // nothing known yet
+    m.told(6400);
+    CHECK(!m.ask(60) && m.ask(40));  // a 64th of 6,400 taken since
+    m.told(64);
+    CHECK(m.ask(1));
+    m.told(0);
+    CHECK(m.ask(0));
     std::puts("ok");
     return 0;
 }
