@@ -195,10 +195,18 @@ int reann_ctx_wait_selftest(reann_ctx* ctx, int64_t polls);
  * after wrapping positions into the cell, excluding only the zero-shift self
  * term (periodic self-images are neighbours).  The returned handle also holds
  * the structure's per-layer device buffers, so it stays resident for repeated
- * evaluations.  Synchronous (waits for the stream).
+ * evaluations; the records of its edges (32 B per row entry) leave a quarter of
+ * the free device memory, and are kept for fewer rows where they would not
+ * (slower, with the same results).  Synchronous (waits for the stream).
  * Errors: REANN_E_ARG (N < 1, species out of range), REANN_E_MISMATCH,
  * REANN_E_GEOM (non-finite position, coincident atoms, singular cell),
  * REANN_E_NOMEM, REANN_E_CUDA.
+ * The handle may be used with other contexts, one call at a time, and outlives
+ * the one that built it.  Calls on another context return REANN_E_MISMATCH where
+ * its model has more features per atom or lacks an element of the atoms.
+ * reann_nlist_free gives the memory back behind the handle's last calls, without
+ * waiting for them on the host; a handle captured into a graph of the caller's
+ * is freed after a device synchronisation, and its graph must not run again.
  */
 int reann_build_nlist(reann_ctx* ctx, int64_t n_atoms, const double* pos, const int32_t* species, const double* cell,
                       double r_c, double skin, reann_nlist** out);
