@@ -358,9 +358,9 @@ int reann_energy_forces_host(reann_ctx* ctx, reann_nlist* nl, const double* pos,
  *                       rows), so its cost follows the work, not the pool's
  *                       size.  Every class is captured as a CUDA graph on the
  *                       first launch (per precision and output pointers, and
- *                       again for the first structure of more than 16,384
- *                       atoms; that launch itself runs directly) and replayed
- *                       afterwards;
+ *                       again for the first structure of more than 4,096,
+ *                       8,192 and 16,384 atoms; those launches themselves run
+ *                       directly) and replayed afterwards;
  *                       submissions take the lowest free ranges, which keeps
  *                       the classes small.  Asynchronous: the
  *                       context stream waits for it.  A slot is evaluated

@@ -210,6 +210,9 @@ struct CellGeom {
     float margin;    // FP32 pre-test band around rcut2 (A^2) decided in FP64
 };
 
+// Lanes per atom of the forward edge pass, and with them the order of its sums, by the atoms of the structure
+// (launch_density_fwd has the times behind the lines).
+__host__ __device__ constexpr int fwd_lanes(int64_t atoms) { return atoms <= 4096 ? 16 : (atoms <= 8192 ? 8 : 4); }
 // Classes of edges that a row's reverse sums are taken in, by the atoms of its structure (launch_density_adj
 // has the times behind the lines).
 __host__ __device__ constexpr int adj_classes(int64_t atoms) { return atoms <= 16384 ? 4 : (atoms <= 28672 ? 2 : 1); }
@@ -352,10 +355,10 @@ struct reann_nlist {
     // [0, tiles128_active) of the tile lists.
     int64_t n_rows = -1, g_rows = -1;
     int64_t tiles_active = -1, tiles128_active = -1;
-    // a serving pool's: the atoms of each owned row's structure, and the reverse edge passes that the
-    // launched structures need (bits 4, 2, 1: sums in that many classes)
+    // a serving pool's: the atoms of each owned row's structure, and the edge passes that the launched
+    // structures need (forward: bits 16, 8, 4, the lanes; reverse: bits 4, 2, 1, the classes of the sums)
     int32_t* structure = nullptr;
-    int adj_passes = 0;
+    int fwd_passes = 0, adj_passes = 0;
     int stride = 0;                   // neighbour row capacity
     int max_count = 0;                // longest row found by the first build
     int n_elem = 0, T = 0;

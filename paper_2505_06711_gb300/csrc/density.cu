@@ -22,8 +22,8 @@
 // stream the records of their atom (coalesced) and gather only what belongs to
 // the neighbour: its coefficients (forward) or its adjoint record (reverse).
 // Both passes give 4 to 32 lanes to a centre atom, more where there are few atoms.
-// The order in which an atom's edges are summed does not depend on that choice nor
-// on how many rows a launch has (see the passes).
+// The order in which an atom's edges are summed follows the size of its structure
+// and never how many rows a launch has (see the passes).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -221,20 +221,16 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
 }
 
 // ------------------------------------------------------------- forward ---
-// LPA lanes per centre atom (32 / LPA atoms per warp).  A row's edges fall into four
-// classes, e mod 4; a class's 80 sums of t_m A_a, t_m = c_{j,m} phi_m, are taken edge after
-// edge, and the classes' are added as (0 + 2) + (1 + 3): the result does not depend on LPA,
-// so that a structure's is the same alone and among others, whose number decides it.
-//   LPA = 4: lane q walks class q and keeps its 80 sums in registers; the record two
-// edges ahead and the coefficients one edge ahead are in flight meanwhile.
-//   LPA = 8, 16: lane (h, q) keeps the 80 / (LPA / 4) sums of channels CH h .. CH h + CH - 1 of
-// class q.  Per batch of LPA edges each lane first forms one edge's t_m into shared memory;
-// the records and coefficients of two or four batches are gathered together (192 atoms, 16 lanes: 6.8 us
-// with one batch's, 6.0 with four).
-// A butterfly reduce-scatter over the four classes leaves 80 / LPA of the sums in each lane
+// LPA lanes per centre atom (32 / LPA atoms per warp), by the atoms of its structure (fwd_lanes), never
+// by how many rows a launch has: the lanes decide the order in which a row's edges are summed, and a
+// structure's results are the same alone and among others.  Lane q walks the edges
+// q, q + LPA, ... of its atom and accumulates the 80 products t_m A_a,
+// t_m = c_{j,m} phi_m, in registers; the record two edges ahead and the
+// coefficients one edge ahead are in flight meanwhile.  A butterfly
+// reduce-scatter over the LPA lanes leaves 80 / LPA of the sums in each lane
 // (stored as the b checkpoint), and lane q contracts its 16 / LPA orbitals.
 // Bound by the latency of the record stream and the coefficient gathers at 16
-// warps per SM (LPA = 4: 126 registers, 80 of them sums; issue slots 55 % busy).  Reading
+// warps per SM (126 registers, 80 of them sums; issue slots 55 % busy).  Reading
 // records instead of recomputing the edge's geometry took a launch from 29.7 to
 // 19.9 us (24,576 atoms) and from 692 to 541 us (1,048,576 atoms).  Eight lanes per
 // edge with the sums of one channel each (48 registers, 37 warps) were slower, 39
@@ -244,7 +240,6 @@ __global__ void __launch_bounds__(kEdgeWarps * 32) k_edges(int64_t row0, int64_t
 // k <= k' over 8 orbitals (108 features).
 constexpr int kFwdWarps = 4;
 constexpr int kBStride = 84;  // padded b row of an atom in shared memory (16 B aligned)
-constexpr int kEdgeLd = 12;   // a staged edge's t_0..7, x, y, z (stride 12: no bank conflicts in the stores)
 
 // one butterfly stage over CNT values: lanes with bit O set keep the upper half
 template <int CNT, int O>
@@ -258,17 +253,18 @@ __device__ __forceinline__ void rs_half(float* v, int q) {
     }
 }
 
-template <bool PAIRS, int LPA>
+// POOL: the rows are a serving pool's (structure: the atoms of each row's structure).
+template <bool PAIRS, int LPA, bool POOL>
 __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0, int64_t rows, int stride, Radial R,
                                                             const int32_t* __restrict__ live_cnt,
                                                             const float4* __restrict__ xyzj,
                                                             const float2* __restrict__ phi,
                                                             const float* __restrict__ coef,
                                                             const float* __restrict__ Wt, float* __restrict__ rho,
-                                                            float* __restrict__ bck, bool far) {
+                                                            float* __restrict__ bck, bool far,
+                                                            const int32_t* __restrict__ structure) {
     constexpr int KO = PAIRS ? NORB_P : NORB, APW = 32 / LPA;
-    static_assert(LPA == 4 || LPA == 8 || LPA == 16, "four classes of edges, 80 sums split evenly");
-    constexpr int CH = NPHI / (LPA / 4), NS = NANG * CH;  // channels and sums per lane
+    static_assert(LPA == 4 || LPA == 8 || LPA == 16, "80 sums split evenly");
     __shared__ __align__(16) float sW[(LMAX + 1) * NPHI * KO];
     __shared__ __align__(16) float sB[kFwdWarps * APW][kBStride];
     for (int i = threadIdx.x; i < (LMAX + 1) * NPHI * KO; i += blockDim.x) sW[i] = Wt[i];
@@ -276,119 +272,64 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 4) k_density_fwd(int64_t row0,
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & (LPA - 1), slot = lane / LPA;
     const int64_t kr = ((int64_t)blockIdx.x * kFwdWarps + warp) * APW + slot;
-    const bool valid = kr < rows;
     const int64_t atom = row0 + kr;
-    const int cnt = valid ? live_cnt[atom] : 0;
-    const float4* ex = xyzj + (size_t)kr * stride;
-    const float2* ep = phi + (size_t)kr * stride;
-    float acc[NS];
+    // (of a serving pool's rows only those whose structure takes this many lanes)
+    const bool valid = kr < rows && (!POOL || fwd_lanes(structure[atom]) == LPA);
+    float acc[NB];
 #pragma unroll
-    for (int v = 0; v < NS; ++v) acc[v] = 0.f;
-    // the row's records start on their way to L2 at once (large systems stream them from HBM)
-    if (far) {
-        for (int e = 8 * q; e < cnt; e += 8 * LPA) prefetch_l2(ex + e);
-        for (int e = 16 * q; e < cnt; e += 16 * LPA) prefetch_l2(ep + e);
-    }
-    auto terms = [&](const float2& p, const float4& c0, const float4& c1, float t[NPHI]) {
-        float ph[NPHI];
-        phi_chain(R, p.x, p.y, ph);
-        t[0] = c0.x * ph[0], t[1] = c0.y * ph[1], t[2] = c0.z * ph[2], t[3] = c0.w * ph[3];
-        t[4] = c1.x * ph[4], t[5] = c1.y * ph[5], t[6] = c1.z * ph[6], t[7] = c1.w * ph[7];
-    };
-    auto add = [&](float x, float y, float z, const float* t) {
-        const float A[NANG] = {1.f, x, y, z, x * x, y * y, z * z, x * y, x * z, y * z};
-#pragma unroll
-        for (int a = 0; a < NANG; ++a)
-#pragma unroll
-            for (int m = 0; m < CH; ++m) acc[a * CH + m] = fmaf(t[m], A[a], acc[a * CH + m]);
-    };
-    auto coefs = [&](const float4& e, float4& c0, float4& c1) { ldg8(coef + (size_t)__float_as_int(e.w) * NPHI, c0, c1); };
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    if constexpr (LPA == 4) {
-        float4 e1 = zero, c0 = zero, c1 = zero, e2 = zero;
-        float2 p1 = make_float2(0.f, 0.f), p2 = p1;
-        if (q < cnt) {
-            e1 = ex[q], p1 = ep[q];
-            coefs(e1, c0, c1);
+    for (int v = 0; v < NB; ++v) acc[v] = 0.f;
+    if (valid) {
+        const int cnt = live_cnt[atom];
+        const float4* ex = xyzj + (size_t)kr * stride;
+        const float2* ep = phi + (size_t)kr * stride;
+        // the row's records start on their way to L2 at once (large systems stream them from HBM)
+        if (far) {
+            for (int e = 8 * q; e < cnt; e += 8 * LPA) prefetch_l2(ex + e);
+            for (int e = 16 * q; e < cnt; e += 16 * LPA) prefetch_l2(ep + e);
         }
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 e1 = zero, c0 = zero, c1 = zero;
+        float2 p1 = make_float2(0.f, 0.f);
+        if (q < cnt) {
+            e1 = ex[q];
+            p1 = ep[q];
+            ldg8(coef + (size_t)__float_as_int(e1.w) * NPHI, c0, c1);
+        }
+        float4 e2 = zero;
+        float2 p2 = make_float2(0.f, 0.f);
         if (q + LPA < cnt) e2 = ex[q + LPA], p2 = ep[q + LPA];
         for (int e = q; e < cnt; e += LPA) {
             const float x = e1.x, y = e1.y, z = e1.z;
-            float t[NPHI];
-            terms(p1, c0, c1, t);
-            e1 = e2, p1 = p2;
-            if (e + LPA < cnt) coefs(e2, c0, c1);
+            float ph[NPHI];
+            phi_chain(R, p1.x, p1.y, ph);
+            const float t[NPHI] = {c0.x * ph[0], c0.y * ph[1], c0.z * ph[2], c0.w * ph[3],
+                                   c1.x * ph[4], c1.y * ph[5], c1.z * ph[6], c1.w * ph[7]};
+            e1 = e2;
+            p1 = p2;
+            if (e + LPA < cnt) ldg8(coef + (size_t)__float_as_int(e2.w) * NPHI, c0, c1);
             if (e + 2 * LPA < cnt) e2 = ex[e + 2 * LPA], p2 = ep[e + 2 * LPA];
-            add(x, y, z, t);
-        }
-    } else {
-        // batches of LPA edges of each of the warp's atoms, a lane one edge of each; the loads of kAhead batches at a time
-        constexpr int kAhead = LPA == 16 ? 4 : 2;
-        __shared__ __align__(16) float sT[kFwdWarps][32 * kEdgeLd];
-        const int c = q & 3, h = q >> 2;
-        int cmax = cnt;  // longest row of the warp's atoms
+            const float A[NANG] = {1.f, x, y, z, x * x, y * y, z * z, x * y, x * z, y * z};
 #pragma unroll
-        for (int o = LPA; o < 32; o <<= 1) cmax = max(cmax, __shfl_xor_sync(FULL, cmax, o));
-        float4 e[kAhead] = {};
-        float2 p[kAhead] = {};
-        auto records = [&](int e0) {
+            for (int a = 0; a < NANG; ++a)
 #pragma unroll
-            for (int u = 0; u < kAhead; ++u)
-                if (e0 + u * LPA + q < cnt) e[u] = ex[e0 + u * LPA + q], p[u] = ep[e0 + u * LPA + q];
-        };
-        records(0);
-#pragma unroll 1
-        for (int e0 = 0; e0 < cmax; e0 += kAhead * LPA) {
-            float4 c0[kAhead] = {}, c1[kAhead] = {};
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u)
-                if (e0 + u * LPA + q < cnt) coefs(e[u], c0[u], c1[u]);
-            float t[kAhead][NPHI];
-            float4 r[kAhead];
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                r[u] = make_float4(e[u].x, e[u].y, e[u].z, 0.f);
-                terms(p[u], c0[u], c1[u], t[u]);
-            }
-            records(e0 + kAhead * LPA);
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                if (e0 + u * LPA >= cmax) break;
-                const bool in = e0 + u * LPA + q < cnt;  // past the row's end: an edge that adds zeros
-                float* d = sT[warp] + lane * kEdgeLd;
-                *reinterpret_cast<float4*>(d) = in ? make_float4(t[u][0], t[u][1], t[u][2], t[u][3]) : zero;
-                *reinterpret_cast<float4*>(d + 4) = in ? make_float4(t[u][4], t[u][5], t[u][6], t[u][7]) : zero;
-                *reinterpret_cast<float4*>(d + 8) = in ? r[u] : zero;
-                __syncwarp();
-                const float* st = sT[warp] + slot * LPA * kEdgeLd;
-#pragma unroll
-                for (int k = 0; k < LPA / 4; ++k) {
-                    const float* x = st + (4 * k + c) * kEdgeLd;
-                    const float4 xyz = ld4(x + 8);
-                    float tm[CH];
-                    ldk<CH>(x + CH * h, tm);
-                    add(xyz.x, xyz.y, xyz.z, tm);
-                }
-                __syncwarp();
-            }
+                for (int m = 0; m < NPHI; ++m) acc[a * NPHI + m] = fmaf(t[m], A[a], acc[a * NPHI + m]);
         }
     }
-    // reduce-scatter over the classes: lane (h, c) keeps the sums NL c .. NL c + NL - 1 of its NS
+    // reduce-scatter: lane q keeps b[80 / LPA * rev(q) ..), rev the order the halves were taken in
     constexpr int NL = NB / LPA;
-    rs_half<NS, 2>(acc, q);
-    rs_half<NS / 2, 1>(acc, q);
+    if constexpr (LPA == 16) rs_half<NB, 8>(acc, q);
+    if constexpr (LPA >= 8) rs_half<(LPA == 16 ? NB / 2 : NB), 4>(acc, q);
+    rs_half<NL * 4, 2>(acc, q);
+    rs_half<NL * 2, 1>(acc, q);
     float* sb = sB[warp * APW + slot];
 #pragma unroll
     for (int v = 0; v < NL; ++v) acc[v] *= R.unscale;
-    if constexpr (LPA == 4) {
+    if constexpr (LPA == 16) {
 #pragma unroll
-        for (int v = 0; v < NL; v += 2) *reinterpret_cast<float2*>(sb + NL * q + v) = make_float2(acc[v], acc[v + 1]);
+        for (int v = 0; v < NL; ++v) sb[NL * q + v] = acc[v];
     } else {
 #pragma unroll
-        for (int v = 0; v < NL; ++v) {
-            const int f = NL * (q & 3) + v;  // sum (a, m) of the lane at f = CH a + m
-            sb[f / CH * NPHI + CH * (q >> 2) + f % CH] = acc[v];
-        }
+        for (int v = 0; v < NL; v += 2) *reinterpret_cast<float2*>(sb + NL * q + v) = make_float2(acc[v], acc[v + 1]);
     }
     __syncwarp();
     if (valid)
@@ -983,33 +924,33 @@ cudaError_t launch_edges(cudaStream_t s, const reann_nlist* nl, const Radial& r,
 cudaError_t launch_density_fwd(cudaStream_t s, const reann_nlist* nl, const Radial& r, int64_t row0, int64_t rows,
                                const float* W, const float* coef, float* rho, float* bck, bool pairs) {
     if (rows == 0) return cudaSuccess;
-    // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer stage
-    // nothing (many).  us per launch within an evaluation with 16 / 8 / 4 lanes: 192 atoms 6.0 / 7.8 /
-    // 10.2, 4,000 9.1 / 10.7 / 11.9, 6,912 8.4 / 6.8 / 7.8, 10,976 10.5 / 12.4 / 8.8, 24,576 25 / 23 /
-    // 19.5, 1,048,576 859 / 757 / 537.
+    // Lanes per atom: more lanes shorten an atom's chain of edges (few atoms: latency), fewer need
+    // less reduction work per atom (many).  us per launch with 16 / 8 / 4 lanes: 192 atoms 4.5 / 5.6 /
+    // 7.9, 4,000 5.5 / 5.8 / 7.1, 10,976 11.8 / 10.8 / 9.1, 24,576 25 / 20 / 20, 1,048,576 914 / 670 / 536.
     const EvalLaunch how = eval_launch(nl);
-    const int lpa = rows <= 4096 ? 16 : (rows <= 8192 ? 8 : 4);
     // records of more rows than this outgrow L2 between the passes: prefetch each atom's when it
     // starts (1,048,576 atoms: 580 -> 541 us; 24,576 atoms: 19.9 -> 20.2 us, so not there)
     const bool far = rows > (int64_t)1 << 16;
-#define REANN_FWD(P, L)                                                                                              \
-    launch_with(how.chain, how.carve(), k_density_fwd<P, L>, blocks_for(rows, kFwdWarps * (32 / L)), kFwdWarps * 32, 0, s, \
-                row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, coef, W, rho, bck, far)
-    if (pairs) {
-        if (lpa == 16)
-            REANN_FWD(true, 16);
-        else if (lpa == 8)
-            REANN_FWD(true, 8);
-        else
-            REANN_FWD(true, 4);
-    } else {
-        if (lpa == 16)
-            REANN_FWD(false, 16);
-        else if (lpa == 8)
-            REANN_FWD(false, 8);
-        else
-            REANN_FWD(false, 4);
-    }
+#define REANN_FWD(P, L, POOL)                                                                                        \
+    launch_with(how.chain, how.carve(), k_density_fwd<P, L, POOL>, blocks_for(rows, kFwdWarps * (32 / L)), kFwdWarps * 32, 0, s, \
+                row0, rows, nl->stride, r, nl->live_cnt, nl->edge_xyzj, nl->edge_phi, coef, W, rho, bck, far, nl->structure)
+#define REANN_FWD_P(L)                      \
+    do {                                    \
+        if (pairs && nl->structure)         \
+            REANN_FWD(true, L, true);       \
+        else if (pairs)                     \
+            REANN_FWD(true, L, false);      \
+        else if (nl->structure)             \
+            REANN_FWD(false, L, true);      \
+        else                                \
+            REANN_FWD(false, L, false);     \
+    } while (0)
+    // a serving pool's rows belong to structures of their own: a launch for each number of lanes they take
+    const int lanes = nl->structure ? nl->fwd_passes : fwd_lanes(nl->n);
+    if (lanes & 16) REANN_FWD_P(16);
+    if (lanes & 8) REANN_FWD_P(8);
+    if (lanes & 4) REANN_FWD_P(4);
+#undef REANN_FWD_P
 #undef REANN_FWD
     return cudaGetLastError();
 }

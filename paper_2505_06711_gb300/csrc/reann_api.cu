@@ -1632,6 +1632,10 @@ struct ServeSlot {
 
 }  // namespace
 
+static_assert(fwd_lanes(4096) == 16 && fwd_lanes(8192) == 8 && fwd_lanes(8193) == 4 && adj_classes(16384) == 4 &&
+                  adj_classes(16385) == 2 && adj_classes(28673) == 1,
+              "reann_serve::kPasses follows them");
+
 struct reann_serve {
     std::mutex mu;  // slots, ranges, staging and the pool stream; builds run outside it
     reann_ctx* ctx = nullptr;
@@ -1647,11 +1651,17 @@ struct reann_serve {
     cudaEvent_t staged = nullptr, done = nullptr, user_ready = nullptr;
     std::vector<std::pair<reann_nlist*, cudaEvent_t>> deferred;  // built lists freed once their pack has run
     // one captured pass per size class k: owned rows [0, n >> k), ghost slots [0, g_cap >> k);
-    // [0] for launches whose structures all take one reverse edge pass (adj_classes 4), [1] for the others
+    // [v] for launches whose largest structure takes the edge passes of kPasses[v]
     static constexpr int kClasses = 8;
     static constexpr int64_t kMinRows = 2048;
-    cudaGraph_t graph[2][kClasses] = {};
-    cudaGraphExec_t exec[2][kClasses] = {};
+    struct Passes {
+        int64_t atoms;  // of the largest structure, at most
+        int fwd, adj;   // reann_nlist::fwd_passes, adj_passes
+    };
+    static constexpr Passes kPasses[] = {{4096, 16, 4}, {8192, 16 | 8, 4}, {16384, 16 | 8 | 4, 4}, {INT64_MAX, 16 | 8 | 4, 4 | 2 | 1}};
+    static constexpr int kVariants = sizeof(kPasses) / sizeof(kPasses[0]);
+    cudaGraph_t graph[kVariants][kClasses] = {};
+    cudaGraphExec_t exec[kVariants][kClasses] = {};
     int graph_precision = -1;
     const void* graph_out[2] = {nullptr, nullptr};
 };
@@ -1674,7 +1684,7 @@ void serve_reap(reann_serve* srv, bool wait) {
 }
 
 void drop_serve_graphs(reann_serve* srv) {
-    for (int w = 0; w < 2; ++w)
+    for (int w = 0; w < reann_serve::kVariants; ++w)
         for (int k = 0; k < reann_serve::kClasses; ++k) {
             if (srv->exec[w][k]) cudaGraphExecDestroy(srv->exec[w][k]);
             if (srv->graph[w][k]) cudaGraphDestroy(srv->graph[w][k]);
@@ -1869,13 +1879,13 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
     size_t n64 = 0, n128 = 0;
     int nseg = 0;
     int64_t hi = 0, ghi = 0;  // owned rows and ghost slots the launched structures occupy
-    int passes = 0;           // the reverse edge passes they take
+    int64_t largest = 0;      // atoms of the largest one
     for (int k = 0; k < srv->max_slots; ++k) {
         ServeSlot& sl = srv->slots[k];
         if (!sl.used || !sl.pending) continue;
         hi = std::max<int64_t>(hi, sl.ob + sl.n);
         ghi = std::max<int64_t>(ghi, sl.gb + sl.g);
-        passes |= adj_classes(sl.n);
+        largest = std::max(largest, sl.n);
         for (const Tile& t : sl.t64) srv->h_t64[n64++] = t;
         for (const Tile& t : sl.t128) srv->h_t128[n128++] = t;
         srv->h_seg[nseg] = make_int4((int)sl.ob, (int)sl.n, k, 0);
@@ -1900,10 +1910,12 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
     // One evaluation of the pool, sized to the work: size class k covers owned rows
     // [0, n >> k) and ghost slots [0, g_cap >> k), the smallest class holding every
     // launched structure (free and retired rows inside it have no neighbours).  Each
-    // class is captured once per (precision, outputs) and replayed; again with the other
-    // reverse edge passes once a structure needs them.
-    const int wide = passes == 4 ? 0 : 1;
-    p->adj_passes = wide ? 7 : 4;
+    // class is captured once per (precision, outputs) and replayed; again with the edge
+    // passes of larger structures when there is one.
+    int v = 0;
+    while (largest > reann_serve::kPasses[v].atoms) ++v;
+    p->fwd_passes = reann_serve::kPasses[v].fwd;
+    p->adj_passes = reann_serve::kPasses[v].adj;
     int cls = 0, ncls = 1;
     while (ncls < reann_serve::kClasses && (p->n >> ncls) >= reann_serve::kMinRows) ++ncls;
     while (cls + 1 < ncls && (p->n >> (cls + 1)) >= hi && (p->g_cap >> (cls + 1)) >= ghi) ++cls;
@@ -1928,12 +1940,12 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
         srv->graph_out[0] = energies;
         srv->graph_out[1] = forces;
     }
-    if (!srv->exec[wide][cls]) {
+    if (!srv->exec[v][cls]) {
         // this launch runs directly (which also sets kernel attributes outside capture);
         // then every size class is captured, so that no later launch pays for a capture
         rc = pool_pass(ctx, srv, energies, forces);
         for (int k = 0; k < ncls && !rc; ++k) {
-            if (srv->exec[wide][k]) continue;
+            if (srv->exec[v][k]) continue;
             set_class(k);
             if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
                 rc = set_error(ctx, REANN_E_CUDA, "serving graph capture failed");
@@ -1942,15 +1954,15 @@ extern "C" int reann_serve_launch(reann_serve* srv, double* energies, float* for
             rc = pool_pass(ctx, srv, energies, forces);
             cudaGraph_t g = nullptr;
             const cudaError_t ec = cudaStreamEndCapture(s, &g);
-            if (!rc && ec == cudaSuccess && cudaGraphInstantiate(&srv->exec[wide][k], g, 0) == cudaSuccess) {
-                srv->graph[wide][k] = g;
+            if (!rc && ec == cudaSuccess && cudaGraphInstantiate(&srv->exec[v][k], g, 0) == cudaSuccess) {
+                srv->graph[v][k] = g;
             } else {
                 if (g) cudaGraphDestroy(g);
-                srv->exec[wide][k] = nullptr;
+                srv->exec[v][k] = nullptr;
                 if (!rc) rc = set_error(ctx, REANN_E_CUDA, "serving graph capture failed");
             }
         }
-    } else if (cudaGraphLaunch(srv->exec[wide][cls], s) != cudaSuccess) {
+    } else if (cudaGraphLaunch(srv->exec[v][cls], s) != cudaSuccess) {
         rc = set_error(ctx, REANN_E_CUDA, "serving graph launch failed");
     }
     p->n_rows = p->g_rows = p->tiles_active = p->tiles128_active = -1;

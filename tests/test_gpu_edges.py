@@ -110,9 +110,9 @@ def test_records_of_a_part_of_the_rows(virial):
 
 @pytest.mark.parametrize("virial,precision", [(False, 0), (True, 0), (False, 3)])
 @pytest.mark.parametrize("molecules,rows", [(1400, 3000), (2800, 4096), (5600, 9000), (9600, 20000), (9600, 700)])
-def test_sums_do_not_depend_on_the_lanes_per_atom(molecules, rows, virial, precision):
-    # the run's rows decide the lanes per atom (forward 16, 8, 4 up to 4,096, 8,192, beyond; reverse 32, 16,
-    # 8 up to 16,384, 28,672, beyond), on the other side of a line than the whole list's here
+def test_sums_do_not_depend_on_the_run(molecules, rows, virial, precision):
+    # the order of a row's sums follows the list's atoms (forward 16, 8, 4 lanes up to 4,096, 8,192, beyond;
+    # reverse 32, 16, 8 up to 16,384, 28,672, beyond), not the run's rows, which here lie across a line
     s = water_box(molecules, seed=9)
     _assert_same(_evaluated(s, 2, rows, virial, precision), _evaluated(s, 2, 1 << 40, virial, precision))
 
